@@ -3,52 +3,61 @@
 // renormalised (Section 3.4).  It produces exmoe_moe_forward's `topk_ids` / `topk_weights` on the device, so a
 // whole stack step can be captured in one CUDA graph without host-side routing.
 //
-// One CTA per token.  The router matrix (E x H BF16, 256 KB for OLMoE) is shared by all tokens and stays in L2;
-// the token's hidden row is staged in shared memory once; warp w computes the logits of experts w, w+8, ...
-// with 128-bit loads, binary32 accumulation in a fixed order (lane-strided partial sums, then a shuffle tree).
-// Warp 0 then does the softmax (expf, binary32) and k rounds of a warp-wide arg-max whose comparison orders
-// equal probabilities by ascending id.  Latency-bound and small next to the expert GEMMs.
+// What bounds it: at decode sizes latency, at prefill sizes the binary32 FMA pipe and the L2 reads of the router
+// matrix (E x H BF16, 256 KB for OLMoE).  So the experts of a group of tokens are spread over a CLUSTER of CTAs: with
+// eight CTAs of eight warps and 64 experts every warp owns one expert, its whole 4 KB row in flight at once, instead
+// of one SM pulling the 256 KB by itself (one CTA per token took 13.8 us at T = 1, weights cold, and 190 us at
+// T = 8192, where every token re-read the matrix from L2).  From a few dozen tokens on a cluster takes several tokens
+// per read of the matrix.  The arithmetic of a logit is the same in both forms, bit for bit (lane-strided chunks of
+// eight products in ascending order, then a shuffle tree).  Above that the logits are a GEMM and run on the tensor
+// cores (route_mma_kernel), with every decision that their rounding could turn repeated in that same arithmetic, so
+// the choice of experts does not depend on the batch size.
+// The logits travel through the cluster's shared memory to the CTA that owns the token; one of its warps does the
+// softmax (expf, binary32) and k rounds of a warp-wide arg-max that orders equal probabilities by ascending id.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
+#include "frag.cuh"
 
 namespace exmoe {
 
 namespace {
 
-constexpr int kRouteThreads = 256;
+namespace cg = cooperative_groups;
 
-__device__ __forceinline__ float dot8(const uint4& a, const uint4& b) {
-    const uint32_t x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.x, b.y, b.z, b.w};
-    float s = 0.f;
+constexpr int kRouteThreads = 256;
+constexpr int kRouteSmemMax = 200 * 1024;
+// Measured crossings (64 experts, d_model 2048, weights cold, launch included), us for the forms in this order:
+//   T = 32: 10.2 / 10.2 / - / -      64: 12.3 / 12.3 / 15.1 / -      256: 22.5 / 17.3 / 16.4 / 24.6
+//   1024: 61 / 39 / 18.5 / 24.6      2048: 115 / 68 / 24.6 / 24.6    4096: 219 / 125 / 37 / 28.7    8192: 430 / 240 / 63 / 47
+constexpr int kRouteFewTokens = 48;       // four tokens per cluster from here on
+constexpr int kRouteMmaTokens = 224;      // tensor cores from here on
+constexpr int kRouteWideTokens = 2304;    // ... with 32 instead of 16 tokens per CTA
+constexpr int kRouteWarps = kRouteThreads / 32;
+
+__device__ __forceinline__ void unpack8(const uint4& a, float (&x)[8]) {
+    const uint32_t r[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        s = fmaf(__uint_as_float(x[i] << 16), __uint_as_float(y[i] << 16), s);
-        s = fmaf(__uint_as_float(x[i] & 0xffff0000u), __uint_as_float(y[i] & 0xffff0000u), s);
+        x[2 * i] = __uint_as_float(r[i] << 16);
+        x[2 * i + 1] = __uint_as_float(r[i] & 0xffff0000u);
     }
+}
+__device__ __forceinline__ float dot8(const float (&w)[8], const float (&x)[8]) {
+    float d = 0.f;
+#pragma unroll
+    for (int n = 0; n < 8; ++n) d = fmaf(w[n], x[n], d);
+    return d;
+}
+__device__ __forceinline__ float warp_sum(float s) {
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
     return s;
 }
 
-__global__ void __launch_bounds__(kRouteThreads)
-route_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* __restrict__ w_router,
-             const float* __restrict__ bias, int H, int E, int k, int32_t* __restrict__ ids_out,
-             float* __restrict__ w_out) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    uint4* xs = reinterpret_cast<uint4*>(smem);                       // [H / 8] the token's hidden row
-    float* prob = reinterpret_cast<float*>(smem + (size_t)H * 2);      // [E] logits, then probabilities
-    const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int chunks = H / 8;
-    const uint4* xrow = reinterpret_cast<const uint4*>(hidden + (size_t)t * H);
-    for (int i = tid; i < chunks; i += kRouteThreads) xs[i] = xrow[i];
-    __syncthreads();
-    for (int e = warp; e < E; e += kRouteThreads / 32) {
-        const uint4* wrow = reinterpret_cast<const uint4*>(w_router + (size_t)e * H);
-        float s = 0.f;
-        for (int i = lane; i < chunks; i += 32) s += dot8(wrow[i], xs[i]);
-#pragma unroll
-        for (int m = 16; m >= 1; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
-        if (lane == 0) prob[e] = s + (bias ? bias[e] : 0.f);
-    }
-    __syncthreads();
-    if (warp != 0) return;
+// Softmax over the E logits in `prob` (this CTA's shared memory) and the k largest, by one warp.
+__device__ __forceinline__ void softmax_topk(float* prob, int E, int k, int lane, int32_t* __restrict__ ids_out,
+                                             float* __restrict__ w_out) {
     float mx = -INFINITY;
     for (int e = lane; e < E; e += 32) mx = fmaxf(mx, prob[e]);
 #pragma unroll
@@ -59,37 +68,424 @@ route_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* __re
         prob[e] = v;
         sum += v;
     }
-#pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, m);
+    sum = warp_sum(sum);
     __syncwarp();
     const float inv = 1.f / sum;
+    // Arg-max over the experts not yet taken.  Probabilities are non-negative, so their bit patterns order as they do:
+    // key = bits + 2, 1 for a NaN (chosen last), 0 for a taken expert; equal keys go to the lower id.
     for (int j = 0; j < k; ++j) {
-        // arg-max over the experts not yet taken (taken ones are marked negative); ties to the lower id
-        float best = -1.f;
+        uint32_t best = 0;
         int best_e = 0x7fffffff;
         for (int e = lane; e < E; e += 32) {
             const float v = prob[e];
-            if (v > best) {                                            // ascending e: the first maximum wins
-                best = v;
+            const uint32_t key = v >= 0.f ? __float_as_uint(v) + 2u : v < 0.f ? 0u : 1u;
+            if (key > best) {                                          // ascending e: the first maximum wins
+                best = key;
                 best_e = e;
             }
         }
-#pragma unroll
-        for (int m = 16; m >= 1; m >>= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, best, m);
-            const int oe = __shfl_xor_sync(0xffffffffu, best_e, m);
-            if (ov > best || (ov == best && oe < best_e)) {
-                best = ov;
-                best_e = oe;
-            }
-        }
+        const uint32_t top = __reduce_max_sync(0xffffffffu, best);
+        const int e = __reduce_min_sync(0xffffffffu, best == top ? best_e : 0x7fffffff);
         if (lane == 0) {
-            ids_out[(size_t)t * k + j] = best_e;
-            w_out[(size_t)t * k + j] = best * inv;
-            prob[best_e] = -2.f;
+            ids_out[j] = e;
+            w_out[j] = prob[e] * inv;
+            prob[e] = -2.f;
         }
         __syncwarp();
     }
+}
+
+// CL: CTAs per cluster; TB: tokens per cluster.
+// Shared memory: the cluster's TB hidden rows (every CTA keeps all of them), then the logits of the ceil(TB / CL) tokens
+// this CTA owns (token i belongs to rank i % CL).
+template <int CL, int TB>
+__global__ void __launch_bounds__(kRouteThreads)
+route_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* __restrict__ w_router,
+             const float* __restrict__ bias, int T, int H, int E, int k, int32_t* __restrict__ ids_out,
+             float* __restrict__ w_out) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint4* xs = reinterpret_cast<uint4*>(smem);                            // [TB][H / 8]
+    float* prob = reinterpret_cast<float*>(smem + (size_t)TB * H * 2);     // [ceil(TB / CL)][E]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = blockIdx.x % CL, t0 = (blockIdx.x / CL) * TB;
+    const int n_tok = min(TB, T - t0);
+    const int chunks = H / 8;
+    // A programmatic dependent of whatever precedes it in the stream: nothing is read before that has completed; and the
+    // kernel after it may be placed at once (it waits for this one in the same way).
+    grid_dependency_wait();
+    grid_launch_dependents();
+    constexpr int JB = 8;                                                  // chunks of an expert in flight
+    const int gw = rank * kRouteWarps + warp;
+    uint4 raw[JB];
+    auto fetch = [&](int e, int j0) {
+#pragma unroll
+        for (int j = 0; j < JB; ++j) {
+            const int i = lane + 32 * (j0 + j);
+            raw[j] = make_uint4(0, 0, 0, 0);
+            if (i < chunks && e < E) raw[j] = reinterpret_cast<const uint4*>(w_router + (size_t)e * H)[i];
+        }
+    };
+    fetch(gw, 0);                                                    // in flight while the hidden rows are staged
+    {
+        const uint4* xrow = reinterpret_cast<const uint4*>(hidden + (size_t)t0 * H);
+        for (int i = tid; i < n_tok * chunks; i += kRouteThreads) xs[i] = xrow[i];
+        for (int i = n_tok * chunks + tid; i < TB * chunks; i += kRouteThreads) xs[i] = make_uint4(0, 0, 0, 0);
+    }
+    cg::cluster_group cluster = cg::this_cluster();
+    __syncthreads();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // every CTA runs: its memory may be written
+    const int nj = (chunks + 31) / 32;
+    bool joined = false;
+    for (int e0 = gw; e0 < E; e0 += CL * kRouteWarps) {
+        float acc[TB];
+#pragma unroll
+        for (int t = 0; t < TB; ++t) acc[t] = 0.f;
+        for (int j0 = 0; j0 < nj; j0 += JB) {
+            if (j0 > 0 || e0 != gw) fetch(e0, j0);
+#pragma unroll
+            for (int j = 0; j < JB; ++j) {
+                if (j0 + j >= nj) break;
+                const int i = lane + 32 * (j0 + j);
+                float w[8];
+                unpack8(raw[j], w);
+#pragma unroll
+                for (int t = 0; t < TB; ++t) {
+                    float x[8];
+                    unpack8(i < chunks ? xs[t * chunks + i] : make_uint4(0, 0, 0, 0), x);
+                    acc[t] += dot8(w, x);
+                }
+            }
+        }
+        if (!joined) {                                                     // before the first store into another CTA's memory
+            asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+            joined = true;
+        }
+        const float b = bias ? bias[e0] : 0.f;
+#pragma unroll
+        for (int t = 0; t < TB; ++t) {
+            const float sum = warp_sum(acc[t]);
+            if (lane == 0 && t < n_tok) {
+                float* dst = cluster.map_shared_rank(prob, t % CL);
+                dst[(t / CL) * E + e0] = sum + b;
+            }
+        }
+    }
+    if (!joined) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    cluster.sync();
+    for (int i = warp; i * CL + rank < n_tok; i += kRouteWarps) {
+        const size_t t = t0 + i * CL + rank;
+        softmax_topk(prob + i * E, E, k, lane, ids_out + t * k, w_out + t * k);
+    }
+}
+
+// every form is a programmatic dependent of the kernel before it in the stream (it waits for it before it reads anything)
+template <typename F>
+int launch_dependent(F kern, int ctas, int cluster, size_t smem, const exmoe_shape& s, const __nv_bfloat16* hidden,
+                     const __nv_bfloat16* w, const float* bias, int T, int32_t* ids, float* wts, cudaStream_t st) {
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3((unsigned)ctas);
+    lc.blockDim = dim3(kRouteThreads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    lc.attrs = attr;
+    lc.numAttrs = cluster > 1 ? 2 : 1;
+    if (cudaLaunchKernelEx(&lc, kern, hidden, w, bias, T, s.d_model, s.num_experts, s.top_k, ids, wts) != cudaSuccess) {
+        cudaGetLastError();
+        return EXMOE_ERR_CUDA;
+    }
+    count_launch();
+    return EXMOE_OK;
+}
+
+template <int CL, int TB>
+int launch_route(const exmoe_shape& s, const __nv_bfloat16* hidden, const __nv_bfloat16* w, const float* bias, int T,
+                 int32_t* ids, float* wts, cudaStream_t st) {
+    const size_t smem = (size_t)TB * s.d_model * 2 + (size_t)((TB + CL - 1) / CL) * s.num_experts * 4;
+    static SmemOnce once;
+    if (!allow_smem(route_kernel<CL, TB>, kRouteSmemMax, once)) return EXMOE_ERR_CUDA;
+    return launch_dependent(route_kernel<CL, TB>, (T + TB - 1) / TB * CL, CL, smem, s, hidden, w, bias, T, ids, wts, st);
+}
+
+// ---- many tokens: the logits as a tensor-core GEMM -------------------------------------------------------------
+// A CTA takes TM tokens; its eight warps split K (32-wide steps, round robin) and their partial logits meet in shared
+// memory.  Operands come straight from L2 in 16-byte loads: a lane's eight consecutive k serve two m16n8k16 steps of both
+// operands, the permutation of K inside the step being the same on both sides.  Batches of a few hundred tokens are
+// latency again: a cluster of four CTAs then splits the experts (16 tokens, 16 experts each, four steps of loads in
+// flight per warp); from a few thousand tokens on two CTAs share 32 tokens, half of the experts each, which
+// reads the matrix half as often (one CTA for all 64 experts needs too many registers to share an SM: 55 us at T = 8192).
+// The experts are an integer decision, and the one made by the binary32 form above is kept: where two of a token's k + 1
+// largest logits are closer than the two forms can be apart, those experts' logits are recomputed in the binary32 form
+// and the choice is made on these.  The forms differ by rounding only: at most 1.5e-7 |x| |w| (5e-8 from d_model 2048 on)
+// in 3.1 million logits of random rows of 128 to 4096 values; the bound taken is 2e-6, so that about one token in
+// eighty is looked at again (64 experts, d_model 2048).
+constexpr int kMmaMaxExperts = 128;
+constexpr int kMmaMaxModel = 4096;                    // |x|^2 and |w|^2 are summed in BF16 over H / 64 terms per lane
+constexpr float kRouteBound = 2e-6f;
+
+// Binary32 logits of the experts marked in `again` (bit i of a lane: expert lane + 32 i), by one warp.
+__device__ __noinline__ void logits_again(float* z, unsigned again, const __nv_bfloat16* __restrict__ x,
+                                          const __nv_bfloat16* __restrict__ w_router, const float* __restrict__ bias, int H,
+                                          int lane) {
+    const uint4* xr = reinterpret_cast<const uint4*>(x);
+    for (int i = 0; i < kMmaMaxExperts / 32; ++i)
+        for (unsigned todo = __ballot_sync(0xffffffffu, (again >> i) & 1u); todo; todo &= todo - 1) {
+            const int e = 32 * i + __ffs(todo) - 1;
+            const uint4* wr = reinterpret_cast<const uint4*>(w_router + (size_t)e * H);
+            float s = 0.f;
+            for (int j0 = 0; j0 < H / 8; j0 += 256) {
+                uint4 wv[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (j0 + 32 * j + lane < H / 8) wv[j] = wr[j0 + 32 * j + lane];
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (j0 + 32 * j + lane < H / 8) {
+                        float wf[8], xf[8];
+                        unpack8(wv[j], wf);
+                        unpack8(xr[j0 + 32 * j + lane], xf);
+                        s += dot8(wf, xf);
+                    }
+            }
+            s = warp_sum(s);
+            if (lane == 0) z[e] = s + (bias ? bias[e] : 0.f);
+        }
+    __syncwarp();
+}
+// One token's choice from its tensor-core logits, by one warp: the k + 1 largest in order; where two of them are within
+// `slack`, both are recomputed (at the cut everything that could displace the k-th) and the choice is made again.  A lane
+// holds the logits of experts lane, lane + 32, ... as order-preserving integers.
+__device__ __forceinline__ void choose(float* z, float slack, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ w_router,
+                                       const float* __restrict__ bias, int H, int E, int k, int lane, int32_t* __restrict__ ids,
+                                       float* __restrict__ wts) {
+    constexpr int PER = kMmaMaxExperts / 32;
+    uint32_t key[PER];                                                     // 0: no expert, or taken
+    bool odd = !(slack < INFINITY);
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int e = lane + 32 * i;
+        key[i] = 0;
+        if (e < E) {
+            const float v = z[e];
+            odd |= !(fabsf(v) < INFINITY);
+            const uint32_t b = __float_as_uint(v);
+            key[i] = b & 0x80000000u ? ~b : b | 0x80000000u;
+        }
+    }
+    odd = __any_sync(0xffffffffu, odd);
+    unsigned again = odd ? ~0u : 0u;
+    float prev = INFINITY;
+    int prev_e = 0, mine = 0;                                              // mine, lane j: the j-th choice (k <= 32)
+    for (int j = 0; j <= k && j < E && !odd; ++j) {
+        uint32_t best = 0;
+        int be = 0x7fffffff;
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (key[i] > best) {
+                best = key[i];
+                be = lane + 32 * i;
+            }
+        const uint32_t top = __reduce_max_sync(0xffffffffu, best);
+        const int e = __reduce_min_sync(0xffffffffu, best == top ? be : 0x7fffffff);
+        const float v = __uint_as_float(top & 0x80000000u ? top & 0x7fffffffu : ~top);
+        const float near = slack + 2.4e-7f * (fabsf(prev) + fabsf(v));
+        if (j > 0 && prev - v <= near) {
+            if (lane == (prev_e & 31)) again |= 1u << (prev_e >> 5);
+            if (lane == (e & 31)) again |= 1u << (e >> 5);
+            if (j == k)                                                    // the rest of the k-th's neighbourhood
+#pragma unroll
+                for (int i = 0; i < PER; ++i)
+                    if (key[i] && z[lane + 32 * i] >= prev - near) again |= 1u << i;
+        }
+        if (j == lane && j < k) mine = e;
+        prev = v;
+        prev_e = e;
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (lane + 32 * i == e) key[i] = 0;
+    }
+    if (odd)
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (lane + 32 * i >= E) again &= ~(1u << i);
+    if (__any_sync(0xffffffffu, again != 0)) {
+        logits_again(z, again, x, w_router, bias, H, lane);
+        softmax_topk(z, E, k, lane, ids, wts);
+        return;
+    }
+    const float mx = __shfl_sync(0xffffffffu, z[mine], 0);
+    float sum = 0.f;
+    for (int e = lane; e < E; e += 32) sum += expf(z[e] - mx);
+    sum = warp_sum(sum);
+    if (lane < k) {
+        ids[lane] = mine;
+        wts[lane] = expf(z[mine] - mx) * (1.f / sum);
+    }
+}
+
+// MT: 16-token tiles per CTA; NT: 8-expert tiles per CTA; CL: CTAs per cluster (CL * NT = 8: 64 experts per pass);
+// U: steps of loads in flight
+template <int MT, int NT, int CL, int U>
+__global__ void __launch_bounds__(kRouteThreads)
+route_mma_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* __restrict__ w_router,
+                 const float* __restrict__ bias, int T, int H, int E, int k, int32_t* __restrict__ ids_out,
+                 float* __restrict__ w_out) {
+    constexpr int TM = 16 * MT, EC = 8 * NT, EB = CL * EC;                  // experts of a CTA / of the cluster per pass
+    constexpr int TOK = TM / CL;                                           // tokens whose choice this CTA makes
+    extern __shared__ __align__(16) unsigned char smem[];
+    float* part = reinterpret_cast<float*>(smem);                          // [warp][TM][EC + 1]
+    float* logit = part + kRouteWarps * TM * (EC + 1);                     // [TOK][kMmaMaxExperts] token i of the cluster: rank i % CL
+    float* xn = logit + TOK * kMmaMaxExperts;                              // [warp][TM] partial |x|^2
+    float* wn = xn + kRouteWarps * TM;                                     // [warp][EC] partial |w|^2
+    float* wmax_of = wn + kRouteWarps * EC;                                // [CL][2] largest |w|^2 of each CTA's experts
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int q = lane >> 2, c = lane & 3;
+    const int rank = blockIdx.x % CL, t0 = (blockIdx.x / CL) * TM, n_tok = min(TM, T - t0);
+    const int steps = H / 32;
+    cg::cluster_group cluster = cg::this_cluster();
+    grid_dependency_wait();
+    grid_launch_dependents();
+    if (CL > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // every CTA runs: its memory may be written
+    const __nv_bfloat162 zero2(__float2bfloat16(0.f), __float2bfloat16(0.f));
+    const uint4* xrow[2 * MT];
+    __nv_bfloat162 xsq[2 * MT];
+#pragma unroll
+    for (int r = 0; r < 2 * MT; ++r) {                                     // rows beyond the last token repeat it
+        xrow[r] = reinterpret_cast<const uint4*>(hidden + (size_t)(t0 + min(8 * r + q, n_tok - 1)) * H) + c;
+        xsq[r] = zero2;
+    }
+    auto square = [](__nv_bfloat162& sum, const uint4& v) {
+        const uint32_t r[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const __nv_bfloat162 p = *reinterpret_cast<const __nv_bfloat162*>(&r[i]);
+            sum = __hfma2(p, p, sum);
+        }
+    };
+    auto quad_sum = [](const __nv_bfloat162& v) {
+        float s = __low2float(v) + __high2float(v);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        return s + __shfl_xor_sync(0xffffffffu, s, 2);
+    };
+    float wtop = 0.f;
+    for (int p0 = 0; p0 < E; p0 += EB) {
+        const int e0 = p0 + rank * EC;
+        float acc[MT][NT][4];
+        __nv_bfloat162 wsq[NT];
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            wsq[n] = zero2;
+#pragma unroll
+            for (int m = 0; m < MT; ++m)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[m][n][i] = 0.f;
+        }
+        const uint4* wrow = reinterpret_cast<const uint4*>(w_router) + (size_t)(e0 + q) * (H / 8) + c;
+        const size_t wstep = (size_t)H;                                    // eight expert rows, in 16-byte chunks
+        for (int s0 = warp; s0 < steps; s0 += U * kRouteWarps) {
+            uint4 a[U][2 * MT], b[U][NT];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int s = s0 + u * kRouteWarps;
+#pragma unroll
+                for (int r = 0; r < 2 * MT; ++r) {
+                    a[u][r] = make_uint4(0, 0, 0, 0);
+                    if (s < steps) a[u][r] = xrow[r][4 * s];
+                }
+#pragma unroll
+                for (int n = 0; n < NT; ++n) {
+                    b[u][n] = make_uint4(0, 0, 0, 0);
+                    if (s < steps && e0 + 8 * n + q < E) b[u][n] = wrow[n * wstep + 4 * s];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+#pragma unroll
+                for (int n = 0; n < NT; ++n)
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) {
+                        const uint4 &lo = a[u][2 * m], &hi = a[u][2 * m + 1];
+                        mma_m16n8k16(acc[m][n], lo.x, hi.x, lo.y, hi.y, b[u][n].x, b[u][n].y);
+                        mma_m16n8k16(acc[m][n], lo.z, hi.z, lo.w, hi.w, b[u][n].z, b[u][n].w);
+                    }
+#pragma unroll
+                for (int n = 0; n < NT; ++n) square(wsq[n], b[u][n]);
+                if (p0 == 0)
+#pragma unroll
+                    for (int r = 0; r < 2 * MT; ++r) square(xsq[r], a[u][r]);
+            }
+        }
+        float* mine = part + warp * TM * (EC + 1);
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int n = 0; n < NT; ++n)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) mine[(16 * m + q + 8 * (i >> 1)) * (EC + 1) + 8 * n + 2 * c + (i & 1)] = acc[m][n][i];
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            const float v = quad_sum(wsq[n]);
+            if (c == 0) wn[warp * EC + 8 * n + q] = v;
+        }
+        if (p0 == 0)
+#pragma unroll
+            for (int r = 0; r < 2 * MT; ++r) {
+                const float v = quad_sum(xsq[r]);
+                if (c == 0) xn[warp * TM + 8 * r + q] = v;
+            }
+        __syncthreads();
+        if (CL > 1 && p0 == 0) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+        for (int i = tid; i < TM * EC; i += kRouteThreads) {
+            const int t = i / EC, e = i % EC;
+            float v = 0.f;
+#pragma unroll
+            for (int w = 0; w < kRouteWarps; ++w) v += part[(w * TM + t) * (EC + 1) + e];
+            if (e0 + e < E) {
+                float* dst = CL == 1 ? logit : cluster.map_shared_rank(logit, t % CL);
+                dst[(t / CL) * kMmaMaxExperts + e0 + e] = v + (bias ? bias[e0 + e] : 0.f);
+            }
+        }
+        if (tid < EC) {
+            float v = 0.f;
+            for (int w = 0; w < kRouteWarps; ++w) v += wn[w * EC + tid];
+            wtop = fmaxf(wtop, v);
+        }
+        __syncthreads();
+    }
+    static_assert(EC <= 64, "threads 0 .. EC - 1 are the first two warps");
+    if (warp < 2) {
+#pragma unroll
+        for (int m = 16; m >= 1; m >>= 1) wtop = fmaxf(wtop, __shfl_xor_sync(0xffffffffu, wtop, m));
+        if (lane < CL) (CL == 1 ? wmax_of : cluster.map_shared_rank(wmax_of, lane))[2 * rank + warp] = wtop;
+    }
+    if (CL > 1) cluster.sync(); else __syncthreads();
+    float wmax = 0.f;
+#pragma unroll
+    for (int r = 0; r < 2 * CL; ++r) wmax = fmaxf(wmax, wmax_of[r]);
+    for (int i = warp; i * CL + rank < n_tok; i += kRouteWarps) {
+        const int t = i * CL + rank;
+        float x2 = 0.f;
+#pragma unroll
+        for (int w = 0; w < kRouteWarps; ++w) x2 += xn[w * TM + t];
+        // of a pair both may be off; the bias addition rounds once more (relative to the logit)
+        choose(logit + i * kMmaMaxExperts, 2.f * kRouteBound * sqrtf(x2) * sqrtf(wmax), hidden + (size_t)(t0 + t) * H, w_router, bias,
+               H, E, k, lane, ids_out + (size_t)(t0 + t) * k, w_out + (size_t)(t0 + t) * k);
+    }
+}
+
+template <int MT, int NT, int CL, int U>
+int launch_route_mma(const exmoe_shape& s, const __nv_bfloat16* hidden, const __nv_bfloat16* w, const float* bias, int T,
+                     int32_t* ids, float* wts, cudaStream_t st) {
+    constexpr int TM = 16 * MT, EC = 8 * NT;
+    constexpr size_t smem = 4 * ((size_t)kRouteWarps * TM * (EC + 1) + (size_t)TM / CL * kMmaMaxExperts + kRouteWarps * (TM + EC) + 2 * CL);
+    static SmemOnce once;
+    if (!allow_smem(route_mma_kernel<MT, NT, CL, U>, (int)smem, once)) return EXMOE_ERR_CUDA;
+    return launch_dependent(route_mma_kernel<MT, NT, CL, U>, (T + TM - 1) / TM * CL, CL, smem, s, hidden, w, bias, T, ids, wts, st);
 }
 
 }  // namespace
@@ -103,15 +499,22 @@ extern "C" int exmoe_route(const exmoe_shape* shape, const void* hidden_bf16, co
     if (T == 0) return EXMOE_OK;
     if (!hidden_bf16 || !router_bf16 || !topk_ids || !topk_weights) return EXMOE_ERR_ARG;
     if ((reinterpret_cast<uintptr_t>(hidden_bf16) | reinterpret_cast<uintptr_t>(router_bf16)) & 15) return EXMOE_ERR_ARG;
-    const size_t smem = (size_t)shape->d_model * 2 + (size_t)shape->num_experts * 4;
-    if (smem > 200 * 1024) return EXMOE_ERR_SHAPE;
-    static SmemOnce smem_once;
-    if (!allow_smem(route_kernel, 200 * 1024, smem_once)) return EXMOE_ERR_CUDA;
-    route_kernel<<<T, kRouteThreads, smem, (cudaStream_t)stream>>>(
-        (const __nv_bfloat16*)hidden_bf16, (const __nv_bfloat16*)router_bf16, bias, shape->d_model, shape->num_experts,
-        shape->top_k, topk_ids, topk_weights);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? EXMOE_OK : EXMOE_ERR_CUDA;
+    const size_t row = (size_t)shape->d_model * 2, logits = (size_t)shape->num_experts * 4;
+    if (row + logits > (size_t)kRouteSmemMax) return EXMOE_ERR_SHAPE;
+    const exmoe_shape& s = *shape;
+    const __nv_bfloat16* x = (const __nv_bfloat16*)hidden_bf16;
+    const __nv_bfloat16* w = (const __nv_bfloat16*)router_bf16;
+    cudaStream_t st = (cudaStream_t)stream;
+    // Clusters of one token while they all find room on the chip at once, then four tokens per read of the matrix, then
+    // the tensor cores (measured crossings, 64 experts, d_model 2048: see the constants).  A shape that a form's shared
+    // memory or tiling does not fit takes the next simpler one; one token per cluster serves every shape.
+    if (T >= kRouteMmaTokens && s.d_model % 32 == 0 && s.d_model <= kMmaMaxModel && s.num_experts <= kMmaMaxExperts &&
+        s.top_k <= 32)
+        return T >= kRouteWideTokens ? launch_route_mma<2, 4, 2, 2>(s, x, w, bias, T, topk_ids, topk_weights, st)
+                                     : launch_route_mma<1, 2, 4, 4>(s, x, w, bias, T, topk_ids, topk_weights, st);
+    if (T >= kRouteFewTokens && 4 * row + logits <= (size_t)kRouteSmemMax)
+        return launch_route<8, 4>(s, x, w, bias, T, topk_ids, topk_weights, st);
+    return launch_route<8, 1>(s, x, w, bias, T, topk_ids, topk_weights, st);
 }
 
 }  // namespace exmoe

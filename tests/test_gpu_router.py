@@ -98,3 +98,25 @@ def test_router_feeds_the_layer(B):
     y, ref = ora.forward(hidden, ids.cpu(), w.cpu())
     helpers.check_output(out, y, ref, "router-fed layer")
     cache.close()
+
+
+@pytest.mark.parametrize("shape,T", [(synth.OLMOE, 47), (synth.OLMOE, 48), (synth.OLMOE, 51), (synth.OLMOE, 223), (synth.OLMOE, 225),
+                                     (synth.OLMOE, 2303), (synth.OLMOE, 2337), (synth.Shape(1280, 128, 72, 5), 300),
+                                     (synth.Shape(1280, 128, 72, 5), 2310), (synth.Shape(128, 128, 3, 2), 240)])
+def test_choice_does_not_depend_on_the_batch_size(B, shape, T):
+    """Every form of the kernel (one or four tokens per cluster, tensor cores with 16 or 32 tokens per CTA; last tiles
+    partly filled, an expert count that is no multiple of 64) picks the experts that one token at a time picks.  Near-ties
+    are planted: rows of the router matrix that differ from another in one element by one BF16 ulp, and equal rows.
+    Weights agree to binary32 rounding: logits of a few units off by 1e-6 at most, so 2e-5 relative as in `check`."""
+    hidden = synth.hidden_states(shape, T, seed=3).cuda()
+    w = synth.router_weights(shape, seed=4)
+    for e in range(1, shape.num_experts, 3):
+        w[e] = w[e - 1]
+        if e % 2:
+            w[e, e % shape.d_model] *= 1.0 + 2.0 ** -7
+    w = w.cuda()
+    ids, p = B.exmoe_route(shape, hidden, w)
+    for t0 in range(0, T, 40):                            # 40 tokens: the one-token-per-cluster form
+        i1, p1 = B.exmoe_route(shape, hidden[t0:t0 + 40].contiguous(), w)
+        assert torch.equal(ids[t0:t0 + 40], i1)
+        torch.testing.assert_close(p[t0:t0 + 40], p1, rtol=2e-5, atol=1e-9)
