@@ -1,10 +1,12 @@
-"""ctypes binding of libexmoe.so: the same entry points as include/exmoe.h, argument marshalling only.
+"""Python binding of libexmoe.so: the same entry points as include/exmoe.h, argument marshalling only (ctypes; the
+calls of a serving loop go through the CPython module `_exmoe_native`, which does the same checks in C++).
 
 PyTorch provides device memory, pinned host memory and streams; every step of the layer runs in
 the library's own CUDA kernels.  There is no fallback: if the library is missing or a call fails,
 an exception is raised.
 """
 import ctypes
+import importlib.util
 import os
 from ctypes import POINTER, byref, c_char_p, c_float, c_int, c_int32, c_size_t, c_uint64, c_void_p
 
@@ -12,6 +14,7 @@ import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libexmoe.so")
+NATIVE_PATH = os.path.join(_PKG, "_exmoe_native.so")
 
 EXMOE_OK = 0
 EXMOE_ERR_ARG = -1
@@ -70,20 +73,28 @@ _SIGNATURES = {
 }
 
 _lib = None
+_native = None
 
 
 def lib():
     """Open libexmoe.so (built in-tree by `paper_2608_15383_b200.build`); fail loudly if absent."""
-    global _lib
+    global _lib, _native
     if _lib is None:
-        if not os.path.exists(LIB_PATH):
-            raise FileNotFoundError(
-                f"{LIB_PATH} is missing: build it with `python -m paper_2608_15383_b200.build` (no CPU fallback exists)")
+        for path in (LIB_PATH, NATIVE_PATH):
+            if not os.path.exists(path):
+                raise FileNotFoundError(
+                    f"{path} is missing: build it with `python -m paper_2608_15383_b200.build` (no CPU fallback exists)")
         h = ctypes.CDLL(LIB_PATH)
         for name, (res, args) in _SIGNATURES.items():
             fn = getattr(h, name)
             fn.restype = res
             fn.argtypes = args
+        spec = importlib.util.spec_from_file_location("_exmoe_native", NATIVE_PATH)
+        native = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(native)
+        native.set_entry_points(*(ctypes.cast(getattr(h, name), c_void_p).value for name in
+                                  ("exmoe_route", "exmoe_moe_forward", "exmoe_moe_forward_host")))
+        _native = native
         _lib = h
     return _lib
 
@@ -160,18 +171,12 @@ def exmoe_moe_forward_static_status():
 
 def exmoe_route(shape, hidden, w_router, bias=None, topk_ids=None, topk_weights=None, stream=None):
     """Eq. 1 on the device: logits, softmax over all experts, top-k.  Returns (ids int32 [T, k], weights fp32 [T, k])."""
-    T = int(hidden.shape[0])
-    if topk_ids is None:
-        topk_ids = torch.empty((T, shape.top_k), dtype=torch.int32, device=hidden.device)
-    if topk_weights is None:
-        topk_weights = torch.empty((T, shape.top_k), dtype=torch.float32, device=hidden.device)
-    rc = lib().exmoe_route(byref(_shape(shape)), _dev(hidden, torch.bfloat16, "hidden"),
-                           _dev(w_router, torch.bfloat16, "w_router"),
-                           _dev(bias, torch.float32, "bias") if bias is not None else None, T,
-                           _dev(topk_ids, torch.int32, "topk_ids"), _dev(topk_weights, torch.float32, "topk_weights"),
-                           _stream_ptr(stream))
-    _check(rc, "exmoe_route")
-    return topk_ids, topk_weights
+    if _native is None:
+        lib()
+    r = _native.route(shape, hidden, w_router, bias, topk_ids, topk_weights, stream)
+    if r.__class__ is int:
+        raise ExmoeError(r, "exmoe_route")
+    return r
 
 
 def exmoe_launch_count():
@@ -253,35 +258,25 @@ class Cache:
                                       self.max_tokens, int(wave_cap))
         _check(rc, "exmoe_cache_create")
         self.handle = h
+        self._address = h.value
         self.max_waves = -(-shape.num_experts // self.wave_cap)
         self.n_keys = self.max_waves * self.C
 
     # exmoe_moe_forward
     def forward(self, layer, hidden, topk_ids, topk_weights, out=None, stream=None):
-        T = hidden.shape[0]
-        if out is None:
-            out = torch.empty_like(hidden)
-        rc = lib().exmoe_moe_forward(self.handle, int(layer), _dev(hidden, torch.bfloat16, "hidden"),
-                                     _dev(topk_ids, torch.int32, "topk_ids"), _dev(topk_weights, torch.float32, "topk_weights"),
-                                     int(T), _dev(out, torch.bfloat16, "out"), _stream_ptr(stream))
-        _check(rc, "exmoe_moe_forward")
-        return out
+        r = _native.forward(self._address, layer, hidden, topk_ids, topk_weights, out, stream)
+        if r.__class__ is int:
+            raise ExmoeError(r, "exmoe_moe_forward")
+        return r
 
     # exmoe_moe_forward_host
     def forward_host(self, layer, hidden, topk_ids, topk_weights, out=None, stream=None):
         """Host tensors in, host tensor out (synchronous): hidden BF16 [T, H], ids int32 [T, k], weights fp32 [T, k]."""
-        T = int(hidden.shape[0])
-        for t, dt, what in ((hidden, torch.bfloat16, "hidden"), (topk_ids, torch.int32, "topk_ids"),
-                            (topk_weights, torch.float32, "topk_weights")):
-            if t.is_cuda or t.dtype != dt or not t.is_contiguous():
-                raise ValueError(f"{what}: need a contiguous CPU tensor of {dt}")
         if out is None:
-            out = torch.empty((T, self.shape.d_model), dtype=torch.bfloat16)
-        elif out.is_cuda or out.dtype != torch.bfloat16 or not out.is_contiguous():
-            raise ValueError("out: need a contiguous CPU tensor of torch.bfloat16")
-        rc = lib().exmoe_moe_forward_host(self.handle, int(layer), c_void_p(hidden.data_ptr()), c_void_p(topk_ids.data_ptr()),
-                                          c_void_p(topk_weights.data_ptr()), T, c_void_p(out.data_ptr()), _stream_ptr(stream))
-        _check(rc, "exmoe_moe_forward_host")
+            out = torch.empty((int(hidden.shape[0]), self.shape.d_model), dtype=torch.bfloat16)
+        r = _native.forward_host(self._address, layer, hidden, topk_ids, topk_weights, out, stream)
+        if r is not None:
+            raise ExmoeError(r, "exmoe_moe_forward_host")
         return out
 
     def state(self, layer):
@@ -387,6 +382,7 @@ class Cache:
         if getattr(self, "handle", None):
             lib().exmoe_cache_destroy(self.handle)
             self.handle = None
+            self._address = 0
 
     def __del__(self):
         try:
