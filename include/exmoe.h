@@ -91,6 +91,16 @@ int exmoe_packed_bytes(const exmoe_shape* shape, size_t* bytes_per_expert);
 int exmoe_pack(const exmoe_shape* shape, const void* w_gate_bf16, const void* w_up_bf16,
                const void* w_down_bf16, void* packed_out, void* stream);
 
+/* The same conversion for `n_experts` experts at once, into host memory (Sec. 3.2's offline step ends in the pinned bank of
+ * Sec. 3.3): expert e of the inputs, each dev BF16 [n_experts, ...], goes to host_bank + e * bytes_per_expert.
+ *   staging   : dev, staging_experts * bytes_per_expert bytes, 16-byte aligned, staging_experts >= 2: one half is filled
+ *               while the other is copied out
+ *   host_bank : host; page-locked memory is copied to at the link's full rate
+ * The host link bounds it (207 MB for 64 OLMoE experts).  Runs on `stream` and a stream of its own and waits for both;
+ * same errors as exmoe_pack. */
+int exmoe_pack_bank(const exmoe_shape* shape, int n_experts, const void* w_gate_bf16, const void* w_up_bf16,
+                    const void* w_down_bf16, void* staging, int staging_experts, void* host_bank, void* stream);
+
 /* Sizes of the two device buffers the caller must allocate for exmoe_cache_create (Sec. 3.3):
  *   slot_bytes_total = num_layers * num_slots * bytes_per_expert
  *   workspace_bytes  = cache state + plan + token grouping + intermediate activations for

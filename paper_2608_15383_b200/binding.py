@@ -46,6 +46,7 @@ _SIGNATURES = {
     "exmoe_strerror": (c_char_p, [c_int]),
     "exmoe_packed_bytes": (c_int, [POINTER(exmoe_shape), POINTER(c_size_t)]),
     "exmoe_pack": (c_int, [POINTER(exmoe_shape), c_void_p, c_void_p, c_void_p, c_void_p, c_void_p]),
+    "exmoe_pack_bank": (c_int, [POINTER(exmoe_shape), c_int, c_void_p, c_void_p, c_void_p, c_void_p, c_int, c_void_p, c_void_p]),
     "exmoe_cache_workspace_bytes": (c_int, [POINTER(exmoe_shape), c_int, c_int, c_int, POINTER(c_size_t), POINTER(c_size_t)]),
     "exmoe_cache_create": (c_int, [POINTER(c_void_p), POINTER(exmoe_shape), c_int, c_int, POINTER(c_void_p), c_void_p,
                                    c_void_p, c_int, c_int]),
@@ -183,16 +184,26 @@ def exmoe_launch_count():
     return int(lib().exmoe_launch_count())
 
 
+PACK_STAGING_EXPERTS = 8      # device staging of pack_bank: two halves of four experts (26 MB for OLMoE's)
+
+
 def pack_bank(shape, w_gate, w_up, w_down, device="cuda"):
     """Pack all experts of one layer ([E,I,H], [E,I,H], [E,H,I] BF16) into a pinned host bank [E, bytes]."""
-    E = shape.num_experts
+    E, I, H = shape.num_experts, shape.d_ff, shape.d_model
+    weights = tuple(w[:E] for w in (w_gate, w_up, w_down))
+    if [tuple(w.shape) for w in weights] != [(E, I, H), (E, I, H), (E, H, I)]:
+        raise ValueError("pack_bank: weight shapes must be [E,I,H], [E,I,H], [E,H,I]")
     n = exmoe_packed_bytes(shape)
-    bank = torch.empty((E, n), dtype=torch.uint8).pin_memory()
-    buf = torch.empty(n, dtype=torch.uint8, device=device)
-    for e in range(E):
-        exmoe_pack(shape, w_gate[e].to(device).contiguous(), w_up[e].to(device).contiguous(),
-                   w_down[e].to(device).contiguous(), buf)
-        bank[e].copy_(buf)
+    bank = torch.empty((E, n), dtype=torch.uint8, pin_memory=True)
+    staging = torch.empty((PACK_STAGING_EXPERTS, n), dtype=torch.uint8, device=device)
+    # weights on the device already are converted in one call, others a few experts at a time as they arrive there
+    step = E if all(w.device == staging.device and w.is_contiguous() for w in weights) else PACK_STAGING_EXPERTS // 2
+    for e in range(0, E, step):
+        part = [w[e:e + step].to(staging.device).contiguous() for w in weights]
+        rc = lib().exmoe_pack_bank(byref(_shape(shape)), part[0].shape[0], *(_dev(w, torch.bfloat16, what) for w, what in
+                                                                             zip(part, ("w_gate", "w_up", "w_down"))),
+                                   c_void_p(staging.data_ptr()), PACK_STAGING_EXPERTS, c_void_p(bank[e:].data_ptr()), _stream_ptr(None))
+        _check(rc, "exmoe_pack_bank")
     return bank
 
 

@@ -287,11 +287,59 @@ int exmoe_pack(const exmoe_shape* shape, const void* w_gate, const void* w_up, c
     int flag = 0;
     rc = EXMOE_OK;
     if (cudaMemsetAsync(d_flag, 0, sizeof(int), st) != cudaSuccess) rc = EXMOE_ERR_CUDA;
-    if (!rc) rc = launch_pack(*shape, w_gate, w_up, w_down, packed_out, d_flag, st);
+    if (!rc) rc = launch_pack(*shape, 1, w_gate, w_up, w_down, packed_out, d_flag, st);
     if (!rc && cudaMemcpyAsync(&flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) rc = EXMOE_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) rc = EXMOE_ERR_CUDA;
     if (!rc && flag) rc = EXMOE_ERR_NONFINITE;
     return rc;
+}
+
+int exmoe_pack_bank(const exmoe_shape* shape, int n_experts, const void* w_gate, const void* w_up, const void* w_down,
+                    void* staging, int staging_experts, void* host_bank, void* stream) {
+    int rc = check_shape(shape);
+    if (rc) return rc;
+    if (n_experts < 0 || staging_experts < 2) return EXMOE_ERR_ARG;
+    if (n_experts == 0) return EXMOE_OK;
+    if (!w_gate || !w_up || !w_down || !staging || !host_bank) return EXMOE_ERR_ARG;
+    if ((reinterpret_cast<uintptr_t>(staging) | reinterpret_cast<uintptr_t>(w_gate) | reinterpret_cast<uintptr_t>(w_up) |
+         reinterpret_cast<uintptr_t>(w_down)) & 15)
+        return EXMOE_ERR_ARG;
+    cudaStream_t st = (cudaStream_t)stream, copy = nullptr;
+    cudaEvent_t packed[2] = {}, copied[2] = {};
+    int* d_flag = pack_flag_word();
+    if (!d_flag) return EXMOE_ERR_CUDA;
+    bool ok = cudaStreamCreateWithFlags(&copy, cudaStreamNonBlocking) == cudaSuccess;
+    for (int b = 0; b < 2; ++b) {
+        ok = ok && cudaEventCreateWithFlags(&packed[b], cudaEventDisableTiming) == cudaSuccess;
+        ok = ok && cudaEventCreateWithFlags(&copied[b], cudaEventDisableTiming) == cudaSuccess;
+    }
+    ok = ok && cudaMemsetAsync(d_flag, 0, sizeof(int), st) == cudaSuccess;
+    const size_t bpe = packed_bytes(*shape), weights = (size_t)shape->d_ff * shape->d_model * 2;
+    const int chunk = staging_experts / 2;
+    int flag = 0, i = 0;
+    for (int e = 0; e < n_experts && ok; e += chunk, ++i) {
+        const int n = n_experts - e < chunk ? n_experts - e : chunk, b = i & 1;
+        uint8_t* half = static_cast<uint8_t*>(staging) + (size_t)b * chunk * bpe;
+        const auto at = [&](const void* w) { return static_cast<const uint8_t*>(w) + (size_t)e * weights; };
+        if (i >= 2) ok = cudaStreamWaitEvent(st, copied[b], 0) == cudaSuccess;       // the half's last copy has read it
+        ok = ok && launch_pack(*shape, n, at(w_gate), at(w_up), at(w_down), half, d_flag, st) == EXMOE_OK;
+        ok = ok && cudaEventRecord(packed[b], st) == cudaSuccess && cudaStreamWaitEvent(copy, packed[b], 0) == cudaSuccess;
+        ok = ok && cudaMemcpyAsync(static_cast<uint8_t*>(host_bank) + (size_t)e * bpe, half, (size_t)n * bpe, cudaMemcpyDeviceToHost, copy) == cudaSuccess;
+        ok = ok && cudaEventRecord(copied[b], copy) == cudaSuccess;
+    }
+    ok = ok && cudaMemcpyAsync(&flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, st) == cudaSuccess;
+    if (copy) ok = (cudaStreamSynchronize(copy) == cudaSuccess) && ok;
+    ok = (cudaStreamSynchronize(st) == cudaSuccess) && ok;
+    for (int b = 0; b < 2; ++b) {
+        if (packed[b]) cudaEventDestroy(packed[b]);
+        if (copied[b]) cudaEventDestroy(copied[b]);
+    }
+    if (copy) cudaStreamDestroy(copy);
+    if (!ok) {
+        cudaGetLastError();
+        return EXMOE_ERR_CUDA;
+    }
+    return flag ? EXMOE_ERR_NONFINITE : EXMOE_OK;
 }
 
 int exmoe_cache_workspace_bytes(const exmoe_shape* shape, int num_layers, int num_slots, int max_tokens,

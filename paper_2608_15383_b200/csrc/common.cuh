@@ -111,7 +111,7 @@ inline bool allow_smem(F kern, int bytes, SmemOnce& once) {
 
 // ---- kernel launchers (defined in the .cu files) ------------------------------------------------
 int* pack_flag_word();      // a device word for one exmoe_pack call's non-finite flag (no allocation)
-int launch_pack(const exmoe_shape& s, const void* wg, const void* wu, const void* wd, void* out,
+int launch_pack(const exmoe_shape& s, int n_experts, const void* wg, const void* wu, const void* wd, void* out,
                 int* d_flag, cudaStream_t st);
 void launch_resolve(const exmoe_shape& s, int C, int Cw, size_t bytes_per_expert, const int32_t* ids, int n_pairs,
                     LayerState state, PlanPtrs plan, int* d_status, cudaStream_t st);

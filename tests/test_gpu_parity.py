@@ -53,6 +53,24 @@ def test_pack_bytes_olmoe_shape(B, olmoe_layer):
         assert np.array_equal(bank[e].numpy(), ora.packed(e)), e
 
 
+@pytest.mark.parametrize("E", [1, 3, 4, 5, 8, 9, 13])
+@pytest.mark.parametrize("where", ["cuda", "cpu", "strided"])
+def test_pack_bank_equals_packing_one_expert_at_a_time(B, E, where):
+    """Staging halves of four experts: fewer, exactly one, one over, a reused half; weights on the device, on the host,
+    and not contiguous.  Bytes against exmoe_pack (itself against the oracle above); one bad weight in the last expert."""
+    s = synth.Shape(d_model=256, d_ff=384, num_experts=E, top_k=1)
+    w = synth.expert_weights(s, seed=E, device="cuda")
+    given = [x.cpu() if where == "cpu" else x.repeat(1, 1, 2)[:, :, :x.shape[2]] if where == "strided" else x for x in w]
+    bank = B.pack_bank(s, *given)
+    assert bank.is_pinned() and bank.shape == (E, B.exmoe_packed_bytes(s))
+    for e in range(E):
+        assert torch.equal(bank[e], B.exmoe_pack(s, *(x[e].contiguous() for x in w)).cpu()), e
+    given[1][-1, -1, -1] = float("inf")
+    with pytest.raises(B.ExmoeError) as err:
+        B.pack_bank(s, *given)
+    assert err.value.code == B.EXMOE_ERR_NONFINITE
+
+
 def test_pack_special_groups_and_errors(B):
     s = synth.Shape(d_model=256, d_ff=128, num_experts=1, top_k=1)
     wg, wu, wd = synth.expert_weights(s, seed=3)
