@@ -52,4 +52,45 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     return true;
 }
 
+// The same by a whole warp, for barriers given by their shared-memory address: control flow that the compiler knows to be
+// uniform (no divergence bookkeeping around the poll, and the code around it keeps its uniform registers), no address
+// conversion per call.
+__device__ __forceinline__ void mbar_arrive_at(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_at(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
+    if (__any_sync(0xffffffffu, mbar_try_at(bar, parity))) return true;
+    const long long t0 = clock64();
+    for (unsigned polls = 1;; ++polls) {
+        if (__any_sync(0xffffffffu, mbar_try_at(bar, parity))) return true;
+        if ((polls & 15u) == 0) {
+            const bool late = clock64() - t0 > kWaitBudget;
+            if (late) {
+                *abort_flag = 1;
+                atomicExch(status, EXMOE_ERR_TIMEOUT);
+            }
+            if (__any_sync(0xffffffffu, late || *abort_flag)) return false;
+        }
+    }
+}
+// one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+template <typename T>
+__device__ __forceinline__ T warp_uniform(T v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 }  // namespace exmoe

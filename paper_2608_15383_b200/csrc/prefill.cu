@@ -8,9 +8,9 @@
 // 16 lanes apart: SwiGLU is one shuffle away in the epilogue.
 //
 // A persistent CTA (one per SM, 28 warps) is specialised by warp:
-//   warp 0        allocates TMEM, then ONE thread issues tcgen05.mma (4 x K16 per 64-wide ring stage) and
+//   warp 0        allocates TMEM, then one elected lane issues tcgen05.mma (4 x K16 per 64-wide ring stage) and
 //                 tcgen05.commit to the stage-empty / accumulator-full mbarriers, from an unrolled ring
-//                 (see the note at the issue loop: what bounds this kernel is what that thread does between MMAs).
+//                 (see the note at the issue loop: what bounds this kernel is what that warp does between MMAs).
 //   warps 4-7,    epilogue (two groups, even / odd 32-column chunks): tcgen05.ld the accumulator (warp w
 //   16-19         reads TMEM lanes 32(w%4)..), SwiGLU -> BF16 activations, or routing weight -> fp32
 //                 pair buffer; two accumulators (2 x 256 columns) let the epilogue of tile i overlap
@@ -82,8 +82,8 @@ struct Tile { int key, n0, nrows, pad; };
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+__device__ __forceinline__ void tc_commit_at(uint32_t bar) {       // barrier by its shared-memory address
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
@@ -272,7 +272,7 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 4);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const int K = GATEUP ? a.H : a.I;
     const int KB = K / BK;
     const int MT = (GATEUP ? 2 * a.I : a.H) / BM;                 // m-tiles of the packed matrix
@@ -299,37 +299,33 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    const uint32_t full_a = smem_u32(full), empty_a = smem_u32(empty), acc_full_a = smem_u32(acc_full), acc_empty_a = smem_u32(acc_empty);
 
     if (warp == 0) {
         // ------------------------------------------------------------------ MMA issuer
-        // ONE thread runs the loop (the other lanes wait at the warp barrier below).  tcgen05.mma issue blocks while
-        // the tensor pipe is busy, and the pipe holds little beyond the MMA it executes: every instruction this
-        // thread spends between two MMAs is time the pipe may drain, and with six busy warps on the same scheduler
-        // each instruction takes many cycles to issue (measured alone: the same four MMAs per stage run at N / 2
-        // cycles each with compile-time operands, at 150-160 cycles each, whatever N, behind run-time ring
-        // arithmetic and a barrier test).  So the ring is unrolled (stage index, barrier addresses and operand offsets
-        // are compile-time constants) and the NEXT stage's barrier is tested before this stage's MMAs are issued,
-        // the answer being read after them.  Shapes whose stage count per tile is not a multiple of the ring depth
-        // take the plain loop.
+        // tcgen05.mma issue blocks while the tensor pipe is busy, and the pipe holds little beyond the MMA it executes: every
+        // instruction between two MMAs is time the pipe may drain, and with six busy warps on the same scheduler each takes
+        // many cycles to issue (measured alone: the four MMAs of a stage run at N / 2 cycles each with compile-time operands,
+        // at 150-160 cycles each, whatever N, behind run-time ring arithmetic and a barrier test).  So the ring is unrolled
+        // (stage index, barrier addresses and operand offsets are compile-time constants), the NEXT stage's barrier is tested
+        // before this stage's MMAs are issued, and the whole warp walks the loop with one elected lane issuing: with
+        // warp-uniform control flow the descriptors live in uniform registers, where the instruction wants them.
+        // Shapes whose stage count per tile is not a multiple of the ring depth take the plain loop.
         PROF_DECL;
-        if (lane == 0) {
+        {
             int tcount = 0;
             bool ok = true;
             const uint64_t da0 = make_desc_a(smem_u32(sA)), db0 = make_desc_b(smem_u32(sB));
             if ((2 * KB) % STAGES == 0) {
-                int ph = 0;                                        // parity of the ring's current turn
+                uint32_t ph = 0;                                   // parity of the ring's current turn
                 bool ready = false;                                // next stage's barrier already seen complete
                 for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++tcount) {
-                    const Tile tl = a.tiles[t / MT];
-                    const int n_mma = (tl.nrows + 15) & ~15;
-                    const uint32_t idesc = make_idesc(n_mma);
+                    const uint32_t idesc = warp_uniform(make_idesc((a.tiles[t / MT].nrows + 15) & ~15));
                     const int buf = tcount & 1;
-                    if (!mbar_try(&acc_empty[buf], ((tcount >> 1) & 1) ^ 1)) {
-                        PROF_WAIT_BEGIN;
-                        ok = mbar_wait(&acc_empty[buf], ((tcount >> 1) & 1) ^ 1, abort_flag, a.status);
-                        PROF_WAIT_END;
-                        if (!ok) break;
-                    }
+                    PROF_WAIT_BEGIN;
+                    ok = mbar_wait_warp(acc_empty_a + 8 * buf, ((tcount >> 1) & 1) ^ 1, abort_flag, a.status);
+                    PROF_WAIT_END;
+                    if (!ok) break;
                     tc_fence_after();
                     const uint32_t d_tmem = tmem_base + buf * BN_T;
                     for (int ks0 = 0; ks0 < 2 * KB && ok; ks0 += STAGES) {
@@ -337,51 +333,56 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
                         for (int st = 0; st < STAGES; ++st) {
                             if (!ready) {
                                 PROF_WAIT_BEGIN;
-                                ok = mbar_wait(&full[st], ph, abort_flag, a.status);
+                                ok = mbar_wait_warp(full_a + 8 * st, ph, abort_flag, a.status);
                                 PROF_WAIT_END;
                                 if (!ok) break;
                             }
                             const int nst = (st + 1) % STAGES;
-                            const bool ready_next = mbar_try(&full[nst], nst ? ph : ph ^ 1);
+                            ready = __any_sync(0xffffffffu, mbar_try_at(full_a + 8 * nst, nst ? ph : ph ^ 1));
                             const uint64_t da = da0 + (uint64_t)(st * (A_STAGE_BYTES >> 4));
                             const uint64_t db = db0 + (uint64_t)(st * (B_STAGE_BYTES >> 4));
+                            if (elect_one()) {
 #pragma unroll
-                            for (int j = 0; j < BKS / 16; ++j)     // K16 step j: A two k-chunks on, B 32 bytes on
-                                tc_mma(d_tmem, da + (uint64_t)(j * 2 * A_LBO >> 4), db + (uint64_t)((j * 32) >> 4), idesc, (ks0 | st | j) ? 1u : 0u);
-                            tc_commit(&empty[st]);                 // stage reusable once these MMAs have read it
-                            ready = ready_next;
+                                for (int j = 0; j < BKS / 16; ++j) // K16 step j: A two k-chunks on, B 32 bytes on
+                                    tc_mma(d_tmem, da + (uint64_t)(j * 2 * A_LBO >> 4), db + (uint64_t)((j * 32) >> 4), idesc, (ks0 | st | j) ? 1u : 0u);
+                                tc_commit_at(empty_a + 8 * st);    // stage reusable once these MMAs have read it
+                            }
+                            __syncwarp();
                         }
                         ph ^= 1;
                     }
-                    if (ok) tc_commit(&acc_full[buf]);             // accumulator complete
+                    if (ok && elect_one()) tc_commit_at(acc_full_a + 8 * buf);     // accumulator complete
+                    __syncwarp();
                 }
             } else {
-                int s = 0, ph = 0;                                 // ring position of the next stage to consume
+                int s = 0;
+                uint32_t ph = 0;                                   // ring position of the next stage to consume
                 for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++tcount) {
-                    const Tile tl = a.tiles[t / MT];
-                    const int n_mma = (tl.nrows + 15) & ~15;
-                    const uint32_t idesc = make_idesc(n_mma);
+                    const uint32_t idesc = warp_uniform(make_idesc((a.tiles[t / MT].nrows + 15) & ~15));
                     const int buf = tcount & 1;
-                    ok = mbar_wait(&acc_empty[buf], ((tcount >> 1) & 1) ^ 1, abort_flag, a.status);
+                    ok = mbar_wait_warp(acc_empty_a + 8 * buf, ((tcount >> 1) & 1) ^ 1, abort_flag, a.status);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t d_tmem = tmem_base + buf * BN_T;
                     for (int ks = 0; ks < 2 * KB; ++ks) {
-                        if (!mbar_try(&full[s], ph)) ok = mbar_wait(&full[s], ph, abort_flag, a.status);
+                        ok = mbar_wait_warp(full_a + 8 * s, ph, abort_flag, a.status);
                         if (!ok) break;
                         const uint64_t da = da0 + (uint64_t)(s * (A_STAGE_BYTES >> 4));
                         const uint64_t db = db0 + (uint64_t)(s * (B_STAGE_BYTES >> 4));
+                        if (elect_one()) {
 #pragma unroll
-                        for (int j = 0; j < BKS / 16; ++j)
-                            tc_mma(d_tmem, da + (uint64_t)(j * 2 * A_LBO >> 4), db + (uint64_t)((j * 32) >> 4), idesc, (ks | j) ? 1u : 0u);
-                        tc_commit(&empty[s]);
+                            for (int j = 0; j < BKS / 16; ++j)
+                                tc_mma(d_tmem, da + (uint64_t)(j * 2 * A_LBO >> 4), db + (uint64_t)((j * 32) >> 4), idesc, (ks | j) ? 1u : 0u);
+                            tc_commit_at(empty_a + 8 * s);
+                        }
+                        __syncwarp();
                         if (++s == STAGES) { s = 0; ph ^= 1; }
                     }
-                    if (ok) tc_commit(&acc_full[buf]);
+                    if (ok && elect_one()) tc_commit_at(acc_full_a + 8 * buf);
+                    __syncwarp();
                 }
             }
         }
-        __syncwarp();
         PROF_REPORT("mma");
     } else if ((warp >= 4 && warp < 8) || (warp >= 16 && warp < 20)) {
         // ------------------------------------------------------------------ epilogue
@@ -397,15 +398,14 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
             constexpr int CHUNKS = (BN_T + 63) / 64;               // 32-column chunks of this warp in a full tile
             const EpiloguePre<CHUNKS> pre = epilogue_prefetch<GATEUP, CHUNKS>(a, tl, odd, lane, offsets, topk_w);
             PROF_WAIT_BEGIN;
-            ok = mbar_wait(&acc_full[buf], (tcount >> 1) & 1, abort_flag, a.status);
+            ok = mbar_wait_warp(acc_full_a + 8 * buf, (tcount >> 1) & 1, abort_flag, a.status);
             PROF_WAIT_END;
-            ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
             epilogue_tile<GATEUP, CHUNKS>(a, tl, mt, e, odd, lane, tmem_base + buf * BN_T, pre, act_out, y_out);
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[buf]);
+            if (elect_one()) mbar_arrive_at(acc_empty_a + 8 * buf);
         }
         PROF_REPORT("epilogue");
     } else if (warp == 1) {
@@ -421,12 +421,11 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
             for (int ks = 0; ks < 2 * KB; ++ks) {
                 {
                     PROF_WAIT_BEGIN;
-                    ok = mbar_wait(&empty[s], ph ^ 1, abort_flag, a.status);
+                    ok = mbar_wait_warp(empty_a + 8 * s, ph ^ 1, abort_flag, a.status);
                     PROF_WAIT_END;
                 }
-                ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                if (lane == 0) {
+                if (elect_one()) {
                     mbar_expect_tx(&full[s], n_mma * 128);
                     tma_load_2d(smem_u32(sB + s * B_STAGE_BYTES), map, ks * BKS, row0, &full[s]);
                 }
@@ -494,14 +493,13 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
         static_assert(STAGES == 4 || STAGES == 8, "ring positions of the conversion warps are precomputed for these depths");
         constexpr int LOG_STAGES = STAGES == 4 ? 2 : 3;
         unsigned char* stage_ptr[2];
-        uint64_t* full_ptr[2];
-        uint64_t* empty_ptr[2];
+        uint32_t full_at[2], empty_at[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int sb = (2 * par + 4 * u) & (STAGES - 1);
             stage_ptr[u] = sA + sb * A_STAGE_BYTES + (2 * pw) * A_SBO + c * A_LBO + q * 16;
-            full_ptr[u] = &full[sb];
-            empty_ptr[u] = &empty[sb];
+            full_at[u] = full_a + 8 * sb;
+            empty_at[u] = empty_a + 8 * sb;
         }
         int n = 2 * par;                                           // stage count of the next block's first half
         for (int g0 = par; g0 < total_blocks && ok; g0 += 2 * PF) {
@@ -517,10 +515,9 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
                 for (int h = 0; h < 2; ++h) {                                         // the block's two halves = two stages
                     {
                         PROF_WAIT_BEGIN;
-                        ok = mbar_wait(empty_ptr[u] + h, ph ^ 1, abort_flag, a.status);
+                        ok = mbar_wait_warp(empty_at[u] + 8 * h, ph ^ 1, abort_flag, a.status);
                         PROF_WAIT_END;
                     }
-                    ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     unsigned char* dst = stage_ptr[u] + h * A_STAGE_BYTES;
                     const uint32_t words[4] = {w[u][h].x, w[u][h].y, w[u][h].z, w[u][h].w};
@@ -532,7 +529,7 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
                     }
                     fence_proxy_async();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(full_ptr[u] + h);
+                    if (elect_one()) mbar_arrive_at(full_at[u] + 8 * h);
                 }
                 if (!ok) break;
                 n += 4;
