@@ -2,21 +2,27 @@
 // grouped expert GEMMs of a wave (Section 3.4, Eq. 2) as HBM-bound streams over the packed expert bytes,
 // with the memory system decoupled from the arithmetic.
 //
-// The work of a wave is cut into units: (active group = expert, pass over up to 8 or 16 of the group's rows,
+// The work of a wave is cut into units: (active group = expert, pass over up to R = 8 or 16 of the group's rows,
 // tile of PP panels; gate/up: PP gate+up panel pairs).  A tile is ONE contiguous range of the packed
 // expert image.  Units are ordered group-major, then pass, then tile, and every persistent CTA (one per
 // SM) takes an equal contiguous share, so that the load is balanced by arithmetic, not by expert, and a
 // CTA's consecutive units share their activation rows.  A group with more rows than one pass holds
 // re-reads its tiles once per pass (they come from L2).  Roles by warp:
-//   warps 0-15  two consumer groups of eight warps that take alternate units: read the tile's packed bytes
-//               from shared memory (the image is already in m16n8k16 fragment order), dequantise in
-//               registers (shift + lop3), mma.sync against the group's activation rows, scale per 128-wide
-//               block in binary32; the K-split partials cross shared memory once and every warp finishes
-//               a slice of the tile (fixed summation order; SwiGLU or routing weight; store).
+//   warps 0-15  two consumer groups of eight warps that take alternate units: read the tile's packed bytes from shared
+//               memory (the image is already in MMA fragment order), turn every word into FP16 operands (one shift, four
+//               ANDs: see frag.cuh), mma.sync against the pass's rows, scale per 128-wide block in binary32; the K-split
+//               partials cross shared memory once and the group's warps finish the tile (fixed summation order; SwiGLU
+//               or routing weight; store).  When a unit starts a new (group, pass), all sixteen warps fetch its rows
+//               (gathered through the plan's permutation for gate/up), convert them and store them.
 //   warp 16     weight producer: one cp.async.bulk per unit into a ring of stages, completion counted in
 //               bytes on the stage's mbarrier; runs as many stages ahead as the ring is deep.
-//   warp 17     activation producer: one cp.async.bulk per activation row (gathered through the plan's
-//               permutation for gate/up) into a row buffer (two of them where shared memory allows).
+// Bound: HBM for the gate/up kernel, 6.2 TB/s (96 % of the measured copy rate) per further expert, plus 7.5 us per launch
+// that do not depend on the number of experts (plan, rows, first and last unit).  The down kernel's units take 2,000 cycles
+// where HBM would take 1,470.  With BF16 operands (128 + u: three shifts and four lop3 a word, a second copy of the block
+// corrections per group) the consumers were the bound: layer 53.2 -> 48.2 us at 16 tokens, 89.2 -> 77.6 at 64.
+// Built and slower at 16 tokens: codes and split activations as e4m3 (mma.sync on e4m3 runs as conversions to FP16 and two
+// FP16 MMAs here), 67 us; sixteen independent warps with their blocks in registers, no ring and no exchange per
+// unit, 62 us (a warp's loads share a few scoreboards: waiting for the oldest block waits for the newest as well).
 // The down kernel is a programmatic dependent of the gate/up kernel: its weight ring fills while the
 // gate/up kernel drains; only its activation producer waits for the dependency.
 // Every mbarrier wait is bounded: on expiry the CTA raises EXMOE_ERR_TIMEOUT, all roles leave their
@@ -24,12 +30,8 @@
 #include "common.cuh"
 #include "frag.cuh"
 #include "mbar.cuh"
-#ifdef EXMOE_STREAM_PROF
-#include <cstdio>
-#define SPROF(...) __VA_ARGS__
-#else
-#define SPROF(...)
-#endif
+
+#include <type_traits>
 
 namespace exmoe {
 
@@ -37,9 +39,9 @@ namespace {
 
 constexpr int kGroupWarps = 8;                       // warps of one consumer group
 constexpr int kGroupThreads = 32 * kGroupWarps;
-constexpr int kGroups = 2;                           // consumer groups, alternate units
+constexpr int kGroups = 2;                           // consumer groups, alternate units (a third one: no change)
 constexpr int kConsumerWarps = kGroups * kGroupWarps;
-constexpr int kStreamThreads = 32 * (kConsumerWarps + 2);
+constexpr int kStreamThreads = 32 * (kConsumerWarps + 1);
 constexpr int kMaxStages = 8;
 constexpr size_t kSmemLimit = 227 * 1024;
 constexpr int kScanChunks = 4;                       // chunks of 32 groups whose plan entries the scan keeps in registers
@@ -61,39 +63,41 @@ __device__ __forceinline__ void group_sync(int grp) {              // named barr
     asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "n"(kGroupThreads) : "memory");
 }
 
+__device__ __forceinline__ void rows_sync() {                      // all consumers
+    asm volatile("bar.sync 8, %0;" ::"n"(32 * kConsumerWarps) : "memory");
+}
+
 struct StreamGeom {
-    int PP, KS, NMW, tiles, n_stages, n_xbuf;
+    int PP, KS, tiles, n_stages, n_xbuf;
     uint32_t stage_bytes, x_stride;
-    size_t off_x, off_part, off_adj, off_bar, total;
+    size_t off_x, off_part, off_cst, off_row, off_bar, total;
 };
 
-constexpr size_t kBarBytes = (2 * kMaxStages + 4) * 8 + 64;          // mbarriers, abort flag, unit range
-constexpr size_t kCtrlBytes = kBarBytes + (size_t)kMetaGroups * 16;  // + plan entries of the CTA's groups
+constexpr size_t kBarBytes = 2 * kMaxStages * 8 + 64;                 // mbarriers, abort flag, unit range
+constexpr size_t kCtrlBytes = kBarBytes + (size_t)kMetaGroups * 16;   // + plan entries of the CTA's groups
 
 #ifndef EXMOE_STREAM_PP
 #define EXMOE_STREAM_PP 0                                              // 0: choose; 1/2/4/8: force where feasible (timing experiments)
 #endif
 
-// Tile shape and shared-memory budget for one matrix kind.  The eight warps of a consumer group are
-// PP panels x (gate | up, when a warp holds one of the two: NMW = 1) x KS ranges of K.
-// Preference: a ring of at least four stages, then two activation buffers over one, then the larger tile.
-__host__ bool stream_geometry(int K, int NR, int NM, int NCH, StreamGeom* out) {
-    const int KB = K / kGroup, R = 8 * NCH;
-    const size_t x_stride = (size_t)K * 2 + 64;
+// Tile shape and shared-memory budget for one matrix kind.  The eight warps of a consumer group are PP panels x
+// (gate | up) x KS ranges of K (ranges differ by one block where KS does not divide it, and are empty where K has fewer).
+// Preference: a ring of at least four stages, then two row buffers over one, then the larger tile.
+__host__ bool stream_geometry(int K, int NR, int NM, int R, StreamGeom* out) {
+    const int KB = K / kGroup;
+    const size_t x_stride = (size_t)K * 2 + 64;                        // bytes of one row; + 64: conflict-free 16-byte fragment loads
     long best = -1;
     for (int NX = 2; NX >= 1; --NX)
-        for (int PP = 8; PP >= 1; PP >>= 1) {
-            const int NMW = (NM == 2 && PP == 8) ? 2 : 1;              // both matrices in one warp only when there is no room to split
-            const int KS = 8 / (PP * (NM / NMW));
-            if (KS < 1 || KB % KS || NR % (kPanelRows * PP)) continue;
+        for (int PP = 8 / NM; PP >= 1; PP >>= 1) {
+            const int KS = 8 / (PP * NM);
+            if (NR % (kPanelRows * PP)) continue;
             if (EXMOE_STREAM_PP && PP != EXMOE_STREAM_PP) continue;
             const size_t stage = (size_t)NM * PP * KB * kBlockBytes;
             if (stage > 96 * 1024) continue;
             const size_t xs = (size_t)NX * R * x_stride;
-            const bool exchange = !(KS == 1 && NMW == NM);             // partials cross shared memory
-            const size_t part = exchange ? (size_t)kGroups * 2 * kGroupWarps * NMW * NCH * 512 : 0;
-            const size_t adj = (size_t)kGroups * NX * KB * R * 4;
-            const size_t fixed = xs + part + adj + kCtrlBytes + 192;
+            const size_t part = (size_t)kGroups * 2 * kGroupWarps * (R / 8) * 128 * 4;
+            const size_t cst = (size_t)NX * KB * R * 8;
+            const size_t fixed = xs + part + cst + (size_t)NX * R * 8 + kCtrlBytes + 256;
             if (fixed + 2 * stage > kSmemLimit) continue;
             int S = (int)((kSmemLimit - fixed) / stage);
             if (S > kMaxStages) S = kMaxStages;
@@ -101,12 +105,13 @@ __host__ bool stream_geometry(int K, int NR, int NM, int NCH, StreamGeom* out) {
             if (score <= best) continue;
             best = score;
             StreamGeom g{};
-            g.PP = PP; g.KS = KS; g.NMW = NMW; g.tiles = NR / (kPanelRows * PP); g.n_stages = S; g.n_xbuf = NX;
+            g.PP = PP; g.KS = KS; g.tiles = NR / (kPanelRows * PP); g.n_stages = S; g.n_xbuf = NX;
             g.stage_bytes = (uint32_t)stage; g.x_stride = (uint32_t)x_stride;
             g.off_x = (size_t)S * stage;
             g.off_part = g.off_x + xs;
-            g.off_adj = g.off_part + part;
-            g.off_bar = (g.off_adj + adj + 63) & ~(size_t)63;
+            g.off_cst = g.off_part + part;
+            g.off_row = g.off_cst + cst;
+            g.off_bar = (g.off_row + (size_t)NX * R * 8 + 63) & ~(size_t)63;
             g.total = g.off_bar + kCtrlBytes;
             *out = g;
         }
@@ -122,7 +127,7 @@ struct StreamArgs {
     int* status;
     int PP, KS, n_stages, n_xbuf;
     uint32_t stage_bytes, x_stride;
-    uint32_t off_x, off_part, off_adj, off_bar;
+    uint32_t off_x, off_part, off_cst, off_row, off_bar;
 };
 
 // position of a unit inside the CTA's share: index into the cached plan entries, pass, tile
@@ -139,50 +144,41 @@ struct Cursor {
     }
 };
 
-// NMW: matrices held by one warp (2 = gate and up of the same panel; 1 = one matrix, gate/up split over warps)
-// KBc, PPc, KSc: blocks along K, panels per tile and K ranges per panel as COMPILE-TIME constants (0 = taken from the
+// R: rows of one pass.  KBc, PPc: blocks along K and panels per tile as COMPILE-TIME constants (0 = taken from the
 // arguments).  With run-time values about a third of the executed instructions were address arithmetic, predicates and
 // loop control around the conversion and the MMAs; the shapes that matter (OLMoE's two matrices) get their own
 // instantiations with the block loop unrolled and every stride a literal, all others run the generic one.
-template <int NCH, bool GATEUP, int NMW, int KBc = 0, int PPc = 0, int KSc = 0>
+template <int R, bool GATEUP, int KBc = 0, int PPc = 0>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 stream_gemm_kernel(const StreamArgs p) {
     constexpr int NM = GATEUP ? 2 : 1;                                // matrices per tile
-    constexpr int MS = NM / NMW;                                      // warps a panel's matrices are split over
-    constexpr int R = 8 * NCH;
-    constexpr int CHN = (NMW * NCH >= 2) ? 1 : 2;                          // accumulator chains per (matrix, chunk): two independent MMA chains per warp at least
+    constexpr int NTM = R / 8;                                        // most column tiles (eight rows) of a pass
     extern __shared__ __align__(128) unsigned char smem[];
     const GemmArgs& a = p.a;
     constexpr bool FIXED = KBc > 0;
-    constexpr int BPWc = KSc > 0 ? KBc / (KSc > 0 ? KSc : 1) : 0;     // blocks per K range when the geometry is fixed
     const int NR = GATEUP ? a.I : a.H;
     const int KB = FIXED ? KBc : (GATEUP ? a.H : a.I) / kGroup, K = KB * kGroup;
-    const int PP = FIXED ? PPc : p.PP, KS = FIXED ? KSc : p.KS, bpw = KB / KS;
+    const int PP = FIXED ? PPc : p.PP, KS = FIXED ? 8 / (PPc * NM) : p.KS;
     const uint32_t x_stride = FIXED ? (uint32_t)(KBc * kGroup * 2 + 64) : p.x_stride;
-    const uint32_t stage_bytes = FIXED ? (uint32_t)((GATEUP ? 2 : 1) * PPc * KBc * kBlockBytes) : p.stage_bytes;
+    const uint32_t stage_bytes = FIXED ? (uint32_t)(NM * PPc * KBc * kBlockBytes) : p.stage_bytes;
     const int tiles = NR / (kPanelRows * PP);
     const int S = p.n_stages, NX = p.n_xbuf;
     unsigned char* wst = smem;
-    unsigned char* xs = smem + p.off_x;
+    unsigned char* xs = smem + p.off_x;                                // [NX][R][x_stride]
     float* part = reinterpret_cast<float*>(smem + p.off_part);
-    float* adj = reinterpret_cast<float*>(smem + p.off_adj);
+    float2* cst = reinterpret_cast<float2*>(smem + p.off_cst);         // [NX][KB][R]
+    int2* rowinfo = reinterpret_cast<int2*>(smem + p.off_row);         // [NX][R] down: (pair, routing weight)
     uint64_t* w_full = reinterpret_cast<uint64_t*>(smem + p.off_bar);
     uint64_t* w_empty = w_full + kMaxStages;
-    uint64_t* x_full = w_empty + kMaxStages;
-    uint64_t* x_empty = x_full + 2;
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(x_empty + 2);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(w_empty + kMaxStages);
     int* s_range = const_cast<int*>(abort_flag) + 4;                   // [0] first unit, [1] end
     const int4* meta = reinterpret_cast<const int4*>(smem + p.off_bar + kBarBytes);   // (key, rows, first row, first unit)
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = warp_uniform(tid >> 5);
     if (tid == 32) {
         for (int s = 0; s < S; ++s) {
             mbar_init(&w_full[s], 1);
             mbar_init(&w_empty[s], kConsumerWarps);                    // both groups: see the consumer loop
-        }
-        for (int b = 0; b < NX; ++b) {
-            mbar_init(&x_full[b], 1);
-            mbar_init(&x_empty[b], kConsumerWarps);                    // both groups
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -249,8 +245,9 @@ stream_gemm_kernel(const StreamArgs p) {
             for (int m = 16; m >= 1; m >>= 1) passes += __shfl_xor_sync(0xffffffffu, passes, m);
             total += passes;
         }
-        const long long U = (long long)total * tiles;
-        int u0 = (int)(U * blockIdx.x / gridDim.x), u1 = (int)(U * (blockIdx.x + 1) / gridDim.x);
+        const int U = total * tiles, share = U / (int)gridDim.x, longer = U - share * (int)gridDim.x;    // the first CTAs take one more
+        int u0 = share * (int)blockIdx.x + min((int)blockIdx.x, longer);
+        int u1 = u0 + share + ((int)blockIdx.x < longer ? 1 : 0);
         int run = 0, found = 0;
         int4* meta_w = const_cast<int4*>(meta);
         for (int chunk = 0; 32 * chunk < n_groups && u0 < u1; ++chunk) {
@@ -321,287 +318,211 @@ stream_gemm_kernel(const StreamArgs p) {
                 while (!mbar_try(&w_full[j % S], (j / S) & 1) && clock64() - t0 < kWaitBudget) {}
             }
         }
-    } else if (warp == kConsumerWarps + 1) {
-        // ---------------------------------------------------------------- activation producer
-        if (!GATEUP) grid_dependency_wait();           // the gate/up kernel's activations are complete and visible
-        int n = 0, b = 0;
-        uint32_t ph = 1;
-        for (int u = u0; u < u1; ++u) {
-            const int4 gm = meta[cur.gi];
-            if (u == u0 || cur.tile == 0) {            // first unit of a (group, pass): stage its rows
-                if (n >= NX && !warp_wait(&x_empty[b], ph, abort_flag, p.status)) break;
-                const int pass0 = cur.pass * R;
-                const int rows_here = min(R, gm.y - pass0);
-                if (lane == 0) mbar_expect_tx(&x_full[b], (uint32_t)rows_here * K * 2);
-                __syncwarp();
-                if (lane < rows_here) {
-                    const size_t src_row = GATEUP ? (size_t)(a.perm[gm.z + pass0 + lane] / a.top_k)
-                                                  : (size_t)(gm.z + pass0 + lane);
-                    bulk_load(xs + ((size_t)b * R + lane) * x_stride, p.x_src + src_row * K, (uint32_t)K * 2, &x_full[b]);
-                }
-                __syncwarp();
-                ++n;
-                if (++b == NX) {
-                    b = 0;
-                    ph ^= 1u;
-                }
-            }
-            cur.advance(tiles, (gm.y + R - 1) / R);
-        }
-        if (*abort_flag && lane == 0) {
-            for (int j = (n > NX ? n - NX : 0); j < n; ++j) {
-                const long long t0 = clock64();
-                while (!mbar_try(&x_full[j % NX], (j / NX) & 1) && clock64() - t0 < kWaitBudget) {}
-            }
-        }
     } else {
         // ---------------------------------------------------------------- consumers
         const int grp = warp / kGroupWarps, cw = warp % kGroupWarps;
         const int q = lane >> 2, c = lane & 3;
-        const int ks = cw % KS, mw = (cw / KS) % MS, pp = cw / (KS * MS);    // K range, matrix (when split), panel
-        const bool exchange = !(KS == 1 && MS == 1);
-        // partials of one unit: [pp][matrix][ks][ch][i][lane], one buffer per group and unit parity
-        const int part_words = kGroupWarps * NMW * NCH * 128;
-        float* adjg = adj + (size_t)grp * NX * KB * R;
+        const int ks = cw % KS, mw = (cw / KS) % NM, pp = cw / (KS * NM);    // K range, matrix, panel
+        const int kb_lo = ks * KB / KS, kb_hi = (ks + 1) * KB / KS;
+        const uint32_t w_full_a = smem_u32(w_full), w_empty_a = smem_u32(w_empty);
+        // partials of one unit: [pp][matrix][ks][column tile][word][lane], one buffer per group and unit parity
+        constexpr int part_words = kGroupWarps * NTM * 128;
+        float* partg = part + (size_t)grp * 2 * part_words;
+        const int panel_local = NM * pp + mw;
+        // this lane's places: packed words and scales of the warp's first block, row q of a column tile, constants of rows 2c, 2c + 1
+        const unsigned char* w_lane = wst + ((size_t)panel_local * KB + kb_lo) * kBlockBytes + lane * 16;
+        const unsigned char* s_lane = wst + ((size_t)panel_local * KB + kb_lo) * kBlockBytes + kCodeBytes + q * 4;
+        const unsigned char* x_lane = xs + (size_t)q * x_stride + (kb_lo * kGroup + 8 * c) * 2;
+        const float2* c_lane = cst + (size_t)kb_lo * R + 2 * c;
+        // fetching rows: item = (row, block), 16 lanes each
+        const int hw = warp * 2 + (lane >> 4), l16 = lane & 15;
         int mine_cnt = 0;
-        int s = -1, xb = -1;                           // weight stage and row buffer of the current unit
-        uint32_t w_ph = 1, x_ph = 1;                   // their barrier parities (flipped when the index wraps to 0)
-        // Both groups walk ALL units in order and observe every phase of every full barrier, also for units and
-        // rows the other group computes on, and release each stage only then: a parity wait is only valid for a
-        // waiter that is at most one phase behind.
-        // A failed (expired or aborted) wait never changes the control flow: the named barriers below need all
-        // eight warps of the group, so the thread runs on over whatever the buffers hold, stores nothing, and
-        // every later wait returns at once because the abort flag is up.
+        int s = -1, xb = 0;                            // weight stage and row buffer of the current unit
+        uint32_t w_ph = 1;                             // the stage's barrier parity (flipped when the index wraps to 0)
+        bool dep = false;
+        // Both groups walk ALL units in order and observe every phase of every full barrier, also for units the other group
+        // computes on, and release each stage only then: a parity wait is only valid for a waiter that is at most one phase
+        // behind.  A failed (expired or aborted) wait never changes the control flow: the named barriers below need
+        // all warps, so the thread runs on over whatever the buffers hold, stores nothing, and every later wait
+        // returns at once because the abort flag is up.
         bool ok = true;
-        SPROF(long long t_x = 0, t_w = 0, t_mma = 0, t_ep = 0, t_other = 0, t_begin = clock64(); int n_mine = 0;)
         for (int u = u0, n = 0; u < u1; ++u, ++n) {
-            SPROF(long long c0 = clock64();)
             const int4 gm = meta[cur.gi];
             const int m_rows = gm.y, row0 = gm.z, tile = cur.tile, pass0 = cur.pass * R;
             const bool fresh = (u == u0 || tile == 0);
-            const bool x_done = (u + 1 == u1 || tile == tiles - 1);
             cur.advance(tiles, (m_rows + R - 1) / R);
-            if (fresh && ++xb == NX) xb = 0;
-            if (fresh && xb == 0) x_ph ^= 1u;
             const int rows_here = min(R, m_rows - pass0);
             if (++s == S) s = 0;
             if (s == 0) w_ph ^= 1u;
-            const unsigned char* xbuf = xs + (size_t)xb * R * x_stride;
-            float* adjb = adjg + (size_t)xb * KB * R;
-            if (fresh) {                               // new rows: each group forms its own copy of the corrections
-                if (!mbar_wait(&x_full[xb], x_ph, abort_flag, p.status)) ok = false;
-                // adj[kb][n] = -136 * sum of the row's activations over block kb (removes the code bias after the MMA);
-                // a block is 16 chunks of 8 values: the 16 lanes of a half-warp hold one block of one row
-                const int chunks_per_row = K >> 3;
-                for (int nn = 0; nn < rows_here; ++nn) {
-                    const unsigned char* xrow = xbuf + (size_t)nn * x_stride;
-                    for (int base = cw * 32; base < chunks_per_row; base += kGroupThreads) {
-                        const int ck = base + lane;
-                        uint4 v = make_uint4(0, 0, 0, 0);
-                        if (ck < chunks_per_row) v = *reinterpret_cast<const uint4*>(xrow + ck * 16);
-                        float sx = sum8_bf16(v);
+            if (fresh) {
+                if (NX == 2) xb ^= 1;
+                else rows_sync();                      // everybody is done with the rows in the only buffer
+                if (!GATEUP && !dep) {
+                    grid_dependency_wait();            // the gate/up kernel's activations are complete and visible
+                    dep = true;
+                }
+                // With two buffers the one written here was last read two passes ago, and every warp has been past that
+                // since the previous pass's barrier.
+                unsigned char* xw = xs + (size_t)xb * R * x_stride + l16 * 16;
+                float2* cwr = cst + (size_t)xb * KB * R;
+                const int items = rows_here * KB;
+                constexpr int FL = 4;                  // items in flight per half-warp
+                for (int it0 = hw; it0 - (lane >> 4) < items; it0 += 2 * kConsumerWarps * FL) {
+                    uint4 raw[FL];
 #pragma unroll
-                        for (int m = 8; m >= 1; m >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, m);
-                        if (ck < chunks_per_row && (ck & 15) == 0) adjb[(ck >> 4) * R + nn] = -136.f * sx;
+                    for (int f = 0; f < FL; ++f) {
+                        const int it = it0 + 2 * kConsumerWarps * f;
+                        raw[f] = make_uint4(0, 0, 0, 0);
+                        if (it < items) {
+                            const int r = row0 + pass0 + it / KB;
+                            const size_t src = GATEUP ? (size_t)(a.perm[r] / a.top_k) : (size_t)r;
+                            raw[f] = reinterpret_cast<const uint4*>(p.x_src + src * K + (it % KB) * kGroup)[l16];
+                        }
+                    }
+#pragma unroll
+                    for (int f = 0; f < FL; ++f) {
+                        const int it = it0 + 2 * kConsumerWarps * f;
+                        if (it - (lane >> 4) >= items) break;          // the same for the whole warp
+                        float2 k2;
+                        const uint4 x = f16_block(raw[f], k2);
+                        if (it < items) {
+                            const int r = it / KB, kb = it % KB;
+                            *reinterpret_cast<uint4*>(xw + (size_t)r * x_stride + kb * kGroup * 2) = x;
+                            if (l16 == 0) cwr[kb * R + r] = k2;
+                        }
                     }
                 }
-                // rows beyond the group's last are zeroed once per staging (both consumer groups write the same zeros:
-                // each reads them only after its own barrier below; no copy targets these rows until every warp
-                // has released the buffer), so the fragment loads of the MMA loop need no row predicate
-                for (int nn = rows_here; nn < R; ++nn) {
-                    unsigned char* xrow = const_cast<unsigned char*>(xbuf) + (size_t)nn * x_stride;
-                    for (int ck = cw * 32 + lane; ck < chunks_per_row; ck += kGroupThreads)
-                        *reinterpret_cast<uint4*>(xrow + ck * 16) = make_uint4(0, 0, 0, 0);
+                if (!GATEUP && warp == 0 && lane < rows_here) {
+                    const int pair = a.perm[row0 + pass0 + lane];
+                    rowinfo[xb * R + lane] = make_int2(pair, __float_as_int(p.topk_w[pair]));
                 }
-                group_sync(grp);
+                rows_sync();
             }
-            SPROF(long long c1 = clock64(); t_x += c1 - c0;)
-            if (!mbar_wait(&w_full[s], w_ph, abort_flag, p.status)) ok = false;
-            SPROF(long long c2 = clock64(); t_w += c2 - c1;)
-            if ((n & 1) != grp) {                      // the other group's unit: nothing of this warp reads it
-                if (lane == 0) {
-                    mbar_arrive(&w_empty[s]);
-                    if (x_done) mbar_arrive(&x_empty[xb]);             // this warp's earlier reads of the rows are complete
-                }
+            ok = mbar_wait_warp(w_full_a + 8 * s, w_ph, abort_flag, p.status) && ok;
+            if (n % kGroups != grp) {                      // the other group's unit: nothing of this warp reads it
+                if (elect_one()) mbar_arrive_at(w_empty_a + 8 * s);
                 continue;
             }
-            const unsigned char* stage = wst + (size_t)s * stage_bytes;
-            float tot[NMW][NCH][4];
-#pragma unroll
-            for (int m = 0; m < NMW; ++m)
-#pragma unroll
-                for (int ch = 0; ch < NCH; ++ch)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) tot[m][ch][i] = 0.f;
-#pragma unroll
-            for (int b = 0; b < (FIXED ? BPWc : bpw); ++b) {
-                const int kb = ks * bpw + b;
-                uint4 wv[NMW][2];
-                uint32_t sv[NMW];
-#pragma unroll
-                for (int m = 0; m < NMW; ++m) {
-                    const int panel_local = GATEUP ? 2 * pp + (NMW == 2 ? m : mw) : pp;
-                    const unsigned char* blk = stage + ((size_t)panel_local * KB + kb) * kBlockBytes;
-                    wv[m][0] = *reinterpret_cast<const uint4*>(blk + lane * 16);
-                    wv[m][1] = *reinterpret_cast<const uint4*>(blk + 512 + lane * 16);
-                    sv[m] = *reinterpret_cast<const uint32_t*>(blk + kCodeBytes + q * 4);
-                }
-                // CHN independent accumulator chains per (matrix, chunk): the block's 8 MMAs would otherwise be one
-                // dependent chain; the chains are added in fixed order below
-                float acc[NMW][NCH][CHN][4];
-#pragma unroll
-                for (int m = 0; m < NMW; ++m)
-#pragma unroll
-                    for (int ch = 0; ch < NCH; ++ch)
-#pragma unroll
-                        for (int cc = 0; cc < CHN; ++cc)
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) acc[m][ch][cc][i] = 0.f;
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int set = 0; set < 2; ++set) {
-                        const int cc = (2 * h + set) % CHN;
-                        const int k0 = kb * kGroup + 64 * h + 32 * set + 8 * c;
-                        uint4 xv[NCH];
-#pragma unroll
-                        for (int ch = 0; ch < NCH; ++ch) {
-                            xv[ch] = *reinterpret_cast<const uint4*>(xbuf + (size_t)(8 * ch + q) * x_stride + k0 * 2);
-                        }
-#pragma unroll
-                        for (int m = 0; m < NMW; ++m) {
-                            const uint32_t wq = set ? wv[m][h].z : wv[m][h].x;        // row q
-                            const uint32_t wq8 = set ? wv[m][h].w : wv[m][h].y;       // row q + 8
-                            uint32_t a0 = code_pair(wq, 0), a1 = code_pair(wq8, 0), a2 = code_pair(wq, 4), a3 = code_pair(wq8, 4);
-#pragma unroll
-                            for (int ch = 0; ch < NCH; ++ch) mma_m16n8k16(acc[m][ch][cc], a0, a1, a2, a3, xv[ch].x, xv[ch].y);
-                            a0 = code_pair(wq, 8), a1 = code_pair(wq8, 8), a2 = code_pair(wq, 12), a3 = code_pair(wq8, 12);
-#pragma unroll
-                            for (int ch = 0; ch < NCH; ++ch) mma_m16n8k16(acc[m][ch][cc], a0, a1, a2, a3, xv[ch].z, xv[ch].w);
-                        }
-                    }
-                float2 cr[NCH];
-#pragma unroll
-                for (int ch = 0; ch < NCH; ++ch)
-                    cr[ch] = *reinterpret_cast<const float2*>(adjb + (size_t)kb * R + 8 * ch + 2 * c);
-#pragma unroll
-                for (int m = 0; m < NMW; ++m) {        // post-scale the block's integer-valued sums (Eq. 3 scale)
-                    const __half2 sc = *reinterpret_cast<const __half2*>(&sv[m]);
-                    const float s_lo = __low2float(sc), s_hi = __high2float(sc);
-#pragma unroll
-                    for (int ch = 0; ch < NCH; ++ch) {
-                        float sum[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            sum[i] = acc[m][ch][0][i];
-#pragma unroll
-                            for (int cc = 1; cc < CHN; ++cc) sum[i] += acc[m][ch][cc][i];
-                        }
-                        tot[m][ch][0] = fmaf(s_lo, sum[0] + cr[ch].x, tot[m][ch][0]);
-                        tot[m][ch][1] = fmaf(s_lo, sum[1] + cr[ch].y, tot[m][ch][1]);
-                        tot[m][ch][2] = fmaf(s_hi, sum[2] + cr[ch].x, tot[m][ch][2]);
-                        tot[m][ch][3] = fmaf(s_hi, sum[3] + cr[ch].y, tot[m][ch][3]);
-                    }
-                }
-            }
-            // this warp is done with the weight stage, and with the rows when the next unit stages others
-            __syncwarp();
-            SPROF(long long c3 = clock64(); t_mma += c3 - c2; ++n_mine;)
-            if (lane == 0) {
-                mbar_arrive(&w_empty[s]);
-                if (x_done) mbar_arrive(&x_empty[xb]);
-            }
-            if (!exchange) {
-                // no K split and both matrices here: the warp finishes its panel from registers
-                if (ok) {
-#pragma unroll
-                    for (int ch = 0; ch < NCH; ++ch)
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int nn = pass0 + 8 * ch + 2 * c + (i & 1);
-                            if (nn >= m_rows) continue;
-                            const int orow = (tile * PP + pp) * kPanelRows + q + 8 * (i >> 1);
-                            if (GATEUP) {
-                                const float gv = tot[0][ch][i], uv = tot[NMW - 1][ch][i];
-                                p.act_out[(size_t)(row0 + nn) * a.I + orow] = __float2bfloat16_rn(gv / (1.f + __expf(-gv)) * uv);
-                            } else {
-                                const int pair = a.perm[row0 + nn];
-                                p.y_out[(size_t)pair * a.H + orow] = p.topk_w[pair] * tot[0][ch][i];
-                            }
-                        }
-                }
-                continue;
-            }
-            // Partials cross shared memory once (buffer alternates with the group's units, so one barrier per unit
-            // is enough); then warp j finishes the slices (panel, chunk, fragment word) = j, j + 8, ...: the sum
-            // over the K ranges in ascending order, SwiGLU or routing weight, store.
-            float* pb = part + (size_t)(grp * 2 + (mine_cnt & 1)) * part_words;
+            const unsigned char* w0 = w_lane + (size_t)s * stage_bytes;
+            const unsigned char* s0 = s_lane + (size_t)s * stage_bytes;
+            const unsigned char* x0 = x_lane + (size_t)xb * R * x_stride;
+            const float2* c0 = c_lane + (size_t)xb * KB * R;
+            float* pb = partg + (mine_cnt & 1) * part_words;
             ++mine_cnt;
+            const int nt = (rows_here + 7) >> 3;
+            // the unit's blocks for NT x 8 rows (columns of rows that the pass does not have hold whatever the buffer does:
+            // columns are independent and theirs are never stored)
+            auto unit = [&](auto NTt) {
+                constexpr int NT = decltype(NTt)::value;
+                float tot[NT][4];
 #pragma unroll
-            for (int m = 0; m < NMW; ++m) {
-                const int mg = (NMW == 2) ? m : mw;                    // matrix index inside the tile
+                for (int j = 0; j < NT; ++j)
 #pragma unroll
-                for (int ch = 0; ch < NCH; ++ch)
+                    for (int i = 0; i < 4; ++i) tot[j][i] = 0.f;
+                [[maybe_unused]] const int nb = kb_hi - kb_lo;
+                [[maybe_unused]] constexpr int NBc = FIXED ? KBc / (8 / ((PPc > 0 ? PPc : 1) * NM)) : 1;
+                auto block = [&](int b) {
+                    const uint4 w[2] = {*reinterpret_cast<const uint4*>(w0 + b * kBlockBytes),
+                                        *reinterpret_cast<const uint4*>(w0 + b * kBlockBytes + 512)};
+                    const uint32_t sv = *reinterpret_cast<const uint32_t*>(s0 + b * kBlockBytes);
+                    float d[NT][2][4];                                 // two chains per column tile
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        pb[((((pp * NM + mg) * KS + ks) * NCH + ch) * 4 + i) * 32 + lane] = tot[m][ch][i];
-            }
+                    for (int j = 0; j < NT; ++j)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) d[j][0][i] = d[j][1][i] = 0.f;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int set = 0; set < 2; ++set) {
+                            const CodeFrag cf(set ? w[h].z : w[h].x, set ? w[h].w : w[h].y);
+                            uint4 x[NT];
+#pragma unroll
+                            for (int j = 0; j < NT; ++j)
+                                x[j] = *reinterpret_cast<const uint4*>(x0 + (size_t)(8 * j) * x_stride + (b * kGroup + 64 * h + 32 * set) * 2);
+#pragma unroll
+                            for (int j = 0; j < NT; ++j) cf.first(d[j][set], x[j]);
+#pragma unroll
+                            for (int j = 0; j < NT; ++j) cf.second(d[j][set], x[j]);
+                        }
+                    const float2 sc = scales16(sv);
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) {
+                        const float4 k4 = *reinterpret_cast<const float4*>(c0 + b * R + 8 * j);     // rows 8 j + 2 c and + 1
+                        tot[j][0] = fmaf(sc.x, fmaf(d[j][0][0] + d[j][1][0], k4.x, k4.y), tot[j][0]);
+                        tot[j][1] = fmaf(sc.x, fmaf(d[j][0][1] + d[j][1][1], k4.z, k4.w), tot[j][1]);
+                        tot[j][2] = fmaf(sc.y, fmaf(d[j][0][2] + d[j][1][2], k4.x, k4.y), tot[j][2]);
+                        tot[j][3] = fmaf(sc.y, fmaf(d[j][0][3] + d[j][1][3], k4.z, k4.w), tot[j][3]);
+                    }
+                };
+                if constexpr (FIXED) {
+#pragma unroll
+                    for (int b = 0; b < NBc; ++b) block(b);
+                } else {
+#pragma unroll 2
+                    for (int b = 0; b < nb; ++b) block(b);
+                }
+                __syncwarp();
+                if (elect_one()) mbar_arrive_at(w_empty_a + 8 * s);    // this warp is done with the weight stage
+                // Partials cross shared memory once (buffer alternates with the group's units, so one barrier per unit
+                // is enough); then the warps finish the slices (panel, N-tile, row half): the sum over the K ranges in
+                // ascending order, SwiGLU or routing weight, store.
+                float* pw = pb + (size_t)((pp * NM + mw) * KS + ks) * (NTM * 128) + lane;
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) pw[(4 * j + i) * 32] = tot[j][i];
+            };
+            if constexpr (NTM == 1) unit(std::integral_constant<int, 1>());
+            else if (nt == 1) unit(std::integral_constant<int, 1>());
+            else unit(std::integral_constant<int, 2>());
             group_sync(grp);
-            const int slices = PP * NCH * 4;
+            const int slices = PP * nt * 4;
             for (int sl = cw; sl < slices; sl += kGroupWarps) {
-                const int i = sl & 3, ch = (sl >> 2) % NCH, spp = sl / (4 * NCH);
+                const int spp = FIXED && PPc == 1 ? 0 : sl / (4 * nt), ji = sl - spp * 4 * nt;
                 float v[NM];
 #pragma unroll
                 for (int mg = 0; mg < NM; ++mg) {
-                    float acc1 = 0.f;
-                    for (int s2 = 0; s2 < KS; ++s2)
-                        acc1 += pb[((((spp * NM + mg) * KS + s2) * NCH + ch) * 4 + i) * 32 + lane];
-                    v[mg] = acc1;
+                    const float* pr = pb + (size_t)((spp * NM + mg) * KS) * (NTM * 128) + ji * 32 + lane;
+                    float sum = pr[0];
+                    for (int k2 = 1; k2 < KS; ++k2) sum += pr[k2 * (NTM * 128)];
+                    v[mg] = sum;
                 }
-                const int nn = pass0 + 8 * ch + 2 * c + (i & 1);
-                if (nn >= m_rows || !ok) continue;
-                const int orow = (tile * PP + spp) * kPanelRows + q + 8 * (i >> 1);
+                const int rr = 8 * (ji >> 2) + 2 * c + (ji & 1);       // row of the pass
+                if (rr >= rows_here || !ok) continue;
+                const int orow = (tile * PP + spp) * kPanelRows + q + 8 * ((ji >> 1) & 1);
                 if (GATEUP) {
                     const float gv = v[0], uv = v[NM - 1];
-                    p.act_out[(size_t)(row0 + nn) * a.I + orow] = __float2bfloat16_rn(gv / (1.f + __expf(-gv)) * uv);
+                    p.act_out[(size_t)(row0 + pass0 + rr) * a.I + orow] = __float2bfloat16_rn(gv / (1.f + __expf(-gv)) * uv);
                 } else {
-                    const int pair = a.perm[row0 + nn];
-                    p.y_out[(size_t)pair * a.H + orow] = p.topk_w[pair] * v[0];
+                    const int2 ri = rowinfo[xb * R + rr];
+                    p.y_out[(size_t)ri.x * a.H + orow] = __int_as_float(ri.y) * v[0];
                 }
             }
-            SPROF(t_ep += clock64() - c3;)
         }
-        SPROF(if (blockIdx.x == 7 && lane == 0 && (cw == 0 || cw == 5))
-                  printf("%s grp %d warp %d: units %d mine %d total %lld xwait %lld wwait %lld mma %lld epi %lld\n", GATEUP ? "gu" : "dn",
-                         grp, cw, u1 - u0, n_mine, clock64() - t_begin, t_x, t_w, t_mma, t_ep);)
     }
 }
 
-template <int NCH, bool GATEUP>
+template <int R, bool GATEUP>
 bool launch_stream_cfg(const GemmArgs& a, const __nv_bfloat16* x, __nv_bfloat16* act, const float* w, float* y, int* status,
                        int max_groups, bool dependent, cudaStream_t st) {
     constexpr int NM = GATEUP ? 2 : 1;
     StreamGeom g;
-    if (!stream_geometry(GATEUP ? a.H : a.I, GATEUP ? a.I : a.H, NM, NCH, &g)) return false;
-    void (*kern)(const StreamArgs) = stream_gemm_kernel<NCH, GATEUP, 1>;
+    if (!stream_geometry(GATEUP ? a.H : a.I, GATEUP ? a.I : a.H, NM, R, &g)) return false;
+    void (*kern)(const StreamArgs) = stream_gemm_kernel<R, GATEUP>;
     int variant = 0;
-    if (GATEUP && g.NMW == 2) {
-        kern = stream_gemm_kernel<NCH, GATEUP, GATEUP ? 2 : 1>;
-        variant = 1;
-    }
 #ifndef EXMOE_STREAM_GENERIC_ONLY
     // OLMoE's two matrices with their geometry as literals (d_model 2048: 16 blocks, one panel pair per tile, K in four
     // ranges; d_ff 1024: 8 blocks, four panels per tile, K in two ranges)
     const int KBv = (GATEUP ? a.H : a.I) / kGroup;
-    if (GATEUP && g.NMW == 1 && KBv == 16 && g.PP == 1 && g.KS == 4) {
-        kern = stream_gemm_kernel<NCH, GATEUP, 1, 16, 1, 4>;
-        variant = 2;
-    } else if (!GATEUP && KBv == 8 && g.PP == 4 && g.KS == 2) {
-        kern = stream_gemm_kernel<NCH, GATEUP, 1, 8, 4, 2>;
-        variant = 2;
+    if (GATEUP && KBv == 16 && g.PP == 1) {
+        kern = stream_gemm_kernel<R, GATEUP, 16, 1>;
+        variant = 1;
+    } else if (!GATEUP && KBv == 8 && g.PP == 4) {
+        kern = stream_gemm_kernel<R, GATEUP, 8, 4>;
+        variant = 1;
     }
 #endif
-    static SmemOnce smem_once[3];
+    static SmemOnce smem_once[2];
     allow_smem(kern, (int)kSmemLimit, smem_once[variant]);
     int sms = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
@@ -621,7 +542,8 @@ bool launch_stream_cfg(const GemmArgs& a, const __nv_bfloat16* x, __nv_bfloat16*
     p.x_stride = g.x_stride;
     p.off_x = (uint32_t)g.off_x;
     p.off_part = (uint32_t)g.off_part;
-    p.off_adj = (uint32_t)g.off_adj;
+    p.off_cst = (uint32_t)g.off_cst;
+    p.off_row = (uint32_t)g.off_row;
     p.off_bar = (uint32_t)g.off_bar;
     const long long units = (long long)max_groups * g.tiles;          // the wave's units when every group takes one pass
     cudaLaunchConfig_t lc{};
@@ -643,12 +565,10 @@ bool launch_stream_cfg(const GemmArgs& a, const __nv_bfloat16* x, __nv_bfloat16*
 
 bool stream_supported(int H, int I) {
     StreamGeom g;
-    return stream_geometry(H, I, 2, 1, &g) && stream_geometry(I, H, 1, 1, &g);
+    return stream_geometry(H, I, 2, 8, &g) && stream_geometry(I, H, 1, 8, &g);
 }
 
-// One wave on the streaming kernels: eight rows of a group per pass.  (Sixteen rows per pass, NCH = 2, halve the
-// shared-memory reads of the weights per row but double the MMAs of every unit; with a few rows per expert that
-// measured slower at every batch size in this path's range.)
+// One wave on the streaming kernels: passes of eight rows of a group.
 bool launch_stream_wave(const GemmArgs& a, const __nv_bfloat16* hidden, __nv_bfloat16* act, const float* topk_w, float* y,
                         int* status, int max_groups, bool gateup, bool down, cudaStream_t st) {
     bool ok = true;
@@ -657,12 +577,12 @@ bool launch_stream_wave(const GemmArgs& a, const __nv_bfloat16* hidden, __nv_bfl
 #else
     const bool entry_dependent = false;
 #endif
-#ifndef EXMOE_STREAM_NCH
-#define EXMOE_STREAM_NCH 1
+#ifndef EXMOE_STREAM_ROWS
+#define EXMOE_STREAM_ROWS 8
 #endif
-    if (gateup) ok = launch_stream_cfg<EXMOE_STREAM_NCH, true>(a, hidden, act, topk_w, y, status, max_groups, entry_dependent, st);
+    if (gateup) ok = launch_stream_cfg<EXMOE_STREAM_ROWS, true>(a, hidden, act, topk_w, y, status, max_groups, entry_dependent, st);
     // a programmatic dependent only when the gate/up kernel of the same wave was launched just before it
-    if (down && ok) ok = launch_stream_cfg<EXMOE_STREAM_NCH, false>(a, act, act, topk_w, y, status, max_groups, gateup, st);
+    if (down && ok) ok = launch_stream_cfg<EXMOE_STREAM_ROWS, false>(a, act, act, topk_w, y, status, max_groups, gateup, st);
     return ok;
 }
 
