@@ -65,9 +65,9 @@ struct exmoe_cache {
     int* arrive;                              // fused-combine arrival counters of the small path
     size_t arrive_words;
     bool last_small;
-    bool last_pair;
+    bool last_pair;                           // ... which formed no plan (per-pair or streaming kernels)
     int last_path;                            // EXMOE_PATH_* of the most recent forward
-    int32_t* saved_ids;                       // ids of the last pairwise call (plan materialised on request)
+    int32_t* saved_ids;                       // ids of the last call without a grouping kernel (plan materialised on request)
     bool stream_ok;                           // the shape fits the streaming middle-regime kernels
     bool pair_ok, small_ok;                   // ... the per-pair kernels / the in-CTA-grouping kernels (shared memory)
     void* tc_scratch;                         // tile list of the tensor-core path
@@ -175,7 +175,7 @@ static void carve_workspace(exmoe_cache* c, uint8_t* ws, size_t* total) {
     c->y = k.take<float>((size_t)c->max_pairs * s.d_model);
     c->arrive_words = (size_t)(kSmallMaxPairs / s.top_k + 1) * (s.d_model / kPanelRows);
     c->arrive = k.take<int>(c->arrive_words);
-    c->saved_ids = k.take<int32_t>(kPairMaxPairs);
+    c->saved_ids = k.take<int32_t>(std::max(kPairMaxPairs, std::min(c->max_pairs, kStreamMaxPairs)));
     c->tc_scratch = k.take<uint8_t>(prefill_scratch_bytes(c->max_pairs, E));
     c->xg = (c->max_pairs > kSmallMaxPairs || !c->small_ok) ? k.take<__nv_bfloat16>((size_t)c->max_pairs * s.d_model) : nullptr;
     c->tc_maps.dev = c->xg ? k.take<uint8_t>(kPrefillMapBytes) : nullptr;
@@ -439,7 +439,9 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
     }
     // timing runs that launch one kernel kind reuse the plan, grouped rows and tile list of the previous full call
     const bool build_plan = (c->prof_only == 0);
-    if (!small && build_plan) {
+    const bool use_stream = !small && c->stream_ok && P <= kStreamMaxPairs;
+    const bool own_plan = use_stream && identity && c->n_keys <= kStreamOwnPlanKeys;     // the kernels group the ids themselves
+    if (!small && build_plan && !own_plan) {
         ProfScope ps(c, PROF_PLAN, st);
         launch_group(s, C, c->n_keys, c->max_waves, identity, topk_ids, P, c->plan, c->d_status, st);
     }
@@ -474,6 +476,9 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
     a.key_miss = c->plan.key_miss;
     a.group_filter = 0;
     a.direct_keys = (C == E && c->n_keys <= 128) ? c->n_keys : 0;
+    a.ids = own_plan ? topk_ids : nullptr;
+    a.n_pairs = P;
+    a.keep_ids = c->saved_ids;
     a.num_slots = C;
     a.top_k = k;
     a.H = s.d_model;
@@ -481,8 +486,7 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
 
     bool tiles_fused = false;
     const bool pairwise = small && P <= kPairMaxPairs && n_waves == 1 && c->pair_ok;
-    c->last_pair = pairwise;
-    const bool use_stream = !small && c->stream_ok && P <= kStreamMaxPairs;
+    c->last_pair = pairwise || own_plan;
     const bool small_n = P <= kPrefillSmallNMaxPairs;      // tensor-core path: which kernel shape
     c->last_path = pairwise ? EXMOE_PATH_PAIR : small ? EXMOE_PATH_SMALL : use_stream ? EXMOE_PATH_STREAM
                    : small_n ? EXMOE_PATH_TENSOR_SMALL_N : EXMOE_PATH_TENSOR;
@@ -773,7 +777,7 @@ int exmoe_debug_last_plan(exmoe_cache* c, int layer, int32_t* n_active, int32_t*
     if (cudaDeviceSynchronize() != cudaSuccess) return EXMOE_ERR_CUDA;
     const int E = c->shape.num_experts;
     if (c->last_pair) {
-        // the pairwise path never groups: run the grouping kernel now on the ids it kept
+        // the call formed no plan: run the grouping kernel now on the ids it kept
         launch_group(c->shape, c->C, c->n_keys, c->max_waves, c->C == E, c->saved_ids, c->last_T * c->shape.top_k,
                      c->plan, c->d_status, nullptr);
         if (cudaDeviceSynchronize() != cudaSuccess) return EXMOE_ERR_CUDA;

@@ -63,6 +63,10 @@ struct GemmArgs {
     int direct_keys;            // > 0: every key 0 .. direct_keys-1 is a (possibly empty) group of the call's only wave
                                 // (all experts resident, key = expert id): kernels may read counts / offsets by key at
                                 // once instead of going through wave_start and group_keys first
+    // Streaming kernels, all experts resident: the ids of the call (null: read the plan).  Every CTA then groups them itself.
+    const int32_t* ids;
+    int n_pairs;
+    int32_t* keep_ids;          // copy of the ids, from which the plan can be materialised on request
     int num_slots;              // C (key % C = slot)
     int top_k;
     int H, I;
@@ -125,6 +129,7 @@ void launch_group(const exmoe_shape& s, int C, int n_keys, int max_waves, bool i
 #define EXMOE_STREAM_MAX_PAIRS 640
 #endif
 constexpr int kStreamMaxPairs = EXMOE_STREAM_MAX_PAIRS;   // above: tensor-core path
+constexpr int kStreamOwnPlanKeys = 128;                    // most experts whose pairs the streaming kernels group themselves
 bool stream_supported(int H, int I);
 bool launch_stream_wave(const GemmArgs& a, const __nv_bfloat16* hidden, __nv_bfloat16* act, const float* topk_w, float* y,
                         int* status, int max_groups, bool gateup, bool down, cudaStream_t st);

@@ -74,7 +74,9 @@ struct StreamGeom {
 };
 
 constexpr size_t kBarBytes = 2 * kMaxStages * 8 + 64;                 // mbarriers, abort flag, unit range
-constexpr size_t kCtrlBytes = kBarBytes + (size_t)kMetaGroups * 16;   // + plan entries of the CTA's groups
+constexpr int kInlineKeys = kStreamOwnPlanKeys;
+constexpr size_t kCtrlBytes = kBarBytes + (size_t)kMetaGroups * 16    // + plan entries of the CTA's groups
+                              + (size_t)kStreamMaxPairs * 4 + kInlineKeys * 4 + kConsumerWarps * 8 * 4;
 
 #ifndef EXMOE_STREAM_PP
 #define EXMOE_STREAM_PP 0                                              // 0: choose; 1/2/4/8: force where feasible (timing experiments)
@@ -172,7 +174,14 @@ stream_gemm_kernel(const StreamArgs p) {
     uint64_t* w_empty = w_full + kMaxStages;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(w_empty + kMaxStages);
     int* s_range = const_cast<int*>(abort_flag) + 4;                   // [0] first unit, [1] end
-    const int4* meta = reinterpret_cast<const int4*>(smem + p.off_bar + kBarBytes);   // (key, rows, first row, first unit)
+    int4* meta_w = reinterpret_cast<int4*>(smem + p.off_bar + kBarBytes);             // (slot, rows, first row, first unit)
+    const int4* meta = meta_w;
+    int* s_key = reinterpret_cast<int*>(meta_w + kMetaGroups);         // [pairs] plan formed here: key of every pair
+    int* s_cnt = s_key + kStreamMaxPairs;                              // [kInlineKeys] pairs per key
+    int* s_rows = s_cnt + kInlineKeys;                                 // [consumer warps][8] pairs of a pass's rows
+    // With every expert resident (key = expert id) and a few hundred pairs, every CTA forms the plan by itself from the ids:
+    // no grouping kernel before this one (2.5 us, and a launch), one L2 round trip before the first weight copy.
+    const bool own_plan = a.ids != nullptr;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = warp_uniform(tid >> 5);
     if (tid == 32) {
@@ -183,13 +192,80 @@ stream_gemm_kernel(const StreamArgs p) {
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (own_plan && tid < kInlineKeys) s_cnt[tid] = 0;
 #ifndef EXMOE_STREAM_NO_ENTRY_PDL
     // The gate/up kernel is itself launched as a programmatic dependent (of the grouping kernel when that runs
-    // just before it): its CTAs are placed and their barriers initialised while the plan is still being
-    // written; the plan is read only after this wait.
+    // just before it, else of whatever does): its CTAs are placed and their barriers initialised while the ids or the plan
+    // are still being written; they are read only after this wait.  The down kernel reads the ids and the plan without
+    // waiting: it starts when every gate/up CTA is past its own wait.
     if (GATEUP) grid_dependency_wait();
 #endif
-    if (warp == 0) {
+    if (own_plan) {
+        constexpr int PT = (kStreamMaxPairs + kStreamThreads - 1) / kStreamThreads;
+        int id[PT];
+#pragma unroll
+        for (int i = 0; i < PT; ++i) {
+            const int pr = tid + i * kStreamThreads;
+            id[i] = pr < a.n_pairs ? a.ids[pr] : -1;
+        }
+        __syncthreads();
+        bool bad = false;
+#pragma unroll
+        for (int i = 0; i < PT; ++i) {
+            const int pr = tid + i * kStreamThreads;
+            if (pr >= a.n_pairs) continue;
+            const bool valid = id[i] >= 0 && id[i] < a.direct_keys;
+            s_key[pr] = valid ? id[i] : -1;
+            if (valid) atomicAdd(&s_cnt[id[i]], 1);
+            bad |= !valid;
+            if (GATEUP && blockIdx.x == 0) a.keep_ids[pr] = id[i];     // the plan can be materialised from these on request
+        }
+        if (GATEUP && blockIdx.x == 0 && bad) atomicExch(p.status, EXMOE_ERR_BAD_EXPERT_ID);
+        __syncthreads();
+        if (warp == 0) {
+            // rows and passes before each key in one scan: passes << 16 | rows
+            constexpr int CH = kInlineKeys / 32;
+            int rows[CH], incl[CH];
+#pragma unroll
+            for (int j = 0; j < CH; ++j) {
+                rows[j] = s_cnt[32 * j + lane];
+                incl[j] = ((rows[j] + R - 1) / R) << 16 | rows[j];
+            }
+#pragma unroll
+            for (int m = 1; m < 32; m <<= 1)
+#pragma unroll
+                for (int j = 0; j < CH; ++j) {
+                    const int v = __shfl_up_sync(0xffffffffu, incl[j], m);
+                    if (lane >= m) incl[j] += v;
+                }
+            int before[CH + 1];
+            before[0] = 0;
+#pragma unroll
+            for (int j = 0; j < CH; ++j) before[j + 1] = before[j] + __shfl_sync(0xffffffffu, incl[j], 31);
+            const int U = (before[CH] >> 16) * tiles, share = U / (int)gridDim.x, longer = U - share * (int)gridDim.x;
+            int u0 = share * (int)blockIdx.x + min((int)blockIdx.x, longer);       // the first CTAs take one more
+            int u1 = u0 + share + ((int)blockIdx.x < longer ? 1 : 0);
+            int found = 0;
+#pragma unroll
+            for (int j = 0; j < CH; ++j) {
+                const int passes = (rows[j] + R - 1) / R, excl = before[j] + incl[j] - (passes << 16 | rows[j]);
+                const int ustart = (excl >> 16) * tiles, uend = ustart + passes * tiles;
+                const bool overlap = passes > 0 && ustart < u1 && uend > u0;
+                const unsigned ballot = __ballot_sync(0xffffffffu, overlap);
+                const int idx = found + __popc(ballot & ((1u << lane) - 1u));
+                if (overlap && idx < kMetaGroups) meta_w[idx] = make_int4(32 * j + lane, rows[j], excl & 0xffff, ustart);
+                found += __popc(ballot);
+            }
+            if (found > kMetaGroups) {
+                if (lane == 0) atomicExch(p.status, EXMOE_ERR_STATE);
+                u1 = u0;
+            }
+            if (lane == 0) {
+                s_range[0] = u0;
+                s_range[1] = u1;
+            }
+        }
+    } else if (warp == 0) {
         // This CTA's share of the wave's units, and the plan entries of the groups it touches (usually one or
         // two).  The plan entries of up to 32 * kScanChunks active groups are fetched in one go and kept in
         // registers for both steps (count the units; find the overlapping groups); beyond that they are re-read.
@@ -249,7 +325,6 @@ stream_gemm_kernel(const StreamArgs p) {
         int u0 = share * (int)blockIdx.x + min((int)blockIdx.x, longer);
         int u1 = u0 + share + ((int)blockIdx.x < longer ? 1 : 0);
         int run = 0, found = 0;
-        int4* meta_w = const_cast<int4*>(meta);
         for (int chunk = 0; 32 * chunk < n_groups && u0 < u1; ++chunk) {
             int key, rows, row0;
             entry(chunk, key, rows, row0);
@@ -363,8 +438,21 @@ stream_gemm_kernel(const StreamArgs p) {
                 }
                 // With two buffers the one written here was last read two passes ago, and every warp has been past that
                 // since the previous pass's barrier.
+                static_assert(R == 8, "the list of a pass's pairs");
                 unsigned char* xw = xs + (size_t)xb * R * x_stride + l16 * 16;
                 float2* cwr = cst + (size_t)xb * KB * R;
+                int* rows_w = s_rows + warp * 8;
+                if (own_plan && (GATEUP || warp == 0)) {               // this warp's own list of the pass's pairs, in pair order
+                    int seen = -pass0;
+                    for (int p0 = 0; p0 < a.n_pairs && seen < rows_here; p0 += 32) {
+                        const bool hit = p0 + lane < a.n_pairs && s_key[p0 + lane] == gm.x;
+                        const unsigned b = __ballot_sync(0xffffffffu, hit);
+                        const int rank = seen + __popc(b & ((1u << lane) - 1u));
+                        if (hit && rank >= 0 && rank < rows_here) rows_w[rank] = p0 + lane;
+                        seen += __popc(b);
+                    }
+                    __syncwarp();
+                }
                 const int items = rows_here * KB;
                 constexpr int FL = 4;                  // items in flight per half-warp
                 for (int it0 = hw; it0 - (lane >> 4) < items; it0 += 2 * kConsumerWarps * FL) {
@@ -374,8 +462,8 @@ stream_gemm_kernel(const StreamArgs p) {
                         const int it = it0 + 2 * kConsumerWarps * f;
                         raw[f] = make_uint4(0, 0, 0, 0);
                         if (it < items) {
-                            const int r = row0 + pass0 + it / KB;
-                            const size_t src = GATEUP ? (size_t)(a.perm[r] / a.top_k) : (size_t)r;
+                            const int r = it / KB, row = row0 + pass0 + r;
+                            const size_t src = GATEUP ? (size_t)((own_plan ? rows_w[r] : a.perm[row]) / a.top_k) : (size_t)row;
                             raw[f] = reinterpret_cast<const uint4*>(p.x_src + src * K + (it % KB) * kGroup)[l16];
                         }
                     }
@@ -393,7 +481,7 @@ stream_gemm_kernel(const StreamArgs p) {
                     }
                 }
                 if (!GATEUP && warp == 0 && lane < rows_here) {
-                    const int pair = a.perm[row0 + pass0 + lane];
+                    const int pair = own_plan ? rows_w[lane] : a.perm[row0 + pass0 + lane];
                     rowinfo[xb * R + lane] = make_int2(pair, __float_as_int(p.topk_w[pair]));
                 }
                 rows_sync();
