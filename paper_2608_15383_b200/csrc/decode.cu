@@ -6,11 +6,10 @@
 // `PP` 16-row panels (gate/up: panel pairs) of one active expert and splits K over `KS` warps per
 // panel; each warp issues ALL of its 128-bit weight loads up front (NB blocks x 2 halves per
 // matrix: up to 8 KB in flight per warp), stages the group's activation rows in shared memory while
-// they fly, then dequantises in registers (one shift and one lop3 per code pair; the code bias of 136 is
-// removed after the MMA with a per-block correction formed while the activations are staged) straight
-// into m16n8k16 fragments: the packed layout IS the fragment order, so no shuffle or shared-memory
-// round trip touches the weights.  Per 128-wide group the integer-valued partial sums are scaled
-// in binary32 by the FP16 group scale (post-scaling: codes and activations enter the MMA exactly).
+// they fly, then feeds the codes to the MMA as FP16 subnormals (one shift and four ANDs per word, see frag.cuh; the
+// activations are converted and their block constants formed while they are staged): the packed layout IS the
+// fragment order, so no shuffle or shared-memory round trip touches the weights.  Per 128-wide group the partial sums
+// are scaled in binary32 by the FP16 group scale (post-scaling: codes and activations enter the MMA exactly).
 // K-split partials are reduced through shared memory in a fixed order.
 //
 // Two flavours share the body:
@@ -159,8 +158,8 @@ decode_gemm_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ x
     const int x_stride = K * 2 + 64;                   // bytes; +64 keeps 128-bit fragment loads conflict-free
     unsigned char* xs = smem;
     float* red = reinterpret_cast<float*>(smem + (size_t)8 * NCH * x_stride);   // [KS-1][PP][NM][NCH][32][4]
-    float* adj = red + (size_t)(KS - 1) * PP * NM * NCH * 128;                  // [KB][8*NCH]
-    int* plan_mem = reinterpret_cast<int*>(adj + (size_t)KB * 8 * NCH);
+    float2* cst = reinterpret_cast<float2*>(red + (size_t)(KS - 1) * PP * NM * NCH * 128);   // [KB][8*NCH] block constants
+    int* plan_mem = reinterpret_cast<int*>(cst + (size_t)KB * 8 * NCH);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int q = lane >> 2, c = lane & 3;
@@ -265,7 +264,7 @@ decode_gemm_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ x
                         waited = true;
                     }
                     __syncthreads();                   // previous readers of xs / red are done
-                    // also: adj[kb][n] = -136 * sum_k x[n][k] over each 128-wide block (see the block loop)
+                    // 16 lanes convert one 128-wide block of a row
                     const int chunks_per_row = K / 8;
                     const int rows_here = min(8 * NCH, m_rows - pass0);   // rows beyond are zero registers, not staged
                     const int total = rows_here * chunks_per_row;
@@ -279,20 +278,19 @@ decode_gemm_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ x
                             else if (GATEUP) src_row = (size_t)(sp.perm[lrow0 + pass0 + n] / a.top_k);
                             else src_row = (size_t)(row0 + pass0 + n);
                             v = *reinterpret_cast<const uint4*>(x_src + src_row * K + ck * 8);
-                            *reinterpret_cast<uint4*>(xs + (size_t)n * x_stride + ck * 16) = v;
                         }
-                        float sx = sum8_bf16(v);
-#pragma unroll
-                        for (int m = 8; m >= 1; m >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, m);   // 16 chunks = one block
-                        if (idx < total && (ck & 15) == 0) adj[(ck >> 4) * (8 * NCH) + n] = -136.f * sx;
+                        float2 k2;
+                        v = f16_block(v, k2);
+                        if (idx < total) {
+                            *reinterpret_cast<uint4*>(xs + (size_t)n * x_stride + ck * 16) = v;
+                            if ((ck & 15) == 0) cst[(ck >> 4) * (8 * NCH) + n] = k2;
+                        }
                     }
                     __syncthreads();
                 }
                 const int rows_here = min(8 * NCH, m_rows - pass0);
 #pragma unroll
                 for (int b = 0; b < NB; ++b) {
-                    // acc = sum (136 + q) x over the block's 128 columns (codes enter the MMA as 128 + u,
-                    // exact in BF16); adj = -136 * sum x was formed while staging; acc + adj = sum q x.
                     float acc[NM][NCH][4];
 #pragma unroll
                     for (int ch = 0; ch < NCH; ++ch)
@@ -316,31 +314,27 @@ decode_gemm_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ x
                             for (int m = 0; m < NM; ++m) {
                                 const uint32_t wq = set ? wreg[m][b][h].z : wreg[m][b][h].x;    // row q
                                 const uint32_t wq8 = set ? wreg[m][b][h].w : wreg[m][b][h].y;   // row q + 8
-                                uint32_t a0 = code_pair(wq, 0), a1 = code_pair(wq8, 0);
-                                uint32_t a2 = code_pair(wq, 4), a3 = code_pair(wq8, 4);
+                                const CodeFrag cf(wq, wq8);
 #pragma unroll
-                                for (int ch = 0; ch < NCH; ++ch) mma_m16n8k16(acc[m][ch], a0, a1, a2, a3, xb[ch].x, xb[ch].y);
-                                a0 = code_pair(wq, 8), a1 = code_pair(wq8, 8);
-                                a2 = code_pair(wq, 12), a3 = code_pair(wq8, 12);
+                                for (int ch = 0; ch < NCH; ++ch) cf.first(acc[m][ch], xb[ch]);
 #pragma unroll
-                                for (int ch = 0; ch < NCH; ++ch) mma_m16n8k16(acc[m][ch], a0, a1, a2, a3, xb[ch].z, xb[ch].w);
+                                for (int ch = 0; ch < NCH; ++ch) cf.second(acc[m][ch], xb[ch]);
                             }
                         }
                     }
-                    float2 cr[NCH];
+                    float4 k4[NCH];                    // constants of rows 2c, 2c + 1
 #pragma unroll
                     for (int ch = 0; ch < NCH; ++ch)
-                        cr[ch] = *reinterpret_cast<const float2*>(adj + (size_t)(kb0 + b) * (8 * NCH) + 8 * ch + 2 * c);
+                        k4[ch] = *reinterpret_cast<const float4*>(cst + (size_t)(kb0 + b) * (8 * NCH) + 8 * ch + 2 * c);
 #pragma unroll
-                    for (int m = 0; m < NM; ++m) {     // post-scale the group's integer-valued sums
-                        const __half2 sc = *reinterpret_cast<const __half2*>(&sreg[m][b]);
-                        const float s_lo = __low2float(sc), s_hi = __high2float(sc);
+                    for (int m = 0; m < NM; ++m) {     // post-scale the group's sums
+                        const float2 sc = scales16(sreg[m][b]);
 #pragma unroll
                         for (int ch = 0; ch < NCH; ++ch) {
-                            tot[m][ch][0] = fmaf(s_lo, acc[m][ch][0] + cr[ch].x, tot[m][ch][0]);
-                            tot[m][ch][1] = fmaf(s_lo, acc[m][ch][1] + cr[ch].y, tot[m][ch][1]);
-                            tot[m][ch][2] = fmaf(s_hi, acc[m][ch][2] + cr[ch].x, tot[m][ch][2]);
-                            tot[m][ch][3] = fmaf(s_hi, acc[m][ch][3] + cr[ch].y, tot[m][ch][3]);
+                            tot[m][ch][0] = fmaf(sc.x, fmaf(acc[m][ch][0], k4[ch].x, k4[ch].y), tot[m][ch][0]);
+                            tot[m][ch][1] = fmaf(sc.x, fmaf(acc[m][ch][1], k4[ch].z, k4[ch].w), tot[m][ch][1]);
+                            tot[m][ch][2] = fmaf(sc.y, fmaf(acc[m][ch][2], k4[ch].x, k4[ch].y), tot[m][ch][2]);
+                            tot[m][ch][3] = fmaf(sc.y, fmaf(acc[m][ch][3], k4[ch].z, k4[ch].w), tot[m][ch][3]);
                         }
                     }
                 }
@@ -455,9 +449,9 @@ token_down_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ ac
     const int K = a.I, KB = K / kGroup, k = a.top_k;
     const int x_stride = K * 2 + 64;
     unsigned char* xs = smem;                                          // [k][x_stride]
-    float* ys = reinterpret_cast<float*>(smem + (size_t)k * x_stride); // [k][16]
+    float2* cst = reinterpret_cast<float2*>(smem + (size_t)k * x_stride);        // [KB][k] block constants
+    float* ys = reinterpret_cast<float*>(cst + (size_t)KB * k);        // [k][16]
     int* s_valid = reinterpret_cast<int*>(ys + k * 16);                // [k]
-    float* adj = reinterpret_cast<float*>(s_valid + k);                // [KB][k]  -136 * block sums of the activations
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int q = lane >> 2, c = lane & 3;
     const int panels = a.H / kPanelRows;
@@ -496,8 +490,8 @@ token_down_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ ac
                 return;                             // timing only: weights requested, dependency met
 #endif
                 // Every warp stages the ONE activation row its expert needs (row j of the token) and forms that row's block
-                // sums itself: all of its 16-byte chunks in flight at once (one L2 round trip), no CTA-wide barrier before
-                // the arithmetic.  Chunk -> lane mapping and butterfly as in the other staging loops: same bits.
+                // constants itself: all of its 16-byte chunks in flight at once (one L2 round trip), no CTA-wide barrier
+                // before the arithmetic.
                 if (j < k) {
                     const int chunks_per_row = K / 8;
                     const uint4* src = reinterpret_cast<const uint4*>(act + (size_t)(t * k + j) * K);
@@ -511,12 +505,14 @@ token_down_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ ac
                         }
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
+                            if (base0 + u * 32 >= chunks_per_row) break;
                             const int ck = base0 + u * 32 + lane;
-                            if (ck < chunks_per_row) *reinterpret_cast<uint4*>(xs + (size_t)j * x_stride + ck * 16) = v[u];
-                            float sx = sum8_bf16(v[u]);
-#pragma unroll
-                            for (int m = 8; m >= 1; m >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, m);
-                            if (ck < chunks_per_row && (ck & 15) == 0) adj[(ck >> 4) * k + j] = -136.f * sx;
+                            float2 k2;
+                            const uint4 x = f16_block(v[u], k2);
+                            if (ck < chunks_per_row) {
+                                *reinterpret_cast<uint4*>(xs + (size_t)j * x_stride + ck * 16) = x;
+                                if ((ck & 15) == 0) cst[(ck >> 4) * k + j] = k2;
+                            }
                         }
                     }
                 }
@@ -539,13 +535,13 @@ token_down_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ ac
                             if (q == 0) xb = *reinterpret_cast<const uint4*>(xs + (size_t)j * x_stride + k0 * 2);
                             const uint32_t wq = set ? wreg[b][h].z : wreg[b][h].x;
                             const uint32_t wq8 = set ? wreg[b][h].w : wreg[b][h].y;
-                            mma_m16n8k16(acc, code_pair(wq, 0), code_pair(wq8, 0), code_pair(wq, 4), code_pair(wq8, 4), xb.x, xb.y);
-                            mma_m16n8k16(acc, code_pair(wq, 8), code_pair(wq8, 8), code_pair(wq, 12), code_pair(wq8, 12), xb.z, xb.w);
+                            const CodeFrag cf(wq, wq8);
+                            cf.first(acc, xb);
+                            cf.second(acc, xb);
                         }
-                    const __half2 sc = *reinterpret_cast<const __half2*>(&sreg[b]);
-                    const float cr = adj[(b0 + b) * k + j];
-                    total[0] = fmaf(__low2float(sc), acc[0] + cr, total[0]);
-                    total[1] = fmaf(__high2float(sc), acc[2] + cr, total[1]);
+                    const float2 sc = scales16(sreg[b]), k2 = cst[(b0 + b) * k + j];
+                    total[0] = fmaf(sc.x, fmaf(acc[0], k2.x, k2.y), total[0]);
+                    total[1] = fmaf(sc.y, fmaf(acc[2], k2.x, k2.y), total[1]);
                     if ((b0 + b + 1) % bpwg == 0) {            // end of one K-split range of the grouped kernel
                         const bool first = (b0 + b + 1 == bpwg);
                         result[0] = first ? total[0] : result[0] + total[0];
@@ -591,7 +587,7 @@ __device__ __forceinline__ void pair_gateup_item(const GemmArgs& a, const SmallA
     const int ks = warp & (KS - 1), pp = warp >> ks_log2;
     unsigned char* xs = smem;                                            // one activation row
     float* red = reinterpret_cast<float*>(smem + K * 2 + 64);            // [KS-1][PP][2][32][4]
-    float* adj = red + (size_t)(KS - 1) * PP * 2 * 128;                  // [KB]
+    float2* cst = reinterpret_cast<float2*>(red + (size_t)(KS - 1) * PP * 2 * 128);      // [KB] block constants
 
     // The hidden row does not depend on the ids: request it first so that it is not queued behind the weights.
     const __nv_bfloat16* xrow = hidden + (size_t)token * K;
@@ -613,19 +609,18 @@ __device__ __forceinline__ void pair_gateup_item(const GemmArgs& a, const SmallA
             wreg[m][b][1] = ldg_stream128(blk + 512 + lane * 16);
             sreg[m][b] = ldg_stream32(blk + kCodeBytes + q * 4);
         }
-    // stage the token's hidden row; adj[kb] = -136 * (sum of the row over block kb)
+    // stage the token's hidden row
     const int total = K / 8;
     for (int base = warp * 32; base < total; base += 256) {
         const int ck = base + lane;
         uint4 v = make_uint4(0, 0, 0, 0);
+        if (ck < total) v = (base < 256) ? xpre : *reinterpret_cast<const uint4*>(xrow + ck * 8);
+        float2 k2;
+        v = f16_block(v, k2);
         if (ck < total) {
-            v = (base < 256) ? xpre : *reinterpret_cast<const uint4*>(xrow + ck * 8);
             *reinterpret_cast<uint4*>(xs + ck * 16) = v;
+            if ((ck & 15) == 0) cst[ck >> 4] = k2;
         }
-        float sx = sum8_bf16(v);
-#pragma unroll
-        for (int m = 8; m >= 1; m >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, m);
-        if (ck < total && (ck & 15) == 0) adj[ck >> 4] = -136.f * sx;
     }
     __syncthreads();
 
@@ -652,17 +647,17 @@ __device__ __forceinline__ void pair_gateup_item(const GemmArgs& a, const SmallA
                 for (int m = 0; m < 2; ++m) {
                     const uint32_t wq = set ? wreg[m][b][h].z : wreg[m][b][h].x;
                     const uint32_t wq8 = set ? wreg[m][b][h].w : wreg[m][b][h].y;
-                    mma_m16n8k16(acc[m], code_pair(wq, 0), code_pair(wq8, 0), code_pair(wq, 4), code_pair(wq8, 4), xb.x, xb.y);
-                    mma_m16n8k16(acc[m], code_pair(wq, 8), code_pair(wq8, 8), code_pair(wq, 12), code_pair(wq8, 12), xb.z, xb.w);
+                    const CodeFrag cf(wq, wq8);
+                    cf.first(acc[m], xb);
+                    cf.second(acc[m], xb);
                 }
             }
-        const float cr = adj[ks * NB + b];             // column 0 is the only live one; others are discarded
+        const float2 k2 = cst[ks * NB + b];            // column 0 is the only live one; others are discarded
 #pragma unroll
         for (int m = 0; m < 2; ++m) {
-            const __half2 sc = *reinterpret_cast<const __half2*>(&sreg[m][b]);
-            const float s_lo = __low2float(sc), s_hi = __high2float(sc);
-            tot[m][0] = fmaf(s_lo, acc[m][0] + cr, tot[m][0]);
-            tot[m][2] = fmaf(s_hi, acc[m][2] + cr, tot[m][2]);
+            const float2 sc = scales16(sreg[m][b]);
+            tot[m][0] = fmaf(sc.x, fmaf(acc[m][0], k2.x, k2.y), tot[m][0]);
+            tot[m][2] = fmaf(sc.y, fmaf(acc[m][2], k2.x, k2.y), tot[m][2]);
         }
     }
     if (ks > 0 && c == 0) {
@@ -713,8 +708,7 @@ pair_gateup_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ h
 // ------------------------------------------------------------------------------------------------
 // Wide variant of the per-pair gate/up kernel: ONE CTA of 16 warps per SM instead of two of 8, each warp one
 // (panel pair, K range) unit held in registers, and every warp a pipeline of its own: its K range of the hidden
-// row goes into a private piece of shared memory, it forms the range's block corrections itself (same chunk ->
-// lane mapping and butterfly as the staging loops above: same bits), requests its blocks AHEAD blocks before it
+// row goes into a private piece of shared memory, it forms the range's block constants itself, requests its blocks AHEAD blocks before it
 // needs them and starts on a block as soon as that block's registers have arrived.  No CTA-wide barrier before the
 // K-range partials meet, so the conversion of the early blocks runs while the late ones are still in flight.
 // Arithmetic and summation orders are those of pair_gateup_item.
@@ -729,7 +723,7 @@ constexpr int kWideMaxPairs = EXMOE_WIDE_MAX_PAIRS;     // pairs up to which the
 #endif
 
 // one 128-wide block of a unit: gate and up words in registers, activations of the warp's K range in `xr`
-__device__ __forceinline__ void wide_block(const uint4 (&wb)[2][2], const uint32_t (&sb)[2], float adj, int b,
+__device__ __forceinline__ void wide_block(const uint4 (&wb)[2][2], const uint32_t (&sb)[2], float2 k2, int b,
                                            const unsigned char* xr, int lane, float (&tot)[2][2]) {
     const int q = lane >> 2, c = lane & 3;
     float acc[2][4];
@@ -748,15 +742,16 @@ __device__ __forceinline__ void wide_block(const uint4 (&wb)[2][2], const uint32
             for (int m = 0; m < 2; ++m) {
                 const uint32_t wq = set ? wb[m][h].z : wb[m][h].x;
                 const uint32_t wq8 = set ? wb[m][h].w : wb[m][h].y;
-                mma_m16n8k16(acc[m], code_pair(wq, 0), code_pair(wq8, 0), code_pair(wq, 4), code_pair(wq8, 4), xb.x, xb.y);
-                mma_m16n8k16(acc[m], code_pair(wq, 8), code_pair(wq8, 8), code_pair(wq, 12), code_pair(wq8, 12), xb.z, xb.w);
+                const CodeFrag cf(wq, wq8);
+                cf.first(acc[m], xb);
+                cf.second(acc[m], xb);
             }
         }
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
-        const __half2 sc = *reinterpret_cast<const __half2*>(&sb[m]);
-        tot[m][0] = fmaf(__low2float(sc), acc[m][0] + adj, tot[m][0]);
-        tot[m][1] = fmaf(__high2float(sc), acc[m][2] + adj, tot[m][1]);
+        const float2 sc = scales16(sb[m]);
+        tot[m][0] = fmaf(sc.x, fmaf(acc[m][0], k2.x, k2.y), tot[m][0]);
+        tot[m][1] = fmaf(sc.y, fmaf(acc[m][2], k2.x, k2.y), tot[m][1]);
     }
 }
 
@@ -808,26 +803,23 @@ pair_gateup_wide_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restric
     constexpr int AHEAD = EXMOE_WIDE_AHEAD < NB ? EXMOE_WIDE_AHEAD : NB;         // blocks requested before the arithmetic starts
 #pragma unroll
     for (int b = 0; b < AHEAD; ++b) issue_block(b);
-    float adjv[NB];
+    float2 cstv[NB];
 #pragma unroll
     for (int i = 0; i < XL; ++i) {
         const int ck = i * 32 + lane;
-        if (ck < NB * 16) *reinterpret_cast<uint4*>(xw + ck * 16) = xpre[i];
-        float sx = sum8_bf16(xpre[i]);
+        float2 k2;
+        const uint4 x = f16_block(xpre[i], k2);
+        if (ck < NB * 16) *reinterpret_cast<uint4*>(xw + ck * 16) = x;
 #pragma unroll
-        for (int m = 8; m >= 1; m >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, m);
-        const float lo = __shfl_sync(0xffffffffu, sx, 0), hi = __shfl_sync(0xffffffffu, sx, 16);
-        // __fmul_rn: the product is rounded on its own, as where pair_gateup_item keeps it in shared memory (left to the
-        // compiler it would be contracted into the accumulator addition that consumes it: different bits)
-        if (2 * i < NB) adjv[2 * i] = __fmul_rn(-136.f, lo);
-        if (2 * i + 1 < NB) adjv[2 * i + 1] = __fmul_rn(-136.f, hi);
+        for (int h = 0; h < 2; ++h)                    // lanes 0-15 hold block 2i, lanes 16-31 block 2i + 1
+            if (2 * i + h < NB) cstv[2 * i + h] = make_float2(__shfl_sync(0xffffffffu, k2.x, 16 * h), __shfl_sync(0xffffffffu, k2.y, 16 * h));
     }
     __syncwarp();
     float tot[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
         if (b + AHEAD < NB) issue_block(b + AHEAD);
-        wide_block(wreg[b], sreg[b], adjv[b], b, xw, lane, tot);
+        wide_block(wreg[b], sreg[b], cstv[b], b, xw, lane, tot);
     }
     if (c == 0) {
         float* r = red + (size_t)warp * 32;            // warp = pp * KS + ks
@@ -885,8 +877,8 @@ token_down_bulk_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict
     unsigned char* xs = smem + (size_t)k * panel_bytes;                  // [k][x_stride]
     float* ys = reinterpret_cast<float*>(xs + (size_t)k * x_stride);     // [k][16]
     int* s_valid = reinterpret_cast<int*>(ys + k * 16);                  // [k]
-    float* adj = reinterpret_cast<float*>(s_valid + 8);                  // [KB][k]
-    uint64_t* bar = reinterpret_cast<uint64_t*>(adj + (((size_t)KB * k + 3) & ~(size_t)3));
+    float2* cst = reinterpret_cast<float2*>(s_valid + 8);                // [KB][k] block constants
+    uint64_t* bar = reinterpret_cast<uint64_t*>(cst + (size_t)KB * k);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(bar + 1);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int q = lane >> 2, c = lane & 3;
@@ -915,7 +907,7 @@ token_down_bulk_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict
     }
     grid_dependency_wait();                                              // the gate/up kernel's activations are complete and visible
     {
-        // four 16-byte chunks per thread in flight at once (one L2 round trip per batch), then the block sums
+        // four 16-byte chunks per thread in flight at once (one L2 round trip per batch), then the conversion
         const int chunks_per_row = K / 8, total = k * chunks_per_row;
         const int cpr_shift = (chunks_per_row & (chunks_per_row - 1)) ? -1 : __ffs(chunks_per_row) - 1;
         const uint4* src = reinterpret_cast<const uint4*>(act + (size_t)t * k * K);         // the token's k rows are contiguous
@@ -929,6 +921,7 @@ token_down_bulk_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
+                if (base0 + u * 256 >= total) break;
                 const int idx = base0 + u * 256 + lane;
                 int n, ck;
                 if (cpr_shift >= 0) {                  // the usual case: no division between the wait and the MMAs
@@ -938,11 +931,12 @@ token_down_bulk_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict
                     n = idx / chunks_per_row;
                     ck = idx - n * chunks_per_row;
                 }
-                if (idx < total) *reinterpret_cast<uint4*>(xs + (size_t)n * x_stride + ck * 16) = v[u];
-                float sx = sum8_bf16(v[u]);
-#pragma unroll
-                for (int m = 8; m >= 1; m >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, m);
-                if (idx < total && (ck & 15) == 0) adj[(ck >> 4) * k + n] = -136.f * sx;
+                float2 k2;
+                const uint4 x = f16_block(v[u], k2);
+                if (idx < total) {
+                    *reinterpret_cast<uint4*>(xs + (size_t)n * x_stride + ck * 16) = x;
+                    if ((ck & 15) == 0) cst[(ck >> 4) * k + n] = k2;
+                }
             }
         }
     }
@@ -969,13 +963,13 @@ token_down_bulk_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict
                         const uint4& wh = h ? w1 : w0;
                         const uint32_t wq = set ? wh.z : wh.x;
                         const uint32_t wq8 = set ? wh.w : wh.y;
-                        mma_m16n8k16(acc, code_pair(wq, 0), code_pair(wq8, 0), code_pair(wq, 4), code_pair(wq8, 4), xb.x, xb.y);
-                        mma_m16n8k16(acc, code_pair(wq, 8), code_pair(wq8, 8), code_pair(wq, 12), code_pair(wq8, 12), xb.z, xb.w);
+                        const CodeFrag cf(wq, wq8);
+                        cf.first(acc, xb);
+                        cf.second(acc, xb);
                     }
-                const __half2 sc = *reinterpret_cast<const __half2*>(&sv);
-                const float cr = adj[(b0 + b) * k + j];
-                total2[0] = fmaf(__low2float(sc), acc[0] + cr, total2[0]);
-                total2[1] = fmaf(__high2float(sc), acc[2] + cr, total2[1]);
+                const float2 sc = scales16(sv), k2 = cst[(b0 + b) * k + j];
+                total2[0] = fmaf(sc.x, fmaf(acc[0], k2.x, k2.y), total2[0]);
+                total2[1] = fmaf(sc.y, fmaf(acc[2], k2.x, k2.y), total2[1]);
                 if ((b0 + b + 1) % bpwg == 0) {                          // end of one K-split range of the grouped kernel
                     const bool first = (b0 + b + 1 == bpwg);
                     result[0] = first ? total2[0] : result[0] + total2[0];
@@ -1022,14 +1016,18 @@ static void launch_pdl(Kern kern, dim3 grid, int block, size_t smem, cudaStream_
     cudaLaunchKernelEx(&lc, kern, args...);
 }
 
+// The limits of pair_path_fits and small_path_fits are those of the published formulas (one word per block and row); the
+// kernels keep two, which these leave room for (at most 6 KB).
+constexpr int kPairSmemMax = 108 * 1024, kSmallSmemMax = 216 * 1024;
+
 template <int NB>
 void launch_pair_gateup(const GemmArgs& a, const SmallArgs& sa, const __nv_bfloat16* hidden, __nv_bfloat16* act, int KS,
                         cudaStream_t st) {
     auto kern = pair_gateup_kernel<NB>;
     const int PP = 8 / KS, tiles = a.I / (kPanelRows * PP);
-    const size_t smem = (size_t)a.H * 2 + 64 + (size_t)(KS - 1) * PP * 2 * 128 * 4 + (size_t)(a.H / kGroup) * 4;
+    const size_t smem = (size_t)a.H * 2 + 64 + (size_t)(KS - 1) * PP * 2 * 128 * 4 + (size_t)(a.H / kGroup) * 8;
     static SmemOnce smem_once;
-    allow_smem(kern, 100 * 1024, smem_once);
+    allow_smem(kern, kPairSmemMax, smem_once);
     int ks_log2 = 0;
     while ((1 << ks_log2) < KS) ++ks_log2;
     launch_pdl(kern, dim3(tiles, a.top_k, sa.n_pairs / a.top_k), 256, smem, st, a, sa, hidden, act, ks_log2);
@@ -1083,12 +1081,12 @@ void launch_cfg(const GemmArgs& a, const SmallArgs& sa, const __nv_bfloat16* x, 
     const int PP = 8 / cfg.KS;
     const int tiles = NR / (kPanelRows * PP);
     size_t smem = (size_t)8 * NCH * (K * 2 + 64) + (size_t)(cfg.KS - 1) * PP * NM * NCH * 128 * 4 +
-                  (size_t)(K / kGroup) * 8 * NCH * 4;
+                  (size_t)(K / kGroup) * 8 * NCH * 8;
     constexpr bool SMALL = (MODE == MODE_SMALL);
     if (SMALL) smem += (size_t)(3 * a.num_slots + 1 + 2 * sa.n_pairs) * 4;
     auto kern = decode_gemm_kernel<NB, NCH, GATEUP, MODE>;
     static SmemOnce smem_once;                      // per instantiation
-    allow_smem(kern, 200 * 1024, smem_once);
+    allow_smem(kern, kSmallSmemMax, smem_once);
     long long items = (long long)max_groups * tiles;
     const int grid = (int)(items < 148 * 8 ? (items < 1 ? 1 : items) : 148 * 8);
     cudaLaunchConfig_t lc{};
@@ -1177,9 +1175,9 @@ template <int NBT>
 void launch_token_down(const GemmArgs& a, const SmallArgs& sa, const __nv_bfloat16* act, const float* w, int T,
                        int bpwg, cudaStream_t st) {
     auto kern = token_down_kernel<NBT>;
-    const size_t smem = (size_t)a.top_k * (a.I * 2 + 64) + (size_t)a.top_k * 17 * 4 + (size_t)(a.I / kGroup) * a.top_k * 4;
+    const size_t smem = (size_t)a.top_k * (a.I * 2 + 64) + (size_t)a.top_k * 17 * 4 + (size_t)(a.I / kGroup) * a.top_k * 8;
     static SmemOnce smem_once;
-    allow_smem(kern, 200 * 1024, smem_once);
+    allow_smem(kern, kSmallSmemMax, smem_once);
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3(T * (a.H / kPanelRows));
     lc.blockDim = dim3(256);
@@ -1204,7 +1202,7 @@ bool launch_token_down_bulk(const GemmArgs& a, const SmallArgs& sa, const __nv_b
     const int K = a.I, KB = K / kGroup, k = a.top_k;
     if (k > 8) return false;
     const size_t smem = (size_t)k * KB * kBlockBytes + (size_t)k * (K * 2 + 64) + (size_t)k * 16 * 4 + 32 +
-                        (((size_t)KB * k + 3) & ~(size_t)3) * 4 + 64;
+                        (size_t)KB * k * 8 + 64;
     if (smem > 100 * 1024) return false;
     auto kern = token_down_bulk_kernel<NBT>;
     static SmemOnce smem_once;

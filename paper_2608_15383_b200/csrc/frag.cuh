@@ -14,13 +14,6 @@ __device__ __forceinline__ void mma_m16n8k16(float (&d)[4], uint32_t a0, uint32_
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-// two offset-binary nibbles (bits s..s+3 of each 16-bit half) -> bf16x2 of 128 + u = 136 + q:
-// 0x4300 | u is that BF16 value exactly (one shift and one lop3 per pair of codes).
-__device__ __forceinline__ uint32_t code_pair(uint32_t w, int s) {
-    uint32_t r;
-    asm("lop3.b32 %0, %1, 0x000f000f, 0x43004300, 0xea;" : "=r"(r) : "r"(w >> s));   // (a & b) | c
-    return r;
-}
 // sum of the 8 BF16 values of a 16-byte chunk, in binary32
 __device__ __forceinline__ float sum8_bf16(const uint4& v) {
     const uint32_t r[4] = {v.x, v.y, v.z, v.w};
@@ -32,7 +25,7 @@ __device__ __forceinline__ float sum8_bf16(const uint4& v) {
 
 // ---- codes as FP16 subnormals ---------------------------------------------------------------------------------------
 // A nibble in bits 0-3 of a 16-bit half IS the FP16 subnormal u * 2^-24, and in bits 4-7 it is 16 u * 2^-24: four code pairs
-// of a word take one shift and four ANDs (BF16 pairs 128 + u: three shifts, four lop3, at the same half rate), and the
+// of a word take one shift and four ANDs (BF16 pairs 128 + u took three shifts and four lop3, at the same half rate), and the
 // products need no bias as large as 136.  The activations go in as FP16 scaled by a power of two per row and 128-wide
 // block: X = x * 2^(14-E), E the exponent of the block's largest value, and X / 16 for the k that meet bits 4-7.  FP16 has
 // three bits more than BF16, so that is exact for values down to 2^-27 of the block's largest and off by less than
