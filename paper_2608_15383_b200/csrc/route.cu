@@ -95,6 +95,45 @@ __device__ __forceinline__ void softmax_topk(float* prob, int E, int k, int lane
     }
 }
 
+// The same by a whole CTA, for one token: the rounds of the arg-max (120 cycles each) are replaced by counting, for every
+// expert, the experts that come before it (four threads per expert).  `pv`: E more floats of shared memory.
+__device__ __forceinline__ void softmax_topk_cta(float* prob, float* pv, int E, int k, int32_t* __restrict__ ids_out,
+                                                 float* __restrict__ w_out) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float mx = -INFINITY;
+    for (int e = lane; e < E; e += 32) mx = fmaxf(mx, prob[e]);
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, m));
+    float sum = 0.f;                                                       // every warp for itself, in the same order
+    for (int e = lane; e < E; e += 32) {
+        const float v = expf(prob[e] - mx);
+        if (warp == 0) pv[e] = v;
+        sum += v;
+    }
+    sum = warp_sum(sum);
+    __syncthreads();
+    if (!(sum < INFINITY)) {                                               // a NaN among the logits
+        if (warp == 0) softmax_topk(prob, E, k, lane, ids_out, w_out);
+        return;
+    }
+    const float inv = 1.f / sum;
+    for (int e0 = 0; e0 < E; e0 += kRouteThreads / 4) {
+        const int e = e0 + (tid >> 2);
+        const float v = e < E ? pv[e] : 0.f;
+        int before = 0;
+        for (int j = tid & 3; j < E; j += 4) {
+            const float o = pv[j];
+            before += o > v || (o == v && j < e);
+        }
+        before += __shfl_xor_sync(0xffffffffu, before, 1);
+        before += __shfl_xor_sync(0xffffffffu, before, 2);
+        if ((tid & 3) == 0 && e < E && before < k) {
+            ids_out[before] = e;
+            w_out[before] = v * inv;
+        }
+    }
+}
+
 // CL: CTAs per cluster; TB: tokens per cluster.
 // Shared memory: the cluster's TB hidden rows (every CTA keeps all of them), then the logits of the ceil(TB / CL) tokens
 // this CTA owns (token i belongs to rank i % CL).
@@ -172,10 +211,8 @@ route_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* __re
     }
     if (!joined) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
     cluster.sync();
-    for (int i = warp; i * CL + rank < n_tok; i += kRouteWarps) {
-        const size_t t = t0 + i * CL + rank;
-        softmax_topk(prob + i * E, E, k, lane, ids_out + t * k, w_out + t * k);
-    }
+    static_assert(TB <= CL, "a CTA owns at most one token");
+    if (rank < n_tok) softmax_topk_cta(prob, prob + E, E, k, ids_out + (size_t)(t0 + rank) * k, w_out + (size_t)(t0 + rank) * k);
 }
 
 // every form is a programmatic dependent of the kernel before it in the stream (it waits for it before it reads anything)
@@ -206,9 +243,9 @@ int launch_dependent(F kern, int ctas, int cluster, size_t smem, const exmoe_sha
 template <int CL, int TB>
 int launch_route(const exmoe_shape& s, const __nv_bfloat16* hidden, const __nv_bfloat16* w, const float* bias, int T,
                  int32_t* ids, float* wts, cudaStream_t st) {
-    const size_t smem = (size_t)TB * s.d_model * 2 + (size_t)((TB + CL - 1) / CL) * s.num_experts * 4;
+    const size_t smem = (size_t)TB * s.d_model * 2 + 2 * (size_t)s.num_experts * 4;
     static SmemOnce once;
-    if (!allow_smem(route_kernel<CL, TB>, kRouteSmemMax, once)) return EXMOE_ERR_CUDA;
+    if (!allow_smem(route_kernel<CL, TB>, kRouteSmemMax + 4096 * 4, once)) return EXMOE_ERR_CUDA;
     return launch_dependent(route_kernel<CL, TB>, (T + TB - 1) / TB * CL, CL, smem, s, hidden, w, bias, T, ids, wts, st);
 }
 
