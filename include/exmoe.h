@@ -141,8 +141,9 @@ int exmoe_moe_forward(exmoe_cache* cache, int layer, const void* hidden_bf16, co
  * The inputs are copied into the library's pinned staging buffer, go to the device in one copy, the layer runs as
  * in exmoe_moe_forward, the result comes back in one copy (results of up to 64 KB are written by the last kernel
  * straight into the pinned staging buffer), and the call returns when out_host holds it (synchronous; `stream`
- * carries the work).  Tiny batches (T * top_k <= 24) whose call contains no host wait (C = E, or the
- * device-initiated miss path) record their launch sequence once per (layer, T) in a CUDA graph and replay it; all
+ * carries the work).  Tiny batches (T * top_k <= 24) of at most 4 KB of activations on a fully resident layer
+ * pass their inputs as kernel parameters, without a copy.  Other tiny batches whose call contains no host wait (C = E, or
+ * the device-initiated miss path) record their launch sequence once per (layer, T) in a CUDA graph and replay it; all
  * other calls issue their launches one by one.  Calls of 256 KB of activations or more whose four tensors are
  * page-locked skip the staging buffer: the device copies use the caller's memory.  Same results, state and errors
  * as exmoe_moe_forward.  Not to be called while `stream` is being captured by the caller. */

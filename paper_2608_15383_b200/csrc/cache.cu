@@ -175,7 +175,7 @@ static void carve_workspace(exmoe_cache* c, uint8_t* ws, size_t* total) {
     c->y = k.take<float>((size_t)c->max_pairs * s.d_model);
     c->arrive_words = (size_t)(kSmallMaxPairs / s.top_k + 1) * (s.d_model / kPanelRows);
     c->arrive = k.take<int>(c->arrive_words);
-    c->saved_ids = k.take<int32_t>(std::max(kPairMaxPairs, std::min(c->max_pairs, kStreamMaxPairs)));
+    c->saved_ids = k.take<int32_t>(std::max(kPairMaxPairs, std::min(c->max_pairs, kStreamOwnPlanPairs)));
     c->tc_scratch = k.take<uint8_t>(prefill_scratch_bytes(c->max_pairs, E));
     c->xg = (c->max_pairs > kSmallMaxPairs || !c->small_ok) ? k.take<__nv_bfloat16>((size_t)c->max_pairs * s.d_model) : nullptr;
     c->tc_maps.dev = c->xg ? k.take<uint8_t>(kPrefillMapBytes) : nullptr;
@@ -440,7 +440,7 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
     // timing runs that launch one kernel kind reuse the plan, grouped rows and tile list of the previous full call
     const bool build_plan = (c->prof_only == 0);
     const bool use_stream = !small && c->stream_ok && P <= kStreamMaxPairs;
-    const bool own_plan = use_stream && identity && c->n_keys <= kStreamOwnPlanKeys;     // the kernels group the ids themselves
+    const bool own_plan = use_stream && identity && c->n_keys <= kStreamOwnPlanKeys && P <= kStreamOwnPlanPairs;     // the kernels group the ids themselves
     if (!small && build_plan && !own_plan) {
         ProfScope ps(c, PROF_PLAN, st);
         launch_group(s, C, c->n_keys, c->max_waves, identity, topk_ids, P, c->plan, c->d_status, st);
@@ -683,6 +683,36 @@ int exmoe_moe_forward_host(exmoe_cache* c, int layer, const void* hidden_host, c
             int rc = ok ? exmoe_moe_forward(c, layer, d_h, d_i, d_w, T, d_o, st) : EXMOE_ERR_CUDA;
             if (!rc && cudaMemcpyAsync(out_host, d_o, nb_h, cudaMemcpyDeviceToHost, st) != cudaSuccess) rc = EXMOE_ERR_CUDA;
             if (cudaStreamSynchronize(st) != cudaSuccess) rc = rc ? rc : EXMOE_ERR_CUDA;
+            return rc;
+        }
+    }
+    // Tiny batches on a fully resident layer: the inputs travel as kernel parameters, two launches and nothing before them.
+    if (c->C == s.num_experts && T * s.top_k <= kSmallMaxPairs && c->C <= kSmallMaxSlots && c->small_ok && c->pair_ok && out_direct &&
+        !c->prof_on && !c->prof_only) {
+        GemmArgs a{};
+        a.slots = c->slot_mem + (size_t)layer * c->C * c->bpe;
+        a.slot_stride = c->bpe;
+        a.num_slots = c->C;
+        a.top_k = s.top_k;
+        a.H = s.d_model;
+        a.I = s.d_ff;
+        SmallWave sw{};
+        sw.n_pairs = T * s.top_k;
+        sw.E = s.num_experts;
+        sw.plan = c->plan;
+        sw.status = c->d_status;
+        sw.act = c->act;
+        sw.out = static_cast<__nv_bfloat16*>(d_o);
+        sw.saved_ids = c->saved_ids;
+        if (launch_pair_inline(a, sw, hidden_host, ids_host, weights_host, st)) {
+            c->last_layer = layer;
+            c->last_T = T;
+            c->last_small = c->last_pair = true;
+            c->last_path = EXMOE_PATH_PAIR;
+            c->last_host_h2d_bytes = off_w + nb_i;
+            int rc = cudaGetLastError() == cudaSuccess ? EXMOE_OK : EXMOE_ERR_CUDA;
+            if (cudaStreamSynchronize(st) != cudaSuccess) rc = EXMOE_ERR_CUDA;
+            if (!rc) std::memcpy(out_host, c->h_stage + c->stage_out_off, nb_h);
             return rc;
         }
     }

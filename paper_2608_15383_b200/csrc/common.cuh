@@ -129,11 +129,13 @@ void launch_group(const exmoe_shape& s, int C, int n_keys, int max_waves, bool i
 #define EXMOE_STREAM_MAX_PAIRS 640
 #endif
 constexpr int kStreamMaxPairs = EXMOE_STREAM_MAX_PAIRS;   // above: tensor-core path
-constexpr int kStreamOwnPlanKeys = 128;                    // most experts whose pairs the streaming kernels group themselves
+constexpr int kStreamOwnPlanKeys = 128, kStreamOwnPlanPairs = 640;    // most experts and pairs that the streaming kernels group themselves
 bool stream_supported(int H, int I);
 bool launch_stream_wave(const GemmArgs& a, const __nv_bfloat16* hidden, __nv_bfloat16* act, const float* topk_w, float* y,
                         int* status, int max_groups, bool gateup, bool down, cudaStream_t st);
 void launch_small_wave(const GemmArgs& a, const SmallWave& w, cudaStream_t st, bool gateup, bool down);
+// the per-pair kernels on HOST inputs that travel as kernel parameters; false (nothing queued) where that does not apply
+bool launch_pair_inline(const GemmArgs& a, const SmallWave& w, const void* hidden, const int32_t* ids, const float* weights, cudaStream_t st);
 bool pair_path_fits(int H, int I, int top_k);                           // shared memory of the per-pair kernels within limits
 bool small_path_fits(int H, int I, int num_slots, int n_pairs);         // ... of the in-CTA-grouping kernels
 size_t prefill_scratch_bytes(int max_pairs, int num_experts);

@@ -23,6 +23,9 @@
 //     pair_gateup_kernel, token_down_kernel (one token) and token_down_bulk_kernel (two or more tokens).
 // Larger batches run on the streaming kernels (stream.cu) or the tensor-core kernels (prefill.cu) with the
 // grouping kernels' global plan and the separate combine kernel defined here.
+#include <cstring>
+#include <type_traits>
+
 #include "common.cuh"
 #include "frag.cuh"
 #include "mbar.cuh"
@@ -79,6 +82,21 @@ struct SmallArgs {
     __nv_bfloat16* out;       // [T, H]
     int32_t* saved_ids;       // [kPairMaxPairs] copy of the ids kept by the pairwise path
 };
+
+// Inputs of a host call inside the launch itself (kernel parameters): hidden rows, ids and mixture weights reach the GPU
+// with the launch instead of through a copy and the dependency on it.  HB: bytes of hidden rows, 0 = none of it.
+template <int HB>
+struct InlineInput {
+    int32_t ids[kSmallMaxPairs];
+    uint4 x[HB / 16];
+};
+template <>
+struct InlineInput<0> {};
+struct InlineIds {
+    int32_t ids[kSmallMaxPairs];
+    float w[kSmallMaxPairs];
+};
+struct NoInlineIds {};
 
 __device__ __forceinline__ void build_small_plan(const SmallArgs& sa, int C, SmallPlan& sp, int* s_scalars) {
     const int tid = threadIdx.x, P = sa.n_pairs;
@@ -440,10 +458,11 @@ decode_gemm_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ x
 #ifndef EXMOE_DOWN_ABLATE
 #define EXMOE_DOWN_ABLATE 0
 #endif
-template <int NBT>
+template <int NBT, typename Inl>
 __global__ void __launch_bounds__(256)
 token_down_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ act, const float* __restrict__ topk_w,
-                  int bpwg) {
+                  int bpwg, const __grid_constant__ Inl in) {
+    constexpr bool INL = std::is_same_v<Inl, InlineIds>;
     extern __shared__ __align__(128) unsigned char smem[];
     grid_launch_dependents();                          // the next kernel in the stream may be placed (it waits for this one)
     const int K = a.I, KB = K / kGroup, k = a.top_k;
@@ -463,9 +482,18 @@ token_down_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ ac
         const int j = j0 + warp;
         const int pair = t * k + j;
         int id = -1;
-        if (j < k) id = sa.ids[pair];
+        float rw = 0.f;
+        if constexpr (INL) {
+            if (j < k) id = in.ids[pair];
+        } else {
+            if (j < k) id = sa.ids[pair];
+        }
         const bool valid = (j < k) && id >= 0 && id < sa.E;
-        const float rw = valid ? ldg_early_f32(topk_w + pair) : 0.f;   // requested early: needed only in the epilogue
+        if constexpr (INL) {
+            if (valid) rw = in.w[pair];
+        } else {
+            if (valid) rw = ldg_early_f32(topk_w + pair);              // requested early: needed only in the epilogue
+        }
         float result[2] = {0.f, 0.f};
         float total[2] = {0.f, 0.f};
         for (int b0 = 0; b0 < KB; b0 += NBT) {
@@ -683,10 +711,10 @@ __device__ __forceinline__ void pair_gateup_item(const GemmArgs& a, const SmallA
 }
 
 // keep the ids of a pairwise call (so the plan can be materialised on request) and flag invalid ones
-__device__ __forceinline__ void keep_pair_ids(const SmallArgs& sa) {
+__device__ __forceinline__ void keep_pair_ids(const SmallArgs& sa, const int32_t* ids) {
     const int tid = threadIdx.x;
     if (tid < sa.n_pairs) {
-        const int v = sa.ids[tid];
+        const int v = ids[tid];
         sa.saved_ids[tid] = v;
         if (v < 0 || v >= sa.E) atomicExch(sa.status, EXMOE_ERR_BAD_EXPERT_ID);
     }
@@ -700,7 +728,7 @@ pair_gateup_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ h
     extern __shared__ __align__(128) unsigned char smem[];
     grid_dependency_wait();                            // launched as a programmatic dependent of whatever precedes it in the stream
     grid_launch_dependents();
-    if ((blockIdx.x | blockIdx.y | blockIdx.z) == 0) keep_pair_ids(sa);
+    if ((blockIdx.x | blockIdx.y | blockIdx.z) == 0) keep_pair_ids(sa, sa.ids);
     pair_gateup_item<NB>(a, sa, hidden, act_out, ks_log2, (int)(blockIdx.z * a.top_k + blockIdx.y), (int)blockIdx.z,
                          (int)blockIdx.x, smem);
 }
@@ -755,10 +783,10 @@ __device__ __forceinline__ void wide_block(const uint4 (&wb)[2][2], const uint32
     }
 }
 
-template <int NB>
+template <int NB, int HB>
 __global__ void __launch_bounds__(32 * kWideWarps, 1)
 pair_gateup_wide_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ hidden,
-                        __nv_bfloat16* __restrict__ act_out, int ks_log2) {
+                        __nv_bfloat16* __restrict__ act_out, int ks_log2, const __grid_constant__ InlineInput<HB> in) {
     // grid = (slices of 16 >> ks_log2 panel pairs, selected expert j, token t): pair p = t * k + j
     extern __shared__ __align__(128) unsigned char smem[];
     // Launched as a programmatic dependent of whatever precedes it in the stream (in a decode loop the previous layer
@@ -766,7 +794,11 @@ pair_gateup_wide_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restric
     // launch latency is off the step; nothing is read or written before the wait.
     grid_dependency_wait();
     grid_launch_dependents();
-    if ((blockIdx.x | blockIdx.y | blockIdx.z) == 0) keep_pair_ids(sa);
+    if constexpr (HB > 0) {
+        if ((blockIdx.x | blockIdx.y | blockIdx.z) == 0) keep_pair_ids(sa, in.ids);
+    } else {
+        if ((blockIdx.x | blockIdx.y | blockIdx.z) == 0) keep_pair_ids(sa, sa.ids);
+    }
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int q = lane >> 2, c = lane & 3;
     const int p = blockIdx.z * a.top_k + blockIdx.y;
@@ -782,9 +814,13 @@ pair_gateup_wide_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restric
 #pragma unroll
     for (int i = 0; i < XL; ++i) {
         xpre[i] = make_uint4(0, 0, 0, 0);
-        if (i * 32 + lane < NB * 16) xpre[i] = ldg_early128(xrow + (size_t)(i * 32 + lane) * 16);
+        if constexpr (HB == 0) {
+            if (i * 32 + lane < NB * 16) xpre[i] = ldg_early128(xrow + (size_t)(i * 32 + lane) * 16);
+        }
     }
-    const int id = sa.ids[p];
+    int id;
+    if constexpr (HB > 0) id = in.ids[p];
+    else id = sa.ids[p];
     if (id < 0 || id >= sa.E) return;                  // uniform over the CTA; the pair contributes nothing
     const int slot = sa.slot_of ? sa.slot_of[id] : id;
     const int panel = blockIdx.x * PP + pp;
@@ -803,6 +839,17 @@ pair_gateup_wide_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restric
     constexpr int AHEAD = EXMOE_WIDE_AHEAD < NB ? EXMOE_WIDE_AHEAD : NB;         // blocks requested before the arithmetic starts
 #pragma unroll
     for (int b = 0; b < AHEAD; ++b) issue_block(b);
+    if constexpr (HB > 0) {
+        // Parameters are read one address at a time, so the CTA reads its row once, all threads together, and the warps take
+        // their ranges from shared memory (each warp reading its own range from the parameters: 2 us longer).
+        uint4* xraw = reinterpret_cast<uint4*>(red + kWideWarps * 32);
+        const int row = blockIdx.z * (a.H / 8);
+        for (int i = tid; i < a.H / 8; i += 32 * kWideWarps) xraw[i] = in.x[row + i];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < XL; ++i)
+            if (i * 32 + lane < NB * 16) xpre[i] = xraw[ks * NB * 16 + i * 32 + lane];
+    }
     float2 cstv[NB];
 #pragma unroll
     for (int i = 0; i < XL; ++i) {
@@ -864,10 +911,11 @@ __device__ __forceinline__ void drain_bar(uint64_t* bar, uint32_t parity) {
     while (!mbar_try(bar, parity) && clock64() - t0 < kWaitBudget) {}
 }
 
-template <int NBT>
+template <int NBT, typename Inl>
 __global__ void __launch_bounds__(256, 1)
 token_down_bulk_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ act, const float* __restrict__ topk_w,
-                       int bpwg) {
+                       int bpwg, const __grid_constant__ Inl in) {
+    constexpr bool INL = std::is_same_v<Inl, InlineIds>;
     extern __shared__ __align__(128) unsigned char smem[];
     grid_launch_dependents();                          // the next kernel in the stream may be placed (it waits for this one)
     const int K = a.I, KB = K / kGroup, k = a.top_k;                     // k <= 8: one warp per selected expert
@@ -892,9 +940,18 @@ token_down_bulk_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict
     const int j = warp;
     const int pair = t * k + j;
     int id = -1;
-    if (j < k) id = sa.ids[pair];
+    float rw = 0.f;
+    if constexpr (INL) {
+        if (j < k) id = in.ids[pair];
+    } else {
+        if (j < k) id = sa.ids[pair];
+    }
     const bool valid = (j < k) && id >= 0 && id < sa.E;
-    const float rw = valid ? ldg_early_f32(topk_w + pair) : 0.f;
+    if constexpr (INL) {
+        if (valid) rw = in.w[pair];
+    } else {
+        if (valid) rw = ldg_early_f32(topk_w + pair);
+    }
     if (j < k && lane == 0) {                                            // the expert's panel: one contiguous range
         if (valid) {
             const int slot = sa.slot_of ? sa.slot_of[id] : id;
@@ -1035,9 +1092,9 @@ void launch_pair_gateup(const GemmArgs& a, const SmallArgs& sa, const __nv_bfloa
 }
 
 // false when the shape does not fit the wide kernel (the caller then takes pair_gateup_kernel)
-template <int NB>
+template <int NB, int HB = 0>
 bool launch_pair_gateup_wide(const GemmArgs& a, const SmallArgs& sa, const __nv_bfloat16* hidden, __nv_bfloat16* act, int KS,
-                             cudaStream_t st) {
+                             cudaStream_t st, const InlineInput<HB>& in = {}) {
 #ifdef EXMOE_NO_WIDE_GATEUP
     return false;
 #endif
@@ -1045,12 +1102,12 @@ bool launch_pair_gateup_wide(const GemmArgs& a, const SmallArgs& sa, const __nv_
     while ((1 << ks_log2) < KS) ++ks_log2;
     const int PP = kWideWarps >> ks_log2;
     if ((1 << ks_log2) != KS || PP < 1 || a.I % (kPanelRows * PP)) return false;
-    auto kern = pair_gateup_wide_kernel<NB>;
-    const size_t smem = (size_t)kWideWarps * NB * kGroup * 2 + (size_t)kWideWarps * 32 * 4;
+    auto kern = pair_gateup_wide_kernel<NB, HB>;
+    const size_t smem = (size_t)kWideWarps * NB * kGroup * 2 + (size_t)kWideWarps * 32 * 4 + (HB > 0 ? (size_t)a.H * 2 : 0);
     static SmemOnce smem_once;
     allow_smem(kern, 100 * 1024, smem_once);
     launch_pdl(kern, dim3(a.I / (kPanelRows * PP), a.top_k, sa.n_pairs / a.top_k), 32 * kWideWarps, smem, st, a, sa, hidden, act,
-               ks_log2);
+               ks_log2, in);
     count_launch();
     return true;
 }
@@ -1171,58 +1228,53 @@ void launch_combine(const float* y, const int32_t* ids, int E, int T, int k, int
 }
 
 
-template <int NBT>
+template <int NBT, typename Inl>
 void launch_token_down(const GemmArgs& a, const SmallArgs& sa, const __nv_bfloat16* act, const float* w, int T,
-                       int bpwg, cudaStream_t st) {
-    auto kern = token_down_kernel<NBT>;
+                       int bpwg, cudaStream_t st, const Inl& in) {
+    auto kern = token_down_kernel<NBT, Inl>;
     const size_t smem = (size_t)a.top_k * (a.I * 2 + 64) + (size_t)a.top_k * 17 * 4 + (size_t)(a.I / kGroup) * a.top_k * 8;
     static SmemOnce smem_once;
     allow_smem(kern, kSmallSmemMax, smem_once);
-    cudaLaunchConfig_t lc{};
-    lc.gridDim = dim3(T * (a.H / kPanelRows));
-    lc.blockDim = dim3(256);
-    lc.dynamicSmemBytes = smem;
-    lc.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = attr;
-    lc.numAttrs = 1;
-#ifdef EXMOE_DISABLE_PDL
-    lc.numAttrs = 0;
-#endif
-    cudaLaunchKernelEx(&lc, kern, a, sa, act, w, bpwg);
+    launch_pdl(kern, dim3(T * (a.H / kPanelRows)), 256, smem, st, a, sa, act, w, bpwg, in);
     count_launch();
 }
 
 // false when the shape does not fit the kernel's shared-memory budget (the caller then takes the register variant)
-template <int NBT>
+template <int NBT, typename Inl>
 bool launch_token_down_bulk(const GemmArgs& a, const SmallArgs& sa, const __nv_bfloat16* act, const float* w, int T, int bpwg,
-                            cudaStream_t st) {
+                            cudaStream_t st, const Inl& in) {
     const int K = a.I, KB = K / kGroup, k = a.top_k;
     if (k > 8) return false;
     const size_t smem = (size_t)k * KB * kBlockBytes + (size_t)k * (K * 2 + 64) + (size_t)k * 16 * 4 + 32 +
                         (size_t)KB * k * 8 + 64;
     if (smem > 100 * 1024) return false;
-    auto kern = token_down_bulk_kernel<NBT>;
+    auto kern = token_down_bulk_kernel<NBT, Inl>;
     static SmemOnce smem_once;
     allow_smem(kern, 100 * 1024, smem_once);
-    cudaLaunchConfig_t lc{};
-    lc.gridDim = dim3(a.H / kPanelRows, T);
-    lc.blockDim = dim3(256);
-    lc.dynamicSmemBytes = smem;
-    lc.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = attr;
-    lc.numAttrs = 1;
-#ifdef EXMOE_DISABLE_PDL
-    lc.numAttrs = 0;
-#endif
-    cudaLaunchKernelEx(&lc, kern, a, sa, act, w, bpwg);
+    launch_pdl(kern, dim3(a.H / kPanelRows, T), 256, smem, st, a, sa, act, w, bpwg, in);
     count_launch();
     return true;
+}
+
+template <typename Inl>
+void launch_pair_down(const GemmArgs& a, const SmallArgs& sa, const __nv_bfloat16* act, const float* w, cudaStream_t st, const Inl& in) {
+    const int KB = a.I / kGroup;
+    const int bpwg = pick_cfg(a.I, a.H).bpw;            // the grouped kernel's K-split range, replayed for rounding
+    const int T = sa.n_pairs / a.top_k;
+    bool done = false;
+#ifndef EXMOE_NO_BULK_DECODE
+    if (T >= 2) {                                       // one token: the register kernel overlaps the gate/up kernel better
+        if (KB % 8 == 0) done = launch_token_down_bulk<8>(a, sa, act, w, T, bpwg, st, in);
+        else if (KB % 4 == 0) done = launch_token_down_bulk<4>(a, sa, act, w, T, bpwg, st, in);
+        else if (KB % 2 == 0) done = launch_token_down_bulk<2>(a, sa, act, w, T, bpwg, st, in);
+        else done = launch_token_down_bulk<1>(a, sa, act, w, T, bpwg, st, in);
+    }
+#endif
+    if (done) return;
+    if (KB % 8 == 0) launch_token_down<8>(a, sa, act, w, T, bpwg, st, in);
+    else if (KB % 4 == 0) launch_token_down<4>(a, sa, act, w, T, bpwg, st, in);
+    else if (KB % 2 == 0) launch_token_down<2>(a, sa, act, w, T, bpwg, st, in);
+    else launch_token_down<1>(a, sa, act, w, T, bpwg, st, in);
 }
 
 // Shared memory the per-pair kernels ask for (launch_pair_gateup, launch_token_down): false when either exceeds its
@@ -1247,8 +1299,7 @@ bool small_path_fits(int H, int I, int num_slots, int n_pairs) {
     return true;
 }
 
-// One wave of the SMALL path: gate/up kernel, then the down kernel with the fused combine.
-void launch_small_wave(const GemmArgs& a, const SmallWave& w, cudaStream_t st, bool gateup, bool down) {
+static SmallArgs small_args(const SmallWave& w) {
     SmallArgs sa{};
     sa.ids = w.ids;
     sa.wave_of = w.wave_of;
@@ -1264,6 +1315,12 @@ void launch_small_wave(const GemmArgs& a, const SmallWave& w, cudaStream_t st, b
     sa.arrive = w.arrive;
     sa.out = w.out;
     sa.saved_ids = w.saved_ids;
+    return sa;
+}
+
+// One wave of the SMALL path: gate/up kernel, then the down kernel with the fused combine.
+void launch_small_wave(const GemmArgs& a, const SmallWave& w, cudaStream_t st, bool gateup, bool down) {
+    const SmallArgs sa = small_args(w);
     if (w.pairwise) {                                   // T*k <= 32, one wave: no grouping, by-token down + combine
         if (gateup) {
             const DecodeCfg cfg = pick_cfg(a.H, a.I);
@@ -1277,29 +1334,36 @@ void launch_small_wave(const GemmArgs& a, const SmallWave& w, cudaStream_t st, b
             else if (cfg.bpw == 1) launch_pair_gateup<1>(a, sa, w.hidden, w.act, cfg.KS, st);
             else launch_decode<true, MODE_PAIR>(a, sa, w.hidden, w.act, nullptr, nullptr, 1, w.n_pairs, st);
         }
-        if (down) {
-            const int KB = a.I / kGroup;
-            const int bpwg = pick_cfg(a.I, a.H).bpw;    // the grouped kernel's K-split range, replayed for rounding
-            const int T = w.n_pairs / a.top_k;
-            bool done = false;
-#ifndef EXMOE_NO_BULK_DECODE
-            if (T >= 2) {                               // one token: the register kernel overlaps the gate/up kernel better
-                if (KB % 8 == 0) done = launch_token_down_bulk<8>(a, sa, w.act, w.topk_w, T, bpwg, st);
-                else if (KB % 4 == 0) done = launch_token_down_bulk<4>(a, sa, w.act, w.topk_w, T, bpwg, st);
-                else if (KB % 2 == 0) done = launch_token_down_bulk<2>(a, sa, w.act, w.topk_w, T, bpwg, st);
-                else done = launch_token_down_bulk<1>(a, sa, w.act, w.topk_w, T, bpwg, st);
-            }
-#endif
-            if (done) {}
-            else if (KB % 8 == 0) launch_token_down<8>(a, sa, w.act, w.topk_w, T, bpwg, st);
-            else if (KB % 4 == 0) launch_token_down<4>(a, sa, w.act, w.topk_w, T, bpwg, st);
-            else if (KB % 2 == 0) launch_token_down<2>(a, sa, w.act, w.topk_w, T, bpwg, st);
-            else launch_token_down<1>(a, sa, w.act, w.topk_w, T, bpwg, st);
-        }
+        if (down) launch_pair_down(a, sa, w.act, w.topk_w, st, NoInlineIds{});
         return;
     }
     if (gateup) launch_decode<true, MODE_SMALL>(a, sa, w.hidden, w.act, nullptr, nullptr, w.max_rows, w.max_groups, st);
     if (down) launch_decode<false, MODE_SMALL>(a, sa, w.act, nullptr, w.topk_w, w.y, w.max_rows, w.max_groups, st);
+}
+
+// The pairwise layer on host inputs that travel as kernel parameters.  A launch with 4 KB of them costs less than a copy and
+// the wait for it (one token of d_model 2048: 27.1 -> 25.6 us per host call); with 12 KB it costs more (two tokens 33.8 ->
+// 35.3), so more than 4 KB of hidden rows are left to the copy.  false, and nothing queued, where it does not apply.
+// (A flag in host memory, set by the last CTA behind a system fence and polled by the host instead of the stream: 29.5 us.)
+constexpr int kInlineHiddenBytes = 4096;
+bool launch_pair_inline(const GemmArgs& a, const SmallWave& w, const void* hidden, const int32_t* ids, const float* weights,
+                        cudaStream_t st) {
+    const SmallArgs sa = small_args(w);
+    const size_t bytes = (size_t)(sa.n_pairs / a.top_k) * a.H * 2;
+    if (sa.n_pairs > kSmallMaxPairs || sa.slot_of || bytes > kInlineHiddenBytes) return false;
+    const DecodeCfg cfg = pick_cfg(a.H, a.I);
+    InlineInput<kInlineHiddenBytes> in;
+    InlineIds in_ids;
+    memcpy(in.x, hidden, bytes);
+    memcpy(in.ids, ids, sa.n_pairs * sizeof(int32_t));
+    memcpy(in_ids.ids, ids, sa.n_pairs * sizeof(int32_t));
+    memcpy(in_ids.w, weights, sa.n_pairs * sizeof(float));
+    const bool ok = cfg.bpw == 4   ? launch_pair_gateup_wide<4, kInlineHiddenBytes>(a, sa, nullptr, w.act, cfg.KS, st, in)
+                    : cfg.bpw == 2 ? launch_pair_gateup_wide<2, kInlineHiddenBytes>(a, sa, nullptr, w.act, cfg.KS, st, in)
+                    : cfg.bpw == 1 ? launch_pair_gateup_wide<1, kInlineHiddenBytes>(a, sa, nullptr, w.act, cfg.KS, st, in)
+                                   : false;
+    if (ok) launch_pair_down(a, sa, w.act, nullptr, st, in_ids);
+    return ok;
 }
 
 // ------------------------------------------------------------------------------------------------

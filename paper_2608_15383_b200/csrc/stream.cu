@@ -80,7 +80,7 @@ struct StreamGeom {
 constexpr size_t kBarBytes = 2 * kMaxStages * 8 + 64;                 // mbarriers, abort flag, unit range
 constexpr int kInlineKeys = kStreamOwnPlanKeys;
 constexpr size_t kCtrlBytes = kBarBytes + (size_t)kMetaGroups * 16    // + plan entries of the CTA's groups
-                              + (size_t)kStreamMaxPairs * 4 + kInlineKeys * 4 + kConsumerWarps * 8 * 4;
+                              + (size_t)kStreamOwnPlanPairs * 4 + kInlineKeys * 4 + kConsumerWarps * 8 * 4;
 
 #ifndef EXMOE_STREAM_PP
 #define EXMOE_STREAM_PP 0                                              // 0: choose; 1/2/4/8: force where feasible (timing experiments)
@@ -181,7 +181,7 @@ stream_gemm_kernel(const StreamArgs p) {
     int4* meta_w = reinterpret_cast<int4*>(smem + p.off_bar + kBarBytes);             // (slot, rows, first row, first unit)
     const int4* meta = meta_w;
     int* s_key = reinterpret_cast<int*>(meta_w + kMetaGroups);         // [pairs] plan formed here: key of every pair
-    int* s_cnt = s_key + kStreamMaxPairs;                              // [kInlineKeys] pairs per key
+    int* s_cnt = s_key + kStreamOwnPlanPairs;                              // [kInlineKeys] pairs per key
     int* s_rows = s_cnt + kInlineKeys;                                 // [consumer warps][8] pairs of a pass's rows
     // With every expert resident (key = expert id) and a few hundred pairs, every CTA forms the plan by itself from the ids:
     // no grouping kernel before this one (2.5 us, and a launch), one L2 round trip before the first weight copy.
@@ -205,7 +205,7 @@ stream_gemm_kernel(const StreamArgs p) {
     if (GATEUP) grid_dependency_wait();
 #endif
     if (own_plan) {
-        constexpr int PT = (kStreamMaxPairs + kStreamThreads - 1) / kStreamThreads;
+        constexpr int PT = (kStreamOwnPlanPairs + kStreamThreads - 1) / kStreamThreads;
         int id[PT];
 #pragma unroll
         for (int i = 0; i < PT; ++i) {
