@@ -441,7 +441,8 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
     const bool build_plan = (c->prof_only == 0);
     const bool use_stream = !small && c->stream_ok && P <= kStreamMaxPairs;
     const bool own_plan = use_stream && identity && c->n_keys <= kStreamOwnPlanKeys && P <= kStreamOwnPlanPairs;     // the kernels group the ids themselves
-    if (!small && build_plan && !own_plan) {
+    const bool plan_with_rows = !small && !use_stream && P <= kPlanGatherPairs && c->n_keys <= kPlanGatherKeys;   // below, with the rows
+    if (!small && build_plan && !own_plan && !plan_with_rows) {
         ProfScope ps(c, PROF_PLAN, st);
         launch_group(s, C, c->n_keys, c->max_waves, identity, topk_ids, P, c->plan, c->d_status, st);
     }
@@ -493,8 +494,12 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
     if (!small && build_plan && !use_stream) {
         ProfScope ps(c, PROF_PLAN, st);                  // hidden rows in plan order, once for all waves
         tiles_fused = (n_waves == 1);                    // one wave: its tile list comes out of the same launch
-        launch_gather_rows((const __nv_bfloat16*)hidden, c->plan.perm, c->plan.offsets + c->n_keys, P, k, s.d_model,
-                           c->xg, tiles_fused ? &a : nullptr, c->plan.wave_start, c->tc_scratch, small_n, st);
+        if (!plan_with_rows)
+            launch_gather_rows((const __nv_bfloat16*)hidden, c->plan.perm, c->plan.offsets + c->n_keys, P, k, s.d_model,
+                               c->xg, tiles_fused ? &a : nullptr, c->plan.wave_start, c->tc_scratch, small_n, st);
+        else
+            launch_plan_gather(s, C, c->n_keys, c->max_waves, identity, (const __nv_bfloat16*)hidden, topk_ids, P, c->plan, c->d_status,
+                               c->xg, tiles_fused, c->tc_scratch, small_n, st);
     }
     if (small && n_waves == 0)                           // no valid id at all: the output is zero
         cudaMemsetAsync(out, 0, (size_t)T * s.d_model * 2, st);

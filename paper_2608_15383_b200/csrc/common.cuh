@@ -145,6 +145,12 @@ constexpr size_t kPrefillMapBytes = 2 * 16 * 128;
 struct PrefillMaps { unsigned char* dev; };
 int prefill_setup(PrefillMaps* maps, const __nv_bfloat16* xg, const __nv_bfloat16* act, int max_pairs, int H, int I);
 void launch_wait_selftest(int* status, long long budget_cycles, int* result, cudaStream_t st);
+// Grouping and grouped copy of the hidden rows in one launch, for calls within these limits.  Its CTAs each count all pairs
+// in shared memory: measured at 64 experts it wins up to 8192 pairs, at 16384 the separate kernels are 3 us faster.
+constexpr int kPlanGatherPairs = 8192, kPlanGatherKeys = 1024;
+void launch_plan_gather(const exmoe_shape& s, int C, int n_keys, int max_waves, bool identity, const __nv_bfloat16* hidden,
+                        const int32_t* ids, int n_pairs, PlanPtrs plan, int* status, __nv_bfloat16* xg, bool single_wave,
+                        void* scratch, bool small_n, cudaStream_t st);
 // grouped copy of the hidden rows; when `single_wave` is given its CTA 0 also builds that wave's tile list in `scratch`
 void launch_gather_rows(const __nv_bfloat16* hidden, const int32_t* perm, const int32_t* n_valid, int n_pairs, int top_k,
                         int H, __nv_bfloat16* xg, const GemmArgs* single_wave, const int32_t* wave_start, void* scratch,

@@ -287,3 +287,33 @@ def test_graph_replay_of_the_larger_paths_is_bit_identical_to_plain_launches(B, 
             assert torch.equal(o.view(torch.int16), p.view(torch.int16)), f"T={T} replay {rep}"
     assert cache.status() == 0
     cache.close()
+
+
+@pytest.mark.parametrize("d_model, E, k, T, slots", [
+    (512, 16, 4, 161, 16),             # 644 pairs, just past the streaming kernels: segments of five pairs, the last one short
+    (512, 16, 4, 300, 6),              # several waves: keys are (wave, slot)
+    (2304, 4, 1, 700, 4),              # rows of more than 256 16-byte pieces (two passes of a warp); one pair per token
+    (512, 16, 4, 2048, 16),            # 8192 pairs, the most that the one-launch grouping takes
+    (512, 16, 4, 2049, 16)])           # ... and the first call behind it
+def test_grouping_together_with_the_row_copy(B, d_model, E, k, T, slots):
+    """Tensor-core calls whose pairs are grouped and whose rows are copied in one launch: plan, permutation and state bit
+    for bit, every 16th token and the last one against the oracle (the repository's output tolerance)."""
+    s = synth.Shape(d_model, 256, E, k)
+    ora, bank = helpers.make_layer(s, seed=31 + d_model + E)
+    hidden, ids, p = helpers.routed_inputs(s, T, seed=5100 + T, alpha=1.0)
+    cache = B.Cache(s, [bank], slots, max_tokens=T)
+    sc = ocache.SlotCache(E, slots, 0, bytes_per_expert=cache.bytes_per_expert)
+    out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    assert cache.last_path() in (B.PATH_TENSOR_SMALL_N, B.PATH_TENSOR)
+    compare_plan(cache, sc, ids)
+    sample = list(range(0, T, 16)) + [T - 1]
+    y, ref = ora.forward(hidden[sample], ids[sample], p[sample])
+    helpers.check_output(out[sample], y, ref, f"{d_model} {E} {k} {T}")
+    assert cache.status() == 0
+    bad = ids.clone()
+    bad[T // 2] = -1                                      # a token without a valid expert: zero row, the others unchanged
+    out2 = cache.forward(0, hidden.cuda(), bad.cuda(), p.cuda())
+    keep = torch.arange(T) != T // 2
+    assert not out2[T // 2].any() and cache.status() != 0
+    assert torch.equal(out2[keep].view(torch.int16), out[keep].view(torch.int16))
+    cache.close()
