@@ -472,36 +472,50 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
         // boundaries.  The load cursor knows its tile's key one tile early, so entering a tile costs no dependent load.
         const int my_tiles = blockIdx.x < total_tiles ? (total_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
         const int total_blocks = my_tiles * KB;                    // of the stream; this warp converts par, par + 2, ...
-        auto panel_row = [&](int t, int key) -> const uint8_t* {
-            const uint8_t* mat = a.slots + (size_t)(key % a.num_slots) * a.slot_stride + (GATEUP ? 0 : w13_bytes);
-            return mat + (size_t)((t % MT) * 8 + pw) * KB * kBlockBytes + lane * 16;
+        // Token tile and weight tile of the cursor's next tile are stepped: with divisions
+        // (128, 333, 1024 tokens: 114.8, 126.7, 167.0 -> 113.2, 123.8, 164.1 us per OLMoE-shaped layer).
+        const int scale_at = kCodeBytes - lane * 16 + q * 4;
+        const int step_ti = (int)gridDim.x / MT, step_mt = (int)gridDim.x % MT;
+        int c_mt = (int)blockIdx.x % MT, n_ti = (int)blockIdx.x / MT, n_mt = c_mt;
+        const uint8_t* const mat0 = a.slots + (GATEUP ? 0 : w13_bytes) + (size_t)pw * KB * kBlockBytes + lane * 16;
+        const size_t mt_stride = (size_t)8 * KB * kBlockBytes;
+        auto panel_row = [&](int key) -> const uint8_t* {          // this lane's codes of weight tile c_mt, block 0
+            const int slot = key < a.num_slots ? key : key % a.num_slots;
+            return mat0 + (size_t)slot * a.slot_stride + (size_t)c_mt * mt_stride;
         };
         int c_t = blockIdx.x, c_kb = par, c_g = par;               // load cursor: tile, block of it, index in the stream
         int c_key_next = 0;
-        const uint8_t* c_pn = nullptr;
+        const uint8_t* c_pn = nullptr;                             // the cursor's block
+        auto look_ahead = [&]() {                                  // key of the tile after the cursor's
+            n_ti += step_ti;
+            n_mt += step_mt;
+            if (n_mt >= MT) { n_mt -= MT; ++n_ti; }
+            if (c_t + (int)gridDim.x < total_tiles) c_key_next = a.tiles[n_ti].key;
+        };
         auto enter_tiles = [&]() {                                 // bring the cursor's block index back inside a tile
             while (c_kb >= KB && c_t < total_tiles) {
                 c_kb -= KB;
                 c_t += gridDim.x;
                 if (c_t < total_tiles) {
-                    c_pn = panel_row(c_t, c_key_next);
-                    if (c_t + (int)gridDim.x < total_tiles) c_key_next = a.tiles[(c_t + gridDim.x) / MT].key;
+                    c_mt = n_mt;
+                    c_pn = panel_row(c_key_next) + (size_t)c_kb * kBlockBytes;
+                    look_ahead();
                 }
             }
         };
         if (my_tiles) {
-            c_pn = panel_row(c_t, a.tiles[c_t / MT].key);
-            if (c_t + (int)gridDim.x < total_tiles) c_key_next = a.tiles[(c_t + gridDim.x) / MT].key;
+            c_pn = panel_row(a.tiles[n_ti].key) + (size_t)c_kb * kBlockBytes;
+            look_ahead();
             enter_tiles();                                         // KB == 1 and par == 1: the first block is the next tile's
         }
         constexpr int PF = 2;                                      // blocks in flight per lane (this one + 1 ahead)
         uint4 w[PF][2];
         uint32_t sc[PF];
         auto fetch = [&](uint4 (&wv)[2], uint32_t& sv) {           // request the cursor's block, move the cursor two on
-            const uint8_t* blk = c_pn + (size_t)c_kb * kBlockBytes;
-            wv[0] = ldg_stream128(blk);
-            wv[1] = ldg_stream128(blk + 512);
-            sv = ldg_stream32(blk - lane * 16 + kCodeBytes + q * 4);
+            wv[0] = ldg_stream128(c_pn);
+            wv[1] = ldg_stream128(c_pn + 512);
+            sv = ldg_stream32(c_pn + scale_at);
+            c_pn += 2 * kBlockBytes;
             c_g += 2;
             c_kb += 2;
             enter_tiles();
