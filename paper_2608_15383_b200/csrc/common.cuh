@@ -150,15 +150,16 @@ void launch_wait_selftest(int* status, long long budget_cycles, int* result, cud
 constexpr int kPlanGatherPairs = 8192, kPlanGatherKeys = 1024;
 void launch_plan_gather(const exmoe_shape& s, int C, int n_keys, int max_waves, bool identity, const __nv_bfloat16* hidden,
                         const int32_t* ids, int n_pairs, PlanPtrs plan, int* status, __nv_bfloat16* xg, bool single_wave,
-                        void* scratch, bool small_n, cudaStream_t st);
+                        void* scratch, int tile_rows, cudaStream_t st);
 // grouped copy of the hidden rows; when `single_wave` is given its CTA 0 also builds that wave's tile list in `scratch`
 void launch_gather_rows(const __nv_bfloat16* hidden, const int32_t* perm, const int32_t* n_valid, int n_pairs, int top_k,
                         int H, __nv_bfloat16* xg, const GemmArgs* single_wave, const int32_t* wave_start, void* scratch,
-                        bool small_n, cudaStream_t st);
+                        int tile_rows, cudaStream_t st);
 // which: bit 0 = gate/up GEMM + SwiGLU, bit 1 = down GEMM x routing weight, bit 2 = (re)build the wave's tile list
 // small_n: the 64-row, eight-stage kernel shape (a few dozen rows per expert) instead of the 256-row, four-stage one
 void launch_prefill_wave(const GemmArgs& g, const int32_t* wave_start, void* scratch, int* status, const PrefillMaps* maps,
-                         __nv_bfloat16* act, const float* topk_w, float* y, int which, bool small_n, cudaStream_t st);
+                         __nv_bfloat16* act, const float* topk_w, float* y, int which, bool small_n, int tile_rows, cudaStream_t st);
+int prefill_tile_rows(const exmoe_shape& s, int n_pairs, int experts_per_wave, bool small_n);     // most grouped rows per tile
 #ifndef EXMOE_PREFILL_SMALL_N_MAX_PAIRS
 #define EXMOE_PREFILL_SMALL_N_MAX_PAIRS 1024
 #endif

@@ -44,6 +44,8 @@
 // the conversion work nor, it turned out, the time.
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "frag.cuh"
 #include "mbar.cuh"
@@ -798,15 +800,27 @@ static int sm_count() {
     return sms;
 }
 
+// The most grouped rows of a tile: all that the kernel shape takes, but halved down to 64 while twice the tiles still fit
+// the SMs in one go.  The smaller tiles convert the weights again, on SMs that would idle, and the launch ends sooner: its
+// end is one tile's epilogue, which takes time by its columns.  512 x 256, 16 experts, 300 tokens: 32.2 -> 26.9 us per layer,
+// 256 x 128, 8 experts, 600 tokens: 26.4 -> 20.6 us; with more tiles than SMs it lost (2048 x 1536, 8 experts, 200 tokens:
+// 57 -> 65 us).
+int prefill_tile_rows(const exmoe_shape& s, int n_pairs, int experts_per_wave, bool small_n) {
+    const int mt = std::min(2 * s.d_ff, s.d_model) / BM, sms = sm_count();
+    int rows = small_n ? BN_SMALL : BN;
+    while (rows > BN_SMALL && 2 * std::max(std::min(n_pairs, experts_per_wave), n_pairs / rows) * mt <= sms) rows /= 2;
+    return rows;
+}
+
 void launch_plan_gather(const exmoe_shape& s, int C, int n_keys, int max_waves, bool identity, const __nv_bfloat16* hidden,
                         const int32_t* ids, int n_pairs, PlanPtrs plan, int* status, __nv_bfloat16* xg, bool single_wave,
-                        void* scratch, bool small_n, cudaStream_t st) {
+                        void* scratch, int tile_rows, cudaStream_t st) {
     const int sms = sm_count(), seg = (n_pairs + sms - 1) / sms, n_seg = (n_pairs + seg - 1) / seg;
     int32_t* n_tiles = reinterpret_cast<int32_t*>(scratch);
     Tile* tiles = single_wave ? reinterpret_cast<Tile*>(reinterpret_cast<unsigned char*>(scratch) + 256) : nullptr;
     launch_dependent(plan_gather_kernel, n_seg + 1, kPlanThreads, (size_t)(2 * n_keys + 1 + seg) * 4, st, hidden, ids, n_pairs,
                      s.top_k, s.d_model, s.num_experts, C, n_keys, max_waves, identity, seg, plan, status, xg, tiles, n_tiles,
-                     small_n ? BN_SMALL : BN);
+                     tile_rows);
 }
 
 size_t prefill_scratch_bytes(int max_pairs, int num_experts) {
@@ -856,18 +870,18 @@ void launch_wait_selftest(int* status, long long budget_cycles, int* result, cud
 
 void launch_gather_rows(const __nv_bfloat16* hidden, const int32_t* perm, const int32_t* n_valid, int n_pairs, int top_k,
                         int H, __nv_bfloat16* xg, const GemmArgs* single_wave, const int32_t* wave_start, void* scratch,
-                        bool small_n, cudaStream_t st) {
+                        int tile_rows, cudaStream_t st) {
     int32_t* n_tiles = reinterpret_cast<int32_t*>(scratch);
     Tile* tiles = single_wave ? reinterpret_cast<Tile*>(reinterpret_cast<unsigned char*>(scratch) + 256) : nullptr;
     gather_rows_kernel<<<(n_pairs + 7) / 8, 256, 0, st>>>(hidden, perm, n_valid, top_k, H, xg, single_wave ? single_wave->counts : nullptr,
                                                  single_wave ? single_wave->group_keys : nullptr, wave_start, tiles, n_tiles,
-                                                 small_n ? BN_SMALL : BN);
+                                                 tile_rows);
     count_launch();
 }
 
 // One wave of the tensor-core path: tile list, gate/up GEMM + SwiGLU, down GEMM x routing weight.
 void launch_prefill_wave(const GemmArgs& g, const int32_t* wave_start, void* scratch, int* status, const PrefillMaps* maps,
-                         __nv_bfloat16* act, const float* topk_w, float* y, int which, bool small_n, cudaStream_t st) {
+                         __nv_bfloat16* act, const float* topk_w, float* y, int which, bool small_n, int tile_rows, cudaStream_t st) {
     int32_t* n_tiles = reinterpret_cast<int32_t*>(scratch);
     Tile* tiles = reinterpret_cast<Tile*>(reinterpret_cast<unsigned char*>(scratch) + 256);
     PrefillArgs a{};
@@ -893,7 +907,7 @@ void launch_prefill_wave(const GemmArgs& g, const int32_t* wave_start, void* scr
     const CUtensorMap* mx = reinterpret_cast<const CUtensorMap*>(maps->dev);
     const CUtensorMap* ma = mx + N_MAPS;
     if (which & 4) {
-        tile_list_kernel<<<1, 1024, 0, st>>>(g.counts, g.group_keys, wave_start, tiles, n_tiles, small_n ? BN_SMALL : BN);
+        tile_list_kernel<<<1, 1024, 0, st>>>(g.counts, g.group_keys, wave_start, tiles, n_tiles, tile_rows);
         count_launch();
     }
     if (which & 1) {
