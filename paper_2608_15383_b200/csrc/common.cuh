@@ -127,10 +127,13 @@ void launch_group(const exmoe_shape& s, int C, int n_keys, int max_waves, bool i
 // Streaming kernels (bulk-copy weight ring in shared memory) above kSmallMaxPairs pairs, up to 640, or fewer than 12 per expert.
 // Their time grows with the eight-row passes over each expert's weights, that of the tensor-core kernels hardly with the
 // rows: 2048 x 1024, top-8: 64 experts 84 tokens (10.5 rows per expert) 105 -> 85 us per layer, 96 experts 128 tokens (10.7)
-// 147 -> 128 us; past 16 rows per expert they lose (64 experts, 192 tokens: 148 against 125 us).
-constexpr int kStreamMaxPairs = 640, kStreamMaxRows = 12;
-constexpr bool stream_range(int n_pairs, int n_experts) { return n_pairs <= kStreamMaxPairs || n_pairs < kStreamMaxRows * n_experts; }
-constexpr int kStreamOwnPlanKeys = 128, kStreamOwnPlanPairs = 640;    // most experts and pairs that the streaming kernels group themselves
+// 147 -> 128 us; past 16 rows per expert they lose (64 experts, 192 tokens: 148 against 125 us).  Up to 128 experts: every
+// CTA walks the plan's groups for its share of the work, the first 128 of them from registers.
+constexpr int kStreamMaxPairs = 640, kStreamMaxRows = 12, kStreamMaxExperts = 128;
+constexpr bool stream_range(int n_pairs, int n_experts) {
+    return n_pairs <= kStreamMaxPairs || (n_experts <= kStreamMaxExperts && n_pairs < kStreamMaxRows * n_experts);
+}
+constexpr int kStreamOwnPlanKeys = 128, kStreamOwnPlanPairs = 640;        // most experts and pairs that the streaming kernels group themselves
 bool stream_supported(int H, int I);
 bool launch_stream_wave(const GemmArgs& a, const __nv_bfloat16* hidden, __nv_bfloat16* act, const float* topk_w, float* y,
                         int* status, int max_groups, bool gateup, bool down, cudaStream_t st);

@@ -12,8 +12,8 @@
 // eight products in ascending order, then a shuffle tree).  Above that the logits are a GEMM and run on the tensor
 // cores (route_mma_kernel), with every decision that their rounding could turn repeated in that same arithmetic, so
 // the choice of experts does not depend on the batch size.
-// The logits travel through the cluster's shared memory to the CTA that owns the token; one of its warps does the
-// softmax (expf, binary32) and k rounds of a warp-wide arg-max that orders equal probabilities by ascending id.
+// The logits travel through the cluster's shared memory to the CTA that owns the token, which does the softmax (expf,
+// binary32) and the choice of the k largest, equal probabilities ordered by ascending id.
 #include <cooperative_groups.h>
 
 #include "common.cuh"

@@ -2,7 +2,7 @@
 // grouped expert GEMMs of a wave (Section 3.4, Eq. 2) as HBM-bound streams over the packed expert bytes,
 // with the memory system decoupled from the arithmetic.
 //
-// The work of a wave is cut into units: (active group = expert, pass over up to R = 8 or 16 of the group's rows,
+// The work of a wave is cut into units: (active group = expert, pass over up to eight of the group's rows,
 // tile of PP panels; gate/up: PP gate+up panel pairs).  A tile is ONE contiguous range of the packed
 // expert image.  Units are ordered group-major, then pass, then tile, and every persistent CTA (one per
 // SM) takes an equal contiguous share, so that the load is balanced by arithmetic, not by expert, and a
@@ -24,7 +24,7 @@
 // FP16 MMAs here), 67 us; sixteen independent warps with their blocks in registers, no ring and no exchange per
 // unit, 62 us (a warp's loads share a few scoreboards: waiting for the oldest block waits for the newest as well).
 // The down kernel is a programmatic dependent of the gate/up kernel: its weight ring fills while the
-// gate/up kernel drains; only its activation producer waits for the dependency.
+// gate/up kernel drains; the consumers wait for the dependency before they fetch rows.
 // Every mbarrier wait is bounded: on expiry the CTA raises EXMOE_ERR_TIMEOUT, all roles leave their
 // loops and the producers wait (bounded) for their copies in flight before the CTA exits.
 #include "common.cuh"

@@ -89,3 +89,24 @@ def test_host_forward_follows_a_miss_path_switch(B, olmoe_layer):
         helpers.compare_plan(host, sc, ids)
     assert host.status() == 0
     full.close(); host.close()
+
+
+@pytest.mark.parametrize("shape, T", [(synth.MID, 1), (synth.MID, 4), (synth.MID, 5),      # 1, 4 and 5 KB of activations
+                                      (synth.Shape(2048, 256, 8, 2), 1), (synth.Shape(2048, 256, 8, 2), 2),    # 4 and 8 KB
+                                      (synth.Shape(256, 128, 8, 3), 8)])                   # 4 KB, 24 pairs
+def test_inputs_as_kernel_parameters_at_their_limits(B, shape, T):
+    """Up to 4 KB of activations the inputs travel with the launches: the bits of the device call on both sides of the
+    limit, with an invalid id reported and left out in both."""
+    _, bank = helpers.make_layer(shape, seed=61)
+    cache = B.Cache(shape, [bank], shape.num_experts, max_tokens=8)
+    stream = torch.cuda.Stream()
+    for rep in range(3):
+        hidden, ids, p = helpers.routed_inputs(shape, T, seed=5500 + T + rep, alpha=0.0)
+        if rep == 2:
+            ids[0, -1] = shape.num_experts
+        want = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda()).cpu()
+        assert cache.status() == (B.EXMOE_ERR_BAD_EXPERT_ID if rep == 2 else 0)
+        got = cache.forward_host(0, hidden, ids, p, stream=stream)
+        assert torch.equal(got.view(torch.int16), want.view(torch.int16)), rep
+        assert cache.status() == (B.EXMOE_ERR_BAD_EXPERT_ID if rep == 2 else 0)
+    cache.close()

@@ -337,3 +337,48 @@ def test_streaming_kernels_past_their_own_grouping(B, olmoe_layer, T):
     assert torch.equal(out2.view(torch.int16), out.view(torch.int16))
     assert cache.status() == 0 and part.status() == 0
     cache.close(); part.close()
+
+
+@pytest.mark.parametrize("E, k, T", [
+    (16, 5, 5),                        # 25 pairs: the smallest streaming call
+    (128, 4, 160),                     # the most experts and pairs that the streaming kernels group themselves
+    (132, 4, 160),                     # ... and the first size that takes the grouping kernel's plan
+    (16, 3, 43)])                      # groups of eight, nine and more rows: remainders of the eight-row passes
+def test_edges_of_the_streaming_kernels_own_grouping(B, E, k, T):
+    s = synth.Shape(256, 128, E, k)
+    ora, bank = helpers.make_layer(s, seed=41 + E + k)
+    hidden, ids, p = helpers.routed_inputs(s, T, seed=5300 + T + E, alpha=0.3)
+    y, ref = ora.forward(hidden, ids, p)
+    cache = B.Cache(s, [bank], E, max_tokens=T)
+    out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    assert cache.last_path() == B.PATH_STREAM
+    compare_plan(cache, ocache.SlotCache(E, E, 0, bytes_per_expert=cache.bytes_per_expert), ids)
+    helpers.check_output(out, y, ref, f"E={E} k={k} T={T}")
+    assert cache.status() == 0
+    cache.close()
+
+
+@pytest.mark.parametrize("T", [1, 4, 40])
+def test_activation_scaling_over_magnitudes(B, T):
+    """The decode and streaming kernels scale every 128-wide block of a row into FP16 by a power of two: rows of 1e-6 to
+    1e6, a row with one block of zeros and rows with one element 4096 times the others keep the repository's tolerance,
+    each row by itself (an element 2^-12 of its block's largest still has all eight of its bits: FP16 reaches 2^-24
+    below 1, scaled blocks start at 2^15)."""
+    s = synth.MID
+    ora, bank = helpers.make_layer(s, seed=55)
+    base, ids, p = helpers.routed_inputs(s, T, seed=5400 + T, alpha=0.5)
+    cache = B.Cache(s, [bank], s.num_experts, max_tokens=T)
+    for what in (1e-6, 1e-3, 1e3, 1e6, "zero block", "outlier"):
+        hidden = base.clone()
+        if what == "zero block":
+            hidden[:, 128:256] = 0
+        elif what == "outlier":
+            hidden[:, 77] = 4096.0
+        else:
+            hidden = (hidden.float() * what).to(torch.bfloat16)
+        y, ref = ora.forward(hidden, ids, p)
+        out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+        for t in range(0, T, 7):
+            helpers.check_output(out[t:t + 1], y[t:t + 1], ref[t:t + 1], f"T={T} row {t} {what}")
+    assert cache.status() == 0
+    cache.close()
