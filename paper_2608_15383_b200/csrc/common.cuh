@@ -62,7 +62,8 @@ struct GemmArgs {
     int group_filter;           // 0 all groups of the wave; 1 only groups whose expert was resident; 2 only the missed ones
     int direct_keys;            // > 0: every key 0 .. direct_keys-1 is a (possibly empty) group of the call's only wave
                                 // (all experts resident, key = expert id): kernels may read counts / offsets by key at
-                                // once instead of going through wave_start and group_keys first
+                                // once instead of going through wave_start and group_keys first.  The size of the key
+                                // space: more than the number of experts where wave_cap is below num_slots
     // Streaming kernels, all experts resident: the ids of the call (null: read the plan).  Every CTA then groups them itself.
     const int32_t* ids;
     int n_pairs;

@@ -218,7 +218,7 @@ stream_gemm_kernel(const StreamArgs p) {
         for (int i = 0; i < PT; ++i) {
             const int pr = tid + i * kStreamThreads;
             if (pr >= a.n_pairs) continue;
-            const bool valid = id[i] >= 0 && id[i] < a.direct_keys;
+            const bool valid = id[i] >= 0 && id[i] < a.num_slots;      // every expert has its slot: num_slots is their number (the key space, direct_keys, may be larger)
             s_key[pr] = valid ? id[i] : -1;
             if (valid) atomicAdd(&s_cnt[id[i]], 1);
             bad |= !valid;

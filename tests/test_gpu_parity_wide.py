@@ -358,6 +358,35 @@ def test_edges_of_the_streaming_kernels_own_grouping(B, E, k, T):
     cache.close()
 
 
+@pytest.mark.parametrize("E, wave_cap, k, T", [(16, 8, 4, 8), (16, 8, 4, 16), (16, 4, 2, 320), (64, 32, 1, 25), (16, 0, 4, 16)])
+def test_ids_beyond_the_experts_in_a_larger_key_space(B, E, wave_cap, k, T):
+    """Every expert resident and a wave_cap below the number of experts: the key space (ceil(E / wave_cap) * E) is larger
+    than the expert count, and ids E .. keys - 1 are as invalid as any other id out of range: sticky status, no
+    contribution, the other tokens' bits unchanged.  Layer 0 of a cache of several layers: the slots such an id would
+    name lie inside the slot memory."""
+    s = synth.Shape(256, 128, E, k)
+    ora, bank = helpers.make_layer(s, seed=61 + E)
+    hidden, ids, p = helpers.routed_inputs(s, T, seed=5500 + T, alpha=0.3)
+    cache = B.Cache(s, [bank] * 5, E, max_tokens=T, wave_cap=wave_cap)
+    clean = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    assert cache.last_path() == B.PATH_STREAM and cache.status() == 0
+    y, ref = ora.forward(hidden, ids, p)
+    helpers.check_output(clean, y, ref, "clean")
+    bad = ids.clone()
+    bad[1], bad[T - 2, 0], bad[T // 2, k - 1] = E, -1, 2 * E - 1
+    out = cache.forward(0, hidden.cuda(), bad.cuda(), p.cuda())
+    assert cache.status() == B.EXMOE_ERR_BAD_EXPERT_ID
+    hit = torch.zeros(T, dtype=torch.bool)
+    hit[[1, T // 2, T - 2]] = True
+    assert torch.equal(out[~hit].view(torch.int16), clean[~hit].view(torch.int16))
+    assert not out[1].any()
+    kept = torch.where((bad >= 0) & (bad < E), bad, torch.full_like(bad, -1))
+    y, ref = ora.forward(hidden, kept, p)
+    helpers.check_output(out, y, ref, "invalid ids add nothing")
+    compare_plan(cache, ocache.SlotCache(E, E, wave_cap, bytes_per_expert=cache.bytes_per_expert), kept)
+    cache.close()
+
+
 @pytest.mark.parametrize("T", [1, 4, 40])
 def test_activation_scaling_over_magnitudes(B, T):
     """The decode and streaming kernels scale every 128-wide block of a row into FP16 by a power of two: rows of 1e-6 to
