@@ -27,12 +27,13 @@ namespace cg = cooperative_groups;
 
 constexpr int kRouteThreads = 256;
 constexpr int kRouteSmemMax = 200 * 1024;
-// Measured crossings (64 experts, d_model 2048, weights cold, launch included), us for the forms in this order:
-//   T = 32: 10.2 / 10.2 / - / -      64: 12.3 / 12.3 / 15.1 / -      256: 22.5 / 17.3 / 16.4 / 24.6
-//   1024: 61 / 39 / 18.5 / 24.6      2048: 115 / 68 / 24.6 / 24.6    4096: 219 / 125 / 37 / 28.7    8192: 430 / 240 / 63 / 47
+// Measured crossings (64 experts, d_model 2048, weights cold, launch included), us for one token per cluster, four tokens per
+// cluster, tensor cores with 16 experts per CTA, with 32:
+//   T = 32: 10.2 / 10.2 / - / -      64: 12.3 / 12.3 / 15.1 / -      256: 22.5 / 17.3 / 16.4 / -
+// and replayed from a graph, for the last two: 1024: 11.8 / 12.4      1184: 16.2 / 13.9      2048: 19.4 / 16.3      8192: 58 / 43
 constexpr int kRouteFewTokens = 48;       // four tokens per cluster from here on
 constexpr int kRouteMmaTokens = 224;      // tensor cores from here on
-constexpr int kRouteWideTokens = 2304;    // ... with 32 instead of 16 tokens per CTA
+constexpr int kRouteWideTokens = 1152;    // ... with 32 instead of 16 experts per CTA
 constexpr int kRouteWarps = kRouteThreads / 32;
 
 __device__ __forceinline__ void unpack8(const uint4& a, float (&x)[8]) {
@@ -250,20 +251,26 @@ int launch_route(const exmoe_shape& s, const __nv_bfloat16* hidden, const __nv_b
 }
 
 // ---- many tokens: the logits as a tensor-core GEMM -------------------------------------------------------------
-// A CTA takes TM tokens; its eight warps split K (32-wide steps, round robin) and their partial logits meet in shared
+// A CTA takes 16 tokens; its eight warps split K (32-wide steps, round robin) and their partial logits meet in shared
 // memory.  Operands come straight from L2 in 16-byte loads: a lane's eight consecutive k serve two m16n8k16 steps of both
 // operands, the permutation of K inside the step being the same on both sides.  Batches of a few hundred tokens are
-// latency again: a cluster of four CTAs then splits the experts (16 tokens, 16 experts each, four steps of loads in
-// flight per warp); from a few thousand tokens on two CTAs share 32 tokens, half of the experts each, which
-// reads the matrix half as often (one CTA for all 64 experts needs too many registers to share an SM: 55 us at T = 8192).
+// latency again: a cluster of four CTAs then splits the experts (16 of them each, four steps of loads in flight per warp);
+// where these no longer find room on the chip at once (two CTAs per SM), two CTAs share the 16 tokens, half of the experts
+// each, and read every row half as often (1024 tokens: 11.8 against 12.4 us, 1184: 16.2 against 13.9, 4096: 33 against 24).
+// An MMA truncates: every product to 2^-25 of the largest one's (and the accumulator's) binade, the result to 24 bits (both
+// measured).  So each starts from zero and its 16 products are added in binary32, to two running sums, which meet with
+// the other warps' in a tree: against 64 bits the logits are off by 1.7e-9 |x| |w| in the root mean square at d_model 2048
+// (the binary32 form 1.65e-9; all the MMAs of a warp in one accumulator 5.2e-9, and up to 3e-6 for rows with their largest
+// values in front), the probabilities by no more than the binary32 form's.
 // The experts are an integer decision, and the one made by the binary32 form above is kept: where two of a token's k + 1
 // largest logits are closer than the two forms can be apart, those experts' logits are recomputed in the binary32 form
-// and the choice is made on these.  The forms differ by rounding only: at most 1.5e-7 |x| |w| (5e-8 from d_model 2048 on)
-// in 3.1 million logits of random rows of 128 to 4096 values; the bound taken is 2e-6, so that about one token in
-// eighty is looked at again (64 experts, d_model 2048).
+// and the choice is made on these.  With S = sum |x_i w_i| <= |x| |w|: the MMAs lose less than 15 / 4 + 1 units of 2^-23 of
+// their products, together under 2^-20 S; every logit passes H / 512 + 6 additions here and 8 + H / 256 + 5 in the
+// binary32 form, each off by 2^-24 S at most; |x| and |w| come out of BF16 sums of H / 64 terms, short of the true ones
+// by (1 - 2^-9)^(H / 128) at most, both together by 1 / 1.14.
 constexpr int kMmaMaxExperts = 128;
 constexpr int kMmaMaxModel = 4096;                    // |x|^2 and |w|^2 are summed in BF16 over H / 64 terms per lane
-constexpr float kRouteBound = 2e-6f;
+__device__ __forceinline__ float route_bound(int H) { return 1.14f * (0x1p-20f + (float)(21 + 3 * H / 512) * 0x1p-24f); }
 
 // Binary32 logits of the experts marked in `again` (bit i of a lane: expert lane + 32 i), by one warp.
 __device__ __noinline__ void logits_again(float* z, unsigned again, const __nv_bfloat16* __restrict__ x,
@@ -361,18 +368,19 @@ __device__ __forceinline__ void choose(float* z, float slack, const __nv_bfloat1
     sum = warp_sum(sum);
     if (lane < k) {
         ids[lane] = mine;
-        wts[lane] = expf(z[mine] - mx) * (1.f / sum);
+        wts[lane] = expf(z[mine] - mx) / sum;
     }
 }
 
-// MT: 16-token tiles per CTA; NT: 8-expert tiles per CTA; CL: CTAs per cluster (CL * NT = 8: 64 experts per pass);
-// U: steps of loads in flight
-template <int MT, int NT, int CL, int U>
-__global__ void __launch_bounds__(kRouteThreads)
+// 16 tokens per CTA; NT: 8-expert tiles per CTA; CL: CTAs per cluster (CL * NT = 8: 64 experts per pass); U: steps of loads in
+// flight (even: they alternate between the two running sums).  Two CTAs share an SM.
+template <int NT, int CL, int U>
+__global__ void __launch_bounds__(kRouteThreads, 2)
 route_mma_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* __restrict__ w_router,
                  const float* __restrict__ bias, int T, int H, int E, int k, int32_t* __restrict__ ids_out,
                  float* __restrict__ w_out) {
-    constexpr int TM = 16 * MT, EC = 8 * NT, EB = CL * EC;                  // experts of a CTA / of the cluster per pass
+    constexpr int TM = 16, EC = 8 * NT, EB = CL * EC;                       // experts of a CTA / of the cluster per pass
+    static_assert(U % 2 == 0, "the two running sums");
     constexpr int TOK = TM / CL;                                           // tokens whose choice this CTA makes
     extern __shared__ __align__(16) unsigned char smem[];
     float* part = reinterpret_cast<float*>(smem);                          // [warp][TM][EC + 1]
@@ -389,10 +397,10 @@ route_mma_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* 
     grid_launch_dependents();
     if (CL > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // every CTA runs: its memory may be written
     const __nv_bfloat162 zero2(__float2bfloat16(0.f), __float2bfloat16(0.f));
-    const uint4* xrow[2 * MT];
-    __nv_bfloat162 xsq[2 * MT];
+    const uint4* xrow[2];
+    __nv_bfloat162 xsq[2];
 #pragma unroll
-    for (int r = 0; r < 2 * MT; ++r) {                                     // rows beyond the last token repeat it
+    for (int r = 0; r < 2; ++r) {                                          // rows beyond the last token repeat it
         xrow[r] = reinterpret_cast<const uint4*>(hidden + (size_t)(t0 + min(8 * r + q, n_tok - 1)) * H) + c;
         xsq[r] = zero2;
     }
@@ -412,25 +420,23 @@ route_mma_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* 
     float wtop = 0.f;
     for (int p0 = 0; p0 < E; p0 += EB) {
         const int e0 = p0 + rank * EC;
-        float acc[MT][NT][4];
+        float acc[2][NT][4];                                           // two running sums
         __nv_bfloat162 wsq[NT];
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
             wsq[n] = zero2;
 #pragma unroll
-            for (int m = 0; m < MT; ++m)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) acc[m][n][i] = 0.f;
+            for (int i = 0; i < 4; ++i) acc[0][n][i] = acc[1][n][i] = 0.f;
         }
         const uint4* wrow = reinterpret_cast<const uint4*>(w_router) + (size_t)(e0 + q) * (H / 8) + c;
         const size_t wstep = (size_t)H;                                    // eight expert rows, in 16-byte chunks
         for (int s0 = warp; s0 < steps; s0 += U * kRouteWarps) {
-            uint4 a[U][2 * MT], b[U][NT];
+            uint4 a[U][2], b[U][NT];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int s = s0 + u * kRouteWarps;
 #pragma unroll
-                for (int r = 0; r < 2 * MT; ++r) {
+                for (int r = 0; r < 2; ++r) {
                     a[u][r] = make_uint4(0, 0, 0, 0);
                     if (s < steps) a[u][r] = xrow[r][4 * s];
                 }
@@ -443,27 +449,26 @@ route_mma_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* 
 #pragma unroll
             for (int u = 0; u < U; ++u) {
 #pragma unroll
-                for (int n = 0; n < NT; ++n)
+                for (int n = 0; n < NT; ++n) {
+                    const uint4 &lo = a[u][0], &hi = a[u][1];
+                    float d[2][4] = {};
+                    mma_m16n8k16(d[0], lo.x, hi.x, lo.y, hi.y, b[u][n].x, b[u][n].y);
+                    mma_m16n8k16(d[1], lo.z, hi.z, lo.w, hi.w, b[u][n].z, b[u][n].w);
 #pragma unroll
-                    for (int m = 0; m < MT; ++m) {
-                        const uint4 &lo = a[u][2 * m], &hi = a[u][2 * m + 1];
-                        mma_m16n8k16(acc[m][n], lo.x, hi.x, lo.y, hi.y, b[u][n].x, b[u][n].y);
-                        mma_m16n8k16(acc[m][n], lo.z, hi.z, lo.w, hi.w, b[u][n].z, b[u][n].w);
-                    }
+                    for (int i = 0; i < 4; ++i) acc[u & 1][n][i] += d[0][i] + d[1][i];
+                }
 #pragma unroll
                 for (int n = 0; n < NT; ++n) square(wsq[n], b[u][n]);
                 if (p0 == 0)
 #pragma unroll
-                    for (int r = 0; r < 2 * MT; ++r) square(xsq[r], a[u][r]);
+                    for (int r = 0; r < 2; ++r) square(xsq[r], a[u][r]);
             }
         }
         float* mine = part + warp * TM * (EC + 1);
 #pragma unroll
-        for (int m = 0; m < MT; ++m)
+        for (int n = 0; n < NT; ++n)
 #pragma unroll
-            for (int n = 0; n < NT; ++n)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) mine[(16 * m + q + 8 * (i >> 1)) * (EC + 1) + 8 * n + 2 * c + (i & 1)] = acc[m][n][i];
+            for (int i = 0; i < 4; ++i) mine[(q + 8 * (i >> 1)) * (EC + 1) + 8 * n + 2 * c + (i & 1)] = acc[0][n][i] + acc[1][n][i];
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
             const float v = quad_sum(wsq[n]);
@@ -471,7 +476,7 @@ route_mma_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* 
         }
         if (p0 == 0)
 #pragma unroll
-            for (int r = 0; r < 2 * MT; ++r) {
+            for (int r = 0; r < 2; ++r) {
                 const float v = quad_sum(xsq[r]);
                 if (c == 0) xn[warp * TM + 8 * r + q] = v;
             }
@@ -479,9 +484,11 @@ route_mma_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* 
         if (CL > 1 && p0 == 0) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
         for (int i = tid; i < TM * EC; i += kRouteThreads) {
             const int t = i / EC, e = i % EC;
-            float v = 0.f;
+            float p[kRouteWarps];
 #pragma unroll
-            for (int w = 0; w < kRouteWarps; ++w) v += part[(w * TM + t) * (EC + 1) + e];
+            for (int w = 0; w < kRouteWarps; ++w) p[w] = part[(w * TM + t) * (EC + 1) + e];
+            static_assert(kRouteWarps == 8, "the tree of the partial sums");
+            const float v = ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
             if (e0 + e < E) {
                 float* dst = CL == 1 ? logit : cluster.map_shared_rank(logit, t % CL);
                 dst[(t / CL) * kMmaMaxExperts + e0 + e] = v + (bias ? bias[e0 + e] : 0.f);
@@ -510,19 +517,19 @@ route_mma_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* 
 #pragma unroll
         for (int w = 0; w < kRouteWarps; ++w) x2 += xn[w * TM + t];
         // of a pair both may be off; the bias addition rounds once more (relative to the logit)
-        choose(logit + i * kMmaMaxExperts, 2.f * kRouteBound * sqrtf(x2) * sqrtf(wmax), hidden + (size_t)(t0 + t) * H, w_router, bias,
+        choose(logit + i * kMmaMaxExperts, 2.f * route_bound(H) * sqrtf(x2) * sqrtf(wmax), hidden + (size_t)(t0 + t) * H, w_router, bias,
                H, E, k, lane, ids_out + (size_t)(t0 + t) * k, w_out + (size_t)(t0 + t) * k);
     }
 }
 
-template <int MT, int NT, int CL, int U>
+template <int NT, int CL, int U>
 int launch_route_mma(const exmoe_shape& s, const __nv_bfloat16* hidden, const __nv_bfloat16* w, const float* bias, int T,
                      int32_t* ids, float* wts, cudaStream_t st) {
-    constexpr int TM = 16 * MT, EC = 8 * NT;
+    constexpr int TM = 16, EC = 8 * NT;
     constexpr size_t smem = 4 * ((size_t)kRouteWarps * TM * (EC + 1) + (size_t)TM / CL * kMmaMaxExperts + kRouteWarps * (TM + EC) + 2 * CL);
     static SmemOnce once;
-    if (!allow_smem(route_mma_kernel<MT, NT, CL, U>, (int)smem, once)) return EXMOE_ERR_CUDA;
-    return launch_dependent(route_mma_kernel<MT, NT, CL, U>, (T + TM - 1) / TM * CL, CL, smem, s, hidden, w, bias, T, ids, wts, st);
+    if (!allow_smem(route_mma_kernel<NT, CL, U>, (int)smem, once)) return EXMOE_ERR_CUDA;
+    return launch_dependent(route_mma_kernel<NT, CL, U>, (T + TM - 1) / TM * CL, CL, smem, s, hidden, w, bias, T, ids, wts, st);
 }
 
 }  // namespace
@@ -547,8 +554,8 @@ extern "C" int exmoe_route(const exmoe_shape* shape, const void* hidden_bf16, co
     // memory or tiling does not fit takes the next simpler one; one token per cluster serves every shape.
     if (T >= kRouteMmaTokens && s.d_model % 32 == 0 && s.d_model <= kMmaMaxModel && s.num_experts <= kMmaMaxExperts &&
         s.top_k <= 32)
-        return T >= kRouteWideTokens ? launch_route_mma<2, 4, 2, 2>(s, x, w, bias, T, topk_ids, topk_weights, st)
-                                     : launch_route_mma<1, 2, 4, 4>(s, x, w, bias, T, topk_ids, topk_weights, st);
+        return T >= kRouteWideTokens ? launch_route_mma<4, 2, 2>(s, x, w, bias, T, topk_ids, topk_weights, st)
+                                     : launch_route_mma<2, 4, 4>(s, x, w, bias, T, topk_ids, topk_weights, st);
     if (T >= kRouteFewTokens && 4 * row + logits <= (size_t)kRouteSmemMax)
         return launch_route<8, 4>(s, x, w, bias, T, topk_ids, topk_weights, st);
     return launch_route<8, 1>(s, x, w, bias, T, topk_ids, topk_weights, st);
