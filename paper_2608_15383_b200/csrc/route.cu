@@ -269,6 +269,7 @@ int launch_route(const exmoe_shape& s, const __nv_bfloat16* hidden, const __nv_b
 // binary32 form, each off by 2^-24 S at most; |x| and |w| come out of BF16 sums of H / 64 terms, short of the true ones
 // by (1 - 2^-9)^(H / 128) at most, both together by 1 / 1.14.
 constexpr int kMmaMaxExperts = 128;
+constexpr float kExpSubnormal = 85.f, kExpZero = 106.f;    // expf(-x): normal below the first (2^-126 is e^-87.3), 0 above the second (2^-150: e^-104)
 constexpr int kMmaMaxModel = 4096;                    // |x|^2 and |w|^2 are summed in BF16 over H / 64 terms per lane
 __device__ __forceinline__ float route_bound(int H) { return 1.14f * (0x1p-20f + (float)(21 + 3 * H / 512) * 0x1p-24f); }
 
@@ -304,6 +305,11 @@ __device__ __noinline__ void logits_again(float* z, unsigned again, const __nv_b
 // One token's choice from its tensor-core logits, by one warp: the k + 1 largest in order; where two of them are within
 // `slack`, both are recomputed (at the cut everything that could displace the k-th) and the choice is made again.  A lane
 // holds the logits of experts lane, lane + 32, ... as order-preserving integers.
+// The other forms order binary32 PROBABILITIES, equal ones by id, and so does the choice made again.  Two logits may share a
+// probability where they differ: closer than expf resolves (its argument z - max is rounded to 2^-24 of itself, the
+// result to a few units of 2^-23), or far enough below the largest that their probabilities are subnormal or zero.  So
+// the first enters `near`, and a choice that reaches the second is made again in any case, with those logits recomputed
+// whose probability is subnormal; the exponential of anything below them is zero in every form.
 __device__ __forceinline__ void choose(float* z, float slack, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ w_router,
                                        const float* __restrict__ bias, int H, int E, int k, int lane, int32_t* __restrict__ ids,
                                        float* __restrict__ wts) {
@@ -316,14 +322,15 @@ __device__ __forceinline__ void choose(float* z, float slack, const __nv_bfloat1
         key[i] = 0;
         if (e < E) {
             const float v = z[e];
-            odd |= !(fabsf(v) < INFINITY);
+            odd |= !(v < INFINITY);                                        // a NaN or +infinity (-infinity: a masked expert)
             const uint32_t b = __float_as_uint(v);
             key[i] = b & 0x80000000u ? ~b : b | 0x80000000u;
         }
     }
     odd = __any_sync(0xffffffffu, odd);
-    unsigned again = odd ? ~0u : 0u;
-    float prev = INFINITY;
+    unsigned again = 0;
+    float prev = INFINITY, top_v = 0.f;
+    bool deep = false;
     int prev_e = 0, mine = 0;                                              // mine, lane j: the j-th choice (k <= 32)
     for (int j = 0; j <= k && j < E && !odd; ++j) {
         uint32_t best = 0;
@@ -337,8 +344,14 @@ __device__ __forceinline__ void choose(float* z, float slack, const __nv_bfloat1
         const uint32_t top = __reduce_max_sync(0xffffffffu, best);
         const int e = __reduce_min_sync(0xffffffffu, best == top ? be : 0x7fffffff);
         const float v = __uint_as_float(top & 0x80000000u ? top & 0x7fffffffu : ~top);
-        const float near = slack + 2.4e-7f * (fabsf(prev) + fabsf(v));
-        if (j > 0 && prev - v <= near) {
+        if (j == 0) {
+            top_v = v;
+            odd = v == -INFINITY;                                          // every expert masked: NaN probabilities
+        } else if (prev < top_v - kExpSubnormal + 2.f * slack) {           // another one follows: both may be subnormal or zero
+            deep = true;
+        }
+        const float near = slack + 2.4e-7f * (fabsf(prev) + fabsf(v) + (top_v - v)) + 1e-6f;
+        if (j > 0 && v > -INFINITY && prev - v <= near) {
             if (lane == (prev_e & 31)) again |= 1u << (prev_e >> 5);
             if (lane == (e & 31)) again |= 1u << (e >> 5);
             if (j == k)                                                    // the rest of the k-th's neighbourhood
@@ -353,11 +366,14 @@ __device__ __forceinline__ void choose(float* z, float slack, const __nv_bfloat1
         for (int i = 0; i < PER; ++i)
             if (lane + 32 * i == e) key[i] = 0;
     }
-    if (odd)
 #pragma unroll
-        for (int i = 0; i < PER; ++i)
-            if (lane + 32 * i >= E) again &= ~(1u << i);
-    if (__any_sync(0xffffffffu, again != 0)) {
+    for (int i = 0; i < PER; ++i) {
+        const int e = lane + 32 * i;
+        if (odd) again |= 1u << i;
+        if (deep && e < E && z[e] < top_v - kExpSubnormal + 2.f * slack && z[e] > top_v - kExpZero - 2.f * slack) again |= 1u << i;
+        if (e >= E) again &= ~(1u << i);
+    }
+    if (deep || __any_sync(0xffffffffu, again != 0)) {
         logits_again(z, again, x, w_router, bias, H, lane);
         softmax_topk(z, E, k, lane, ids, wts);
         return;

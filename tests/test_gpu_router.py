@@ -164,3 +164,38 @@ def test_near_ties_in_rows_of_one_sign(B):
         i1, p1 = B.exmoe_route(s, hidden[t:t + 40].contiguous(), w)
         assert torch.equal(ids[t:t + 40], i1)
         torch.testing.assert_close(p[t:t + 40], p1, rtol=2e-5, atol=1e-9)
+
+
+@pytest.mark.parametrize("what", ["small hidden states", "zero hidden states", "fewer than k unmasked", "masked with -inf", "all but one far below",
+                                  "subnormal probabilities", "large logits"])
+def test_choice_where_probabilities_cannot_tell(B, what):
+    """Logits that differ and share a binary32 probability (closer than expf resolves, or so far below the largest that the
+    probabilities are subnormal or zero) are ordered by id in every form: a batch that takes the tensor cores chooses what
+    calls of 40 tokens choose."""
+    s = synth.OLMOE
+    E, k, T = s.num_experts, s.top_k, 400
+    hidden, w, bias = synth.hidden_states(s, T, seed=21), synth.router_weights(s, seed=22), None
+    g = torch.Generator().manual_seed(23)
+    rows = torch.randperm(E, generator=g)
+    if what == "small hidden states":
+        hidden = (hidden.float() * torch.logspace(-12, -1, T)[:, None]).to(torch.bfloat16)
+    elif what == "zero hidden states":
+        hidden = torch.zeros_like(hidden)
+        bias = torch.randint(0, 40, (E,), generator=g).float() * 1e-9
+    elif what == "large logits":
+        bias = torch.rand(E, generator=g) * 90.0
+        bias[rows[:k]] = 90.0 + torch.arange(k) * 1e-6
+    else:
+        bias = torch.zeros(E)
+        if what == "subnormal probabilities":
+            bias[rows[3:]] = -torch.linspace(80.0, 115.0, E - 3)
+        elif what == "all but one far below":
+            bias[rows[1:]] = -200.0
+        else:
+            bias[rows[k - 2:]] = -1e4 if what == "fewer than k unmasked" else float("-inf")
+    hidden, w, bias = hidden.cuda(), w.cuda(), None if bias is None else bias.cuda()
+    ids, p = B.exmoe_route(s, hidden, w, bias)
+    for t in range(0, T, 40):
+        i1, p1 = B.exmoe_route(s, hidden[t:t + 40].contiguous(), w, bias)
+        assert torch.equal(ids[t:t + 40], i1), t
+        torch.testing.assert_close(p[t:t + 40], p1, rtol=2e-5, atol=1e-9)
