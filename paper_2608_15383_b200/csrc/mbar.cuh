@@ -54,7 +54,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 
 // The same by a whole warp, for barriers given by their shared-memory address: control flow that the compiler knows to be
 // uniform (no divergence bookkeeping around the poll, and the code around it keeps its uniform registers), no address
-// conversion per call.
+// conversion per call.  The wait ends when EVERY lane has seen the phase complete: what the barrier guards is ordered only
+// behind a lane's own successful wait.
 __device__ __forceinline__ void mbar_arrive_at(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -70,10 +71,10 @@ __device__ __forceinline__ bool mbar_try_at(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
-    if (__any_sync(0xffffffffu, mbar_try_at(bar, parity))) return true;
+    if (__all_sync(0xffffffffu, mbar_try_at(bar, parity))) return true;
     const long long t0 = clock64();
     for (unsigned polls = 1;; ++polls) {
-        if (__any_sync(0xffffffffu, mbar_try_at(bar, parity))) return true;
+        if (__all_sync(0xffffffffu, mbar_try_at(bar, parity))) return true;
         if ((polls & 15u) == 0) {
             const bool late = clock64() - t0 > kWaitBudget;
             if (late) {

@@ -351,7 +351,7 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
                                 if (!ok) break;
                             }
                             const int nst = (st + 1) % STAGES;
-                            ready = __any_sync(0xffffffffu, mbar_try_at(full_a + 8 * nst, nst ? ph : ph ^ 1));
+                            ready = __all_sync(0xffffffffu, mbar_try_at(full_a + 8 * nst, nst ? ph : ph ^ 1));
                             const uint64_t da = da0 + (uint64_t)(st * (A_STAGE_BYTES >> 4));
                             const uint64_t db = db0 + (uint64_t)(st * (B_STAGE_BYTES >> 4));
                             if (elect_one()) {

@@ -1,0 +1,19 @@
+"""Rules of the kernels' barrier code that no run on a GPU can show broken (a missing order between a wait and what it
+guards, a wait where only a look is meant): read from the sources."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2608_15383_b200", "csrc")
+
+
+def sources():
+    for name in sorted(os.listdir(CSRC)):
+        with open(os.path.join(CSRC, name)) as f:
+            yield name, re.sub(r"//[^\n]*", "", f.read())
+
+
+def test_a_warp_goes_on_only_when_every_lane_has_seen_the_barrier():
+    """A lane's memory accesses are ordered behind its own successful wait on an mbarrier, not behind another lane's: a vote
+    on the outcome has to ask for all lanes."""
+    votes = [(name, v) for name, text in sources() for v in re.findall(r"__(any|all)_sync\(\s*0xffffffffu\s*,\s*mbar_", text)]
+    assert votes and all(v == "all" for _, v in votes), votes
