@@ -70,6 +70,18 @@ __device__ __forceinline__ bool mbar_try_at(uint32_t bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// A look that never blocks (try_wait suspends the thread until the phase completes or a time limit of the hardware's).
+__device__ __forceinline__ bool mbar_look_at(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
     if (__all_sync(0xffffffffu, mbar_try_at(bar, parity))) return true;
     const long long t0 = clock64();

@@ -320,8 +320,10 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
         // instruction between two MMAs is time the pipe may drain, and with six busy warps on the same scheduler each takes
         // many cycles to issue (measured alone: the four MMAs of a stage run at N / 2 cycles each with compile-time operands,
         // at 150-160 cycles each, whatever N, behind run-time ring arithmetic and a barrier test).  So the ring is unrolled
-        // (stage index, barrier addresses and operand offsets are compile-time constants), the NEXT stage's barrier is tested
-        // before this stage's MMAs are issued, and the whole warp walks the loop with one elected lane issuing: with
+        // (stage index, barrier addresses and operand offsets are compile-time constants), the NEXT stage's barrier is looked at
+        // before this stage's MMAs are issued and the answer used after them (a look, not a try_wait, which suspends: that held
+        // this stage's MMAs back until the next stage came, and a tile's last ones for a time limit: 333 tokens 127 -> 117 us
+        // per OLMoE-shaped layer, 512/256/16/4 at 300 tokens 26.7 -> 19.1), and the whole warp walks the loop with one elected lane issuing: with
         // warp-uniform control flow the descriptors live in uniform registers, where the instruction wants them.
         // Shapes whose stage count per tile is not a multiple of the ring depth take the plain loop.
         PROF_DECL;
@@ -351,7 +353,7 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
                                 if (!ok) break;
                             }
                             const int nst = (st + 1) % STAGES;
-                            ready = __all_sync(0xffffffffu, mbar_try_at(full_a + 8 * nst, nst ? ph : ph ^ 1));
+                            const bool seen = mbar_look_at(full_a + 8 * nst, nst ? ph : ph ^ 1);
                             const uint64_t da = da0 + (uint64_t)(st * (A_STAGE_BYTES >> 4));
                             const uint64_t db = db0 + (uint64_t)(st * (B_STAGE_BYTES >> 4));
                             if (elect_one()) {
@@ -361,6 +363,7 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
                                 tc_commit_at(empty_a + 8 * st);    // stage reusable once these MMAs have read it
                             }
                             __syncwarp();
+                            ready = __all_sync(0xffffffffu, seen);
                         }
                         ph ^= 1;
                     }

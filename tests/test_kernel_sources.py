@@ -17,3 +17,13 @@ def test_a_warp_goes_on_only_when_every_lane_has_seen_the_barrier():
     on the outcome has to ask for all lanes."""
     votes = [(name, v) for name, text in sources() for v in re.findall(r"__(any|all)_sync\(\s*0xffffffffu\s*,\s*mbar_", text)]
     assert votes and all(v == "all" for _, v in votes), votes
+
+
+def test_the_issue_loop_only_looks_ahead():
+    """mbarrier.try_wait may suspend its thread: outside the waits themselves (mbar.cuh's, and loops that spin on it) a
+    barrier is looked at with test_wait, so that work in hand is not held back by a barrier that is not due yet."""
+    for name, text in sources():
+        if name == "mbar.cuh":
+            continue
+        ahead = [line.strip() for line in text.splitlines() if re.search(r"mbar_try(_at)?\(", line) and not re.search(r"\bwhile\s*\(", line)]
+        assert not ahead, (name, ahead)
