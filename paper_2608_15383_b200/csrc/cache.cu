@@ -439,7 +439,7 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
     }
     // timing runs that launch one kernel kind reuse the plan, grouped rows and tile list of the previous full call
     const bool build_plan = (c->prof_only == 0);
-    const bool use_stream = !small && c->stream_ok && stream_range(P, E);
+    const bool use_stream = !small && c->stream_ok && P <= kStreamMaxPairs;
     const bool own_plan = use_stream && identity && c->n_keys <= kStreamOwnPlanKeys && P <= kStreamOwnPlanPairs;     // the kernels group the ids themselves
     const bool plan_with_rows = !small && !use_stream && P <= kPlanGatherPairs && c->n_keys <= kPlanGatherKeys;   // below, with the rows
     if (!small && build_plan && !own_plan && !plan_with_rows) {

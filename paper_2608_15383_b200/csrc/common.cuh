@@ -125,15 +125,12 @@ void launch_fetch_misses(const PlanPtrs& plan, int wave, const uint8_t* bank_dev
                          cudaStream_t st, bool small_grid = false, bool follows_resolve = true);
 void launch_group(const exmoe_shape& s, int C, int n_keys, int max_waves, bool identity, const int32_t* ids,
                   int n_pairs, PlanPtrs plan, int* d_status, cudaStream_t st);
-// Streaming kernels (bulk-copy weight ring in shared memory) above kSmallMaxPairs pairs, up to 640, or fewer than 12 per expert.
-// Their time grows with the eight-row passes over each expert's weights, that of the tensor-core kernels hardly with the
-// rows: 2048 x 1024, top-8: 64 experts 84 tokens (10.5 rows per expert) 105 -> 85 us per layer, 96 experts 128 tokens (10.7)
-// 147 -> 128 us; past 16 rows per expert they lose (64 experts, 192 tokens: 148 against 125 us).  Up to 128 experts: every
-// CTA walks the plan's groups for its share of the work, the first 128 of them from registers.
-constexpr int kStreamMaxPairs = 640, kStreamMaxRows = 12, kStreamMaxExperts = 128;
-constexpr bool stream_range(int n_pairs, int n_experts) {
-    return n_pairs <= kStreamMaxPairs || (n_experts <= kStreamMaxExperts && n_pairs < kStreamMaxRows * n_experts);
-}
+// Streaming kernels (bulk-copy weight ring in shared memory) above kSmallMaxPairs pairs, up to 640.  Their time grows with the
+// eight-row passes over the experts' weights, that of the tensor-core kernels with the experts that have rows, and the
+// host knows neither.  Up to twelve rows per expert they would win beyond 640 pairs where the routing is uniform (64 experts
+// of 2048 x 1024, top-8, 81 tokens: 82 against 97 us per layer) and lose where it is skewed (Zipf of strength 1.5: 74 against
+// 63; 128 experts of 896 x 2048, 427 tokens: 124 against 48).
+constexpr int kStreamMaxPairs = 640;
 constexpr int kStreamOwnPlanKeys = 128, kStreamOwnPlanPairs = 640;        // most experts and pairs that the streaming kernels group themselves
 bool stream_supported(int H, int I);
 bool launch_stream_wave(const GemmArgs& a, const __nv_bfloat16* hidden, __nv_bfloat16* act, const float* topk_w, float* y,
