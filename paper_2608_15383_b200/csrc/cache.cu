@@ -68,7 +68,7 @@ struct exmoe_cache {
     bool last_pair;                           // ... which formed no plan (per-pair or streaming kernels)
     int last_path;                            // EXMOE_PATH_* of the most recent forward
     int32_t* saved_ids;                       // ids of the last call without a grouping kernel (plan materialised on request)
-    bool stream_ok;                           // the shape fits the streaming middle-regime kernels
+    int stream_pairs;                         // most pairs that go to the streaming kernels (0: the shape does not fit them)
     bool pair_ok, small_ok;                   // ... the per-pair kernels / the in-CTA-grouping kernels (shared memory)
     void* tc_scratch;                         // tile list of the tensor-core path
     __nv_bfloat16* xg;                        // [max_pairs, H] hidden rows in plan order (tensor-core path only)
@@ -381,7 +381,7 @@ int exmoe_cache_create(exmoe_cache** out, const exmoe_shape* shape, int num_laye
     c->slot_last_seq.assign(num_layers, std::vector<uint64_t>(num_slots, 0));
     c->last_layer = -1;
     c->last_T = 0;
-    c->stream_ok = stream_supported(c->shape.d_model, c->shape.d_ff);
+    c->stream_pairs = stream_max_pairs(c->shape);
     c->miss_path = map_banks(c) ? EXMOE_MISS_DEVICE_FETCH : EXMOE_MISS_HOST_COPIES;
     bool ok = cudaMallocHost(&c->h_plan, c->plan_d2h_bytes) == cudaSuccess;
     ok = ok && cudaMallocHost(&c->h_stage, c->stage_bytes) == cudaSuccess;
@@ -439,7 +439,7 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
     }
     // timing runs that launch one kernel kind reuse the plan, grouped rows and tile list of the previous full call
     const bool build_plan = (c->prof_only == 0);
-    const bool use_stream = !small && c->stream_ok && P <= kStreamMaxPairs;
+    const bool use_stream = !small && P <= c->stream_pairs;
     const bool own_plan = use_stream && identity && c->n_keys <= kStreamOwnPlanKeys && P <= kStreamOwnPlanPairs;     // the kernels group the ids themselves
     const bool plan_with_rows = !small && !use_stream && P <= kPlanGatherPairs && c->n_keys <= kPlanGatherKeys;   // below, with the rows
     if (!small && build_plan && !own_plan && !plan_with_rows) {

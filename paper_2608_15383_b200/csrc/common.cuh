@@ -131,8 +131,16 @@ void launch_group(const exmoe_shape& s, int C, int n_keys, int max_waves, bool i
 // of 2048 x 1024, top-8, 81 tokens: 82 against 97 us per layer) and lose where it is skewed (Zipf of strength 1.5: 74 against
 // 63; 128 experts of 896 x 2048, 427 tokens: 124 against 48).
 constexpr int kStreamMaxPairs = 640;
+// ... and up to 14 rows per expert on average, or 28 where the tensor-core kernels would leave SMs idle (the 128-row weight
+// tiles of all experts are no more than the SMs): against the tensor-core kernels at 14 / 20 / 28 rows per expert, 16 experts
+// of 1920 x 512 0.85 / 1.0 / 1.3 of their time, 24 of 2304 x 2048 1.05 / 1.3 / 1.5, 16 of 512 x 256 0.8 / 0.85 / 1.0.
+constexpr int kStreamMaxRows = 14, kStreamMaxRowsFew = 28;
+// ... and up to 192 pairs where the eight warps of a consumer group cannot share K evenly (7, 9, 11, 13, 15 ... blocks): a group's
+// time is its longest range's. 48 experts of 2048 x 1920, 480 pairs, Zipf 1.5: 1.36 of the tensor-core kernels' time;
+// an offloaded cache of 16 of 48 experts of 1024 x 1664, top-1, no misses: 200 pairs 1.2, 341 pairs 1.3, 500 pairs 1.5.
+constexpr int kStreamMaxPairsUneven = 192;
 constexpr int kStreamOwnPlanKeys = 128, kStreamOwnPlanPairs = 640;        // most experts and pairs that the streaming kernels group themselves
-bool stream_supported(int H, int I);
+int stream_max_pairs(const exmoe_shape& s);      // most pairs of a call that the streaming kernels take; 0: not this shape
 bool launch_stream_wave(const GemmArgs& a, const __nv_bfloat16* hidden, __nv_bfloat16* act, const float* topk_w, float* y,
                         int* status, int max_groups, bool gateup, bool down, cudaStream_t st);
 void launch_small_wave(const GemmArgs& a, const SmallWave& w, cudaStream_t st, bool gateup, bool down);

@@ -31,6 +31,7 @@
 #include "frag.cuh"
 #include "mbar.cuh"
 
+#include <algorithm>
 #include <type_traits>
 
 namespace exmoe {
@@ -669,9 +670,16 @@ bool launch_stream_cfg(const GemmArgs& a, const __nv_bfloat16* x, __nv_bfloat16*
 
 }  // namespace
 
-bool stream_supported(int H, int I) {
-    StreamGeom g;
-    return stream_geometry(H, I, 2, 8, &g) && stream_geometry(I, H, 1, 8, &g);
+int stream_max_pairs(const exmoe_shape& s) {
+    StreamGeom gu, dn;
+    if (!stream_geometry(s.d_model, s.d_ff, 2, 8, &gu) || !stream_geometry(s.d_ff, s.d_model, 1, 8, &dn)) return 0;
+    const bool even = (s.d_model / kGroup) % gu.KS == 0 && (s.d_ff / kGroup) % dn.KS == 0;
+    int sms = 0, dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+        sms = 148;
+    const int tiles = s.num_experts * std::max(2 * s.d_ff, s.d_model) / 128;
+    const int rows = tiles <= sms ? kStreamMaxRowsFew : kStreamMaxRows;
+    return std::min(even ? kStreamMaxPairs : kStreamMaxPairsUneven, rows * s.num_experts);
 }
 
 // One wave on the streaming kernels: passes of eight rows of a group.

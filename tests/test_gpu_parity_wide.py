@@ -334,6 +334,27 @@ def test_streaming_kernels_end_at_640_pairs(B, E, k, T, path):
     cache.close()
 
 
+@pytest.mark.parametrize("d_model, d_ff, E, k, slots, last", [
+    (512, 256, 64, 4, 64, 160),        # 640 pairs
+    (1024, 768, 24, 4, 24, 84),        # 14 rows per expert (288 weight tiles: more than SMs)
+    (512, 256, 16, 4, 16, 112),        # 28 rows per expert (64 weight tiles)
+    (2816, 256, 6, 6, 6, 28),          # 22 blocks do not split into four ranges: 28 rows per expert come first
+    (1664, 640, 32, 4, 32, 48),        # 13 and 5 blocks: 192 pairs
+    (1664, 640, 32, 4, 8, 48)])        # ... and the same with misses
+def test_where_the_streaming_kernels_end(B, d_model, d_ff, E, k, slots, last):
+    """The last token count that goes to the streaming kernels and the first that does not."""
+    s = synth.Shape(d_model, d_ff, E, k)
+    ora, bank = helpers.make_layer(s, seed=81 + d_model)
+    cache = B.Cache(s, [bank], slots, max_tokens=last + 1)
+    for T, path in ((last, B.PATH_STREAM), (last + 1, B.PATH_TENSOR_SMALL_N)):
+        hidden, ids, p = helpers.routed_inputs(s, T, seed=5700 + T, alpha=0.5)
+        out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+        assert cache.last_path() == path and cache.status() == 0
+        y, ref = ora.forward(hidden[::17], ids[::17], p[::17])
+        helpers.check_output(out[::17], y, ref, f"T={T}")
+    cache.close()
+
+
 @pytest.mark.parametrize("E, k, T", [
     (16, 5, 5),                        # 25 pairs: the smallest streaming call
     (128, 4, 160),                     # the most experts and pairs that the streaming kernels group themselves
@@ -353,7 +374,7 @@ def test_edges_of_the_streaming_kernels_own_grouping(B, E, k, T):
     cache.close()
 
 
-@pytest.mark.parametrize("E, wave_cap, k, T", [(16, 8, 4, 8), (16, 8, 4, 16), (16, 4, 2, 320), (64, 32, 1, 25), (16, 0, 4, 16)])
+@pytest.mark.parametrize("E, wave_cap, k, T", [(16, 8, 4, 8), (16, 8, 4, 16), (16, 4, 2, 200), (64, 32, 1, 25), (16, 0, 4, 16)])
 def test_ids_beyond_the_experts_in_a_larger_key_space(B, E, wave_cap, k, T):
     """Every expert resident and a wave_cap below the number of experts: the key space (ceil(E / wave_cap) * E) is larger
     than the expert count, and ids E .. keys - 1 are as invalid as any other id out of range: sticky status, no
