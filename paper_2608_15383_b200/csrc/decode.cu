@@ -1239,18 +1239,26 @@ void launch_token_down(const GemmArgs& a, const SmallArgs& sa, const __nv_bfloat
     count_launch();
 }
 
+// The bulk kernel is taken where its panels, rows and one word per block and expert fit 100 KB, the line that was measured
+// (1024 x 1408, top-7: with it 16.8 and 19.1 us per layer at two and three tokens, the register variant 19.7 and 24.3); the
+// second word of the block constants is on top of that.
+constexpr size_t bulk_smem(int k, int KB, int words) {
+    return (size_t)k * KB * kBlockBytes + (size_t)k * (KB * kGroup * 2 + 64) + (size_t)k * 16 * 4 + 32 + (size_t)words * 4 + 64;
+}
+constexpr bool bulk_fits(int k, int KB) { return k <= 8 && bulk_smem(k, KB, (KB * k + 3) & ~3) <= 100 * 1024; }
+static_assert(bulk_fits(7, 11) && bulk_fits(8, 9) && bulk_fits(1, 77) && !bulk_fits(8, 10) && !bulk_fits(7, 12) && !bulk_fits(9, 1));
+static_assert(bulk_smem(7, 11, 2 * 7 * 11) <= (size_t)kPairSmemMax && bulk_smem(1, 77, 2 * 77) <= (size_t)kPairSmemMax);
+
 // false when the shape does not fit the kernel's shared-memory budget (the caller then takes the register variant)
 template <int NBT, typename Inl>
 bool launch_token_down_bulk(const GemmArgs& a, const SmallArgs& sa, const __nv_bfloat16* act, const float* w, int T, int bpwg,
                             cudaStream_t st, const Inl& in) {
-    const int K = a.I, KB = K / kGroup, k = a.top_k;
-    if (k > 8) return false;
-    const size_t smem = (size_t)k * KB * kBlockBytes + (size_t)k * (K * 2 + 64) + (size_t)k * 16 * 4 + 32 +
-                        (size_t)KB * k * 8 + 64;
-    if (smem > 100 * 1024) return false;
+    const int KB = a.I / kGroup, k = a.top_k;
+    if (!bulk_fits(k, KB)) return false;
+    const size_t smem = bulk_smem(k, KB, 2 * KB * k);
     auto kern = token_down_bulk_kernel<NBT, Inl>;
     static SmemOnce smem_once;
-    allow_smem(kern, 100 * 1024, smem_once);
+    allow_smem(kern, kPairSmemMax, smem_once);
     launch_pdl(kern, dim3(a.H / kPanelRows, T), 256, smem, st, a, sa, act, w, bpwg, in);
     count_launch();
     return true;

@@ -427,3 +427,17 @@ def test_activation_scaling_over_magnitudes(B, T):
             helpers.check_output(out[t:t + 1], y[t:t + 1], ref[t:t + 1], f"T={T} row {t} {what}")
     assert cache.status() == 0
     cache.close()
+
+
+@pytest.mark.parametrize("T", [1, 2, 3])
+def test_largest_panels_of_the_bulk_down_kernel(B, T):
+    """Seven selected experts of eleven blocks: the shape that fills the shared memory of the by-token down kernel."""
+    s = synth.Shape(1024, 1408, 12, 7)
+    ora, bank = helpers.make_layer(s, seed=91)
+    hidden, ids, p = helpers.routed_inputs(s, T, seed=5800 + T, alpha=0.5)
+    cache = B.Cache(s, [bank], 12, max_tokens=T)
+    out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    y, ref = ora.forward(hidden, ids, p)
+    helpers.check_output(out, y, ref, f"T={T}")
+    assert cache.last_path() == B.PATH_PAIR and cache.status() == 0
+    cache.close()
