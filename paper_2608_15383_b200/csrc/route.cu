@@ -331,7 +331,7 @@ __device__ __forceinline__ void choose(float* z, float slack, const __nv_bfloat1
     unsigned again = 0;
     float prev = INFINITY, top_v = 0.f;
     bool deep = false;
-    int prev_e = 0, mine = 0;                                              // mine, lane j: the j-th choice (k <= 32)
+    int prev_e = 0, first_e = 0, mine = 0;                                              // mine, lane j: the j-th choice (k <= 32)
     for (int j = 0; j <= k && j < E && !odd; ++j) {
         uint32_t best = 0;
         int be = 0x7fffffff;
@@ -346,6 +346,7 @@ __device__ __forceinline__ void choose(float* z, float slack, const __nv_bfloat1
         const float v = __uint_as_float(top & 0x80000000u ? top & 0x7fffffffu : ~top);
         if (j == 0) {
             top_v = v;
+            first_e = e;
             odd = v == -INFINITY;                                          // every expert masked: NaN probabilities
         } else if (prev < top_v - kExpSubnormal + 2.f * slack) {           // another one follows: both may be subnormal or zero
             deep = true;
@@ -374,6 +375,7 @@ __device__ __forceinline__ void choose(float* z, float slack, const __nv_bfloat1
         if (e >= E) again &= ~(1u << i);
     }
     if (deep || __any_sync(0xffffffffu, again != 0)) {
+        if (lane == (first_e & 31)) again |= 1u << (first_e >> 5);         // the maximum, from which expf's arguments are measured
         logits_again(z, again, x, w_router, bias, H, lane);
         softmax_topk(z, E, k, lane, ids, wts);
         return;
