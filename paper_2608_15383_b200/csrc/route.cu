@@ -27,11 +27,8 @@ namespace cg = cooperative_groups;
 
 constexpr int kRouteThreads = 256;
 constexpr int kRouteSmemMax = 200 * 1024;
-// Measured crossings (64 experts, d_model 2048, weights cold, launch included), us for one token per cluster, four tokens per
-// cluster, tensor cores with 16 experts per CTA, with 32:
-//   T = 32: 10.2 / 10.2 / - / -      64: 12.3 / 12.3 / 15.1 / -      256: 22.5 / 17.3 / 16.4 / -
-// and replayed from a graph, for the last two: 1024: 11.8 / 12.4      1184: 16.2 / 13.9      2048: 19.4 / 16.3      8192: 58 / 43
-constexpr int kRouteFewTokens = 48;       // four tokens per cluster from here on
+constexpr int kRouteFewTokens = 48;       // several tokens per cluster from here on
+constexpr int kRouteTokenTokens = 192;    // one CTA per token, few experts, from here on
 constexpr int kRouteMmaTokens = 224;      // tensor cores from here on
 constexpr int kRouteWideTokens = 1152;    // ... with 32 instead of 16 experts per CTA
 constexpr int kRouteWarps = kRouteThreads / 32;
@@ -97,7 +94,12 @@ __device__ __forceinline__ void softmax_topk(float* prob, int E, int k, int lane
 }
 
 // The same by a whole CTA, for one token: the rounds of the arg-max (120 cycles each) are replaced by counting, for every
-// expert, the experts that come before it (four threads per expert).  `pv`: E more floats of shared memory.
+// expert, the experts that come before it (four threads per expert).  `pv`: E more floats of shared memory.  The counting
+// takes time by E * E, the rounds by k: equal at about 160 experts for eight choices (one token, d_model 2048, rounds against
+// counting: 64 experts 5.1 / 3.9 us, 128: 6.1 / 5.8, 192: 7.6 / 8.0, 256: 8.2 / 10.3; 4096 experts, d_model 1024: 58 / 755).
+constexpr bool choose_by_counting(int E, int k) { return (long long)E * E <= 3200ll * k; }
+static_assert(choose_by_counting(64, 8) && choose_by_counting(128, 8) && choose_by_counting(8, 2) && choose_by_counting(256, 64));
+static_assert(!choose_by_counting(192, 8) && !choose_by_counting(256, 8) && !choose_by_counting(4096, 8));
 __device__ __forceinline__ void softmax_topk_cta(float* prob, float* pv, int E, int k, int32_t* __restrict__ ids_out,
                                                  float* __restrict__ w_out) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -135,10 +137,10 @@ __device__ __forceinline__ void softmax_topk_cta(float* prob, float* pv, int E, 
     }
 }
 
-// CL: CTAs per cluster; TB: tokens per cluster.
+// CL: CTAs per cluster; TB: tokens per cluster; COUNT: the choice by counting.
 // Shared memory: the cluster's TB hidden rows (every CTA keeps all of them), then the logits of the ceil(TB / CL) tokens
 // this CTA owns (token i belongs to rank i % CL).
-template <int CL, int TB>
+template <int CL, int TB, bool COUNT>
 __global__ void __launch_bounds__(kRouteThreads)
 route_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* __restrict__ w_router,
              const float* __restrict__ bias, int T, int H, int E, int k, int32_t* __restrict__ ids_out,
@@ -213,7 +215,48 @@ route_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* __re
     if (!joined) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
     cluster.sync();
     static_assert(TB <= CL, "a CTA owns at most one token");
-    if (rank < n_tok) softmax_topk_cta(prob, prob + E, E, k, ids_out + (size_t)(t0 + rank) * k, w_out + (size_t)(t0 + rank) * k);
+    if constexpr (COUNT) {
+        if (rank < n_tok) softmax_topk_cta(prob, prob + E, E, k, ids_out + (size_t)(t0 + rank) * k, w_out + (size_t)(t0 + rank) * k);
+    } else {
+        if (rank < n_tok && warp == 0) softmax_topk(prob, E, k, lane, ids_out + (size_t)(t0 + rank) * k, w_out + (size_t)(t0 + rank) * k);
+    }
+}
+
+// One CTA per token, no cluster and nothing held ahead in registers: many CTAs per SM.  For calls with more tokens than
+// there is room for clusters and so few experts that reading the matrix again for every token costs little.  Same arithmetic.
+__global__ void __launch_bounds__(kRouteThreads)
+route_token_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* __restrict__ w_router,
+                   const float* __restrict__ bias, int T, int H, int E, int k, int32_t* __restrict__ ids_out,
+                   float* __restrict__ w_out) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint4* xs = reinterpret_cast<uint4*>(smem);                            // [H / 8]
+    float* prob = reinterpret_cast<float*>(smem + (size_t)H * 2);          // [E]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, chunks = H / 8;
+    grid_dependency_wait();
+    const uint4* xrow = reinterpret_cast<const uint4*>(hidden + (size_t)blockIdx.x * H);
+    for (int i = tid; i < chunks; i += kRouteThreads) xs[i] = xrow[i];
+    __syncthreads();
+    for (int e = warp; e < E; e += kRouteWarps) {
+        const uint4* wrow = reinterpret_cast<const uint4*>(w_router + (size_t)e * H);
+        float s = 0.f;
+        for (int i = lane; i < chunks; i += 32) {
+            const uint4 wv = wrow[i], xv = xs[i];
+            const uint32_t wr[4] = {wv.x, wv.y, wv.z, wv.w}, xr[4] = {xv.x, xv.y, xv.z, xv.w};
+            float d = 0.f;                                                 // dot8 without the sixteen unpacked values
+#pragma unroll
+            for (int n = 0; n < 4; ++n) {
+                d = fmaf(__uint_as_float(wr[n] << 16), __uint_as_float(xr[n] << 16), d);
+                d = fmaf(__uint_as_float(wr[n] & 0xffff0000u), __uint_as_float(xr[n] & 0xffff0000u), d);
+            }
+            s += d;
+        }
+        s = warp_sum(s);
+        if (lane == 0) prob[e] = s + (bias ? bias[e] : 0.f);
+    }
+    // not earlier: CTAs of the next kernel that wait in their places keep this kernel's from spreading evenly
+    grid_launch_dependents();
+    __syncthreads();
+    if (warp == 0) softmax_topk(prob, E, k, lane, ids_out + (size_t)blockIdx.x * k, w_out + (size_t)blockIdx.x * k);
 }
 
 // every form is a programmatic dependent of the kernel before it in the stream (it waits for it before it reads anything)
@@ -245,9 +288,18 @@ template <int CL, int TB>
 int launch_route(const exmoe_shape& s, const __nv_bfloat16* hidden, const __nv_bfloat16* w, const float* bias, int T,
                  int32_t* ids, float* wts, cudaStream_t st) {
     const size_t smem = (size_t)TB * s.d_model * 2 + 2 * (size_t)s.num_experts * 4;
+    static SmemOnce once[2];
+    const bool count = choose_by_counting(s.num_experts, s.top_k);
+    const auto kern = count ? route_kernel<CL, TB, true> : route_kernel<CL, TB, false>;
+    if (!allow_smem(kern, kRouteSmemMax + 4096 * 4, once[count])) return EXMOE_ERR_CUDA;
+    return launch_dependent(kern, (T + TB - 1) / TB * CL, CL, smem, s, hidden, w, bias, T, ids, wts, st);
+}
+
+int launch_route_token(const exmoe_shape& s, const __nv_bfloat16* hidden, const __nv_bfloat16* w, const float* bias, int T,
+                       int32_t* ids, float* wts, cudaStream_t st) {
     static SmemOnce once;
-    if (!allow_smem(route_kernel<CL, TB>, kRouteSmemMax + 4096 * 4, once)) return EXMOE_ERR_CUDA;
-    return launch_dependent(route_kernel<CL, TB>, (T + TB - 1) / TB * CL, CL, smem, s, hidden, w, bias, T, ids, wts, st);
+    if (!allow_smem(route_token_kernel, kRouteSmemMax, once)) return EXMOE_ERR_CUDA;
+    return launch_dependent(route_token_kernel, T, 1, (size_t)s.d_model * 2 + (size_t)s.num_experts * 4, s, hidden, w, bias, T, ids, wts, st);
 }
 
 // ---- many tokens: the logits as a tensor-core GEMM -------------------------------------------------------------
@@ -550,6 +602,39 @@ int launch_route_mma(const exmoe_shape& s, const __nv_bfloat16* hidden, const __
     return launch_dependent(route_mma_kernel<NT, CL, U>, (T + TM - 1) / TM * CL, CL, smem, s, hidden, w, bias, T, ids, wts, st);
 }
 
+// Which form a call takes.  All give the same bits but the tensor-core ones (see there).  One token per cluster of eight CTAs
+// while the clusters find room on the chip at once, and for what nothing else fits; then four tokens per read of the
+// matrix, by clusters of eight, or of four where these have a warp per expert or the calls are large; with few experts one
+// CTA per token; then the tensor cores.  us, replayed from a graph, in the order one / four / four narrow / token / tensor
+// cores (16 experts per CTA / 32):
+//   64 experts, d_model 2048:  32 tokens 5.1 / 4.9 / - / - / 5.8         64: - / 5.4 / 6.5 / - / 5.7     224: - / 10.0 / 10.9 / - / 10.6
+//   16 experts, d_model 512:   64 tokens 5.2 / 3.5 / 3.3 / 3.9 / 6.8    223: - / 5.7 / 4.1 / 4.1 / 7.0   800: - / 13 / 7.4 / 4.7 / 7.8 / 7.7
+//   16 experts, d_model 2048: 128 tokens 9.5 / 7.0 / 4.6 / 5.1 / 9.6    300: - / 9.8 / 7.3 / 5.4 / 9.7   900: - / 22 / 14 / 12 / 11 / 11
+//   8 experts, d_model 256:    64 tokens 5.0 / 3.3 / 3.2 / 2.7 / 3.8   1024: - / 14 / 9.1 / 4.9 / 6.7 / 6.7   2048: - / 26 / 15 / 6.8 / 8.4 / 7.4
+//   256 experts, d_model 1024 (no tensor-core form): 256 tokens 31 / 21 / 22 / 26    1024: 104 / 58 / 55 / 70    4000: 387 / 205 / 178 / 195
+//   20 experts, d_model 1000 (none either): 300 tokens 15 / 8.2 / 5.3 / 6.4          4000: 162 / 71 / 40 / 29
+enum class RouteForm { One, Four, FourNarrow, Token, Mma, MmaWide };
+constexpr RouteForm route_form(int E, int H, int k, int T) {
+    const bool mma = H % 32 == 0 && H <= kMmaMaxModel && E <= kMmaMaxExperts && k <= 32;
+    const bool four = 8 * (size_t)H + 4 * (size_t)E <= (size_t)kRouteSmemMax;
+    const bool small = E * H <= 40000;                                     // 80 KB of matrix
+    if (T < kRouteFewTokens) return RouteForm::One;
+    if (small && E <= 32) {
+        if (T >= (E <= 8 ? kRouteFewTokens : kRouteTokenTokens) && (!mma || T < (E <= 8 ? 1536 : 896))) return RouteForm::Token;
+        if (T < kRouteTokenTokens && four) return RouteForm::FourNarrow;
+    }
+    if (mma && T >= kRouteMmaTokens) return T >= kRouteWideTokens ? RouteForm::MmaWide : RouteForm::Mma;
+    if (small && !mma && T >= 2048) return RouteForm::Token;
+    return four ? (T >= 512 ? RouteForm::FourNarrow : RouteForm::Four) : RouteForm::One;
+}
+static_assert(route_form(64, 2048, 8, 47) == RouteForm::One && route_form(64, 2048, 8, 48) == RouteForm::Four);
+static_assert(route_form(64, 2048, 8, 223) == RouteForm::Four && route_form(64, 2048, 8, 224) == RouteForm::Mma);
+static_assert(route_form(64, 2048, 8, 1152) == RouteForm::MmaWide && route_form(16, 512, 4, 896) == RouteForm::Mma);
+static_assert(route_form(16, 512, 4, 191) == RouteForm::FourNarrow && route_form(16, 512, 4, 192) == RouteForm::Token);
+static_assert(route_form(16, 512, 4, 895) == RouteForm::Token && route_form(8, 256, 2, 48) == RouteForm::Token);
+static_assert(route_form(20, 1000, 3, 4000) == RouteForm::Token && route_form(256, 1024, 8, 4000) == RouteForm::FourNarrow);
+static_assert(route_form(4096, 1024, 8, 256) == RouteForm::Four && route_form(64, 40000, 8, 4000) == RouteForm::One);
+
 }  // namespace
 
 extern "C" int exmoe_route(const exmoe_shape* shape, const void* hidden_bf16, const void* router_bf16, const float* bias,
@@ -567,16 +652,15 @@ extern "C" int exmoe_route(const exmoe_shape* shape, const void* hidden_bf16, co
     const __nv_bfloat16* x = (const __nv_bfloat16*)hidden_bf16;
     const __nv_bfloat16* w = (const __nv_bfloat16*)router_bf16;
     cudaStream_t st = (cudaStream_t)stream;
-    // Clusters of one token while they all find room on the chip at once, then four tokens per read of the matrix, then
-    // the tensor cores (measured crossings, 64 experts, d_model 2048: see the constants).  A shape that a form's shared
-    // memory or tiling does not fit takes the next simpler one; one token per cluster serves every shape.
-    if (T >= kRouteMmaTokens && s.d_model % 32 == 0 && s.d_model <= kMmaMaxModel && s.num_experts <= kMmaMaxExperts &&
-        s.top_k <= 32)
-        return T >= kRouteWideTokens ? launch_route_mma<4, 2, 2>(s, x, w, bias, T, topk_ids, topk_weights, st)
-                                     : launch_route_mma<2, 4, 4>(s, x, w, bias, T, topk_ids, topk_weights, st);
-    if (T >= kRouteFewTokens && 4 * row + logits <= (size_t)kRouteSmemMax)
-        return launch_route<8, 4>(s, x, w, bias, T, topk_ids, topk_weights, st);
-    return launch_route<8, 1>(s, x, w, bias, T, topk_ids, topk_weights, st);
+    switch (route_form(s.num_experts, s.d_model, s.top_k, T)) {
+        case RouteForm::One: return launch_route<8, 1>(s, x, w, bias, T, topk_ids, topk_weights, st);
+        case RouteForm::Four: return launch_route<8, 4>(s, x, w, bias, T, topk_ids, topk_weights, st);
+        case RouteForm::FourNarrow: return launch_route<4, 4>(s, x, w, bias, T, topk_ids, topk_weights, st);
+        case RouteForm::Token: return launch_route_token(s, x, w, bias, T, topk_ids, topk_weights, st);
+        case RouteForm::Mma: return launch_route_mma<2, 4, 4>(s, x, w, bias, T, topk_ids, topk_weights, st);
+        case RouteForm::MmaWide: return launch_route_mma<4, 2, 2>(s, x, w, bias, T, topk_ids, topk_weights, st);
+    }
+    return EXMOE_ERR_STATE;
 }
 
 }  // namespace exmoe

@@ -103,7 +103,11 @@ def test_router_feeds_the_layer(B):
 @pytest.mark.parametrize("shape,T", [(synth.OLMOE, 47), (synth.OLMOE, 48), (synth.OLMOE, 51), (synth.OLMOE, 223), (synth.OLMOE, 225),
                                      (synth.OLMOE, 2303), (synth.OLMOE, 2337), (synth.Shape(1280, 128, 72, 5), 300),
                                      (synth.Shape(1280, 128, 72, 5), 2310), (synth.Shape(128, 128, 3, 2), 240),
-                                     (synth.Shape(512, 128, 16, 4), 896), (synth.Shape(512, 128, 16, 4), 4000)])
+                                     (synth.Shape(512, 128, 16, 4), 896), (synth.Shape(512, 128, 16, 4), 4000),
+                                     (synth.Shape(512, 128, 16, 4), 191), (synth.Shape(512, 128, 16, 4), 895),
+                                     (synth.Shape(256, 128, 8, 2), 49), (synth.Shape(256, 128, 8, 2), 1536), (synth.Shape(1000, 128, 20, 3), 300),
+                                     (synth.Shape(1024, 128, 256, 8), 130), (synth.Shape(1024, 128, 256, 8), 515), (synth.Shape(8192, 128, 64, 8), 530),
+                                     (synth.Shape(256, 128, 132, 4), 2050), (synth.Shape(512, 128, 1030, 3), 50)])
 def test_choice_does_not_depend_on_the_batch_size(B, shape, T):
     """Every form of the kernel (one or four tokens per cluster, tensor cores with 16 or 32 tokens per CTA; last tiles
     partly filled, an expert count that is no multiple of 64) picks the experts that one token at a time picks.  Near-ties
