@@ -188,20 +188,28 @@ PACK_STAGING_EXPERTS = 8      # device staging of pack_bank: two halves of four 
 
 
 def pack_bank(shape, w_gate, w_up, w_down, device="cuda"):
-    """Pack all experts of one layer ([E,I,H], [E,I,H], [E,H,I] BF16) into a pinned host bank [E, bytes]."""
+    """Pack all experts of one layer ([E,I,H], [E,I,H], [E,H,I] BF16: tensors, or anything that gives expert e's matrix for
+    index e) into a pinned host bank [E, bytes]."""
     E, I, H = shape.num_experts, shape.d_ff, shape.d_model
-    weights = tuple(w[:E] for w in (w_gate, w_up, w_down))
-    if [tuple(w.shape) for w in weights] != [(E, I, H), (E, I, H), (E, H, I)]:
-        raise ValueError("pack_bank: weight shapes must be [E,I,H], [E,I,H], [E,H,I]")
     n = exmoe_packed_bytes(shape)
     bank = torch.empty((E, n), dtype=torch.uint8, pin_memory=True)
     staging = torch.empty((PACK_STAGING_EXPERTS, n), dtype=torch.uint8, device=device)
+    matrices = ((w_gate, (I, H)), (w_up, (I, H)), (w_down, (H, I)))
+
+    def on_device(w, size, e, m):
+        part = w[e:e + m] if torch.is_tensor(w) else torch.stack([w[j].to(staging.device) for j in range(e, e + m)])
+        if tuple(part.shape) != (m, *size):
+            raise ValueError("pack_bank: weight shapes must be [E,I,H], [E,I,H], [E,H,I]")
+        return part.to(staging.device).contiguous()
+
     # weights on the device already are converted in one call, others a few experts at a time as they arrive there
-    step = E if all(w.device == staging.device and w.is_contiguous() for w in weights) else PACK_STAGING_EXPERTS // 2
+    resident = all(torch.is_tensor(w) and w.device == staging.device and w.is_contiguous() for w, _ in matrices)
+    step = E if resident else PACK_STAGING_EXPERTS // 2
     for e in range(0, E, step):
-        part = [w[e:e + step].to(staging.device).contiguous() for w in weights]
-        rc = lib().exmoe_pack_bank(byref(_shape(shape)), part[0].shape[0], *(_dev(w, torch.bfloat16, what) for w, what in
-                                                                             zip(part, ("w_gate", "w_up", "w_down"))),
+        m = min(step, E - e)
+        part = [on_device(w, size, e, m) for w, size in matrices]
+        rc = lib().exmoe_pack_bank(byref(_shape(shape)), m, *(_dev(w, torch.bfloat16, what) for w, what in
+                                                              zip(part, ("w_gate", "w_up", "w_down"))),
                                    c_void_p(staging.data_ptr()), PACK_STAGING_EXPERTS, c_void_p(bank[e:].data_ptr()), _stream_ptr(None))
         _check(rc, "exmoe_pack_bank")
     return bank

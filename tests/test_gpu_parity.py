@@ -71,6 +71,21 @@ def test_pack_bank_equals_packing_one_expert_at_a_time(B, E, where):
     assert err.value.code == B.EXMOE_ERR_NONFINITE
 
 
+@pytest.mark.parametrize("E", [1, 4, 6])
+@pytest.mark.parametrize("where", ["list", "list on the host", "dict"])
+def test_pack_bank_takes_one_matrix_per_expert(B, E, where):
+    """A checkpoint's weights as they are loaded, a matrix per expert: the bank of the stacked tensors."""
+    s = synth.Shape(d_model=256, d_ff=384, num_experts=E, top_k=1)
+    w = synth.expert_weights(s, seed=E, device="cuda")
+    given = [[x[e].cpu() if where == "list on the host" else x[e].clone() for e in range(E)] for x in w]
+    if where == "dict":
+        given = [dict(enumerate(x)) for x in given]
+    assert torch.equal(B.pack_bank(s, *given), B.pack_bank(s, *w))
+    given[2][E - 1] = given[2][E - 1][:-1]
+    with pytest.raises(ValueError):
+        B.pack_bank(s, *given)
+
+
 def test_pack_special_groups_and_errors(B):
     s = synth.Shape(d_model=256, d_ff=128, num_experts=1, top_k=1)
     wg, wu, wd = synth.expert_weights(s, seed=3)
