@@ -32,14 +32,22 @@ const at::Tensor* tensor(PyObject* o, at::ScalarType dt, bool cuda, const char* 
 }
 constexpr const char *kBf16 = "torch.bfloat16", *kF32 = "torch.float32", *kI32 = "torch.int32";
 
-bool int_attr(PyObject* o, PyObject* name, int* v) {
-    PyObject* a = PyObject_GetAttr(o, name);
-    if (!a) return false;
-    const long x = PyLong_AsLong(a);
-    Py_DECREF(a);
+// int(o): whatever Python's int() takes, a float or a zero-dimensional array among them
+bool to_int(PyObject* o, int* v) {
+    PyObject* i = PyLong_CheckExact(o) ? Py_NewRef(o) : PyNumber_Long(o);
+    if (!i) return false;
+    const long x = PyLong_AsLong(i);
+    Py_DECREF(i);
     if (x == -1 && PyErr_Occurred()) return false;
     *v = (int)x;
     return true;
+}
+bool int_attr(PyObject* o, PyObject* name, int* v) {
+    PyObject* a = PyObject_GetAttr(o, name);
+    if (!a) return false;
+    const bool ok = to_int(a, v);
+    Py_DECREF(a);
+    return ok;
 }
 bool shape_of(PyObject* o, exmoe_shape* s) {
     if (!int_attr(o, s_d_model, &s->d_model) || !int_attr(o, s_d_ff, &s->d_ff) || !int_attr(o, s_experts, &s->num_experts) ||
@@ -112,8 +120,8 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (n != 7) return PyErr_Format(PyExc_TypeError, "forward: 7 arguments");
     return guarded([&]() -> PyObject* {
         exmoe_cache* c = static_cast<exmoe_cache*>(PyLong_AsVoidPtr(a[0]));
-        const int layer = (int)PyLong_AsLong(a[1]);
-        if (PyErr_Occurred()) return nullptr;
+        int layer;
+        if (PyErr_Occurred() || !to_int(a[1], &layer)) return nullptr;
         const at::Tensor *h, *i, *p, *o = nullptr;
         if (!(h = tensor(a[2], at::kBFloat16, true, "hidden", kBf16))) return nullptr;
         if (!(i = tensor(a[3], at::kInt, true, "topk_ids", kI32))) return nullptr;
@@ -137,8 +145,8 @@ PyObject* forward_host(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (n != 7) return PyErr_Format(PyExc_TypeError, "forward_host: 7 arguments");
     return guarded([&]() -> PyObject* {
         exmoe_cache* c = static_cast<exmoe_cache*>(PyLong_AsVoidPtr(a[0]));
-        const int layer = (int)PyLong_AsLong(a[1]);
-        if (PyErr_Occurred()) return nullptr;
+        int layer;
+        if (PyErr_Occurred() || !to_int(a[1], &layer)) return nullptr;
         const at::Tensor *h, *i, *p, *o;
         if (!(h = tensor(a[2], at::kBFloat16, false, "hidden", kBf16))) return nullptr;
         if (!(i = tensor(a[3], at::kInt, false, "topk_ids", kI32))) return nullptr;

@@ -63,3 +63,25 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(binding, "LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(FileNotFoundError):
         binding.lib()
+
+
+def test_serving_calls_take_what_int_takes(libpath):
+    """Layer numbers and shape dimensions go through int(): floats, strings of digits, numpy scalars.  With host tensors where
+    device tensors belong, a call that got past its numbers ends at the tensors."""
+    import types
+
+    import numpy as np
+    import torch
+
+    from paper_2608_15383_b200 import binding
+    binding.lib()
+    h = torch.zeros((1, 256), dtype=torch.bfloat16)
+    for layer in (0, 1.0, np.int64(1), np.float32(2.0), "1", torch.tensor(1), True):
+        with pytest.raises(ValueError, match="hidden"):
+            binding.Cache.forward(types.SimpleNamespace(_address=0), layer, h, None, None)
+    for bad in (None, "x", [1]):
+        with pytest.raises((TypeError, ValueError), match="int"):
+            binding.Cache.forward(types.SimpleNamespace(_address=0), bad, h, None, None)
+    for d in (256, 256.0, np.float64(256), "256"):
+        with pytest.raises(ValueError, match="hidden"):
+            binding.exmoe_route(types.SimpleNamespace(d_model=d, d_ff=128, num_experts=8, top_k=2), h, h)
