@@ -12,6 +12,8 @@ from ctypes import POINTER, byref, c_char_p, c_float, c_int, c_int32, c_size_t, 
 
 import torch
 
+from . import build
+
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libexmoe.so")
 NATIVE_PATH = os.path.join(_PKG, "_exmoe_native.so")
@@ -77,27 +79,40 @@ _lib = None
 _native = None
 
 
+def _must_exist(path):
+    if not os.path.exists(path):
+        raise FileNotFoundError(f"{path} is missing: build it with `python -m paper_2608_15383_b200.build` (no CPU fallback exists)")
+
+
 def lib():
     """Open libexmoe.so (built in-tree by `paper_2608_15383_b200.build`); fail loudly if absent."""
-    global _lib, _native
+    global _lib
     if _lib is None:
-        for path in (LIB_PATH, NATIVE_PATH):
-            if not os.path.exists(path):
-                raise FileNotFoundError(
-                    f"{path} is missing: build it with `python -m paper_2608_15383_b200.build` (no CPU fallback exists)")
+        _must_exist(LIB_PATH)
         h = ctypes.CDLL(LIB_PATH)
         for name, (res, args) in _SIGNATURES.items():
             fn = getattr(h, name)
             fn.restype = res
             fn.argtypes = args
+        _lib = h
+    return _lib
+
+
+def _serving():
+    """The CPython module of the serving calls, opened on the first of them: the rest of the binding needs libexmoe.so only.
+    It uses torch's C++ interface, which holds for one version: another one's build is refused, not loaded."""
+    global _native
+    if _native is None:
+        _must_exist(NATIVE_PATH)
+        if not build.native_is_current(NATIVE_PATH):
+            raise ImportError(f"{NATIVE_PATH} was built for another torch than {torch.__version__}: run `python -m paper_2608_15383_b200.build`")
         spec = importlib.util.spec_from_file_location("_exmoe_native", NATIVE_PATH)
         native = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(native)
-        native.set_entry_points(*(ctypes.cast(getattr(h, name), c_void_p).value for name in
+        native.set_entry_points(*(ctypes.cast(getattr(lib(), name), c_void_p).value for name in
                                   ("exmoe_route", "exmoe_moe_forward", "exmoe_moe_forward_host")))
         _native = native
-        _lib = h
-    return _lib
+    return _native
 
 
 def strerror(code):
@@ -172,9 +187,7 @@ def exmoe_moe_forward_static_status():
 
 def exmoe_route(shape, hidden, w_router, bias=None, topk_ids=None, topk_weights=None, stream=None):
     """Eq. 1 on the device: logits, softmax over all experts, top-k.  Returns (ids int32 [T, k], weights fp32 [T, k])."""
-    if _native is None:
-        lib()
-    r = _native.route(shape, hidden, w_router, bias, topk_ids, topk_weights, stream)
+    r = (_native or _serving()).route(shape, hidden, w_router, bias, topk_ids, topk_weights, stream)
     if r.__class__ is int:
         raise ExmoeError(r, "exmoe_route")
     return r
@@ -283,7 +296,7 @@ class Cache:
 
     # exmoe_moe_forward
     def forward(self, layer, hidden, topk_ids, topk_weights, out=None, stream=None):
-        r = _native.forward(self._address, layer, hidden, topk_ids, topk_weights, out, stream)
+        r = (_native or _serving()).forward(self._address, layer, hidden, topk_ids, topk_weights, out, stream)
         if r.__class__ is int:
             raise ExmoeError(r, "exmoe_moe_forward")
         return r
@@ -293,7 +306,7 @@ class Cache:
         """Host tensors in, host tensor out (synchronous): hidden BF16 [T, H], ids int32 [T, k], weights fp32 [T, k]."""
         if out is None:
             out = torch.empty((int(hidden.shape[0]), self.shape.d_model), dtype=torch.bfloat16)
-        r = _native.forward_host(self._address, layer, hidden, topk_ids, topk_weights, out, stream)
+        r = (_native or _serving()).forward_host(self._address, layer, hidden, topk_ids, topk_weights, out, stream)
         if r is not None:
             raise ExmoeError(r, "exmoe_moe_forward_host")
         return out

@@ -25,6 +25,17 @@ def _stale(target, sources):
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _torch_tag():
+    import torch
+    return f"built for torch {torch.__version__}"
+
+
+def native_is_current(path=NATIVE):
+    """Whether the CPython module at `path` was built for the torch of this process (it says so in a string of its own)."""
+    with open(path, "rb") as f:
+        return _torch_tag().encode() + b"\0" in f.read()
+
+
 def _run(cmd, verbose, target):
     res = subprocess.run(cmd, capture_output=True, text=True)
     if verbose or res.returncode:
@@ -40,13 +51,13 @@ def build(force=False, verbose=False):
         extra = os.environ.get("EXMOE_NVCC_EXTRA", "").split()      # e.g. -DEXMOE_DISABLE_PDL for an A/B timing
         _run([nvcc] + NVCC_FLAGS + extra + (["-Xptxas", "-v"] if verbose else []) +
              [os.path.join(CSRC, s) for s in SOURCES] + ["-o", LIB, "-lcudart"], verbose, LIB)
-    if force or _stale(NATIVE, [NATIVE_SOURCE]):
+    if force or _stale(NATIVE, [NATIVE_SOURCE]) or not native_is_current():
         import torch
         from torch.utils.cpp_extension import include_paths
         libdir = os.path.join(os.path.dirname(torch.__file__), "lib")
         cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
         inc = [f"-I{d}" for d in include_paths() + [sysconfig.get_paths()["include"], cuda]]
-        _run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] +
+        _run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f'-DEXMOE_TORCH_TAG="{_torch_tag()}"', f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] +
              inc + [os.path.join(CSRC, NATIVE_SOURCE), "-o", NATIVE, f"-L{libdir}", "-ltorch_python", "-ltorch_cuda",
                     "-ltorch_cpu", "-lc10_cuda", "-lc10"], verbose, NATIVE)
     return LIB

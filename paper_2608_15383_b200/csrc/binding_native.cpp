@@ -10,6 +10,9 @@
 
 #include "../../include/exmoe.h"
 
+// read from the file before it is loaded (build.native_is_current)
+extern "C" __attribute__((used)) const char exmoe_native_torch_tag[] = EXMOE_TORCH_TAG;
+
 namespace {
 
 decltype(&exmoe_route) g_route = nullptr;

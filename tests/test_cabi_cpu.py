@@ -85,3 +85,30 @@ def test_serving_calls_take_what_int_takes(libpath):
     for d in (256, 256.0, np.float64(256), "256"):
         with pytest.raises(ValueError, match="hidden"):
             binding.exmoe_route(types.SimpleNamespace(d_model=d, d_ff=128, num_experts=8, top_k=2), h, h)
+
+
+def test_only_the_serving_calls_need_the_native_module(libpath, monkeypatch, tmp_path):
+    import torch
+
+    from paper_2608_15383_b200 import binding, synth
+    monkeypatch.setattr(binding, "_lib", None)
+    monkeypatch.setattr(binding, "_native", None)
+    monkeypatch.setattr(binding, "NATIVE_PATH", str(tmp_path / "nope.so"))
+    assert binding.exmoe_packed_bytes(synth.TINY) == 50688
+    with pytest.raises(FileNotFoundError):
+        binding.exmoe_route(synth.TINY, torch.zeros((1, 256)), torch.zeros((8, 256)))
+
+
+def test_a_native_module_of_another_torch_is_rebuilt_and_not_loaded(libpath, monkeypatch, tmp_path):
+    import torch
+
+    from paper_2608_15383_b200 import binding, build, synth
+    assert build.native_is_current()
+    other = tmp_path / "other.so"
+    with open(build.NATIVE, "rb") as f:
+        other.write_bytes(f.read().replace(torch.__version__.encode(), b"9" * len(torch.__version__)))
+    assert not build.native_is_current(str(other))
+    monkeypatch.setattr(binding, "_native", None)
+    monkeypatch.setattr(binding, "NATIVE_PATH", str(other))
+    with pytest.raises(ImportError, match="another torch"):
+        binding.exmoe_route(synth.TINY, torch.zeros((1, 256)), torch.zeros((8, 256)))
