@@ -813,9 +813,10 @@ int exmoe_debug_last_plan(exmoe_cache* c, int layer, int32_t* n_active, int32_t*
     if (cudaDeviceSynchronize() != cudaSuccess) return EXMOE_ERR_CUDA;
     const int E = c->shape.num_experts;
     if (c->last_pair) {
-        // the call formed no plan: run the grouping kernel now on the ids it kept
+        // the call formed no plan: run the grouping kernel now on the ids it kept (the call has raised the status for
+        // invalid ones, and the caller may have read it since: this run reports to a spare word)
         launch_group(c->shape, c->C, c->n_keys, c->max_waves, c->C == E, c->saved_ids, c->last_T * c->shape.top_k,
-                     c->plan, c->d_status, nullptr);
+                     c->plan, c->d_status + 16, nullptr);
         if (cudaDeviceSynchronize() != cudaSuccess) return EXMOE_ERR_CUDA;
         c->last_pair = false;
         c->last_small = false;

@@ -441,3 +441,19 @@ def test_largest_panels_of_the_bulk_down_kernel(B, T):
     helpers.check_output(out, y, ref, f"T={T}")
     assert cache.last_path() == B.PATH_PAIR and cache.status() == 0
     cache.close()
+
+
+@pytest.mark.parametrize("T", [3, 12, 60, 300])
+def test_reading_the_plan_leaves_the_status_alone(B, T):
+    """One invalid id raises the sticky status once: reading the plan afterwards (which some calls form only then) does not
+    raise it again."""
+    s = synth.MID
+    _, bank = helpers.make_layer(s, seed=95)
+    hidden, ids, p = helpers.routed_inputs(s, T, seed=5900 + T)
+    ids[T // 2, 1] = -3
+    cache = B.Cache(s, [bank], s.num_experts, max_tokens=T)
+    cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    assert cache.status() == B.EXMOE_ERR_BAD_EXPERT_ID
+    assert cache.last_plan(0, ids.numel())["counts"].sum() == T * s.top_k - 1
+    assert cache.status() == 0
+    cache.close()
