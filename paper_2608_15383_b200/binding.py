@@ -210,10 +210,12 @@ def pack_bank(shape, w_gate, w_up, w_down, device="cuda"):
     matrices = ((w_gate, (I, H)), (w_up, (I, H)), (w_down, (H, I)))
 
     def on_device(w, size, e, m):
-        part = w[e:e + m] if torch.is_tensor(w) else torch.stack([w[j].to(staging.device) for j in range(e, e + m)])
-        if tuple(part.shape) != (m, *size):
+        part = w[e:e + m] if torch.is_tensor(w) else [w[j] for j in range(e, e + m)]
+        if (tuple(part.shape) != (m, *size)) if torch.is_tensor(part) else any(tuple(x.shape) != size for x in part):
             raise ValueError("pack_bank: weight shapes must be [E,I,H], [E,I,H], [E,H,I]")
-        return part.to(staging.device).contiguous()
+        if torch.is_tensor(part):
+            return part.to(staging.device).contiguous()
+        return torch.stack([x.to(staging.device) for x in part])
 
     # weights on the device already are converted in one call, others a few experts at a time as they arrive there
     resident = all(torch.is_tensor(w) and w.device == staging.device and w.is_contiguous() for w, _ in matrices)
