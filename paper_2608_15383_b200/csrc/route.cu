@@ -617,10 +617,10 @@ enum class RouteForm { One, Four, FourNarrow, Token, Mma, MmaWide };
 constexpr RouteForm route_form(int E, int H, int k, int T) {
     const bool mma = H % 32 == 0 && H <= kMmaMaxModel && E <= kMmaMaxExperts && k <= 32;
     const bool four = 8 * (size_t)H + 4 * (size_t)E <= (size_t)kRouteSmemMax;
-    const bool small = E * H <= 40000;                                     // 80 KB of matrix
+    const bool small = E * H <= 40000, few = E <= 32 && E * H <= 65536;    // 80 KB of matrix; 128 KB
     if (T < kRouteFewTokens) return RouteForm::One;
-    if (small && E <= 32) {
-        if (T >= (E <= 8 ? kRouteFewTokens : kRouteTokenTokens) && (!mma || T < (E <= 8 ? 1536 : 896))) return RouteForm::Token;
+    if (few) {
+        if (T >= (E <= 8 ? kRouteFewTokens : kRouteTokenTokens) && (!mma || T < (E <= 8 ? 1536 : small ? 896 : 600))) return RouteForm::Token;
         if (T < kRouteTokenTokens && four) return RouteForm::FourNarrow;
     }
     if (mma && T >= kRouteMmaTokens) return T >= kRouteWideTokens ? RouteForm::MmaWide : RouteForm::Mma;
@@ -632,6 +632,7 @@ static_assert(route_form(64, 2048, 8, 223) == RouteForm::Four && route_form(64, 
 static_assert(route_form(64, 2048, 8, 1152) == RouteForm::MmaWide && route_form(16, 512, 4, 896) == RouteForm::Mma);
 static_assert(route_form(16, 512, 4, 191) == RouteForm::FourNarrow && route_form(16, 512, 4, 192) == RouteForm::Token);
 static_assert(route_form(16, 512, 4, 895) == RouteForm::Token && route_form(8, 256, 2, 48) == RouteForm::Token);
+static_assert(route_form(32, 2048, 8, 599) == RouteForm::Token && route_form(32, 2048, 8, 600) == RouteForm::Mma);
 static_assert(route_form(20, 1000, 3, 4000) == RouteForm::Token && route_form(256, 1024, 8, 4000) == RouteForm::FourNarrow);
 static_assert(route_form(4096, 1024, 8, 256) == RouteForm::Four && route_form(64, 40000, 8, 4000) == RouteForm::One);
 

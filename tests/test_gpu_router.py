@@ -105,6 +105,7 @@ def test_router_feeds_the_layer(B):
                                      (synth.Shape(1280, 128, 72, 5), 2310), (synth.Shape(128, 128, 3, 2), 240),
                                      (synth.Shape(512, 128, 16, 4), 896), (synth.Shape(512, 128, 16, 4), 4000),
                                      (synth.Shape(512, 128, 16, 4), 191), (synth.Shape(512, 128, 16, 4), 895),
+                                     (synth.Shape(2048, 128, 32, 8), 599),
                                      (synth.Shape(256, 128, 8, 2), 49), (synth.Shape(256, 128, 8, 2), 1536), (synth.Shape(1000, 128, 20, 3), 300),
                                      (synth.Shape(1024, 128, 256, 8), 130), (synth.Shape(1024, 128, 256, 8), 515), (synth.Shape(8192, 128, 64, 8), 530),
                                      (synth.Shape(256, 128, 132, 4), 2050), (synth.Shape(512, 128, 1030, 3), 50)])
