@@ -257,7 +257,8 @@ enum {
     EXMOE_PATH_PAIR = 2,           /* per-pair gate/up kernel + by-token down kernel (T*k <= 24, one wave) */
     EXMOE_PATH_SMALL = 3,          /* grouping rebuilt inside the GEMM CTAs (T*k <= 24, several waves) */
     EXMOE_PATH_STREAM = 4,         /* bulk-copy weight ring + register dequantisation (T*k <= 640, at most 14 to 28 rows
-                                    * per expert by the shape; <= 192 where K does not split evenly over the warps) */
+                                    * per expert by the shape; < 12 per expert of at most 64 for 2048 x 1024; <= 192 where
+                                    * K does not split evenly over the warps) */
     EXMOE_PATH_TENSOR_SMALL_N = 5, /* tcgen05 kernels, 64-row token tiles (T*k <= 1024) */
     EXMOE_PATH_TENSOR = 6          /* tcgen05 kernels, 256-row token tiles */
 };

@@ -131,6 +131,10 @@ void launch_group(const exmoe_shape& s, int C, int n_keys, int max_waves, bool i
 // of 2048 x 1024, top-8, 81 tokens: 82 against 97 us per layer) and lose where it is skewed (Zipf of strength 1.5: 74 against
 // 63; 128 experts of 896 x 2048, 427 tokens: 124 against 48).
 constexpr int kStreamMaxPairs = 640;
+// ... and up to twelve rows per expert of at most 64 where both matrices run with their geometry as literals (d_model 2048,
+// d_ff 1024): the kernels are faster there. 64 experts, top-8, 94 tokens, uniform / Zipf 1.0 / 1.5: 0.86 / 1.0 / 1.29 of the
+// tensor-core kernels' time (0.75 / 0.85 / 1.08 of what these took before their look-ahead), and the weights are not rounded.
+constexpr int kStreamMaxRowsLiteral = 12, kStreamMaxExpertsLiteral = 64;
 // ... and up to 14 rows per expert on average, or 28 where the tensor-core kernels would leave SMs idle (the 128-row weight
 // tiles of all experts are no more than the SMs): against the tensor-core kernels at 14 / 20 / 28 rows per expert, 16 experts
 // of 1920 x 512 0.85 / 1.0 / 1.3 of their time, 24 of 2304 x 2048 1.05 / 1.3 / 1.5, 16 of 512 x 256 0.8 / 0.85 / 1.0.

@@ -125,6 +125,10 @@ __host__ bool stream_geometry(int K, int NR, int NM, int R, StreamGeom* out) {
     return best >= 0;
 }
 
+// OLMoE's two matrices have instantiations with their geometry as literals (d_model 2048: 16 blocks, one panel pair per tile, K in
+// four ranges; d_ff 1024: 8 blocks, four panels per tile, K in two ranges)
+inline bool literal_geometry(bool gateup, int K, const StreamGeom& g) { return gateup ? K / kGroup == 16 && g.PP == 1 : K / kGroup == 8 && g.PP == 4; }
+
 struct StreamArgs {
     GemmArgs a;
     const __nv_bfloat16* x_src;     // gate/up: hidden [T, H]; down: activations [pairs, I] in grouped row order
@@ -618,14 +622,8 @@ bool launch_stream_cfg(const GemmArgs& a, const __nv_bfloat16* x, __nv_bfloat16*
     void (*kern)(const StreamArgs) = stream_gemm_kernel<R, GATEUP>;
     int variant = 0;
 #ifndef EXMOE_STREAM_GENERIC_ONLY
-    // OLMoE's two matrices with their geometry as literals (d_model 2048: 16 blocks, one panel pair per tile, K in four
-    // ranges; d_ff 1024: 8 blocks, four panels per tile, K in two ranges)
-    const int KBv = (GATEUP ? a.H : a.I) / kGroup;
-    if (GATEUP && KBv == 16 && g.PP == 1) {
-        kern = stream_gemm_kernel<R, GATEUP, 16, 1>;
-        variant = 1;
-    } else if (!GATEUP && KBv == 8 && g.PP == 4) {
-        kern = stream_gemm_kernel<R, GATEUP, 8, 4>;
+    if (literal_geometry(GATEUP, GATEUP ? a.H : a.I, g)) {
+        kern = stream_gemm_kernel<R, GATEUP, GATEUP ? 16 : 8, GATEUP ? 1 : 4>;
         variant = 1;
     }
 #endif
@@ -679,7 +677,10 @@ int stream_max_pairs(const exmoe_shape& s) {
         sms = 148;
     const int tiles = s.num_experts * std::max(2 * s.d_ff, s.d_model) / 128;
     const int rows = tiles <= sms ? kStreamMaxRowsFew : kStreamMaxRows;
-    return std::min(even ? kStreamMaxPairs : kStreamMaxPairsUneven, rows * s.num_experts);
+    int pairs = even ? kStreamMaxPairs : kStreamMaxPairsUneven;
+    if (literal_geometry(true, s.d_model, gu) && literal_geometry(false, s.d_ff, dn) && s.num_experts <= kStreamMaxExpertsLiteral)
+        pairs = std::max(pairs, kStreamMaxRowsLiteral * s.num_experts - 1);
+    return std::min(pairs, rows * s.num_experts);
 }
 
 // One wave on the streaming kernels: passes of eight rows of a group.

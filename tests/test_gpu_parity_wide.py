@@ -319,10 +319,30 @@ def test_grouping_together_with_the_row_copy(B, d_model, E, k, T, slots):
     cache.close()
 
 
+@pytest.mark.parametrize("T", [81, 95])
+def test_streaming_kernels_past_their_own_grouping(B, olmoe_layer, T):
+    """648 and 760 pairs over 64 experts, fewer than 12 per expert: the streaming kernels on the grouping kernel's plan,
+    every token against the oracle, and bit for bit the same from a cache with misses and several waves."""
+    ora, bank = olmoe_layer
+    s = synth.OLMOE
+    hidden, ids, p = helpers.routed_inputs(s, T, seed=7300 + T, alpha=1.0)
+    y, ref = ora.forward(hidden, ids, p)
+    cache = B.Cache(s, [bank], 64, max_tokens=T)
+    out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    assert cache.last_path() == B.PATH_STREAM
+    compare_plan(cache, ocache.SlotCache(64, 64, 0, bytes_per_expert=cache.bytes_per_expert), ids)
+    helpers.check_output(out, y, ref, f"T={T}")
+    part = B.Cache(s, [bank], 24, max_tokens=T, wave_cap=10)
+    out2 = part.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    assert torch.equal(out2.view(torch.int16), out.view(torch.int16))
+    assert cache.status() == 0 and part.status() == 0
+    cache.close(); part.close()
+
+
 @pytest.mark.parametrize("E, k, T, path", [(64, 8, 80, "PATH_STREAM"), (64, 8, 81, "PATH_TENSOR_SMALL_N"), (96, 7, 110, "PATH_TENSOR_SMALL_N"),
                                            (128, 4, 300, "PATH_TENSOR")])
 def test_streaming_kernels_end_at_640_pairs(B, E, k, T, path):
-    """... however few rows that is per expert: what they cost under skewed routing the host cannot see."""
+    """... however few rows that is per expert (but for 2048 x 1024): what they cost under skewed routing the host cannot see."""
     s = synth.Shape(256, 128, E, k)
     ora, bank = helpers.make_layer(s, seed=71 + E)
     hidden, ids, p = helpers.routed_inputs(s, T, seed=5600 + T, alpha=1.0)
