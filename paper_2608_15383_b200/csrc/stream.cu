@@ -44,6 +44,7 @@ constexpr int kGroups = 2;                           // consumer groups, alterna
 constexpr int kConsumerWarps = kGroups * kGroupWarps;
 constexpr int kStreamThreads = 32 * (kConsumerWarps + 1);
 constexpr int kMaxStages = 8;
+constexpr int kPassRows = 8;                         // rows of one pass: the columns of one MMA tile (sixteen: slower at every size)
 constexpr size_t kSmemLimit = 227 * 1024;
 constexpr int kScanChunks = 4;                       // chunks of 32 groups whose plan entries the scan keeps in registers
 constexpr int kMetaGroups = 64;                      // most groups one CTA's share of the units can touch (see stream_geometry)
@@ -155,15 +156,15 @@ struct Cursor {
     }
 };
 
-// R: rows of one pass.  KBc, PPc: blocks along K and panels per tile as COMPILE-TIME constants (0 = taken from the
+// KBc, PPc: blocks along K and panels per tile as COMPILE-TIME constants (0 = taken from the
 // arguments).  With run-time values about a third of the executed instructions were address arithmetic, predicates and
 // loop control around the conversion and the MMAs; the shapes that matter (OLMoE's two matrices) get their own
 // instantiations with the block loop unrolled and every stride a literal, all others run the generic one.
-template <int R, bool GATEUP, int KBc = 0, int PPc = 0>
+template <bool GATEUP, int KBc = 0, int PPc = 0>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 stream_gemm_kernel(const StreamArgs p) {
     constexpr int NM = GATEUP ? 2 : 1;                                // matrices per tile
-    constexpr int NTM = R / 8;                                        // most column tiles (eight rows) of a pass
+    constexpr int R = kPassRows;
     extern __shared__ __align__(128) unsigned char smem[];
     const GemmArgs& a = p.a;
     constexpr bool FIXED = KBc > 0;
@@ -417,11 +418,11 @@ stream_gemm_kernel(const StreamArgs p) {
         const int ks = cw % KS, mw = (cw / KS) % NM, pp = cw / (KS * NM);    // K range, matrix, panel
         const int kb_lo = ks * KB / KS, kb_hi = (ks + 1) * KB / KS;
         const uint32_t w_full_a = smem_u32(w_full), w_empty_a = smem_u32(w_empty);
-        // partials of one unit: [pp][matrix][ks][column tile][word][lane], one buffer per group and unit parity
-        constexpr int part_words = kGroupWarps * NTM * 128;
+        // partials of one unit: [pp][matrix][ks][word][lane], one buffer per group and unit parity
+        constexpr int part_words = kGroupWarps * 128;
         float* partg = part + (size_t)grp * 2 * part_words;
         const int panel_local = NM * pp + mw;
-        // this lane's places: packed words and scales of the warp's first block, row q of a column tile, constants of rows 2c, 2c + 1
+        // this lane's places: packed words and scales of the warp's first block, row q, constants of rows 2c, 2c + 1
         const unsigned char* w_lane = wst + ((size_t)panel_local * KB + kb_lo) * kBlockBytes + lane * 16;
         const unsigned char* s_lane = wst + ((size_t)panel_local * KB + kb_lo) * kBlockBytes + kCodeBytes + q * 4;
         const unsigned char* x_lane = xs + (size_t)q * x_stride + (kb_lo * kGroup + 8 * c) * 2;
@@ -455,7 +456,6 @@ stream_gemm_kernel(const StreamArgs p) {
                 }
                 // With two buffers the one written here was last read two passes ago, and every warp has been past that
                 // since the previous pass's barrier.
-                static_assert(R == 8, "the list of a pass's pairs");
                 unsigned char* xw = xs + (size_t)xb * R * x_stride + l16 * 16;
                 float2* cwr = cst + (size_t)xb * KB * R;
                 int* rows_w = s_rows + warp * 8;
@@ -519,88 +519,65 @@ stream_gemm_kernel(const StreamArgs p) {
             const float2* c0 = c_lane + (size_t)xb * KB * R;
             float* pb = partg + (mine_cnt & 1) * part_words;
             ++mine_cnt;
-            const int nt = NTM == 1 ? 1 : (rows_here + 7) >> 3;
-            // the unit's blocks for NT x 8 rows (columns of rows that the pass does not have hold whatever the buffer does:
-            // columns are independent and theirs are never stored)
-            auto unit = [&](auto NTt) {
-                constexpr int NT = decltype(NTt)::value;
-                float tot[NT][4];
+            // the unit's blocks (columns of rows that the pass does not have hold whatever the buffer does: columns are
+            // independent and theirs are never stored)
+            float tot[4] = {0.f, 0.f, 0.f, 0.f};
+            [[maybe_unused]] const int nb = kb_hi - kb_lo;
+            [[maybe_unused]] constexpr int NBc = FIXED ? KBc / (8 / ((PPc > 0 ? PPc : 1) * NM)) : 1;
+            auto block = [&](int b) {
+                const uint4 w[2] = {*reinterpret_cast<const uint4*>(w0 + b * kBlockBytes),
+                                    *reinterpret_cast<const uint4*>(w0 + b * kBlockBytes + 512)};
+                const uint32_t sv = *reinterpret_cast<const uint32_t*>(s0 + b * kBlockBytes);
+                float d[2][4];                                         // two chains
 #pragma unroll
-                for (int j = 0; j < NT; ++j)
+                for (int i = 0; i < 4; ++i) d[0][i] = d[1][i] = 0.f;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) tot[j][i] = 0.f;
-                [[maybe_unused]] const int nb = kb_hi - kb_lo;
-                [[maybe_unused]] constexpr int NBc = FIXED ? KBc / (8 / ((PPc > 0 ? PPc : 1) * NM)) : 1;
-                auto block = [&](int b) {
-                    const uint4 w[2] = {*reinterpret_cast<const uint4*>(w0 + b * kBlockBytes),
-                                        *reinterpret_cast<const uint4*>(w0 + b * kBlockBytes + 512)};
-                    const uint32_t sv = *reinterpret_cast<const uint32_t*>(s0 + b * kBlockBytes);
-                    float d[NT][2][4];                                 // two chains per column tile
+                for (int h = 0; h < 2; ++h)
 #pragma unroll
-                    for (int j = 0; j < NT; ++j)
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) d[j][0][i] = d[j][1][i] = 0.f;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-#pragma unroll
-                        for (int set = 0; set < 2; ++set) {
-                            const CodeFrag cf(set ? w[h].z : w[h].x, set ? w[h].w : w[h].y);
-                            uint4 x[NT];
-#pragma unroll
-                            for (int j = 0; j < NT; ++j)
-                                x[j] = *reinterpret_cast<const uint4*>(x0 + (size_t)(8 * j) * x_stride + (b * kGroup + 64 * h + 32 * set) * 2);
-#pragma unroll
-                            for (int j = 0; j < NT; ++j) cf.first(d[j][set], x[j]);
-#pragma unroll
-                            for (int j = 0; j < NT; ++j) cf.second(d[j][set], x[j]);
-                        }
-                    const float2 sc = scales16(sv);
-#pragma unroll
-                    for (int j = 0; j < NT; ++j) {
-                        const float4 k4 = *reinterpret_cast<const float4*>(c0 + b * R + 8 * j);     // rows 8 j + 2 c and + 1
-                        tot[j][0] = fmaf(sc.x, fmaf(d[j][0][0] + d[j][1][0], k4.x, k4.y), tot[j][0]);
-                        tot[j][1] = fmaf(sc.x, fmaf(d[j][0][1] + d[j][1][1], k4.z, k4.w), tot[j][1]);
-                        tot[j][2] = fmaf(sc.y, fmaf(d[j][0][2] + d[j][1][2], k4.x, k4.y), tot[j][2]);
-                        tot[j][3] = fmaf(sc.y, fmaf(d[j][0][3] + d[j][1][3], k4.z, k4.w), tot[j][3]);
+                    for (int set = 0; set < 2; ++set) {
+                        const CodeFrag cf(set ? w[h].z : w[h].x, set ? w[h].w : w[h].y);
+                        const uint4 x = *reinterpret_cast<const uint4*>(x0 + (b * kGroup + 64 * h + 32 * set) * 2);
+                        cf.first(d[set], x);
+                        cf.second(d[set], x);
                     }
-                };
-                if constexpr (FIXED) {
-#pragma unroll
-                    for (int b = 0; b < NBc; ++b) block(b);
-                } else {
-#pragma unroll 2
-                    for (int b = 0; b < nb; ++b) block(b);
-                }
-                __syncwarp();
-                if (elect_one()) mbar_arrive_at(w_empty_a + 8 * s);    // this warp is done with the weight stage
-                // Partials cross shared memory once (buffer alternates with the group's units, so one barrier per unit
-                // is enough); then the warps finish the slices (panel, N-tile, row half): the sum over the K ranges in
-                // ascending order, SwiGLU or routing weight, store.
-                float* pw = pb + (size_t)((pp * NM + mw) * KS + ks) * (NTM * 128) + lane;
-#pragma unroll
-                for (int j = 0; j < NT; ++j)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) pw[(4 * j + i) * 32] = tot[j][i];
+                const float2 sc = scales16(sv);
+                const float4 k4 = *reinterpret_cast<const float4*>(c0 + b * R);            // rows 2 c and 2 c + 1
+                tot[0] = fmaf(sc.x, fmaf(d[0][0] + d[1][0], k4.x, k4.y), tot[0]);
+                tot[1] = fmaf(sc.x, fmaf(d[0][1] + d[1][1], k4.z, k4.w), tot[1]);
+                tot[2] = fmaf(sc.y, fmaf(d[0][2] + d[1][2], k4.x, k4.y), tot[2]);
+                tot[3] = fmaf(sc.y, fmaf(d[0][3] + d[1][3], k4.z, k4.w), tot[3]);
             };
-            if constexpr (NTM == 1) unit(std::integral_constant<int, 1>());
-            else if (nt == 1) unit(std::integral_constant<int, 1>());
-            else unit(std::integral_constant<int, 2>());
+            if constexpr (FIXED) {
+#pragma unroll
+                for (int b = 0; b < NBc; ++b) block(b);
+            } else {
+#pragma unroll 2
+                for (int b = 0; b < nb; ++b) block(b);
+            }
+            __syncwarp();
+            if (elect_one()) mbar_arrive_at(w_empty_a + 8 * s);        // this warp is done with the weight stage
+            // Partials cross shared memory once (buffer alternates with the group's units, so one barrier per unit
+            // is enough); then the warps finish the slices (panel, word): the sum over the K ranges in ascending
+            // order, SwiGLU or routing weight, store.
+            float* pw = pb + (size_t)((pp * NM + mw) * KS + ks) * 128 + lane;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) pw[i * 32] = tot[i];
             group_sync(grp);
-            const int slices = PP * nt * 4;
-#pragma unroll(FIXED && NTM == 1 ? (PPc > 1 ? PPc / 2 : 1) : 1)
+            const int slices = PP * 4;
+#pragma unroll(FIXED ? (PPc > 1 ? PPc / 2 : 1) : 1)
             for (int sl = cw; sl < slices; sl += kGroupWarps) {
-                const int spp = FIXED && PPc == 1 ? 0 : sl / (4 * nt), ji = sl - spp * 4 * nt;
+                const int spp = FIXED && PPc == 1 ? 0 : sl / 4, ji = sl - spp * 4;
                 float v[NM];
 #pragma unroll
                 for (int mg = 0; mg < NM; ++mg) {
-                    const float* pr = pb + (size_t)((spp * NM + mg) * KS) * (NTM * 128) + ji * 32 + lane;
+                    const float* pr = pb + (size_t)((spp * NM + mg) * KS) * 128 + ji * 32 + lane;
                     float sum = pr[0];
-                    for (int k2 = 1; k2 < KS; ++k2) sum += pr[k2 * (NTM * 128)];
+                    for (int k2 = 1; k2 < KS; ++k2) sum += pr[k2 * 128];
                     v[mg] = sum;
                 }
-                const int rr = 8 * (ji >> 2) + 2 * c + (ji & 1);       // row of the pass
+                const int rr = 2 * c + (ji & 1);                       // row of the pass
                 if (rr >= rows_here || !ok) continue;
-                const int orow = (tile * PP + spp) * kPanelRows + q + 8 * ((ji >> 1) & 1);
+                const int orow = (tile * PP + spp) * kPanelRows + q + 8 * (ji >> 1);
                 if (GATEUP) {
                     const float gv = v[0], uv = v[NM - 1];
                     p.act_out[(size_t)(row0 + pass0 + rr) * a.I + orow] = __float2bfloat16_rn(gv / (1.f + __expf(-gv)) * uv);
@@ -613,17 +590,17 @@ stream_gemm_kernel(const StreamArgs p) {
     }
 }
 
-template <int R, bool GATEUP>
+template <bool GATEUP>
 bool launch_stream_cfg(const GemmArgs& a, const __nv_bfloat16* x, __nv_bfloat16* act, const float* w, float* y, int* status,
                        int max_groups, bool dependent, cudaStream_t st) {
     constexpr int NM = GATEUP ? 2 : 1;
     StreamGeom g;
-    if (!stream_geometry(GATEUP ? a.H : a.I, GATEUP ? a.I : a.H, NM, R, &g)) return false;
-    void (*kern)(const StreamArgs) = stream_gemm_kernel<R, GATEUP>;
+    if (!stream_geometry(GATEUP ? a.H : a.I, GATEUP ? a.I : a.H, NM, kPassRows, &g)) return false;
+    void (*kern)(const StreamArgs) = stream_gemm_kernel<GATEUP>;
     int variant = 0;
 #ifndef EXMOE_STREAM_GENERIC_ONLY
     if (literal_geometry(GATEUP, GATEUP ? a.H : a.I, g)) {
-        kern = stream_gemm_kernel<R, GATEUP, GATEUP ? 16 : 8, GATEUP ? 1 : 4>;
+        kern = stream_gemm_kernel<GATEUP, GATEUP ? 16 : 8, GATEUP ? 1 : 4>;
         variant = 1;
     }
 #endif
@@ -670,7 +647,7 @@ bool launch_stream_cfg(const GemmArgs& a, const __nv_bfloat16* x, __nv_bfloat16*
 
 int stream_max_pairs(const exmoe_shape& s) {
     StreamGeom gu, dn;
-    if (!stream_geometry(s.d_model, s.d_ff, 2, 8, &gu) || !stream_geometry(s.d_ff, s.d_model, 1, 8, &dn)) return 0;
+    if (!stream_geometry(s.d_model, s.d_ff, 2, kPassRows, &gu) || !stream_geometry(s.d_ff, s.d_model, 1, kPassRows, &dn)) return 0;
     const bool even = (s.d_model / kGroup) % gu.KS == 0 && (s.d_ff / kGroup) % dn.KS == 0;
     int sms = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
@@ -692,12 +669,9 @@ bool launch_stream_wave(const GemmArgs& a, const __nv_bfloat16* hidden, __nv_bfl
 #else
     const bool entry_dependent = false;
 #endif
-#ifndef EXMOE_STREAM_ROWS
-#define EXMOE_STREAM_ROWS 8
-#endif
-    if (gateup) ok = launch_stream_cfg<EXMOE_STREAM_ROWS, true>(a, hidden, act, topk_w, y, status, max_groups, entry_dependent, st);
+    if (gateup) ok = launch_stream_cfg<true>(a, hidden, act, topk_w, y, status, max_groups, entry_dependent, st);
     // a programmatic dependent only when the gate/up kernel of the same wave was launched just before it
-    if (down && ok) ok = launch_stream_cfg<EXMOE_STREAM_ROWS, false>(a, act, act, topk_w, y, status, max_groups, gateup, st);
+    if (down && ok) ok = launch_stream_cfg<false>(a, act, act, topk_w, y, status, max_groups, gateup, st);
     return ok;
 }
 
