@@ -260,7 +260,7 @@ enum {
                                     * per expert by the shape; < 12 per expert of at most 64 for 2048 x 1024; <= 192 where
                                     * K does not split evenly over the warps) */
     EXMOE_PATH_TENSOR_SMALL_N = 5, /* tcgen05 kernels, 64-row token tiles (T*k <= 1024) */
-    EXMOE_PATH_TENSOR = 6          /* tcgen05 kernels, 256-row token tiles */
+    EXMOE_PATH_TENSOR = 6          /* tcgen05 kernels, token tiles of up to 256 rows */
 };
 int exmoe_debug_last_path(exmoe_cache* cache);
 

@@ -30,7 +30,7 @@
 //                 127 -> 119 us, 1024 tokens 177 -> 174 us, 2048 tokens unchanged per OLMoE-shaped layer.
 // Producers -> MMA through full[stage] mbarriers, MMA -> producers through tcgen05.commit on empty[stage].
 // The gate/up GEMM reads its tokens from a grouped copy of the hidden states (rows in plan order),
-// written once per call by gather_rows_kernel, so that both GEMMs load B with plain tiled TMA.
+// written once per call (plan_gather_kernel, or gather_rows_kernel for large calls), so that both GEMMs load B with plain tiled TMA.
 // Every wait is bounded: on expiry the CTA raises EXMOE_ERR_TIMEOUT, all roles drain, TMEM is freed.
 //
 // Measured alone on one SM (one CTA, operands in place): an MMA of this shape takes N / 2 cycles issued back to
@@ -71,7 +71,7 @@ constexpr int A_STAGE_BYTES = 16 * A_SBO;      // 20 KB
 // B (tokens): TMA 128-byte swizzle; 64 columns x up to 256 rows of 128 B; 8-row atoms of 1024 B
 constexpr int B_SBO = 1024;
 constexpr int N_MAPS = 16;         // tensor maps per operand: boxes of 16, 32, ..., 256 rows
-constexpr int NUM_THREADS = 896;   // 28 warps: MMA, TMA, 2 idle, 4 + 4 epilogue, 8 + 8 dequant
+constexpr int NUM_THREADS = 896;   // 28 warps: MMA, TMA, relay, 1 idle, 4 + 4 epilogue, 8 + 8 dequant
 
 struct Tile { int key, n0, nrows, pad; };
 
