@@ -132,12 +132,13 @@ void launch_group(const exmoe_shape& s, int C, int n_keys, int max_waves, bool i
 // 63; 128 experts of 896 x 2048, 427 tokens: 124 against 48).
 constexpr int kStreamMaxPairs = 640;
 // ... and up to twelve rows per expert of at most 64 where both matrices run with their geometry as literals (d_model 2048,
-// d_ff 1024): the kernels are faster there. 64 experts, top-8, 94 tokens, uniform / Zipf 1.0 / 1.5: 0.86 / 1.0 / 1.29 of the
-// tensor-core kernels' time (0.75 / 0.85 / 1.08 of what these took before their look-ahead), and the weights are not rounded.
+// d_ff 1024): the kernels are faster there. 64 experts, top-8, 81 and 94 tokens: uniform routing 0.84 and 0.93 of the
+// tensor-core kernels' time, Zipf 1.0 1.03 and 1.00, Zipf 1.5 1.17 and 1.28; and the weights are not rounded to BF16.
 constexpr int kStreamMaxRowsLiteral = 12, kStreamMaxExpertsLiteral = 64;
 // ... and up to 14 rows per expert on average, or 28 where the tensor-core kernels would leave SMs idle (the 128-row weight
-// tiles of all experts are no more than the SMs): against the tensor-core kernels at 14 / 20 / 28 rows per expert, 16 experts
-// of 1920 x 512 0.85 / 1.0 / 1.3 of their time, 24 of 2304 x 2048 1.05 / 1.3 / 1.5, 16 of 512 x 256 0.8 / 0.85 / 1.0.
+// tiles of all experts are no more than the SMs). Against the tensor-core kernels at 12 / 14 / 20 / 24 rows per expert, uniform
+// routing: 32 experts of 1024 x 512 0.94 / 0.95 / 1.21 / 1.28 of their time, 24 of 1536 x 768 0.99 / 1.11 / 1.34 / 1.52; with
+// fewer tiles than SMs 16 of 512 x 256 0.64 / 0.91 / 0.97 / 0.99 (32 rows: 1.28), 8 of 256 x 128 0.65 / 0.92 / 0.98 / 1.02.
 constexpr int kStreamMaxRows = 14, kStreamMaxRowsFew = 28;
 // ... and up to 192 pairs where the eight warps of a consumer group cannot share K evenly (7, 9, 11, 13, 15 ... blocks): a group's
 // time is its longest range's. 48 experts of 2048 x 1920, 480 pairs, Zipf 1.5: 1.36 of the tensor-core kernels' time;
