@@ -259,8 +259,9 @@ enum {
     EXMOE_PATH_STREAM = 4,         /* bulk-copy weight ring + register dequantisation (T*k <= 640, at most 14 to 28 rows
                                     * per expert by the shape; < 12 per expert of at most 64 for 2048 x 1024; <= 192 where
                                     * K does not split evenly over the warps) */
-    EXMOE_PATH_TENSOR_SMALL_N = 5, /* tcgen05 kernels, 64-row token tiles (T*k <= 1024) */
-    EXMOE_PATH_TENSOR = 6          /* tcgen05 kernels, token tiles of up to 256 rows */
+    EXMOE_PATH_TENSOR_SMALL_N = 5, /* tcgen05 kernels up to T*k = 1024: 64-row token tiles */
+    EXMOE_PATH_TENSOR = 6          /* tcgen05 kernels beyond: token tiles of up to 256 rows.  Large layers of d_model >= 2048 take
+                                    * the streaming tcgen05 kernels on either side of 1024, up to 24 rows per expert */
 };
 int exmoe_debug_last_path(exmoe_cache* cache);
 

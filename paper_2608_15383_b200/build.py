@@ -12,7 +12,7 @@ CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libexmoe.so")
 NATIVE = os.path.join(PKG, "_exmoe_native.so")
 NATIVE_SOURCE = "binding_native.cpp"
-SOURCES = ["pack.cu", "plan.cu", "decode.cu", "stream.cu", "prefill.cu", "route.cu", "cache.cu"]
+SOURCES = ["pack.cu", "plan.cu", "decode.cu", "stream.cu", "prefill.cu", "tcstream.cu", "route.cu", "cache.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--shared", "--threads", "8"]
 

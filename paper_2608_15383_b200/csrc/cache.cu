@@ -489,7 +489,8 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
     const bool pairwise = small && P <= kPairMaxPairs && n_waves == 1 && c->pair_ok;
     c->last_pair = pairwise || own_plan;
     const bool small_n = P <= kPrefillSmallNMaxPairs;      // tensor-core path: which kernel shape
-    const int tile_rows = prefill_tile_rows(s, P, c->Cw, small_n);
+    const int tc_kind = tc_stream_takes(s, P) ? TC_STREAM : small_n ? TC_SMALL_N : TC_LARGE;
+    const int tile_rows = prefill_tile_rows(s, P, c->Cw, tc_kind);
     c->last_path = pairwise ? EXMOE_PATH_PAIR : small ? EXMOE_PATH_SMALL : use_stream ? EXMOE_PATH_STREAM
                    : small_n ? EXMOE_PATH_TENSOR_SMALL_N : EXMOE_PATH_TENSOR;
     if (!small && build_plan && !use_stream) {
@@ -497,10 +498,10 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
         tiles_fused = (n_waves == 1);                    // one wave: its tile list comes out of the same launch
         if (!plan_with_rows)
             launch_gather_rows((const __nv_bfloat16*)hidden, c->plan.perm, c->plan.offsets + c->n_keys, P, k, s.d_model,
-                               c->xg, tiles_fused ? &a : nullptr, c->plan.wave_start, c->tc_scratch, tile_rows, st);
+                               c->xg, tiles_fused ? &a : nullptr, c->plan.wave_start, c->tc_scratch, tile_rows, tc_kind == TC_STREAM, st);
         else
             launch_plan_gather(s, C, c->n_keys, c->max_waves, identity, (const __nv_bfloat16*)hidden, topk_ids, P, c->plan, c->d_status,
-                               c->xg, tiles_fused, c->tc_scratch, tile_rows, st);
+                               c->xg, tiles_fused, c->tc_scratch, tile_rows, tc_kind == TC_STREAM, st);
     }
     if (small && n_waves == 0)                           // no valid id at all: the output is zero
         cudaMemsetAsync(out, 0, (size_t)T * s.d_model * 2, st);
@@ -616,16 +617,16 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
         } else {
             // many rows per expert: dense contraction on the tensor cores (tcgen05 / TMEM)
             if (build_plan && !tiles_fused)
-                launch_prefill_wave(a, a.wave_start, c->tc_scratch, c->d_status, &c->tc_maps, c->act, topk_weights, c->y, 4, small_n, tile_rows, st);
+                launch_prefill_wave(a, a.wave_start, c->tc_scratch, c->d_status, &c->tc_maps, c->act, topk_weights, c->y, 4, tc_kind, tile_rows, st);
             if (!c->prof_only || c->prof_only == PROF_GATEUP) {
                 ProfScope ps(c, PROF_GATEUP, st);
                 launch_prefill_wave(a, a.wave_start, c->tc_scratch, c->d_status, &c->tc_maps, c->act, topk_weights, c->y, 1,
-                                    small_n, tile_rows, st);
+                                    tc_kind, tile_rows, st);
             }
             if (!c->prof_only || c->prof_only == PROF_DOWN) {
                 ProfScope ps(c, PROF_DOWN, st);
                 launch_prefill_wave(a, a.wave_start, c->tc_scratch, c->d_status, &c->tc_maps, c->act, topk_weights, c->y, 2,
-                                    small_n, tile_rows, st);
+                                    tc_kind, tile_rows, st);
             }
         }
         if (!identity && !dev_fetch) {

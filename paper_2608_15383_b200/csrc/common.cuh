@@ -159,22 +159,37 @@ size_t prefill_scratch_bytes(int max_pairs, int num_experts);
 constexpr size_t kPrefillMapBytes = 2 * 16 * 128;
 struct PrefillMaps { unsigned char* dev; };
 int prefill_setup(PrefillMaps* maps, const __nv_bfloat16* xg, const __nv_bfloat16* act, int max_pairs, int H, int I);
+struct Tile;
+// one wave on the streaming tensor-core kernels (token matrices in their K order); false: not possible on this device
+bool launch_tc_stream_wave(const GemmArgs& g, const Tile* tiles, int tile_cap, const int32_t* n_tiles, int* status, const PrefillMaps* maps, __nv_bfloat16* act,
+                           const float* topk_w, float* y, bool gateup, bool down, cudaStream_t st);
 void launch_wait_selftest(int* status, long long budget_cycles, int* result, cudaStream_t st);
 // Grouping and grouped copy of the hidden rows in one launch, for calls within these limits.  Its CTAs each count all pairs
 // in shared memory: measured at 64 experts it wins up to 8192 pairs, at 16384 the separate kernels are 3 us faster.
 constexpr int kPlanGatherPairs = 8192, kPlanGatherKeys = 1024;
 void launch_plan_gather(const exmoe_shape& s, int C, int n_keys, int max_waves, bool identity, const __nv_bfloat16* hidden,
                         const int32_t* ids, int n_pairs, PlanPtrs plan, int* status, __nv_bfloat16* xg, bool single_wave,
-                        void* scratch, int tile_rows, cudaStream_t st);
+                        void* scratch, int tile_rows, bool k_order, cudaStream_t st);
 // grouped copy of the hidden rows; when `single_wave` is given its CTA 0 also builds that wave's tile list in `scratch`
 void launch_gather_rows(const __nv_bfloat16* hidden, const int32_t* perm, const int32_t* n_valid, int n_pairs, int top_k,
                         int H, __nv_bfloat16* xg, const GemmArgs* single_wave, const int32_t* wave_start, void* scratch,
-                        int tile_rows, cudaStream_t st);
+                        int tile_rows, bool k_order, cudaStream_t st);
 // which: bit 0 = gate/up GEMM + SwiGLU, bit 1 = down GEMM x routing weight, bit 2 = (re)build the wave's tile list
-// small_n: the 64-row, eight-stage kernel shape (a few dozen rows per expert) instead of the 256-row, four-stage one
+// kind: the 64-row, eight-stage kernel shape (a few dozen rows per expert), the 256-row, four-stage one, or the streaming kernels
 void launch_prefill_wave(const GemmArgs& g, const int32_t* wave_start, void* scratch, int* status, const PrefillMaps* maps,
-                         __nv_bfloat16* act, const float* topk_w, float* y, int which, bool small_n, int tile_rows, cudaStream_t st);
-int prefill_tile_rows(const exmoe_shape& s, int n_pairs, int experts_per_wave, bool small_n);     // most grouped rows per tile
+                         __nv_bfloat16* act, const float* topk_w, float* y, int which, int kind, int tile_rows, cudaStream_t st);
+enum { TC_SMALL_N = 0, TC_LARGE = 1, TC_STREAM = 2 };     // kind of a tensor-core call
+// The streaming tensor-core kernels: beyond the streaming kernels' range up to 24 rows per expert, for layers whose gate/up
+// matrices come to 100 blocks of 128 x 128 per SM and whose K is at least 2048 (their launches take 2.5 us longer to their first MMA than
+// the other tensor-core kernels, which smaller layers and few active experts do not earn back).  Of the other kernels' time, with
+// routing uniform / Zipf 0.5 / Zipf 1.5: 64 experts of 2048 x 1024, top-8, 100 tokens 0.79 / 0.78 / 1.02, 150 0.86 / 0.88 / 1.01,
+// 250 (31 rows) 0.92 / 0.92 / 1.09; 60 of 2048 x 1408, top-4, 161 tokens 0.74 / 0.78 / 0.89, 200 0.78 / 0.77 / 1.03, 300
+// 0.81 / 0.83 / 1.15.  Not taken: 96 of 1024 x 1408, top-2, 500 tokens 0.80 / 0.90 / 1.13; 40 of 896 x 1152, top-5, 150 tokens
+// 1.02 / 0.96 / 1.16; 16 of 512 x 256, top-4, 200 tokens 1.33 / 1.27 / 1.29.  By the layer's experts, not the cache's slots: a call's bits
+// do not depend on these.
+constexpr int kTcStreamMaxRows = 24, kTcStreamMinBlocksPerSm = 100, kTcStreamMinModel = 2048;
+bool tc_stream_takes(const exmoe_shape& s, int n_pairs);
+int prefill_tile_rows(const exmoe_shape& s, int n_pairs, int experts_per_wave, int kind);     // most grouped rows per tile
 #ifndef EXMOE_PREFILL_SMALL_N_MAX_PAIRS
 #define EXMOE_PREFILL_SMALL_N_MAX_PAIRS 1024
 #endif

@@ -50,6 +50,7 @@
 #include "frag.cuh"
 #include "mbar.cuh"
 #include "plan.cuh"
+#include "tc.cuh"
 #ifdef EXMOE_PREFILL_PROF
 #include <cstdio>
 #endif
@@ -58,7 +59,6 @@ namespace exmoe {
 
 namespace {
 
-constexpr int BM = 128;            // weight rows per tile
 constexpr int BN = 256;            // max grouped rows (tokens) per tile of the large-N kernel shape
 constexpr int BN_SMALL = 64;       // ... and of the small-N shape (a few dozen rows per expert: eight stages fit)
 constexpr int BK = 128;            // one packed block / one scale group
@@ -68,12 +68,8 @@ constexpr int BKS = 64;            // K per ring stage = half a packed block (th
 constexpr int A_LBO = 160;
 constexpr int A_SBO = (BKS / 8) * A_LBO;
 constexpr int A_STAGE_BYTES = 16 * A_SBO;      // 20 KB
-// B (tokens): TMA 128-byte swizzle; 64 columns x up to 256 rows of 128 B; 8-row atoms of 1024 B
-constexpr int B_SBO = 1024;
-constexpr int N_MAPS = 16;         // tensor maps per operand: boxes of 16, 32, ..., 256 rows
+// B (tokens): TMA 128-byte swizzle; 64 columns x up to 256 rows of 128 B
 constexpr int NUM_THREADS = 896;   // 28 warps: MMA, TMA, relay, 1 idle, 4 + 4 epilogue, 8 + 8 dequant
-
-struct Tile { int key, n0, nrows, pad; };
 
 #ifdef EXMOE_PREFILL_PROF
 #define PROF_DECL long long prof_t0 = clock64(), prof_wait = 0
@@ -88,11 +84,6 @@ struct Tile { int key, n0, nrows, pad; };
 #endif
 
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit_at(uint32_t bar) {       // barrier by its shared-memory address
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
 __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -101,19 +92,7 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-}
-__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// shared-memory matrix descriptors, K-major, version 1 (sm_100)
+// shared-memory matrix descriptor of the weights, K-major, version 1 (sm_100)
 __device__ __forceinline__ uint64_t make_desc_a(uint32_t saddr) {            // no swizzle
     uint64_t d = 0;
     d |= (uint64_t)((saddr >> 4) & 0x3fff);
@@ -121,25 +100,6 @@ __device__ __forceinline__ uint64_t make_desc_a(uint32_t saddr) {            // 
     d |= (uint64_t)((A_SBO >> 4) & 0x3fff) << 32;
     d |= (uint64_t)1 << 46;
     return d;
-}
-__device__ __forceinline__ uint64_t make_desc_b(uint32_t saddr) {            // 128-byte swizzle
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3fff);
-    d |= (uint64_t)1 << 16;                                                  // leading offset unused with swizzle
-    d |= (uint64_t)((B_SBO >> 4) & 0x3fff) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-        : "memory");
-}
-// instruction descriptor: D fp32, A/B BF16, both K-major, M = 128, N = n
-__device__ __forceinline__ uint32_t make_idesc(int n) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 __device__ __forceinline__ uint4 ldg_stream128(const void* p) {
     uint4 v;
@@ -200,10 +160,9 @@ struct EpiloguePre {
 };
 template <bool GATEUP, int CHUNKS>
 __device__ __forceinline__ EpiloguePre<CHUNKS> epilogue_prefetch(const PrefillArgs& a, const Tile& tl, int first, int lane,
-                                                                 const int32_t* __restrict__ offsets,
                                                                  const float* __restrict__ topk_w) {
     EpiloguePre<CHUNKS> p;
-    p.row0 = offsets[tl.key] + tl.n0;
+    p.row0 = tl.row0;
 #pragma unroll
     for (int i = 0; i < CHUNKS; ++i) {
         p.pair[i] = 0;
@@ -266,7 +225,7 @@ __device__ __forceinline__ void epilogue_tile(const PrefillArgs& a, const Tile& 
 template <bool GATEUP, int BN_T, int STAGES>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bfloat16* __restrict__ act_out,
-                    const float* __restrict__ topk_w, const int32_t* __restrict__ offsets, float* __restrict__ y_out) {
+                    const float* __restrict__ topk_w, float* __restrict__ y_out) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // swizzled tiles need 1 KB alignment
     constexpr int B_STAGE_BYTES = BN_T * 128;                     // BN_T rows x 64 columns
@@ -412,7 +371,7 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
             const int mt = t % MT;
             const int buf = tcount & 1;
             constexpr int CHUNKS = (BN_T + 63) / 64;               // 32-column chunks of this warp in a full tile
-            const EpiloguePre<CHUNKS> pre = epilogue_prefetch<GATEUP, CHUNKS>(a, tl, odd, lane, offsets, topk_w);
+            const EpiloguePre<CHUNKS> pre = epilogue_prefetch<GATEUP, CHUNKS>(a, tl, odd, lane, topk_w);
             PROF_WAIT_BEGIN;
             ok = mbar_wait_warp(acc_full_a + 8 * buf, (tcount >> 1) & 1, abort_flag, a.status);
             PROF_WAIT_END;
@@ -431,7 +390,7 @@ prefill_gemm_kernel(PrefillArgs a, const CUtensorMap* __restrict__ maps, __nv_bf
         PROF_DECL;
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
             const Tile tl = a.tiles[t / MT];
-            const int row0 = offsets[tl.key] + tl.n0;
+            const int row0 = tl.row0;
             const int n_mma = (tl.nrows + 15) & ~15;               // rows of the box = rows the MMAs read
             const CUtensorMap* map = maps + (n_mma / 16 - 1);
             for (int ks = 0; ks < 2 * KB; ++ks) {
@@ -602,53 +561,87 @@ __global__ void wait_timeout_selftest_kernel(int* status, long long budget, int*
 }
 
 // n-tiles of one wave: every active group is cut into balanced runs of at most `bn` grouped rows (multiples of 16).
-// Executed by one whole CTA (any multiple of 32 threads up to 1024): thread g handles group g, an exclusive scan of
+// With each tile goes the weight of those before it (tile_weight).  Executed by one whole CTA (any multiple of 32 threads up to 1024): thread g handles group g, an exclusive scan of
 // the piece counts places its tiles.
-__device__ void build_tile_list(const int32_t* __restrict__ counts, const int32_t* __restrict__ group_keys,
+__device__ void build_tile_list(const int32_t* __restrict__ counts, const int32_t* __restrict__ offsets, const int32_t* __restrict__ group_keys,
                                 const int32_t* __restrict__ wave_start, Tile* __restrict__ tiles,
                                 int32_t* __restrict__ n_tiles, int bn) {
-    __shared__ int s_warp[32];
-    __shared__ int s_running;
+    __shared__ int s_warp[32], s_weight[32];
+    __shared__ int s_running, s_running_w;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x, nwarp = nthr >> 5;
     const int g0 = wave_start[0], ng = wave_start[1] - g0;
-    if (tid == 0) s_running = 0;
+    if (tid == 0) s_running = s_running_w = 0;
     __syncthreads();
     for (int base = 0; base < ng; base += nthr) {
         const int g = base + tid;
-        int key = 0, cnt = 0, pieces = 0, per = 0;
+        int key = 0, cnt = 0, row0 = 0, pieces = 0, per = 0;
         if (g < ng) {
             key = group_keys[g0 + g];
             cnt = counts[key];
+            row0 = offsets[key];
             pieces = (cnt + bn - 1) / bn;
             per = ((cnt + pieces - 1) / pieces + 15) & ~15;
             pieces = (cnt + per - 1) / per;
         }
-        int incl = pieces;
+        const int mine = pieces ? (pieces - 1) * tile_weight(per) + tile_weight(cnt - (pieces - 1) * per) : 0;
+        int incl = pieces, incl_w = mine;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            const int o = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += o;
+            const int o = __shfl_up_sync(0xffffffffu, incl, d), ow = __shfl_up_sync(0xffffffffu, incl_w, d);
+            if (lane >= d) {
+                incl += o;
+                incl_w += ow;
+            }
         }
-        if (lane == 31) s_warp[warp] = incl;
+        if (lane == 31) {
+            s_warp[warp] = incl;
+            s_weight[warp] = incl_w;
+        }
         __syncthreads();
-        int wbase = 0, total = 0;
+        int wbase = 0, total = 0, wbase_w = 0, total_w = 0;
         for (int w = 0; w < nwarp; ++w) {
-            if (w < warp) wbase += s_warp[w];
+            if (w < warp) {
+                wbase += s_warp[w];
+                wbase_w += s_weight[w];
+            }
             total += s_warp[w];
+            total_w += s_weight[w];
         }
-        int pos = s_running + wbase + incl - pieces;
-        for (int n0 = 0; n0 < cnt; n0 += per) tiles[pos++] = Tile{key, n0, min(per, cnt - n0), 0};
+        int pos = s_running + wbase + incl - pieces, weight = s_running_w + wbase_w + incl_w - mine;
+        for (int n0 = 0; n0 < cnt; n0 += per) {
+            tiles[pos++] = Tile{key, weight, min(per, cnt - n0), row0 + n0};
+            weight += tile_weight(min(per, cnt - n0));
+        }
         __syncthreads();
-        if (tid == 0) s_running += total;
+        if (tid == 0) {
+            s_running += total;
+            s_running_w += total_w;
+        }
         __syncthreads();
     }
-    if (tid == 0) *n_tiles = s_running;
+    if (tid == 0) {
+        n_tiles[0] = s_running;
+        n_tiles[1] = s_running_w;                      // weight of all tiles
+    }
 }
 
 __global__ void __launch_bounds__(1024)
-tile_list_kernel(const int32_t* __restrict__ counts, const int32_t* __restrict__ group_keys,
+tile_list_kernel(const int32_t* __restrict__ counts, const int32_t* __restrict__ offsets, const int32_t* __restrict__ group_keys,
                  const int32_t* __restrict__ wave_start, Tile* __restrict__ tiles, int32_t* __restrict__ n_tiles, int bn) {
-    build_tile_list(counts, group_keys, wave_start, tiles, n_tiles, bn);
+    build_tile_list(counts, offsets, group_keys, wave_start, tiles, n_tiles, bn);
+}
+
+// 16-byte chunk of a row, by its place in the row's order or in the K order of the kernels whose weights are in tensor memory
+// (k_position: the pairs (c, s) of four neighbouring chunks as (s, c), a transposition among four lanes).  By whole warps.
+__device__ __forceinline__ uint4 ordered_chunk(uint4 v, int lane, bool k_order) {
+    if (k_order) {
+        const bool odd = lane & 1, high = lane & 2;
+        const uint32_t a = __shfl_xor_sync(0xffffffffu, odd ? v.x : v.y, 1), b = __shfl_xor_sync(0xffffffffu, odd ? v.z : v.w, 1);
+        v = odd ? make_uint4(a, v.y, b, v.w) : make_uint4(v.x, a, v.z, b);
+        const uint32_t c = __shfl_xor_sync(0xffffffffu, high ? v.x : v.z, 2), d = __shfl_xor_sync(0xffffffffu, high ? v.y : v.w, 2);
+        v = high ? make_uint4(c, d, v.z, v.w) : make_uint4(v.x, v.y, c, d);
+    }
+    return v;
 }
 
 // grouped copy of the hidden states: row r of the plan order = hidden row of token perm[r] / k
@@ -656,9 +649,9 @@ tile_list_kernel(const int32_t* __restrict__ counts, const int32_t* __restrict__
 __global__ void __launch_bounds__(256)
 gather_rows_kernel(const __nv_bfloat16* __restrict__ hidden, const int32_t* __restrict__ perm,
                    const int32_t* __restrict__ n_valid, int top_k, int H, __nv_bfloat16* __restrict__ xg,
-                   const int32_t* __restrict__ counts, const int32_t* __restrict__ group_keys,
-                   const int32_t* __restrict__ wave_start, Tile* __restrict__ tiles, int32_t* __restrict__ n_tiles, int bn) {
-    if (blockIdx.x == 0 && tiles) build_tile_list(counts, group_keys, wave_start, tiles, n_tiles, bn);
+                   const int32_t* __restrict__ counts, const int32_t* __restrict__ offsets, const int32_t* __restrict__ group_keys,
+                   const int32_t* __restrict__ wave_start, Tile* __restrict__ tiles, int32_t* __restrict__ n_tiles, int bn, bool k_order) {
+    if (blockIdx.x == 0 && tiles) build_tile_list(counts, offsets, group_keys, wave_start, tiles, n_tiles, bn);
     // one warp per row, eight rows per CTA; a lane keeps up to eight 16-byte loads in flight before it stores
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r = blockIdx.x * 8 + warp;
@@ -679,7 +672,8 @@ gather_rows_kernel(const __nv_bfloat16* __restrict__ hidden, const int32_t* __re
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const int i = base + lane + 32 * j;
-            if (i < n16) dst[i] = v[j];
+            const uint4 o = ordered_chunk(v[j], lane, k_order);
+            if (i < n16) dst[i] = o;
         }
     }
 }
@@ -696,7 +690,7 @@ static_assert(kPlanGatherPairs < 65536, "two counts in one word");
 __global__ void __launch_bounds__(kPlanThreads)
 plan_gather_kernel(const __nv_bfloat16* __restrict__ hidden, const int32_t* __restrict__ ids, int n_pairs, int top_k, int H, int E,
                    int C, int n_keys, int max_waves, bool identity, int seg, PlanPtrs plan, int* __restrict__ status,
-                   __nv_bfloat16* __restrict__ xg, Tile* __restrict__ tiles, int32_t* __restrict__ n_tiles, int bn) {
+                   __nv_bfloat16* __restrict__ xg, Tile* __restrict__ tiles, int32_t* __restrict__ n_tiles, int bn, bool k_order) {
     extern __shared__ __align__(16) int s_int[];
     int* s_cnt = s_int;                    // [n_keys]: pairs of the key | those before the segment << 16
     int* s_off = s_cnt + n_keys;           // [n_keys + 1]
@@ -737,7 +731,7 @@ plan_gather_kernel(const __nv_bfloat16* __restrict__ hidden, const int32_t* __re
             plan.header[HDR_BAD_ID] = 0;
         }
         __syncthreads();
-        if (tiles) build_tile_list(plan.counts, plan.group_keys, plan.wave_start, tiles, n_tiles, bn);
+        if (tiles) build_tile_list(plan.counts, plan.offsets, plan.group_keys, plan.wave_start, tiles, n_tiles, bn);
         return;
     }
     if (warp == 0) {                       // place of the segment's first pair of every key
@@ -764,12 +758,15 @@ plan_gather_kernel(const __nv_bfloat16* __restrict__ hidden, const int32_t* __re
         for (int j = lane; j < i; j += 32) before += s_key[j] == key;
         const int pos = s_off[key] + (int)__reduce_add_sync(0xffffffffu, (unsigned)before);
         if (lane == 0) plan.perm[pos] = start + i;
-        uint4* dst = reinterpret_cast<uint4*>(xg + (size_t)pos * H) + lane;
+        uint4* dst = reinterpret_cast<uint4*>(xg + (size_t)pos * H);
         for (int base = 0; base < n16; base += 256) {
             if (i != warp || base) load(i, base);
 #pragma unroll
             for (int j = 0; j < 8; ++j)
-                if (base + lane + 32 * j < n16) dst[base + 32 * j] = v[j];
+                if (base + 32 * j < n16) {             // the same for the whole warp
+                    const uint4 o = ordered_chunk(v[j], lane, k_order);
+                    if (base + lane + 32 * j < n16) dst[base + lane + 32 * j] = o;
+                }
         }
     }
 }
@@ -808,22 +805,27 @@ static int sm_count() {
 // end is one tile's epilogue, which takes time by its columns.  512 x 256, 16 experts, 300 tokens: 32.2 -> 26.9 us per layer,
 // 256 x 128, 8 experts, 600 tokens: 26.4 -> 20.6 us; with more tiles than SMs it lost (2048 x 1536, 8 experts, 200 tokens:
 // 57 -> 65 us).
-int prefill_tile_rows(const exmoe_shape& s, int n_pairs, int experts_per_wave, bool small_n) {
+int prefill_tile_rows(const exmoe_shape& s, int n_pairs, int experts_per_wave, int kind) {
     const int mt = std::min(2 * s.d_ff, s.d_model) / BM, sms = sm_count();
-    int rows = small_n ? BN_SMALL : BN;
+    int rows = kind == TC_LARGE ? BN : BN_SMALL;
     while (rows > BN_SMALL && 2 * std::max(std::min(n_pairs, experts_per_wave), n_pairs / rows) * mt <= sms) rows /= 2;
     return rows;
 }
 
+bool tc_stream_takes(const exmoe_shape& s, int n_pairs) {
+    const long long blocks = (long long)s.num_experts * (2 * s.d_ff / BM) * (s.d_model / BK);
+    return n_pairs <= kTcStreamMaxRows * s.num_experts && s.d_model >= kTcStreamMinModel && blocks >= (long long)kTcStreamMinBlocksPerSm * sm_count();
+}
+
 void launch_plan_gather(const exmoe_shape& s, int C, int n_keys, int max_waves, bool identity, const __nv_bfloat16* hidden,
                         const int32_t* ids, int n_pairs, PlanPtrs plan, int* status, __nv_bfloat16* xg, bool single_wave,
-                        void* scratch, int tile_rows, cudaStream_t st) {
+                        void* scratch, int tile_rows, bool k_order, cudaStream_t st) {
     const int sms = sm_count(), seg = (n_pairs + sms - 1) / sms, n_seg = (n_pairs + seg - 1) / seg;
     int32_t* n_tiles = reinterpret_cast<int32_t*>(scratch);
     Tile* tiles = single_wave ? reinterpret_cast<Tile*>(reinterpret_cast<unsigned char*>(scratch) + 256) : nullptr;
     launch_dependent(plan_gather_kernel, n_seg + 1, kPlanThreads, (size_t)(2 * n_keys + 1 + seg) * 4, st, hidden, ids, n_pairs,
                      s.top_k, s.d_model, s.num_experts, C, n_keys, max_waves, identity, seg, plan, status, xg, tiles, n_tiles,
-                     tile_rows);
+                     tile_rows, k_order);
 }
 
 size_t prefill_scratch_bytes(int max_pairs, int num_experts) {
@@ -873,18 +875,19 @@ void launch_wait_selftest(int* status, long long budget_cycles, int* result, cud
 
 void launch_gather_rows(const __nv_bfloat16* hidden, const int32_t* perm, const int32_t* n_valid, int n_pairs, int top_k,
                         int H, __nv_bfloat16* xg, const GemmArgs* single_wave, const int32_t* wave_start, void* scratch,
-                        int tile_rows, cudaStream_t st) {
+                        int tile_rows, bool k_order, cudaStream_t st) {
     int32_t* n_tiles = reinterpret_cast<int32_t*>(scratch);
     Tile* tiles = single_wave ? reinterpret_cast<Tile*>(reinterpret_cast<unsigned char*>(scratch) + 256) : nullptr;
     gather_rows_kernel<<<(n_pairs + 7) / 8, 256, 0, st>>>(hidden, perm, n_valid, top_k, H, xg, single_wave ? single_wave->counts : nullptr,
+                                                 single_wave ? single_wave->offsets : nullptr,
                                                  single_wave ? single_wave->group_keys : nullptr, wave_start, tiles, n_tiles,
-                                                 tile_rows);
+                                                 tile_rows, k_order);
     count_launch();
 }
 
 // One wave of the tensor-core path: tile list, gate/up GEMM + SwiGLU, down GEMM x routing weight.
 void launch_prefill_wave(const GemmArgs& g, const int32_t* wave_start, void* scratch, int* status, const PrefillMaps* maps,
-                         __nv_bfloat16* act, const float* topk_w, float* y, int which, bool small_n, int tile_rows, cudaStream_t st) {
+                         __nv_bfloat16* act, const float* topk_w, float* y, int which, int kind, int tile_rows, cudaStream_t st) {
     int32_t* n_tiles = reinterpret_cast<int32_t*>(scratch);
     Tile* tiles = reinterpret_cast<Tile*>(reinterpret_cast<unsigned char*>(scratch) + 256);
     PrefillArgs a{};
@@ -910,20 +913,25 @@ void launch_prefill_wave(const GemmArgs& g, const int32_t* wave_start, void* scr
     const CUtensorMap* mx = reinterpret_cast<const CUtensorMap*>(maps->dev);
     const CUtensorMap* ma = mx + N_MAPS;
     if (which & 4) {
-        tile_list_kernel<<<1, 1024, 0, st>>>(g.counts, g.group_keys, wave_start, tiles, n_tiles, tile_rows);
+        tile_list_kernel<<<1, 1024, 0, st>>>(g.counts, g.offsets, g.group_keys, wave_start, tiles, n_tiles, tile_rows);
         count_launch();
     }
+    if (kind == TC_STREAM) {
+        launch_tc_stream_wave(g, tiles, g.n_pairs / 16 + g.num_slots + 16, n_tiles, status, maps, act, topk_w, y, which & 1, which & 2, st);
+        return;
+    }
+    const bool small_n = kind == TC_SMALL_N;
     if (which & 1) {
         if (small_n)
-            launch_dependent(prefill_gemm_kernel<true, BN_SMALL, kStagesSmall>, sms, NUM_THREADS, smem_small, st, a, mx, act, (const float*)nullptr, (const int32_t*)g.offsets, (float*)nullptr);
+            launch_dependent(prefill_gemm_kernel<true, BN_SMALL, kStagesSmall>, sms, NUM_THREADS, smem_small, st, a, mx, act, (const float*)nullptr, (float*)nullptr);
         else
-            launch_dependent(prefill_gemm_kernel<true, BN, kStagesLarge>, sms, NUM_THREADS, smem_large, st, a, mx, act, (const float*)nullptr, (const int32_t*)g.offsets, (float*)nullptr);
+            launch_dependent(prefill_gemm_kernel<true, BN, kStagesLarge>, sms, NUM_THREADS, smem_large, st, a, mx, act, (const float*)nullptr, (float*)nullptr);
     }
     if (which & 2) {
         if (small_n)
-            launch_dependent(prefill_gemm_kernel<false, BN_SMALL, kStagesSmall>, sms, NUM_THREADS, smem_small, st, a, ma, (__nv_bfloat16*)nullptr, topk_w, (const int32_t*)g.offsets, y);
+            launch_dependent(prefill_gemm_kernel<false, BN_SMALL, kStagesSmall>, sms, NUM_THREADS, smem_small, st, a, ma, (__nv_bfloat16*)nullptr, topk_w, y);
         else
-            launch_dependent(prefill_gemm_kernel<false, BN, kStagesLarge>, sms, NUM_THREADS, smem_large, st, a, ma, (__nv_bfloat16*)nullptr, topk_w, (const int32_t*)g.offsets, y);
+            launch_dependent(prefill_gemm_kernel<false, BN, kStagesLarge>, sms, NUM_THREADS, smem_large, st, a, ma, (__nv_bfloat16*)nullptr, topk_w, y);
     }
 }
 

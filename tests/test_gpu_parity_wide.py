@@ -477,3 +477,32 @@ def test_reading_the_plan_leaves_the_status_alone(B, T):
     assert cache.last_plan(0, ids.numel())["counts"].sum() == T * s.top_k - 1
     assert cache.status() == 0
     cache.close()
+
+
+def test_streaming_tensor_core_kernels_at_tile_edges(B):
+    """Groups of 1 to 129 rows (tiles of 64, their remainders and 16-row steps) on odd numbers of K blocks (17 and 11) and of
+    weight tiles (17): the first and last rows of every token tile against the oracle, and the same bits in waves of 20 experts."""
+    s = synth.Shape(d_model=2176, d_ff=1408, num_experts=48, top_k=1)
+    ora, bank = helpers.make_layer(s, seed=4100)
+    sizes = [1, 15, 16, 17, 31, 32, 33, 47, 48, 49, 63, 64, 65, 80, 127, 128, 129, 2]
+    ids = torch.tensor([[(5 * e + 3) % 48] for e, n in enumerate(sizes) for _ in range(n)], dtype=torch.int32)
+    T = ids.shape[0]
+    ids = ids[torch.randperm(T, generator=torch.Generator().manual_seed(1))].contiguous()
+    hidden = synth.hidden_states(s, T, seed=4200)
+    p = torch.rand((T, 1), generator=torch.Generator().manual_seed(2)) + 0.5
+    cache = B.Cache(s, [bank], 48, max_tokens=T)
+    out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    assert cache.last_path() == B.PATH_TENSOR_SMALL_N and cache.status() == 0
+    sample = set()
+    for e in range(48):
+        rows = (ids[:, 0] == e).nonzero()[:, 0].tolist()
+        for n0 in tile_rows(len(rows), 64) if rows else []:
+            sample.update(rows[i] for i in (n0 - 1, n0, len(rows) - 1) if i >= 0)
+    sample = sorted(sample)
+    y, ref = ora.forward(hidden[sample], ids[sample], p[sample])
+    helpers.check_output(out[sample], y, ref, f"{len(sample)} tokens")
+    cache.close()
+    part = B.Cache(s, [bank], 20, max_tokens=T)
+    again = part.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    assert torch.equal(out.view(torch.int16), again.view(torch.int16)) and part.status() == 0
+    part.close()
