@@ -29,7 +29,7 @@ constexpr int kRouteThreads = 256;
 constexpr int kRouteSmemMax = 200 * 1024;
 constexpr int kRouteFewTokens = 48;       // several tokens per cluster from here on
 constexpr int kRouteTokenTokens = 192;    // one CTA per token, few experts, from here on
-constexpr int kRouteMmaTokens = 224;      // tensor cores from here on
+constexpr int kRouteMmaTokens = 193;      // tensor cores from here on
 constexpr int kRouteWideTokens = 1152;    // ... with 32 instead of 16 experts per CTA
 constexpr int kRouteWarps = kRouteThreads / 32;
 
@@ -325,45 +325,92 @@ constexpr float kExpSubnormal = 85.f, kExpZero = 106.f;    // expf(-x): normal b
 constexpr int kMmaMaxModel = 4096;                    // |x|^2 and |w|^2 are summed in BF16 over H / 64 terms per lane
 __device__ __forceinline__ float route_bound(int H) { return 1.14f * (0x1p-20f + (float)(21 + 3 * H / 512) * 0x1p-24f); }
 
-// Binary32 logits of the experts marked in `again` (bit i of a lane: expert lane + 32 i), by one warp.
-__device__ __noinline__ void logits_again(float* z, unsigned again, const __nv_bfloat16* __restrict__ x,
-                                          const __nv_bfloat16* __restrict__ w_router, const float* __restrict__ bias, int H,
-                                          int lane) {
-    const uint4* xr = reinterpret_cast<const uint4*>(x);
-    for (int i = 0; i < kMmaMaxExperts / 32; ++i)
-        for (unsigned todo = __ballot_sync(0xffffffffu, (again >> i) & 1u); todo; todo &= todo - 1) {
-            const int e = 32 * i + __ffs(todo) - 1;
-            const uint4* wr = reinterpret_cast<const uint4*>(w_router + (size_t)e * H);
-            float s = 0.f;
-            for (int j0 = 0; j0 < H / 8; j0 += 256) {
-                uint4 wv[8];
+// Binary32 logit of one expert, by one warp.
+__device__ __noinline__ float logit_again(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ w, int H, int lane) {
+    const uint4 *xr = reinterpret_cast<const uint4*>(x), *wr = reinterpret_cast<const uint4*>(w);
+    float s = 0.f;
+    for (int j0 = 0; j0 < H / 8; j0 += 256) {
+        uint4 wv[8], xv[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (j0 + 32 * j + lane < H / 8) wv[j] = wr[j0 + 32 * j + lane];
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (j0 + 32 * j + lane < H / 8) {
-                        float wf[8], xf[8];
-                        unpack8(wv[j], wf);
-                        unpack8(xr[j0 + 32 * j + lane], xf);
-                        s += dot8(wf, xf);
-                    }
+        for (int j = 0; j < 8; ++j)
+            if (j0 + 32 * j + lane < H / 8) {
+                wv[j] = wr[j0 + 32 * j + lane];
+                xv[j] = xr[j0 + 32 * j + lane];
             }
-            s = warp_sum(s);
-            if (lane == 0) z[e] = s + (bias ? bias[e] : 0.f);
-        }
-    __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (j0 + 32 * j + lane < H / 8) {
+                float wf[8], xf[8];
+                unpack8(wv[j], wf);
+                unpack8(xv[j], xf);
+                s += dot8(wf, xf);
+            }
+    }
+    return warp_sum(s);
 }
+// softmax_topk for at most kMmaMaxExperts experts and 32 choices: the same arithmetic and order, keys in registers, one store at the end
+// (2.4 -> 1.0 us in a call's tail).
+__device__ __forceinline__ void softmax_topk_few(const float* z, int E, int k, int lane, int32_t* __restrict__ ids, float* __restrict__ wts) {
+    constexpr int PER = kMmaMaxExperts / 32;
+    float mx = -INFINITY, v[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+        if (lane + 32 * i < E) mx = fmaxf(mx, z[lane + 32 * i]);
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, m));
+    float sum = 0.f;
+    uint32_t key[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        key[i] = 0;
+        v[i] = 0.f;
+        if (lane + 32 * i < E) {
+            v[i] = expf(z[lane + 32 * i] - mx);
+            key[i] = v[i] >= 0.f ? __float_as_uint(v[i]) + 2u : 1u;        // 1: a NaN, chosen last
+            sum += v[i];
+        }
+    }
+    const float inv = 1.f / warp_sum(sum);
+    int mine = 0;
+    float weight = 0.f;
+    for (int j = 0; j < k; ++j) {
+        uint32_t best = 0;
+        int at = 0;
+        float p = 0.f;
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (key[i] > best) {                                           // ascending experts: the first maximum wins
+                best = key[i];
+                at = i;
+                p = v[i];
+            }
+        const uint32_t top = __reduce_max_sync(0xffffffffu, best);
+        const int e = (int)__reduce_min_sync(0xffffffffu, best == top ? (unsigned)(lane + 32 * at) : 0x7fffffffu);
+        p = __shfl_sync(0xffffffffu, p, e & 31);
+        if (j == lane) {
+            mine = e;
+            weight = p * inv;
+        }
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (lane + 32 * i == e) key[i] = 0;
+    }
+    if (lane < k) {
+        ids[lane] = mine;
+        wts[lane] = weight;
+    }
+}
+
 // One token's choice from its tensor-core logits, by one warp: the k + 1 largest in order; where two of them are within
 // `slack`, both are recomputed (at the cut everything that could displace the k-th) and the choice is made again.  A lane
-// holds the logits of experts lane, lane + 32, ... as order-preserving integers.
+// holds the logits of experts lane, lane + 32, ... as order-preserving integers.  What is to be recomputed is left in `todo` (a bit
+// per expert) for the whole CTA, and true returned.
 // The other forms order binary32 PROBABILITIES, equal ones by id, and so does the choice made again.  Two logits may share a
 // probability where they differ: closer than expf resolves (its argument z - max is rounded to 2^-24 of itself, the
 // result to a few units of 2^-23), or far enough below the largest that their probabilities are subnormal or zero.  So
 // the first enters `near`, and a choice that reaches the second is made again in any case, with those logits recomputed
 // whose probability is subnormal; the exponential of anything below them is zero in every form.
-__device__ __forceinline__ void choose(float* z, float slack, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ w_router,
-                                       const float* __restrict__ bias, int H, int E, int k, int lane, int32_t* __restrict__ ids,
+__device__ __forceinline__ bool choose(const float* z, float slack, int E, int k, int lane, uint32_t* todo, int32_t* __restrict__ ids,
                                        float* __restrict__ wts) {
     constexpr int PER = kMmaMaxExperts / 32;
     uint32_t key[PER];                                                     // 0: no expert, or taken
@@ -428,9 +475,12 @@ __device__ __forceinline__ void choose(float* z, float slack, const __nv_bfloat1
     }
     if (deep || __any_sync(0xffffffffu, again != 0)) {
         if (lane == (first_e & 31)) again |= 1u << (first_e >> 5);         // the maximum, from which expf's arguments are measured
-        logits_again(z, again, x, w_router, bias, H, lane);
-        softmax_topk(z, E, k, lane, ids, wts);
-        return;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const unsigned b = __ballot_sync(0xffffffffu, (again >> i) & 1u);
+            if (lane == 0) todo[i] = b;
+        }
+        return true;
     }
     const float mx = __shfl_sync(0xffffffffu, z[mine], 0);
     float sum = 0.f;
@@ -440,6 +490,7 @@ __device__ __forceinline__ void choose(float* z, float slack, const __nv_bfloat1
         ids[lane] = mine;
         wts[lane] = expf(z[mine] - mx) / sum;
     }
+    return false;
 }
 
 // 16 tokens per CTA; NT: 8-expert tiles per CTA; CL: CTAs per cluster (CL * NT = 8: 64 experts per pass); U: steps of loads in
@@ -581,14 +632,42 @@ route_mma_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* 
     float wmax = 0.f;
 #pragma unroll
     for (int r = 0; r < 2 * CL; ++r) wmax = fmaxf(wmax, wmax_of[r]);
+    static_assert(TOK <= 32, "a bit per token");
+    __shared__ uint32_t todo[TOK][kMmaMaxExperts / 32];
+    unsigned again = 0;                                                    // this warp's tokens that are chosen again
     for (int i = warp; i * CL + rank < n_tok; i += kRouteWarps) {
         const int t = i * CL + rank;
         float x2 = 0.f;
 #pragma unroll
         for (int w = 0; w < kRouteWarps; ++w) x2 += xn[w * TM + t];
         // of a pair both may be off; the bias addition rounds once more (relative to the logit)
-        choose(logit + i * kMmaMaxExperts, 2.f * route_bound(H) * sqrtf(x2) * sqrtf(wmax), hidden + (size_t)(t0 + t) * H, w_router, bias,
-               H, E, k, lane, ids_out + (size_t)(t0 + t) * k, w_out + (size_t)(t0 + t) * k);
+        if (choose(logit + i * kMmaMaxExperts, 2.f * route_bound(H) * sqrtf(x2) * sqrtf(wmax), E, k, lane, todo[i], ids_out + (size_t)(t0 + t) * k,
+                   w_out + (size_t)(t0 + t) * k))
+            again |= 1u << i;
+    }
+    // One token in fifty is chosen again (64 experts of 2048), so every call of some size has one, and it is the call's tail: its
+    // logits are spread over all warps, and its choice keeps its keys in registers: 333 tokens 12.0 -> 9.8 -> 8.3 us, 2048 17.2 -> 15.6 -> 14.1.
+    if (!__syncthreads_or(again != 0)) return;
+    __shared__ unsigned flagged;
+    if (tid == 0) flagged = 0;
+    __syncthreads();
+    if (lane == 0 && again) atomicOr(&flagged, again);
+    __syncthreads();
+    int item = 0;
+    for (unsigned toks = flagged; toks; toks &= toks - 1) {
+        const int i = __ffs(toks) - 1;
+        for (int b = 0; b < kMmaMaxExperts / 32; ++b)
+            for (unsigned es = todo[i][b]; es; es &= es - 1, ++item) {
+                if (item % kRouteWarps != warp) continue;
+                const int e = 32 * b + __ffs(es) - 1;
+                const float v = logit_again(hidden + (size_t)(t0 + i * CL + rank) * H, w_router + (size_t)e * H, H, lane);
+                if (lane == 0) logit[i * kMmaMaxExperts + e] = v + (bias ? bias[e] : 0.f);
+            }
+    }
+    __syncthreads();
+    for (; again; again &= again - 1) {
+        const int i = __ffs(again) - 1, t = i * CL + rank;
+        softmax_topk_few(logit + i * kMmaMaxExperts, E, k, lane, ids_out + (size_t)(t0 + t) * k, w_out + (size_t)(t0 + t) * k);
     }
 }
 
@@ -607,7 +686,7 @@ int launch_route_mma(const exmoe_shape& s, const __nv_bfloat16* hidden, const __
 // matrix, by clusters of eight, or of four where these have a warp per expert or the calls are large; with few experts one
 // CTA per token; then the tensor cores.  us, replayed from a graph, in the order one / four / four narrow / token / tensor
 // cores (16 experts per CTA / 32):
-//   64 experts, d_model 2048:  32 tokens 5.1 / 4.9 / - / - / 5.8         64: - / 5.4 / 6.5 / - / 5.7     224: - / 10.0 / 10.9 / - / 10.6
+//   64 experts, d_model 2048:  32 tokens 5.1 / 4.9 / - / - / 5.8         64: - / 5.1 / 6.5 / - / 6.8     192: - / 7.7 / - / - / 7.7     208: - / 9.1 / 10.9 / - / 7.8
 //   16 experts, d_model 512:   64 tokens 5.2 / 3.5 / 3.3 / 3.9 / 6.8    223: - / 5.7 / 4.1 / 4.1 / 7.0   800: - / 13 / 7.4 / 4.7 / 7.8 / 7.7
 //   16 experts, d_model 2048: 128 tokens 9.5 / 7.0 / 4.6 / 5.1 / 9.6    300: - / 9.8 / 7.3 / 5.4 / 9.7   900: - / 22 / 14 / 12 / 11 / 11
 //   8 experts, d_model 256:    64 tokens 5.0 / 3.3 / 3.2 / 2.7 / 3.8   1024: - / 14 / 9.1 / 4.9 / 6.7 / 6.7   2048: - / 26 / 15 / 6.8 / 8.4 / 7.4
@@ -628,7 +707,7 @@ constexpr RouteForm route_form(int E, int H, int k, int T) {
     return four ? (T >= 512 ? RouteForm::FourNarrow : RouteForm::Four) : RouteForm::One;
 }
 static_assert(route_form(64, 2048, 8, 47) == RouteForm::One && route_form(64, 2048, 8, 48) == RouteForm::Four);
-static_assert(route_form(64, 2048, 8, 223) == RouteForm::Four && route_form(64, 2048, 8, 224) == RouteForm::Mma);
+static_assert(route_form(64, 2048, 8, 192) == RouteForm::Four && route_form(64, 2048, 8, 193) == RouteForm::Mma);
 static_assert(route_form(64, 2048, 8, 1152) == RouteForm::MmaWide && route_form(16, 512, 4, 896) == RouteForm::Mma);
 static_assert(route_form(16, 512, 4, 191) == RouteForm::FourNarrow && route_form(16, 512, 4, 192) == RouteForm::Token);
 static_assert(route_form(16, 512, 4, 895) == RouteForm::Token && route_form(8, 256, 2, 48) == RouteForm::Token);
