@@ -1189,7 +1189,7 @@ void launch_decode(const GemmArgs& a, const SmallArgs& sa, const __nv_bfloat16* 
 // 8192 tokens 25.8 and 101.5 us before, 28.6 and 119 with eight, 24.2 and 90.6 (6.3 TB/s) with four.
 template <int AHEAD>
 __global__ void __launch_bounds__(256)
-combine_kernel(const float* __restrict__ y, const int32_t* __restrict__ ids, int E, int T, int k, int H,
+combine_kernel(const float* y, const int32_t* __restrict__ ids, int E, int T, int k, int H,
                __nv_bfloat16* __restrict__ out) {
     grid_launch_dependents();                          // the next kernel in the stream may be placed (it waits for this one)
     const int per_row = H / 4;
@@ -1215,7 +1215,7 @@ combine_kernel(const float* __restrict__ y, const int32_t* __restrict__ ids, int
         float4 v[AHEAD];
 #pragma unroll
         for (int j = 0; j < AHEAD; ++j)
-            if (valid[j]) v[j] = *(row + (size_t)(j0 + j) * per_row);
+            if (valid[j]) v[j] = load_behind_wait(row + (size_t)(j0 + j) * per_row);
 #pragma unroll
         for (int j = 0; j < AHEAD; ++j)
             if (valid[j]) {

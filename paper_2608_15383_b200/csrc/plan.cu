@@ -3,6 +3,7 @@
 // exclusive prefix sum and stable permutation of token-expert pairs (the grouping step of Figure 1's caption).
 // Integer work only; every result is deterministic and bit-exact.
 #include "common.cuh"
+#include "frag.cuh"
 #include "plan.cuh"
 
 namespace exmoe {
@@ -370,15 +371,17 @@ constexpr int kChunk = 512;
 #endif
 
 __global__ void __launch_bounds__(kChunk)
-group_chunk_count_kernel(const int32_t* __restrict__ ids, int n_pairs, int E, int C, int n_keys, int max_waves,
-                         bool identity, PlanPtrs plan, int32_t* __restrict__ table, int32_t* __restrict__ done,
-                         int* __restrict__ status) {
+group_chunk_count_kernel(const int32_t* ids, int n_pairs, int E, int C, int n_keys, int max_waves,
+                         bool identity, PlanPtrs plan, int32_t* table, int32_t* done,
+                         int* status) {
     extern __shared__ __align__(16) int s_hist[];          // [n_keys] (+ [n_keys + 1] scratch offsets for the last CTA)
     __shared__ int s_last, s_bad;
     const int tid = threadIdx.x, chunk = blockIdx.x, n_chunks = gridDim.x;
     if (tid == 0) s_bad = 0;
     for (int i = tid; i < n_keys; i += kChunk) s_hist[i] = 0;
     __syncthreads();
+    grid_dependency_wait();
+    grid_launch_dependents();
     const int p = chunk * kChunk + tid;
     if (p < n_pairs) {
         const int key = pair_key(ids[p], E, C, identity, plan.wave_of, plan.slot_of);
@@ -388,7 +391,7 @@ group_chunk_count_kernel(const int32_t* __restrict__ ids, int n_pairs, int E, in
     __syncthreads();
     for (int i = tid; i < n_keys; i += kChunk) table[(size_t)i * n_chunks + chunk] = s_hist[i];
     if (tid == 0 && s_bad) {
-        plan.header[HDR_BAD_ID] = 1;
+        atomicOr(done + 1, 1);
         atomicExch(status, EXMOE_ERR_BAD_EXPERT_ID);
     }
     __threadfence();
@@ -397,7 +400,11 @@ group_chunk_count_kernel(const int32_t* __restrict__ ids, int n_pairs, int E, in
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    if (tid == 0) *done = 0;                               // ready for the next call
+    if (tid == 0) {
+        const int bad = __ldcg(done + 1);
+        if (identity || bad) plan.header[HDR_BAD_ID] = bad;    // with fewer slots the resolution kernel has set the word
+        done[0] = done[1] = 0;                             // ready for the next call
+    }
     // totals per key -> plan.counts (one warp per key, lanes over chunks); warp 0 then scans the keys
     const int lane = tid & 31, warp = tid >> 5;
     for (int i = warp; i < n_keys; i += kChunk / 32) {
@@ -432,11 +439,13 @@ group_chunk_count_kernel(const int32_t* __restrict__ ids, int n_pairs, int E, in
 }
 
 __global__ void __launch_bounds__(kChunk)
-group_chunk_scatter_kernel(const int32_t* __restrict__ ids, int n_pairs, int E, int C, int n_keys, bool identity,
-                           PlanPtrs plan, const int32_t* __restrict__ table) {
+group_chunk_scatter_kernel(const int32_t* ids, int n_pairs, int E, int C, int n_keys, bool identity,
+                           PlanPtrs plan, const int32_t* table) {
     extern __shared__ __align__(16) int s_cur[];           // [n_keys] pairs of this chunk already placed, per key
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, chunk = blockIdx.x, n_chunks = gridDim.x;
     for (int i = tid; i < n_keys; i += kChunk) s_cur[i] = 0;
+    grid_dependency_wait();
+    grid_launch_dependents();
     const int p = chunk * kChunk + tid;
     int key = -1;
     if (p < n_pairs) key = pair_key(ids[p], E, C, identity, plan.wave_of, plan.slot_of);
@@ -482,11 +491,24 @@ void launch_group(const exmoe_shape& s, int C, int n_keys, int max_waves, bool i
     }
     const int n_chunks = (n_pairs + kChunk - 1) / kChunk;
     if (plan.chunk_table && (size_t)n_keys * n_chunks <= plan.chunk_table_words && n_keys <= 5000) {
-        if (identity) cudaMemsetAsync(plan.header + HDR_BAD_ID, 0, 4, st);
-        group_chunk_count_kernel<<<n_chunks, kChunk, (size_t)(2 * n_keys + 1) * 4, st>>>(
-            ids, n_pairs, E, C, n_keys, max_waves, identity, plan, plan.chunk_table, plan.chunk_done, d_status);
-        group_chunk_scatter_kernel<<<n_chunks, kChunk, (size_t)n_keys * 4, st>>>(ids, n_pairs, E, C, n_keys, identity, plan,
-                                                                               plan.chunk_table);
+        // programmatic dependents, each of the kernel before it (16384 pairs: XXX)
+        cudaLaunchConfig_t lc{};
+        lc.gridDim = dim3((unsigned)n_chunks);
+        lc.blockDim = dim3(kChunk);
+        lc.dynamicSmemBytes = (size_t)(2 * n_keys + 1) * 4;
+        lc.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        lc.attrs = attr;
+        lc.numAttrs = 1;
+#ifdef EXMOE_DISABLE_PDL
+        lc.numAttrs = 0;
+#endif
+        cudaLaunchKernelEx(&lc, group_chunk_count_kernel, ids, n_pairs, E, C, n_keys, max_waves, identity, plan, plan.chunk_table, plan.chunk_done,
+                           d_status);
+        lc.dynamicSmemBytes = (size_t)n_keys * 4;
+        cudaLaunchKernelEx(&lc, group_chunk_scatter_kernel, ids, n_pairs, E, C, n_keys, identity, plan, (const int32_t*)plan.chunk_table);
         count_launch(2);
         return;
     }

@@ -56,7 +56,9 @@ __device__ __forceinline__ void scan_keys_warp0(const int32_t* cnt, int n_keys, 
     __syncwarp();
     for (int w = lane; w <= max_waves; w += 32) {          // wave_start[w] = #active keys below w*C
         int c = 0;
-        for (int g = 0; g < ng; ++g) c += (plan.group_keys[g] < w * C);
+        if (w * C >= n_keys) c = ng;                       // a single wave: nothing to read back
+        else
+            for (int g = 0; g < (w ? ng : 0); ++g) c += (plan.group_keys[g] < w * C);
         plan.wave_start[w] = c;
     }
 }

@@ -561,24 +561,25 @@ __global__ void wait_timeout_selftest_kernel(int* status, long long budget, int*
 }
 
 // n-tiles of one wave: every active group is cut into balanced runs of at most `bn` grouped rows (multiples of 16).
-// With each tile goes the weight of those before it (tile_weight).  Executed by one whole CTA (any multiple of 32 threads up to 1024): thread g handles group g, an exclusive scan of
-// the piece counts places its tiles.
-__device__ void build_tile_list(const int32_t* __restrict__ counts, const int32_t* __restrict__ offsets, const int32_t* __restrict__ group_keys,
-                                const int32_t* __restrict__ wave_start, Tile* __restrict__ tiles,
-                                int32_t* __restrict__ n_tiles, int bn) {
+// With each tile goes the weight of those before it (tile_weight).  Executed by one whole CTA (any multiple of 32 threads up to 1024):
+// thread g handles group g, an exclusive scan of the piece counts places its tiles.  Without `group_keys` the groups are the keys
+// themselves, empty ones among them (the plan of a single wave, from the counts and offsets in shared memory).
+__device__ void build_tile_list(const int32_t* counts, const int32_t* offsets, const int32_t* group_keys, int g0, int ng,
+                                Tile* tiles, int32_t* n_tiles, int bn) {
     __shared__ int s_warp[32], s_weight[32];
     __shared__ int s_running, s_running_w;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x, nwarp = nthr >> 5;
-    const int g0 = wave_start[0], ng = wave_start[1] - g0;
     if (tid == 0) s_running = s_running_w = 0;
     __syncthreads();
     for (int base = 0; base < ng; base += nthr) {
         const int g = base + tid;
         int key = 0, cnt = 0, row0 = 0, pieces = 0, per = 0;
         if (g < ng) {
-            key = group_keys[g0 + g];
+            key = group_keys ? group_keys[g0 + g] : g;
             cnt = counts[key];
             row0 = offsets[key];
+        }
+        if (cnt > 0) {
             pieces = (cnt + bn - 1) / bn;
             per = ((cnt + pieces - 1) / pieces + 15) & ~15;
             pieces = (cnt + per - 1) / per;
@@ -626,9 +627,9 @@ __device__ void build_tile_list(const int32_t* __restrict__ counts, const int32_
 }
 
 __global__ void __launch_bounds__(1024)
-tile_list_kernel(const int32_t* __restrict__ counts, const int32_t* __restrict__ offsets, const int32_t* __restrict__ group_keys,
-                 const int32_t* __restrict__ wave_start, Tile* __restrict__ tiles, int32_t* __restrict__ n_tiles, int bn) {
-    build_tile_list(counts, offsets, group_keys, wave_start, tiles, n_tiles, bn);
+tile_list_kernel(const int32_t* counts, const int32_t* offsets, const int32_t* group_keys,
+                 const int32_t* wave_start, Tile* tiles, int32_t* n_tiles, int bn) {
+    build_tile_list(counts, offsets, group_keys, wave_start[0], wave_start[1] - wave_start[0], tiles, n_tiles, bn);
 }
 
 // 16-byte chunk of a row, by its place in the row's order or in the K order of the kernels whose weights are in tensor memory
@@ -647,11 +648,13 @@ __device__ __forceinline__ uint4 ordered_chunk(uint4 v, int lane, bool k_order) 
 // grouped copy of the hidden states: row r of the plan order = hidden row of token perm[r] / k
 // CTA 0 also builds the tile list of the call's only wave when `tiles` is given (one launch less).
 __global__ void __launch_bounds__(256)
-gather_rows_kernel(const __nv_bfloat16* __restrict__ hidden, const int32_t* __restrict__ perm,
-                   const int32_t* __restrict__ n_valid, int top_k, int H, __nv_bfloat16* __restrict__ xg,
-                   const int32_t* __restrict__ counts, const int32_t* __restrict__ offsets, const int32_t* __restrict__ group_keys,
-                   const int32_t* __restrict__ wave_start, Tile* __restrict__ tiles, int32_t* __restrict__ n_tiles, int bn, bool k_order) {
-    if (blockIdx.x == 0 && tiles) build_tile_list(counts, offsets, group_keys, wave_start, tiles, n_tiles, bn);
+gather_rows_kernel(const __nv_bfloat16* hidden, const int32_t* perm,
+                   const int32_t* n_valid, int top_k, int H, __nv_bfloat16* xg,
+                   const int32_t* counts, const int32_t* offsets, const int32_t* group_keys,
+                   const int32_t* wave_start, Tile* tiles, int32_t* n_tiles, int bn, bool k_order) {
+    grid_dependency_wait();
+    grid_launch_dependents();
+    if (blockIdx.x == 0 && tiles) build_tile_list(counts, offsets, group_keys, wave_start[0], wave_start[1] - wave_start[0], tiles, n_tiles, bn);
     // one warp per row, eight rows per CTA; a lane keeps up to eight 16-byte loads in flight before it stores
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r = blockIdx.x * 8 + warp;
@@ -688,9 +691,9 @@ gather_rows_kernel(const __nv_bfloat16* __restrict__ hidden, const int32_t* __re
 constexpr int kPlanThreads = 1024;
 static_assert(kPlanGatherPairs < 65536, "two counts in one word");
 __global__ void __launch_bounds__(kPlanThreads)
-plan_gather_kernel(const __nv_bfloat16* __restrict__ hidden, const int32_t* __restrict__ ids, int n_pairs, int top_k, int H, int E,
-                   int C, int n_keys, int max_waves, bool identity, int seg, PlanPtrs plan, int* __restrict__ status,
-                   __nv_bfloat16* __restrict__ xg, Tile* __restrict__ tiles, int32_t* __restrict__ n_tiles, int bn, bool k_order) {
+plan_gather_kernel(const __nv_bfloat16* hidden, const int32_t* ids, int n_pairs, int top_k, int H, int E,
+                   int C, int n_keys, int max_waves, bool identity, int seg, PlanPtrs plan, int* status,
+                   __nv_bfloat16* xg, Tile* tiles, int32_t* n_tiles, int bn, bool k_order) {
     extern __shared__ __align__(16) int s_int[];
     int* s_cnt = s_int;                    // [n_keys]: pairs of the key | those before the segment << 16
     int* s_off = s_cnt + n_keys;           // [n_keys + 1]
@@ -731,7 +734,7 @@ plan_gather_kernel(const __nv_bfloat16* __restrict__ hidden, const int32_t* __re
             plan.header[HDR_BAD_ID] = 0;
         }
         __syncthreads();
-        if (tiles) build_tile_list(plan.counts, plan.offsets, plan.group_keys, plan.wave_start, tiles, n_tiles, bn);
+        if (tiles) build_tile_list(s_cnt, s_off, nullptr, 0, n_keys, tiles, n_tiles, bn);
         return;
     }
     if (warp == 0) {                       // place of the segment's first pair of every key
@@ -878,11 +881,9 @@ void launch_gather_rows(const __nv_bfloat16* hidden, const int32_t* perm, const 
                         int tile_rows, bool k_order, cudaStream_t st) {
     int32_t* n_tiles = reinterpret_cast<int32_t*>(scratch);
     Tile* tiles = single_wave ? reinterpret_cast<Tile*>(reinterpret_cast<unsigned char*>(scratch) + 256) : nullptr;
-    gather_rows_kernel<<<(n_pairs + 7) / 8, 256, 0, st>>>(hidden, perm, n_valid, top_k, H, xg, single_wave ? single_wave->counts : nullptr,
-                                                 single_wave ? single_wave->offsets : nullptr,
-                                                 single_wave ? single_wave->group_keys : nullptr, wave_start, tiles, n_tiles,
-                                                 tile_rows, k_order);
-    count_launch();
+    launch_dependent(gather_rows_kernel, (n_pairs + 7) / 8, 256, 0, st, hidden, perm, n_valid, top_k, H, xg,
+                     (const int32_t*)(single_wave ? single_wave->counts : nullptr), (const int32_t*)(single_wave ? single_wave->offsets : nullptr),
+                     (const int32_t*)(single_wave ? single_wave->group_keys : nullptr), wave_start, tiles, n_tiles, tile_rows, k_order);
 }
 
 // One wave of the tensor-core path: tile list, gate/up GEMM + SwiGLU, down GEMM x routing weight.

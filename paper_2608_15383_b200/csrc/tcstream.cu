@@ -144,7 +144,7 @@ __device__ __forceinline__ void codes_bf16(uint32_t w, uint32_t (&out)[4]) {
 
 // Tile t of the list, past L1: the list's memory is another call's before this one.
 __device__ __forceinline__ Tile listed_tile(const Tile* tiles, const int4* listed, int t) {
-    const int4 v = t < kListed ? listed[t] : __ldcg(reinterpret_cast<const int4*>(tiles) + t);
+    const int4 v = t < kListed ? listed[t] : load_behind_wait_cg(reinterpret_cast<const int4*>(tiles) + t);
     return Tile{v.x, v.y, v.z, v.w};
 }
 
@@ -228,9 +228,9 @@ tc_stream_kernel(const TcStreamArgs a, const CUtensorMap* __restrict__ maps, __n
         int4 tl[kListed / 32];
 #pragma unroll
         for (int j = 0; j < kListed / 32; ++j)
-            tl[j] = 32 * j + lane < a.tile_cap ? __ldcg(reinterpret_cast<const int4*>(a.tiles) + 32 * j + lane) : make_int4(0, 0, 0, 0);
-        const int n = __ldcg(a.n_tiles);
-        const long long total = (long long)__ldcg(a.n_tiles + 1) * MT;
+            tl[j] = 32 * j + lane < a.tile_cap ? load_behind_wait_cg(reinterpret_cast<const int4*>(a.tiles) + 32 * j + lane) : make_int4(0, 0, 0, 0);
+        const int n = load_behind_wait_cg(a.n_tiles);
+        const long long total = (long long)load_behind_wait_cg(a.n_tiles + 1) * MT;
 #pragma unroll
         for (int j = 0; j < kListed / 32; ++j) s_tiles[32 * j + lane] = tl[j];
         __syncwarp();
@@ -243,7 +243,7 @@ tc_stream_kernel(const TcStreamArgs a, const CUtensorMap* __restrict__ maps, __n
             for (int j = 0; j < kListed / 32; ++j)
                 count += __popc(__ballot_sync(0xffffffffu, 32 * j + lane < n && (long long)tl[j].y * MT <= edge));
             for (int base = kListed; base < n; base += 32)
-                count += __popc(__ballot_sync(0xffffffffu, base + lane < n && (long long)__ldcg(&a.tiles[base + lane].before) * MT <= edge));
+                count += __popc(__ballot_sync(0xffffffffu, base + lane < n && (long long)load_behind_wait_cg(&a.tiles[base + lane].before) * MT <= edge));
             if (count > 0) {
                 const Tile v = listed_tile(a.tiles, s_tiles, count - 1);
                 const int w = tile_weight(v.nrows);
