@@ -265,6 +265,19 @@ enum {
 };
 int exmoe_debug_last_path(exmoe_cache* cache);
 
+/* Which tensor-core kernels served the most recent exmoe_moe_forward (test and measurement hook; no paper counterpart):
+ * EXMOE_TENSOR_*, EXMOE_ERR_STATE where that call was not on EXMOE_PATH_TENSOR_SMALL_N or EXMOE_PATH_TENSOR.  Does not
+ * synchronise. */
+enum {
+    EXMOE_TENSOR_ROWS64 = 0,       /* scaled weights through shared memory, token tiles of 64 rows */
+    EXMOE_TENSOR_ROWS256 = 1,      /* ... of up to 256 rows */
+    EXMOE_TENSOR_STREAM = 2        /* codes through tensor memory, token tiles of 64 rows */
+};
+int exmoe_debug_last_tensor_kernels(exmoe_cache* cache);
+/* Test hook: non-zero, and the cache behaves as on a device that cannot run the streaming tensor-core kernels (their share
+ * of shared memory or registers refused); zero, and it asks the device again.  Affects later calls. */
+int exmoe_debug_refuse_tensor_stream(exmoe_cache* cache, int refuse);
+
 /* Bytes of the staged host-to-device input copy of the most recent exmoe_moe_forward_host (test hook; no paper
  * counterpart): T * d_model * 2 + 2 * T * top_k * 4 rounded up to 16-byte pieces, whatever max_tokens is. */
 int exmoe_debug_last_host_copy_bytes(exmoe_cache* cache, size_t* h2d_bytes);

@@ -61,6 +61,8 @@ _SIGNATURES = {
     "exmoe_cache_get_state": (c_int, [c_void_p, c_int, c_void_p, c_void_p, c_void_p, c_void_p]),
     "exmoe_debug_last_plan": (c_int, [c_void_p, c_int] + [c_void_p] * 9),
     "exmoe_debug_last_path": (c_int, [c_void_p]),
+    "exmoe_debug_last_tensor_kernels": (c_int, [c_void_p]),
+    "exmoe_debug_refuse_tensor_stream": (c_int, [c_void_p, c_int]),
     "exmoe_debug_read_slot": (c_int, [c_void_p, c_int, c_int, c_void_p]),
     "exmoe_debug_wait_timeout": (c_int, [c_void_p, ctypes.c_longlong, POINTER(c_int)]),
     "exmoe_cache_stats": (c_int, [c_void_p, c_int, POINTER(exmoe_stats)]),
@@ -256,6 +258,7 @@ def pad_hidden(hidden, d_model_padded):
 
 MISS_HOST_COPIES, MISS_DEVICE_FETCH = 0, 1
 PATH_PAIR, PATH_SMALL, PATH_STREAM, PATH_TENSOR_SMALL_N, PATH_TENSOR = 2, 3, 4, 5, 6
+TENSOR_ROWS64, TENSOR_ROWS256, TENSOR_STREAM = 0, 1, 2
 
 
 class Cache:
@@ -349,6 +352,17 @@ class Cache:
         if rc < 0:
             raise ExmoeError(rc, "exmoe_debug_last_path")
         return rc
+
+    def last_tensor_kernels(self):
+        """TENSOR_* of the tensor-core kernels that served the most recent forward (exmoe_debug_last_tensor_kernels)."""
+        rc = int(lib().exmoe_debug_last_tensor_kernels(self.handle))
+        if rc < 0:
+            raise ExmoeError(rc, "exmoe_debug_last_tensor_kernels")
+        return rc
+
+    def refuse_tensor_stream(self, refuse=True):
+        """Later calls go as on a device that cannot run the streaming tensor-core kernels (exmoe_debug_refuse_tensor_stream)."""
+        _check(lib().exmoe_debug_refuse_tensor_stream(self.handle, int(refuse)), "exmoe_debug_refuse_tensor_stream")
 
     def last_host_copy_bytes(self):
         n = c_size_t()

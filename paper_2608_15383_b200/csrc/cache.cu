@@ -67,6 +67,8 @@ struct exmoe_cache {
     bool last_small;
     bool last_pair;                           // ... which formed no plan (per-pair or streaming kernels)
     int last_path;                            // EXMOE_PATH_* of the most recent forward
+    int last_tensor;                          // EXMOE_TENSOR_* of the most recent forward, -1: none of them
+    bool tc_stream_ok;                        // the streaming tensor-core kernels run on this device
     int32_t* saved_ids;                       // ids of the last call without a grouping kernel (plan materialised on request)
     int stream_pairs;                         // most pairs that go to the streaming kernels (0: the shape does not fit them)
     bool pair_ok, small_ok;                   // ... the per-pair kernels / the in-CTA-grouping kernels (shared memory)
@@ -95,7 +97,7 @@ struct exmoe_cache {
     struct HostGraph {
         cudaGraphExec_t exec;
         bool last_small, last_pair;
-        int last_path;
+        int last_path, last_tensor;
     };
     std::map<long long, HostGraph> host_graphs;
 };
@@ -397,6 +399,7 @@ int exmoe_cache_create(exmoe_cache** out, const exmoe_shape* shape, int num_laye
     ok = ok && cudaMemset(c->arrive, 0, c->arrive_words * 4) == cudaSuccess;
     ok = ok && cudaMemset(c->plan.chunk_done, 0, 256) == cudaSuccess;
     for (int l = 0; l < num_layers && ok; ++l) ok = reset_layer(c, l) == EXMOE_OK;
+    c->tc_stream_ok = tc_stream_runs();
     if (ok && c->xg) ok = prefill_setup(&c->tc_maps, c->xg, c->act, c->max_pairs, c->shape.d_model, c->shape.d_ff) == EXMOE_OK;
     if (ok && c->C == c->shape.num_experts) {            // full residency: preload, slot = expert id
         for (int l = 0; l < num_layers && ok; ++l)
@@ -489,10 +492,11 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
     const bool pairwise = small && P <= kPairMaxPairs && n_waves == 1 && c->pair_ok;
     c->last_pair = pairwise || own_plan;
     const bool small_n = P <= kPrefillSmallNMaxPairs;      // tensor-core path: which kernel shape
-    const int tc_kind = tc_stream_takes(s, P) ? TC_STREAM : small_n ? TC_SMALL_N : TC_LARGE;
+    const int tc_kind = c->tc_stream_ok && tc_stream_takes(s, P) ? TC_STREAM : small_n ? TC_SMALL_N : TC_LARGE;
     const int tile_rows = prefill_tile_rows(s, P, c->Cw, tc_kind);
     c->last_path = pairwise ? EXMOE_PATH_PAIR : small ? EXMOE_PATH_SMALL : use_stream ? EXMOE_PATH_STREAM
                    : small_n ? EXMOE_PATH_TENSOR_SMALL_N : EXMOE_PATH_TENSOR;
+    c->last_tensor = small || use_stream ? -1 : tc_kind;
     if (!small && build_plan && !use_stream) {
         ProfScope ps(c, PROF_PLAN, st);                  // hidden rows in plan order, once for all waves
         tiles_fused = (n_waves == 1);                    // one wave: its tile list comes out of the same launch
@@ -506,7 +510,8 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
     if (small && n_waves == 0)                           // no valid id at all: the output is zero
         cudaMemsetAsync(out, 0, (size_t)T * s.d_model * 2, st);
     int mi = 0;
-    for (int w = 0; w < n_waves; ++w) {
+    bool launched = true;                                // false: a kernel was refused, and what follows would read stale buffers
+    for (int w = 0; w < n_waves && launched; ++w) {
         int groups = identity ? (E < P ? E : P) : 0;
         bool split = false;                              // the wave's kernels run twice: resident groups, then fetched ones
         if (dev_fetch) {
@@ -596,36 +601,36 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
                 a.group_filter = 1;
                 {
                     ProfScope ps(c, PROF_GATEUP, st);
-                    launch_stream_wave(a, (const __nv_bfloat16*)hidden, c->act, topk_weights, c->y, c->d_status, groups, true, true, st);
+                    launched = launched && launch_stream_wave(a, (const __nv_bfloat16*)hidden, c->act, topk_weights, c->y, c->d_status, groups, true, true, st);
                 }
                 cudaStreamWaitEvent(st, c->ev_copy[c->copy_seq % kEventRing], 0);     // the wave's fetched experts are in their slots
                 a.group_filter = 2;
                 {
                     ProfScope ps(c, PROF_GATEUP, st);
-                    launch_stream_wave(a, (const __nv_bfloat16*)hidden, c->act, topk_weights, c->y, c->d_status, groups, true, true, st);
+                    launched = launched && launch_stream_wave(a, (const __nv_bfloat16*)hidden, c->act, topk_weights, c->y, c->d_status, groups, true, true, st);
                 }
                 a.group_filter = 0;
             } else if (!c->prof_only) {
                 ProfScope ps(c, PROF_GATEUP, st);    // both kernels: the down kernel is a programmatic dependent
-                launch_stream_wave(a, (const __nv_bfloat16*)hidden, c->act, topk_weights, c->y, c->d_status, groups, true, true,
+                launched = launched && launch_stream_wave(a, (const __nv_bfloat16*)hidden, c->act, topk_weights, c->y, c->d_status, groups, true, true,
                                    st);
             } else if (c->prof_only == PROF_GATEUP || c->prof_only == PROF_DOWN) {
                 ProfScope ps(c, c->prof_only, st);
-                launch_stream_wave(a, (const __nv_bfloat16*)hidden, c->act, topk_weights, c->y, c->d_status, groups,
+                launched = launched && launch_stream_wave(a, (const __nv_bfloat16*)hidden, c->act, topk_weights, c->y, c->d_status, groups,
                                    c->prof_only == PROF_GATEUP, c->prof_only == PROF_DOWN, st);
             }
         } else {
             // many rows per expert: dense contraction on the tensor cores (tcgen05 / TMEM)
             if (build_plan && !tiles_fused)
-                launch_prefill_wave(a, a.wave_start, c->tc_scratch, c->d_status, &c->tc_maps, c->act, topk_weights, c->y, 4, tc_kind, tile_rows, st);
+                launched = launched && launch_prefill_wave(a, a.wave_start, c->tc_scratch, c->d_status, &c->tc_maps, c->act, topk_weights, c->y, 4, tc_kind, tile_rows, st);
             if (!c->prof_only || c->prof_only == PROF_GATEUP) {
                 ProfScope ps(c, PROF_GATEUP, st);
-                launch_prefill_wave(a, a.wave_start, c->tc_scratch, c->d_status, &c->tc_maps, c->act, topk_weights, c->y, 1,
+                launched = launched && launch_prefill_wave(a, a.wave_start, c->tc_scratch, c->d_status, &c->tc_maps, c->act, topk_weights, c->y, 1,
                                     tc_kind, tile_rows, st);
             }
             if (!c->prof_only || c->prof_only == PROF_DOWN) {
                 ProfScope ps(c, PROF_DOWN, st);
-                launch_prefill_wave(a, a.wave_start, c->tc_scratch, c->d_status, &c->tc_maps, c->act, topk_weights, c->y, 2,
+                launched = launched && launch_prefill_wave(a, a.wave_start, c->tc_scratch, c->d_status, &c->tc_maps, c->act, topk_weights, c->y, 2,
                                     tc_kind, tile_rows, st);
             }
         }
@@ -635,6 +640,10 @@ int exmoe_moe_forward(exmoe_cache* c, int layer, const void* hidden, const int32
             for (int e = 0; e < E; ++e)
                 if (h_wave_of[e] == w) c->slot_last_seq[layer][h_slot_of[e]] = c->seq;
         }
+    }
+    if (!launched) {
+        cudaGetLastError();
+        return EXMOE_ERR_CUDA;
     }
     if (!small && (!c->prof_only || c->prof_only == PROF_COMBINE)) {
         ProfScope ps(c, PROF_COMBINE, st);
@@ -716,6 +725,7 @@ int exmoe_moe_forward_host(exmoe_cache* c, int layer, const void* hidden_host, c
             c->last_T = T;
             c->last_small = c->last_pair = true;
             c->last_path = EXMOE_PATH_PAIR;
+            c->last_tensor = -1;
             c->last_host_h2d_bytes = off_w + nb_i;
             int rc = cudaGetLastError() == cudaSuccess ? EXMOE_OK : EXMOE_ERR_CUDA;
             if (cudaStreamSynchronize(st) != cudaSuccess) rc = EXMOE_ERR_CUDA;
@@ -753,6 +763,7 @@ int exmoe_moe_forward_host(exmoe_cache* c, int layer, const void* hidden_host, c
         c->last_small = it->second.last_small;
         c->last_pair = it->second.last_pair;
         c->last_path = it->second.last_path;
+        c->last_tensor = it->second.last_tensor;
         if (cudaGraphLaunch(it->second.exec, st) != cudaSuccess) rc = EXMOE_ERR_CUDA;
     } else {
         rc = enqueue();                                                   // this call runs as plain launches
@@ -770,7 +781,7 @@ int exmoe_moe_forward_host(exmoe_cache* c, int layer, const void* hidden_host, c
         }
         ok = ok && cudaGraphInstantiate(&exec, g, 0) == cudaSuccess;
         if (g) cudaGraphDestroy(g);
-        if (ok) c->host_graphs[key] = exmoe_cache::HostGraph{exec, c->last_small, c->last_pair, c->last_path};
+        if (ok) c->host_graphs[key] = exmoe_cache::HostGraph{exec, c->last_small, c->last_pair, c->last_path, c->last_tensor};
         else cudaGetLastError();                                          // stay on plain launches for this key
     }
     return rc;
@@ -856,6 +867,17 @@ int exmoe_debug_last_path(exmoe_cache* c) {
     if (!c) return EXMOE_ERR_ARG;
     if (c->last_layer < 0) return EXMOE_ERR_STATE;
     return c->last_path;
+}
+
+int exmoe_debug_last_tensor_kernels(exmoe_cache* c) {
+    if (!c) return EXMOE_ERR_ARG;
+    return c->last_layer < 0 || c->last_tensor < 0 ? EXMOE_ERR_STATE : c->last_tensor;
+}
+
+int exmoe_debug_refuse_tensor_stream(exmoe_cache* c, int refuse) {
+    if (!c) return EXMOE_ERR_ARG;
+    c->tc_stream_ok = !refuse && tc_stream_runs();
+    return EXMOE_OK;
 }
 
 int exmoe_debug_last_host_copy_bytes(exmoe_cache* c, size_t* h2d_bytes) {

@@ -146,11 +146,11 @@ constexpr int kStreamMaxRows = 14, kStreamMaxRowsFew = 28;
 constexpr int kStreamMaxPairsUneven = 192;
 constexpr int kStreamOwnPlanKeys = 128, kStreamOwnPlanPairs = 640;        // most experts and pairs that the streaming kernels group themselves
 int stream_max_pairs(const exmoe_shape& s);      // most pairs of a call that the streaming kernels take; 0: not this shape
-bool launch_stream_wave(const GemmArgs& a, const __nv_bfloat16* hidden, __nv_bfloat16* act, const float* topk_w, float* y,
+[[nodiscard]] bool launch_stream_wave(const GemmArgs& a, const __nv_bfloat16* hidden, __nv_bfloat16* act, const float* topk_w, float* y,
                         int* status, int max_groups, bool gateup, bool down, cudaStream_t st);
 void launch_small_wave(const GemmArgs& a, const SmallWave& w, cudaStream_t st, bool gateup, bool down);
 // the per-pair kernels on HOST inputs that travel as kernel parameters; false (nothing queued) where that does not apply
-bool launch_pair_inline(const GemmArgs& a, const SmallWave& w, const void* hidden, const int32_t* ids, const float* weights, cudaStream_t st);
+[[nodiscard]] bool launch_pair_inline(const GemmArgs& a, const SmallWave& w, const void* hidden, const int32_t* ids, const float* weights, cudaStream_t st);
 bool pair_path_fits(int H, int I, int top_k);                           // shared memory of the per-pair kernels within limits
 bool small_path_fits(int H, int I, int num_slots, int n_pairs);         // ... of the in-CTA-grouping kernels
 size_t prefill_scratch_bytes(int max_pairs, int num_experts);
@@ -160,8 +160,8 @@ constexpr size_t kPrefillMapBytes = 2 * 16 * 128;
 struct PrefillMaps { unsigned char* dev; };
 int prefill_setup(PrefillMaps* maps, const __nv_bfloat16* xg, const __nv_bfloat16* act, int max_pairs, int H, int I);
 struct Tile;
-// one wave on the streaming tensor-core kernels (token matrices in their K order); false: not possible on this device
-bool launch_tc_stream_wave(const GemmArgs& g, const Tile* tiles, int tile_cap, const int32_t* n_tiles, int* status, const PrefillMaps* maps, __nv_bfloat16* act,
+// one wave on the streaming tensor-core kernels (token matrices in their K order); false: not launched
+[[nodiscard]] bool launch_tc_stream_wave(const GemmArgs& g, const Tile* tiles, int tile_cap, const int32_t* n_tiles, int* status, const PrefillMaps* maps, __nv_bfloat16* act,
                            const float* topk_w, float* y, bool gateup, bool down, cudaStream_t st);
 void launch_wait_selftest(int* status, long long budget_cycles, int* result, cudaStream_t st);
 // Grouping and grouped copy of the hidden rows in one launch, for calls within these limits.  Its CTAs each count all pairs
@@ -176,9 +176,13 @@ void launch_gather_rows(const __nv_bfloat16* hidden, const int32_t* perm, const 
                         int tile_rows, bool k_order, cudaStream_t st);
 // which: bit 0 = gate/up GEMM + SwiGLU, bit 1 = down GEMM x routing weight, bit 2 = (re)build the wave's tile list
 // kind: the 64-row, eight-stage kernel shape (a few dozen rows per expert), the 256-row, four-stage one, or the streaming kernels
-void launch_prefill_wave(const GemmArgs& g, const int32_t* wave_start, void* scratch, int* status, const PrefillMaps* maps,
+// false: not launched
+[[nodiscard]] bool launch_prefill_wave(const GemmArgs& g, const int32_t* wave_start, void* scratch, int* status, const PrefillMaps* maps,
                          __nv_bfloat16* act, const float* topk_w, float* y, int which, int kind, int tile_rows, cudaStream_t st);
-enum { TC_SMALL_N = 0, TC_LARGE = 1, TC_STREAM = 2 };     // kind of a tensor-core call
+enum { TC_SMALL_N = EXMOE_TENSOR_ROWS64, TC_LARGE = EXMOE_TENSOR_ROWS256, TC_STREAM = EXMOE_TENSOR_STREAM };     // kind of a tensor-core call
+// Whether this device can run the streaming tensor-core kernels.  Asked when a cache is created: a call's rows are copied in
+// these kernels' own K order, so the choice cannot be taken back where they are launched.
+bool tc_stream_runs();
 // The streaming tensor-core kernels: beyond the streaming kernels' range up to 24 rows per expert, for layers whose gate/up
 // matrices come to 100 blocks of 128 x 128 per SM and whose K is at least 2048 (their launches take 2.5 us longer to their first MMA than
 // the other tensor-core kernels, which smaller layers and few active experts do not earn back).  Of the other kernels' time, with

@@ -887,7 +887,7 @@ void launch_gather_rows(const __nv_bfloat16* hidden, const int32_t* perm, const 
 }
 
 // One wave of the tensor-core path: tile list, gate/up GEMM + SwiGLU, down GEMM x routing weight.
-void launch_prefill_wave(const GemmArgs& g, const int32_t* wave_start, void* scratch, int* status, const PrefillMaps* maps,
+bool launch_prefill_wave(const GemmArgs& g, const int32_t* wave_start, void* scratch, int* status, const PrefillMaps* maps,
                          __nv_bfloat16* act, const float* topk_w, float* y, int which, int kind, int tile_rows, cudaStream_t st) {
     int32_t* n_tiles = reinterpret_cast<int32_t*>(scratch);
     Tile* tiles = reinterpret_cast<Tile*>(reinterpret_cast<unsigned char*>(scratch) + 256);
@@ -917,10 +917,8 @@ void launch_prefill_wave(const GemmArgs& g, const int32_t* wave_start, void* scr
         tile_list_kernel<<<1, 1024, 0, st>>>(g.counts, g.offsets, g.group_keys, wave_start, tiles, n_tiles, tile_rows);
         count_launch();
     }
-    if (kind == TC_STREAM) {
-        launch_tc_stream_wave(g, tiles, g.n_pairs / 16 + g.num_slots + 16, n_tiles, status, maps, act, topk_w, y, which & 1, which & 2, st);
-        return;
-    }
+    if (kind == TC_STREAM)
+        return launch_tc_stream_wave(g, tiles, g.n_pairs / 16 + g.num_slots + 16, n_tiles, status, maps, act, topk_w, y, which & 1, which & 2, st);
     const bool small_n = kind == TC_SMALL_N;
     if (which & 1) {
         if (small_n)
@@ -934,6 +932,7 @@ void launch_prefill_wave(const GemmArgs& g, const int32_t* wave_start, void* scr
         else
             launch_dependent(prefill_gemm_kernel<false, BN, kStagesLarge>, sms, NUM_THREADS, smem_large, st, a, ma, (__nv_bfloat16*)nullptr, topk_w, y);
     }
+    return true;
 }
 
 }  // namespace exmoe

@@ -555,15 +555,16 @@ tc_stream_kernel(const TcStreamArgs a, const CUtensorMap* __restrict__ maps, __n
 }
 
 template <bool GATEUP>
-bool launch_tc_stream(const TcStreamArgs& a, const CUtensorMap* maps, __nv_bfloat16* act, const float* topk_w, float* y, cudaStream_t st) {
+bool tc_stream_kernel_runs() {
     static SmemOnce once;
-    if (!allow_smem(tc_stream_kernel<GATEUP>, (int)kSmemBytes, once)) return false;
+    cudaFuncAttributes at{};
     // the warpgroups' shares come out of the registers that the launch brings: fewer, and the split would wait for good
-    static const int regs = [] {
-        cudaFuncAttributes at{};
-        return cudaFuncGetAttributes(&at, tc_stream_kernel<GATEUP>) == cudaSuccess ? at.numRegs : 0;
-    }();
-    if (regs * kThreads < kRegsSplit) return false;
+    return allow_smem(tc_stream_kernel<GATEUP>, (int)kSmemBytes, once) && cudaFuncGetAttributes(&at, tc_stream_kernel<GATEUP>) == cudaSuccess &&
+           at.numRegs * kThreads >= kRegsSplit;
+}
+
+template <bool GATEUP>
+bool launch_tc_stream(const TcStreamArgs& a, const CUtensorMap* maps, __nv_bfloat16* act, const float* topk_w, float* y, cudaStream_t st) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
         sms = 148;
@@ -577,12 +578,18 @@ bool launch_tc_stream(const TcStreamArgs& a, const CUtensorMap* maps, __nv_bfloa
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    cudaLaunchKernelEx(&lc, tc_stream_kernel<GATEUP>, a, maps, act, topk_w, y);
+    if (cudaLaunchKernelEx(&lc, tc_stream_kernel<GATEUP>, a, maps, act, topk_w, y) != cudaSuccess) return false;
     count_launch();
     return true;
 }
 
 }  // namespace
+
+bool tc_stream_runs() {
+    const bool runs = tc_stream_kernel_runs<true>() && tc_stream_kernel_runs<false>();
+    if (!runs) cudaGetLastError();
+    return runs;
+}
 
 bool launch_tc_stream_wave(const GemmArgs& g, const Tile* tiles, int tile_cap, const int32_t* n_tiles, int* status, const PrefillMaps* maps, __nv_bfloat16* act,
                            const float* topk_w, float* y, bool gateup, bool down, cudaStream_t st) {

@@ -506,3 +506,26 @@ def test_streaming_tensor_core_kernels_at_tile_edges(B):
     again = part.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
     assert torch.equal(out.view(torch.int16), again.view(torch.int16)) and part.status() == 0
     part.close()
+
+
+@pytest.mark.parametrize("T", [96, 150])
+def test_device_that_cannot_run_the_streaming_tensor_core_kernels(B, olmoe_layer, T):
+    """Where the device refuses these kernels their shared memory or registers, the other tensor-core kernels take the call
+    (with the rows in their own order), on both sides of 1024 pairs; nothing is combined from an earlier call's buffers."""
+    ora, bank = olmoe_layer
+    s = synth.OLMOE
+    cache = B.Cache(s, [bank], 64, max_tokens=T)
+    hidden, ids, p = helpers.routed_inputs(s, T, seed=7600 + T, alpha=0.5)
+    first = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda()).clone()
+    assert cache.last_tensor_kernels() == B.TENSOR_STREAM
+    cache.refuse_tensor_stream()
+    hidden = hidden.flip(0).contiguous()                 # other rows than those that the buffers hold
+    out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    assert cache.last_tensor_kernels() == (B.TENSOR_ROWS64 if T * s.top_k <= 1024 else B.TENSOR_ROWS256)
+    y, ref = ora.forward(hidden, ids, p)
+    helpers.check_output(out, y, ref, f"T={T}, refused")
+    cache.refuse_tensor_stream(False)
+    out = cache.forward(0, hidden.flip(0).contiguous().cuda(), ids.cuda(), p.cuda())
+    assert cache.last_tensor_kernels() == B.TENSOR_STREAM and torch.equal(out.view(torch.int16), first.view(torch.int16))
+    assert cache.status() == 0
+    cache.close()

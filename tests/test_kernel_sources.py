@@ -27,3 +27,19 @@ def test_the_issue_loop_only_looks_ahead():
             continue
         ahead = [line.strip() for line in text.splitlines() if re.search(r"mbar_try(_at)?\(", line) and not re.search(r"\bwhile\s*\(", line)]
         assert not ahead, (name, ahead)
+
+
+def test_a_refused_launch_is_not_dropped():
+    """A launcher that answers whether it launched is [[nodiscard]], and no call of one stands by itself: what comes behind it
+    would read the buffers of an earlier call."""
+    launchers = set()
+    for name, text in sources():
+        if name == "common.cuh":
+            for mark, fn in re.findall(r"^(\[\[nodiscard\]\] )?bool (launch_\w+)\(", text, re.M):
+                assert mark, fn
+                launchers.add(fn)
+    assert {"launch_stream_wave", "launch_tc_stream_wave", "launch_prefill_wave"} <= launchers
+    for name, text in sources():
+        for fn in launchers:
+            alone = re.findall(r"[;{})]\s*%s\(" % fn, text)
+            assert not alone, (name, fn)
