@@ -162,7 +162,7 @@ enum { MODE_SMALL = 1, MODE_PAIR = 2 };
 // MODE_PAIR  : one item per token-expert pair, no grouping at all (T*k <= 32, gate/up only)
 template <int NB, int NCH, bool GATEUP, int MODE>
 __global__ void __launch_bounds__(256, 1)
-decode_gemm_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ x_src,
+decode_gemm_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* x_src,
                    __nv_bfloat16* __restrict__ act_out, const float* __restrict__ topk_w, float* __restrict__ y_out,
                    int KS, int blocks_per_warp) {
     constexpr int NM = GATEUP ? 2 : 1;
@@ -460,7 +460,7 @@ decode_gemm_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ x
 #endif
 template <int NBT, typename Inl>
 __global__ void __launch_bounds__(256)
-token_down_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ act, const float* __restrict__ topk_w,
+token_down_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* act, const float* __restrict__ topk_w,
                   int bpwg, const __grid_constant__ Inl in) {
     constexpr bool INL = std::is_same_v<Inl, InlineIds>;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -604,7 +604,7 @@ token_down_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ ac
 // one resident wave; the arithmetic and its order are those of decode_gemm_kernel.
 template <int NB>
 __device__ __forceinline__ void pair_gateup_item(const GemmArgs& a, const SmallArgs& sa,
-                                                 const __nv_bfloat16* __restrict__ hidden,
+                                                 const __nv_bfloat16* hidden,
                                                  __nv_bfloat16* __restrict__ act_out, int ks_log2, int p, int token,
                                                  int tile, unsigned char* smem) {
     // No integer division anywhere before the first loads are issued (a runtime division is a dependent chain of
@@ -722,7 +722,7 @@ __device__ __forceinline__ void keep_pair_ids(const SmallArgs& sa, const int32_t
 
 template <int NB>
 __global__ void __launch_bounds__(256, 2)
-pair_gateup_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ hidden,
+pair_gateup_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* hidden,
                    __nv_bfloat16* __restrict__ act_out, int ks_log2) {
     // grid = (tiles of the intermediate dimension, selected expert j, token t): pair p = t * k + j
     extern __shared__ __align__(128) unsigned char smem[];
@@ -785,7 +785,7 @@ __device__ __forceinline__ void wide_block(const uint4 (&wb)[2][2], const uint32
 
 template <int NB, int HB>
 __global__ void __launch_bounds__(32 * kWideWarps, 1)
-pair_gateup_wide_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ hidden,
+pair_gateup_wide_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* hidden,
                         __nv_bfloat16* __restrict__ act_out, int ks_log2, const __grid_constant__ InlineInput<HB> in) {
     // grid = (slices of 16 >> ks_log2 panel pairs, selected expert j, token t): pair p = t * k + j
     extern __shared__ __align__(128) unsigned char smem[];
@@ -913,7 +913,7 @@ __device__ __forceinline__ void drain_bar(uint64_t* bar, uint32_t parity) {
 
 template <int NBT, typename Inl>
 __global__ void __launch_bounds__(256, 1)
-token_down_bulk_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* __restrict__ act, const float* __restrict__ topk_w,
+token_down_bulk_kernel(GemmArgs a, SmallArgs sa, const __nv_bfloat16* act, const float* __restrict__ topk_w,
                        int bpwg, const __grid_constant__ Inl in) {
     constexpr bool INL = std::is_same_v<Inl, InlineIds>;
     extern __shared__ __align__(128) unsigned char smem[];

@@ -168,7 +168,7 @@ constexpr int kFetchVec = 8;
 constexpr int kFetchPiece = kFetchThreads * kFetchVec * 16;           // 32,768 B
 
 __global__ void __launch_bounds__(kFetchThreads)
-fetch_misses_kernel(const int32_t* __restrict__ header, const int32_t* __restrict__ misses, int wave,
+fetch_misses_kernel(const int32_t* header, const int32_t* misses, int wave,
                     const uint8_t* __restrict__ bank, uint8_t* __restrict__ slots, unsigned long long bpe, int E, int C) {
     __shared__ int s_lo, s_hi;
     asm volatile("griddepcontrol.wait;" ::: "memory");  // launched as a programmatic dependent of the resolution kernel (wave 0)
@@ -236,7 +236,7 @@ void launch_fetch_misses(const PlanPtrs& plan, int wave, const uint8_t* bank_dev
 
 // Small problems (up to 2048 pairs): one CTA does histogram, scan and the stable permutation.
 __global__ void __launch_bounds__(256)
-group_small_kernel(const int32_t* __restrict__ ids, int n_pairs, int E, int C, int n_keys, int max_waves,
+group_small_kernel(const int32_t* ids, int n_pairs, int E, int C, int n_keys, int max_waves,
                    bool identity, PlanPtrs plan, int* __restrict__ status) {
     extern __shared__ __align__(16) int s_int[];
     int* s_cnt = s_int;                    // [n_keys]

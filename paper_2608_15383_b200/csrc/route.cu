@@ -142,7 +142,7 @@ __device__ __forceinline__ void softmax_topk_cta(float* prob, float* pv, int E, 
 // this CTA owns (token i belongs to rank i % CL).
 template <int CL, int TB, bool COUNT>
 __global__ void __launch_bounds__(kRouteThreads)
-route_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* __restrict__ w_router,
+route_kernel(const __nv_bfloat16* hidden, const __nv_bfloat16* __restrict__ w_router,
              const float* __restrict__ bias, int T, int H, int E, int k, int32_t* __restrict__ ids_out,
              float* __restrict__ w_out) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -225,7 +225,7 @@ route_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* __re
 // One CTA per token, no cluster and nothing held ahead in registers: many CTAs per SM.  For calls with more tokens than
 // there is room for clusters and so few experts that reading the matrix again for every token costs little.  Same arithmetic.
 __global__ void __launch_bounds__(kRouteThreads)
-route_token_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* __restrict__ w_router,
+route_token_kernel(const __nv_bfloat16* hidden, const __nv_bfloat16* __restrict__ w_router,
                    const float* __restrict__ bias, int T, int H, int E, int k, int32_t* __restrict__ ids_out,
                    float* __restrict__ w_out) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -326,7 +326,7 @@ constexpr int kMmaMaxModel = 4096;                    // |x|^2 and |w|^2 are sum
 __device__ __forceinline__ float route_bound(int H) { return 1.14f * (0x1p-20f + (float)(21 + 3 * H / 512) * 0x1p-24f); }
 
 // Binary32 logit of one expert, by one warp.
-__device__ __noinline__ float logit_again(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ w, int H, int lane) {
+__device__ __noinline__ float logit_again(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w, int H, int lane) {
     const uint4 *xr = reinterpret_cast<const uint4*>(x), *wr = reinterpret_cast<const uint4*>(w);
     float s = 0.f;
     for (int j0 = 0; j0 < H / 8; j0 += 256) {
@@ -497,7 +497,7 @@ __device__ __forceinline__ bool choose(const float* z, float slack, int E, int k
 // flight (even: they alternate between the two running sums).  Two CTAs share an SM.
 template <int NT, int CL, int U>
 __global__ void __launch_bounds__(kRouteThreads, 2)
-route_mma_kernel(const __nv_bfloat16* __restrict__ hidden, const __nv_bfloat16* __restrict__ w_router,
+route_mma_kernel(const __nv_bfloat16* hidden, const __nv_bfloat16* __restrict__ w_router,
                  const float* __restrict__ bias, int T, int H, int E, int k, int32_t* __restrict__ ids_out,
                  float* __restrict__ w_out) {
     constexpr int TM = 16, EC = 8 * NT, EB = CL * EC;                       // experts of a CTA / of the cluster per pass

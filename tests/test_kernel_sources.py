@@ -43,3 +43,33 @@ def test_a_refused_launch_is_not_dropped():
         for fn in launchers:
             alone = re.findall(r"[;{})]\s*%s\(" % fn, text)
             assert not alone, (name, fn)
+
+
+# const __restrict__ parameters of kernels that wait for the kernel in front of them: data that are complete before they start
+COMPLETE_BEFORE = {
+    "w_router": None, "bias": None, "w": None, "maps": None, "bank": None,                 # never written by a kernel of a serving loop
+    # written by the router, and read by kernels in front of these, which let them start only behind their own wait
+    "topk_w": {"decode_gemm_kernel", "token_down_kernel", "token_down_bulk_kernel", "prefill_gemm_kernel", "tc_stream_kernel",
+               "epilogue_prefetch"},
+    "ids": {"combine_kernel"},
+}
+
+
+def test_nothing_read_behind_a_launch_dependency_counts_as_read_only():
+    """A load through const __restrict__ may move in front of griddepcontrol.wait, where its data are still being written: only
+    parameters that are complete before the kernel starts have it, and so with the device functions that such kernels call."""
+    seen = set()
+    for name, text in sources():
+        if not re.search(r"grid_dependency_wait\(\)|griddepcontrol\.wait", text):
+            continue
+        text = re.sub(r"__launch_bounds__\([^)]*\)", "", text)
+        functions = list(re.finditer(r"(__global__|__device__)[^;{}]*?(\w+)\(([^{};]*)\)\s*\{", text))
+        for i, m in enumerate(functions):
+            end = functions[i + 1].start() if i + 1 < len(functions) else len(text)
+            if m[1] == "__global__" and not re.search(r"grid_dependency_wait\(\)|griddepcontrol\.wait", text[m.end():end]):
+                continue                                       # an ordinary launch: everything in front of it is complete
+            for param in re.findall(r"const [\w ]+\*\s*__restrict__ (\w+)", m[3]):
+                assert param in COMPLETE_BEFORE and m[2] in (COMPLETE_BEFORE[param] or {m[2]}), (name, m[2], param)
+            seen.add(m[2])
+    assert {"route_kernel", "route_token_kernel", "route_mma_kernel", "group_small_kernel", "plan_gather_kernel", "combine_kernel",
+            "stream_gemm_kernel", "tc_stream_kernel", "pair_gateup_wide_kernel", "fetch_misses_kernel"} <= seen
