@@ -381,7 +381,6 @@ group_chunk_count_kernel(const int32_t* ids, int n_pairs, int E, int C, int n_ke
     for (int i = tid; i < n_keys; i += kChunk) s_hist[i] = 0;
     __syncthreads();
     grid_dependency_wait();
-    grid_launch_dependents();
     const int p = chunk * kChunk + tid;
     if (p < n_pairs) {
         const int key = pair_key(ids[p], E, C, identity, plan.wave_of, plan.slot_of);
@@ -445,7 +444,6 @@ group_chunk_scatter_kernel(const int32_t* ids, int n_pairs, int E, int C, int n_
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, chunk = blockIdx.x, n_chunks = gridDim.x;
     for (int i = tid; i < n_keys; i += kChunk) s_cur[i] = 0;
     grid_dependency_wait();
-    grid_launch_dependents();
     const int p = chunk * kChunk + tid;
     int key = -1;
     if (p < n_pairs) key = pair_key(ids[p], E, C, identity, plan.wave_of, plan.slot_of);
@@ -491,7 +489,9 @@ void launch_group(const exmoe_shape& s, int C, int n_keys, int max_waves, bool i
     }
     const int n_chunks = (n_pairs + kChunk - 1) / kChunk;
     if (plan.chunk_table && (size_t)n_keys * n_chunks <= plan.chunk_table_words && n_keys <= 5000) {
-        // programmatic dependents, each of the kernel before it (16384 pairs: XXX)
+        // Programmatic dependents, each of the kernel before it, and none lets the next one in early (with it 303 and 1005 us below).
+        // Against plain launches and a memset, 64 experts of 2048 x 1024, us per layer, the row copy's launch included: 16384 pairs
+        // 309 -> 302, 32768 540 -> 533, 65536 1010 -> 1001.
         cudaLaunchConfig_t lc{};
         lc.gridDim = dim3((unsigned)n_chunks);
         lc.blockDim = dim3(kChunk);

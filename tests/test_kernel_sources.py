@@ -73,3 +73,14 @@ def test_nothing_read_behind_a_launch_dependency_counts_as_read_only():
             seen.add(m[2])
     assert {"route_kernel", "route_token_kernel", "route_mma_kernel", "group_small_kernel", "plan_gather_kernel", "combine_kernel",
             "stream_gemm_kernel", "tc_stream_kernel", "pair_gateup_wide_kernel", "fetch_misses_kernel"} <= seen
+
+
+def test_kernels_of_many_ctas_keep_the_next_one_out():
+    """A kernel that releases its dependents at its start shares its SMs with their waiting CTAs: the row copy has thousands of
+    CTAs, and behind it stands a GEMM whose one CTA per SM takes half of the threads."""
+    text = dict(sources())
+    for name, kernel in (("prefill.cu", "gather_rows_kernel"), ("plan.cu", "group_chunk_count_kernel"), ("plan.cu", "group_chunk_scatter_kernel")):
+        start = text[name].index("\n%s(" % kernel)
+        end = text[name].index("\n}\n", start)
+        body = text[name][start:end]
+        assert "grid_dependency_wait();" in body and "grid_launch_dependents" not in body, kernel
