@@ -29,7 +29,8 @@ constexpr int kRouteThreads = 256;
 constexpr int kRouteSmemMax = 200 * 1024;
 constexpr int kRouteFewTokens = 48;       // several tokens per cluster from here on
 constexpr int kRouteTokenTokens = 192;    // one CTA per token, few experts, from here on
-constexpr int kRouteMmaTokens = 193;      // tensor cores from here on
+constexpr int kRouteMmaTokens = 193;      // tensor cores from here on,
+constexpr int kRouteMmaTokensShort = 224; // ... from here on up to 64 experts of d_model below 640
 constexpr int kRouteWideTokens = 1152;    // ... with 32 instead of 16 experts per CTA
 constexpr int kRouteWarps = kRouteThreads / 32;
 
@@ -690,6 +691,9 @@ int launch_route_mma(const exmoe_shape& s, const __nv_bfloat16* hidden, const __
 //   16 experts, d_model 512:   64 tokens 5.2 / 3.5 / 3.3 / 3.9 / 6.8    223: - / 5.7 / 4.1 / 4.1 / 7.0   800: - / 13 / 7.4 / 4.7 / 7.8 / 7.7
 //   16 experts, d_model 2048: 128 tokens 9.5 / 7.0 / 4.6 / 5.1 / 9.6    300: - / 9.8 / 7.3 / 5.4 / 9.7   900: - / 22 / 14 / 12 / 11 / 11
 //   8 experts, d_model 256:    64 tokens 5.0 / 3.3 / 3.2 / 2.7 / 3.8   1024: - / 14 / 9.1 / 4.9 / 6.7 / 6.7   2048: - / 26 / 15 / 6.8 / 8.4 / 7.4
+//   193 / 223 tokens, four and tensor cores, in calls with a near-tie (most at 1024 and more; without one the tensor cores take 2 us less):
+//   64 experts, d_model 256: 5.7 / 6.0 and 6.6 / 6.7    48, 512: 6.1 / 6.3 and 6.8 / 6.8    64, 640: 6.7 / 7.2 and - / 6.9    64, 768: 6.9 / 7.3 and 6.9 / 6.9
+//   64, 1024: 7.2 / 8.0 and 7.3 / 7.3    64, 4096: 13.3 / 14.5 and 10.6 / 10.7    128, 128: 8.7 / 9.1 and 7.6 / 7.7    128, 256: 8.7 / 9.2 and 8.3 / 8.3
 //   256 experts, d_model 1024 (no tensor-core form): 256 tokens 31 / 21 / 22 / 26    1024: 104 / 58 / 55 / 70    4000: 387 / 205 / 178 / 195
 //   20 experts, d_model 1000 (none either): 300 tokens 15 / 8.2 / 5.3 / 6.4          4000: 162 / 71 / 40 / 29
 enum class RouteForm { One, Four, FourNarrow, Token, Mma, MmaWide };
@@ -702,12 +706,14 @@ constexpr RouteForm route_form(int E, int H, int k, int T) {
         if (T >= (E <= 8 ? kRouteFewTokens : kRouteTokenTokens) && (!mma || T < (E <= 8 ? 1536 : small ? 896 : 600))) return RouteForm::Token;
         if (T < kRouteTokenTokens && four) return RouteForm::FourNarrow;
     }
-    if (mma && T >= kRouteMmaTokens) return T >= kRouteWideTokens ? RouteForm::MmaWide : RouteForm::Mma;
+    if (mma && T >= (E <= 64 && H < 640 ? kRouteMmaTokensShort : kRouteMmaTokens)) return T >= kRouteWideTokens ? RouteForm::MmaWide : RouteForm::Mma;
     if (small && !mma && T >= 2048) return RouteForm::Token;
     return four ? (T >= 512 ? RouteForm::FourNarrow : RouteForm::Four) : RouteForm::One;
 }
 static_assert(route_form(64, 2048, 8, 47) == RouteForm::One && route_form(64, 2048, 8, 48) == RouteForm::Four);
 static_assert(route_form(64, 2048, 8, 192) == RouteForm::Four && route_form(64, 2048, 8, 193) == RouteForm::Mma);
+static_assert(route_form(64, 640, 8, 193) == RouteForm::Mma && route_form(128, 128, 8, 193) == RouteForm::Mma);
+static_assert(route_form(64, 512, 8, 223) == RouteForm::Four && route_form(48, 512, 8, 224) == RouteForm::Mma);
 static_assert(route_form(64, 2048, 8, 1152) == RouteForm::MmaWide && route_form(16, 512, 4, 896) == RouteForm::Mma);
 static_assert(route_form(16, 512, 4, 191) == RouteForm::FourNarrow && route_form(16, 512, 4, 192) == RouteForm::Token);
 static_assert(route_form(16, 512, 4, 895) == RouteForm::Token && route_form(8, 256, 2, 48) == RouteForm::Token);
