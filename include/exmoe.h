@@ -261,7 +261,8 @@ enum {
                                     * K does not split evenly over the warps) */
     EXMOE_PATH_TENSOR_SMALL_N = 5, /* tcgen05 kernels up to T*k = 1024: 64-row token tiles */
     EXMOE_PATH_TENSOR = 6          /* tcgen05 kernels beyond: token tiles of up to 256 rows.  Large layers of d_model >= 2048 take
-                                    * the streaming tcgen05 kernels on either side of 1024, up to 24 rows per expert */
+                                    * the streaming tcgen05 kernels on either side of 1024, up to 24 rows per expert (beyond 1024:
+                                    * up to 144 tokens) */
 };
 int exmoe_debug_last_path(exmoe_cache* cache);
 

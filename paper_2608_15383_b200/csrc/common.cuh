@@ -185,13 +185,19 @@ enum { TC_SMALL_N = EXMOE_TENSOR_ROWS64, TC_LARGE = EXMOE_TENSOR_ROWS256, TC_STR
 bool tc_stream_runs();
 // The streaming tensor-core kernels: beyond the streaming kernels' range up to 24 rows per expert, for layers whose gate/up
 // matrices come to 100 blocks of 128 x 128 per SM and whose K is at least 2048 (their launches take 2.5 us longer to their first MMA than
-// the other tensor-core kernels, which smaller layers and few active experts do not earn back).  Of the other kernels' time, with
-// routing uniform / Zipf 0.5 / Zipf 1.5: 64 experts of 2048 x 1024, top-8, 100 tokens 0.79 / 0.78 / 1.02, 150 0.86 / 0.88 / 1.01,
-// 250 (31 rows) 0.92 / 0.92 / 1.09; 60 of 2048 x 1408, top-4, 161 tokens 0.74 / 0.78 / 0.89, 200 0.78 / 0.77 / 1.03, 300
-// 0.81 / 0.83 / 1.15.  Not taken: 96 of 1024 x 1408, top-2, 500 tokens 0.80 / 0.90 / 1.13; 40 of 896 x 1152, top-5, 150 tokens
-// 1.02 / 0.96 / 1.16; 16 of 512 x 256, top-4, 200 tokens 1.33 / 1.27 / 1.29.  By the layer's experts, not the cache's slots: a call's bits
-// do not depend on these.
-constexpr int kTcStreamMaxRows = 24, kTcStreamMinBlocksPerSm = 100, kTcStreamMinModel = 2048;
+// the other tensor-core kernels, which smaller layers and few active experts do not earn back).  Up to 1024 pairs, where the others
+// have tiles of 64 rows too and convert a hot expert's weights as often; beyond, where these take up to 256 rows per conversion, up to
+// 144 tokens (an expert has no more rows than that).  Of the other kernels' time, routing uniform / Zipf 0.5 / 1.0 / 1.25 / 1.5, means
+// of four routings:
+//   64 experts of 2048 x 1024, top-8: 100 tokens 0.82 / 0.81 / 0.87 / 0.89 / 1.02    128: 0.87 / 0.81 / 0.91 / 0.93 / 0.94    144: 0.86 / 0.87 / 0.92 / 0.98 / 1.00
+//                                     160: 0.87 / 0.88 / 0.94 / 0.99 / 1.02 (not taken)   192: 0.86 / 0.88 / 0.91 / 1.02 / 1.03 (not taken)   top-6, 192: Zipf 1.5 1.10 (not taken)
+//   60 of 2048 x 1408, top-4: 170 tokens 0.78 / 0.83 / 0.86 / 0.93 / 0.92    256: 0.83 / 0.82 / 0.88 / 0.91 / 0.98    300: 0.83 / 0.85 / 0.92 / - / 1.17 (not taken)
+//   96 of 4096 x 512, top-2: 400 tokens 0.79 / 0.84 / 0.95 / 0.87 / 1.04    1150: 0.85 / 0.89 / 1.01 / - / 1.19 (not taken)
+//   48 of 2304 x 1536, top-2: 500 tokens 0.84 / 0.82 / 0.89 / 0.94 / 0.93    570: 0.83 / 0.89 / 0.98 / - / 1.27 (not taken)
+//   Not taken for their size: 96 of 1024 x 1408, top-2, 500 tokens 0.80 / 0.90 / - / - / 1.13; 40 of 896 x 1152, top-5, 150 1.02 / 0.96 / - / - / 1.16; 16 of 512 x 256,
+//   top-4, 200 1.33 / 1.27 / - / - / 1.29.
+// By the layer's experts, not the cache's slots: a call's bits do not depend on these.
+constexpr int kTcStreamMaxRows = 24, kTcStreamMaxTokens = 144, kTcStreamMinBlocksPerSm = 100, kTcStreamMinModel = 2048;
 bool tc_stream_takes(const exmoe_shape& s, int n_pairs);
 int prefill_tile_rows(const exmoe_shape& s, int n_pairs, int experts_per_wave, int kind);     // most grouped rows per tile
 #ifndef EXMOE_PREFILL_SMALL_N_MAX_PAIRS

@@ -819,6 +819,7 @@ int prefill_tile_rows(const exmoe_shape& s, int n_pairs, int experts_per_wave, i
 
 bool tc_stream_takes(const exmoe_shape& s, int n_pairs) {
     const long long blocks = (long long)s.num_experts * (2 * s.d_ff / BM) * (s.d_model / BK);
+    if (n_pairs > kPrefillSmallNMaxPairs && n_pairs > kTcStreamMaxTokens * s.top_k) return false;
     return n_pairs <= kTcStreamMaxRows * s.num_experts && s.d_model >= kTcStreamMinModel && blocks >= (long long)kTcStreamMinBlocksPerSm * sm_count();
 }
 

@@ -508,7 +508,7 @@ def test_streaming_tensor_core_kernels_at_tile_edges(B):
     part.close()
 
 
-@pytest.mark.parametrize("T", [96, 150])
+@pytest.mark.parametrize("T", [96, 140])
 def test_device_that_cannot_run_the_streaming_tensor_core_kernels(B, olmoe_layer, T):
     """Where the device refuses these kernels their shared memory or registers, the other tensor-core kernels take the call
     (with the rows in their own order), on both sides of 1024 pairs; nothing is combined from an earlier call's buffers."""
@@ -527,5 +527,27 @@ def test_device_that_cannot_run_the_streaming_tensor_core_kernels(B, olmoe_layer
     cache.refuse_tensor_stream(False)
     out = cache.forward(0, hidden.flip(0).contiguous().cuda(), ids.cuda(), p.cuda())
     assert cache.last_tensor_kernels() == B.TENSOR_STREAM and torch.equal(out.view(torch.int16), first.view(torch.int16))
+    assert cache.status() == 0
+    cache.close()
+
+
+@pytest.mark.parametrize("shape, T, kind", [
+    (synth.OLMOE, 96, "STREAM"),                                                 # the first call behind the streaming kernels
+    (synth.OLMOE, 128, "STREAM"), (synth.OLMOE, 129, "STREAM"), (synth.OLMOE, 144, "STREAM"), (synth.OLMOE, 145, "ROWS256"),
+    (synth.Shape(2048, 1408, 60, 4), 256, "STREAM"), (synth.Shape(2048, 1408, 60, 4), 257, "ROWS256"),
+    (synth.Shape(2560, 1280, 40, 4), 240, "STREAM"), (synth.Shape(2560, 1280, 40, 4), 241, "ROWS64"),     # 24 rows per expert, one more pair each
+    (synth.Shape(1920, 1408, 60, 4), 200, "ROWS64"),                             # d_model
+    (synth.Shape(2048, 640, 92, 4), 200, "ROWS64"), (synth.Shape(2048, 640, 93, 4), 200, "STREAM")])       # 99.5 and 100.5 blocks per SM
+def test_range_of_the_streaming_tensor_core_kernels(B, shape, T, kind):
+    """Which tensor-core kernels take a call, at the edges of the rule; rounding apart, both give the same rows."""
+    bank = B.pack_bank(shape, *synth.expert_weights(shape, 4300, device="cuda"))
+    cache = B.Cache(shape, [bank], shape.num_experts, max_tokens=T)
+    hidden, ids, p = (x.cuda() for x in helpers.routed_inputs(shape, T, seed=4310 + T, alpha=1.0))
+    out = cache.forward(0, hidden, ids, p).float()
+    assert cache.last_tensor_kernels() == getattr(B, "TENSOR_" + kind)
+    cache.refuse_tensor_stream()
+    other = cache.forward(0, hidden, ids, p).float()
+    assert cache.last_tensor_kernels() != B.TENSOR_STREAM
+    assert torch.linalg.norm(out - other) <= 2 * helpers.REL_FRO * torch.linalg.norm(other)      # each within REL_FRO of the oracle
     assert cache.status() == 0
     cache.close()
