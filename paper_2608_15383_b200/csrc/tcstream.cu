@@ -2,7 +2,7 @@
 // expert, where the bound is the stream of packed bytes and the tensor cores are fed straight from it.
 //
 // As in the large-row kernels the weights are the UMMA A operand (128 rows = 8 panels) and the tokens the B operand, but
-//   - A is the CODES, q = u - 8 as BF16 (exact, 11 instructions per eight codes against 19 with the scale multiplied in),
+//   - A is the CODES, (u - 8) x 2^-10 as BF16 (exact, 11 instructions per eight codes against 19 with the scale multiplied in),
 //     in TENSOR MEMORY: written by tcgen05.st.16x128b, which hands a lane the cells of its fragment-ordered codes;
 //   - every 128-wide block gets an accumulator of its own, and the drain warps add scale x accumulator to binary32 sums in
 //     registers: the weights are not rounded to BF16;
@@ -129,15 +129,18 @@ __device__ __forceinline__ void tma_load_at(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
         : "memory");
 }
-// eight codes of one word -> (q, q') pairs as BF16, K order
+// eight codes of one word -> (q, q') x 2^-10 pairs as BF16, K order.  A block's sum of 128 products is then no larger than its
+// largest activation, whatever the codes are, so that what the scaled sum can hold the accumulator can hold too; the drain's scales
+// give the 2^10 back.  (Codes as integers overflowed from activations of 3e35 on.)
+constexpr float kCodeUnit = 1024.f;
 __device__ __forceinline__ void codes_bf16(uint32_t w, uint32_t (&out)[4]) {
-    uint32_t bias = 0x43084308u;                                   // BF16 136 twice
+    uint32_t bias = 0x3e083e08u;                                   // BF16 136 x 2^-10 twice
     const __nv_bfloat162 b2 = *reinterpret_cast<__nv_bfloat162*>(&bias);
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
         uint32_t v;
-        asm("lop3.b32 %0, %1, 0x000f000f, 0x43004300, 0xea;" : "=r"(v) : "r"(w >> (4 * s)));   // (128+u, 128+u')
-        const __nv_bfloat162 q2 = __hsub2(*reinterpret_cast<__nv_bfloat162*>(&v), b2);         // exact small integers
+        asm("lop3.b32 %0, %1, 0x000f000f, 0x3e003e00, 0xea;" : "=r"(v) : "r"(w >> (4 * s)));   // (128+u, 128+u') x 2^-10
+        const __nv_bfloat162 q2 = __hsub2(*reinterpret_cast<__nv_bfloat162*>(&v), b2);         // exact: integers of 2^-10
         out[s] = *reinterpret_cast<const uint32_t*>(&q2);
     }
 }
@@ -403,7 +406,7 @@ tc_stream_kernel(const TcStreamArgs a, const CUtensorMap* __restrict__ maps, __n
                 for (int u = 0; u < AHEAD; ++u) {
                     const int kb = kb0 + u;
                     if (kb >= KB) break;
-                    const float s = __half2float(__ushort_as_half(sc[u]));
+                    const float s = __half2float(__ushort_as_half(sc[u])) * kCodeUnit;     // exact
                     if (kb + AHEAD < KB) sc[u] = __ldg(reinterpret_cast<const unsigned short*>(sp + (size_t)(kb + AHEAD) * kBlockBytes));
                     ok = mbar_wait_warp(done_a + 8 * sg, ph, abort_flag, a.status);
                     if (!ok) break;

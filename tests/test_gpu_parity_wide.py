@@ -551,3 +551,26 @@ def test_range_of_the_streaming_tensor_core_kernels(B, shape, T, kind):
     assert torch.linalg.norm(out - other) <= 2 * helpers.REL_FRO * torch.linalg.norm(other)      # each within REL_FRO of the oracle
     assert cache.status() == 0
     cache.close()
+
+
+def test_streaming_tensor_core_kernels_with_large_activations(B):
+    """Activations up to binary32's end in one block of 128: the block's sum of code x activation must not overflow where the
+    layer's own values do not (up values near 1e37, gates near 1, outputs near 1e36)."""
+    s = synth.Shape(d_model=2048, d_ff=1024, num_experts=64, top_k=8)
+    wg, wu, wd = synth.expert_weights(s, 4400)
+    wg[:, :, 128:] = 0                                   # gates read the first block, up projections the second
+    wu[:, :, :128] = 0
+    wu[:, :, 256:] = 0
+    ora, bank = helpers.OracleLayer(s, wg, wu, wd), B.pack_bank(s, wg, wu, wd)
+    T = 100
+    hidden, ids, p = helpers.routed_inputs(s, T, seed=4410)
+    hidden[:, 128:256] = (hidden[:, 128:256].float().clamp(-3, 3) * 1e38).to(torch.bfloat16)
+    cache = B.Cache(s, [bank], 64, max_tokens=T)
+    out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    assert cache.last_tensor_kernels() == B.TENSOR_STREAM
+    sample = list(range(0, T, 9))
+    y, ref = ora.forward(hidden[sample], ids[sample], p[sample])
+    assert 1e35 < abs(ref).max() < 3e38
+    helpers.check_output(out[sample], y, ref, "activations of 3e38")
+    assert cache.status() == 0
+    cache.close()
