@@ -277,6 +277,10 @@ int launch_dependent(F kern, int ctas, int cluster, size_t smem, const exmoe_sha
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     lc.attrs = attr;
     lc.numAttrs = cluster > 1 ? 2 : 1;
+#ifdef EXMOE_DISABLE_PDL
+    lc.attrs = attr + 1;
+    --lc.numAttrs;
+#endif
     if (cudaLaunchKernelEx(&lc, kern, hidden, w, bias, T, s.d_model, s.num_experts, s.top_k, ids, wts) != cudaSuccess) {
         cudaGetLastError();
         return EXMOE_ERR_CUDA;

@@ -638,6 +638,9 @@ bool launch_stream_cfg(const GemmArgs& a, const __nv_bfloat16* x, __nv_bfloat16*
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = dependent ? 1 : 0;
+#ifdef EXMOE_DISABLE_PDL
+    lc.numAttrs = 0;
+#endif
     cudaLaunchKernelEx(&lc, kern, p);
     count_launch();
     return true;

@@ -581,6 +581,9 @@ bool launch_tc_stream(const TcStreamArgs& a, const CUtensorMap* maps, __nv_bfloa
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = 1;
+#ifdef EXMOE_DISABLE_PDL
+    lc.numAttrs = 0;
+#endif
     if (cudaLaunchKernelEx(&lc, tc_stream_kernel<GATEUP>, a, maps, act, topk_w, y) != cudaSuccess) return false;
     count_launch();
     return true;

@@ -84,3 +84,14 @@ def test_kernels_of_many_ctas_keep_the_next_one_out():
         end = text[name].index("\n}\n", start)
         body = text[name][start:end]
         assert "grid_dependency_wait();" in body and "grid_launch_dependents" not in body, kernel
+
+
+def test_every_programmatic_launch_can_be_switched_off():
+    """-DEXMOE_DISABLE_PDL is for timing without programmatic launches: every launcher that asks for one honours it."""
+    found = 0
+    for name, text in sources():
+        for m in re.finditer(r"programmaticStreamSerializationAllowed = 1;", text):
+            launch = text[m.end():text.index("cudaLaunchKernelEx(", m.end())]
+            assert "#ifdef EXMOE_DISABLE_PDL" in launch, (name, text[:m.start()].count("\n") + 1)
+            found += 1
+    assert found >= 8
