@@ -80,9 +80,15 @@ def test_small_n_tensor_core_kernels_at_olmoe_shape(B, olmoe_layer, T):
     hidden, ids, p = helpers.routed_inputs(s, T, seed=7100 + T, alpha=1.0)
     y, ref = ora.forward(hidden, ids, p)
     cache = B.Cache(s, [bank], 64, max_tokens=T)
+    cache.refuse_tensor_stream()                          # they take these calls where the device can run them
     out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
     assert cache.last_path() == B.PATH_TENSOR_SMALL_N
+    assert cache.last_tensor_kernels() == B.TENSOR_ROWS64
     helpers.check_output(out, y, ref, f"T={T}")
+    cache.refuse_tensor_stream(False)
+    out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    assert cache.last_path() == B.PATH_TENSOR_SMALL_N and cache.last_tensor_kernels() == B.TENSOR_STREAM
+    helpers.check_output(out, y, ref, f"T={T}, streaming tensor-core kernels")
     assert cache.status() == 0
     cache.close()
 
@@ -188,6 +194,8 @@ def test_no_kernel_writes_outside_its_buffers(B, case):
                       "streaming": (40, 6, 0, B.PATH_STREAM), "tensor small-N": (200, 6, 3, B.PATH_TENSOR_SMALL_N),
                       "tensor large-N": (300, 16, 0, B.PATH_TENSOR), "chunked grouping": (700, 6, 0, B.PATH_TENSOR),
                       "host copies": (40, 5, 2, B.PATH_STREAM), "prefetch": (3, 8, 0, None)}[case]
+    if case == "chunked grouping":                           # beyond 8192 pairs: fewer are grouped together with the row copy
+        T = 2100
     cache = B.Cache(s, [bank], C, max_tokens=T, wave_cap=Cw, guard_bytes=1 << 16)
     if case == "host copies":
         cache.set_miss_path(B.MISS_HOST_COPIES)
@@ -202,6 +210,26 @@ def test_no_kernel_writes_outside_its_buffers(B, case):
         assert cache.last_path() == want
     assert cache.guards_intact() and out_guards_intact(whole, first, last)
     helpers.check_output(out, y, ref, case)
+    assert cache.status() == 0
+    cache.close()
+
+
+@pytest.mark.parametrize("slots, wave_cap", [(64, 0), (20, 7)])
+def test_streaming_tensor_core_kernels_write_only_their_buffers(B, olmoe_layer, slots, wave_cap):
+    """The same margins around the streaming tensor-core kernels, which the small shape above does not reach: one wave and several,
+    with the rows of the last token in the buffers' last rows."""
+    ora, bank = olmoe_layer
+    s, T = synth.OLMOE, 101
+    cache = B.Cache(s, [bank], slots, max_tokens=T, wave_cap=wave_cap, guard_bytes=1 << 16)
+    hidden, ids, p = helpers.routed_inputs(s, T, seed=9350, alpha=1.0)
+    out, whole, first, last = guarded_out(T, s.d_model)
+    for _ in range(2):
+        cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda(), out=out)
+    assert cache.last_tensor_kernels() == B.TENSOR_STREAM
+    assert cache.guards_intact() and out_guards_intact(whole, first, last)
+    sample = list(range(0, T, 5))
+    y, ref = ora.forward(hidden[sample], ids[sample], p[sample])
+    helpers.check_output(out[sample], y, ref, f"{slots} slots")
     assert cache.status() == 0
     cache.close()
 
@@ -266,10 +294,12 @@ def test_graph_replay_of_the_larger_paths_is_bit_identical_to_plain_launches(B, 
     _, bank = olmoe_layer
     s = synth.OLMOE
     cache = B.Cache(s, [bank], 64, max_tokens=T)
+    cache.refuse_tensor_stream()                          # T = 128: the 64-row shape; the kernels that it stands in for are below
     inputs = [tuple(x.cuda() for x in helpers.routed_inputs(s, T, seed=8800 + T + i, alpha=0.5)) for i in range(2)]
     plain = [cache.forward(0, h, i, w).clone() for h, i, w in inputs]
     want = {16: B.PATH_STREAM, 128: B.PATH_TENSOR_SMALL_N, 2048: B.PATH_TENSOR}[T]
     assert cache.last_path() == want
+    assert T == 16 or cache.last_tensor_kernels() == (B.TENSOR_ROWS64 if T == 128 else B.TENSOR_ROWS256)
     outs = [torch.zeros_like(plain[0]) for _ in inputs]
     stream = torch.cuda.Stream()
     stream.wait_stream(torch.cuda.current_stream())
@@ -285,6 +315,36 @@ def test_graph_replay_of_the_larger_paths_is_bit_identical_to_plain_launches(B, 
         stream.synchronize()
         for o, p in zip(outs, plain):
             assert torch.equal(o.view(torch.int16), p.view(torch.int16)), f"T={T} replay {rep}"
+    assert cache.status() == 0
+    cache.close()
+
+
+@pytest.mark.parametrize("T", [100, 140])
+def test_graph_replay_of_the_streaming_tensor_core_kernels(B, olmoe_layer, T):
+    """The same for the streaming tensor-core kernels, on both sides of 1024 pairs: two layer calls per graph, replayed on rows
+    and routing that change between the replays."""
+    _, bank = olmoe_layer
+    s = synth.OLMOE
+    cache = B.Cache(s, [bank, bank], 64, max_tokens=T)
+    inputs = [tuple(x.cuda() for x in helpers.routed_inputs(s, T, seed=8900 + T + i, alpha=0.5)) for i in range(3)]
+    plain = [[cache.forward(l, *x).clone() for l in range(2)] for x in inputs]
+    assert cache.last_tensor_kernels() == B.TENSOR_STREAM
+    held, outs = [x.clone() for x in inputs[0]], [torch.zeros_like(plain[0][0]) for _ in range(2)]
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        for l in range(2):
+            cache.forward(l, *held, out=outs[l], stream=stream)
+    for i in (1, 2, 0):
+        for x, y in zip(held, inputs[i]):
+            x.copy_(y)
+        stream.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(stream):
+            g.replay()
+        stream.synchronize()
+        for o, p in zip(outs, plain[i]):
+            assert torch.equal(o.view(torch.int16), p.view(torch.int16)), i
     assert cache.status() == 0
     cache.close()
 
@@ -493,6 +553,7 @@ def test_streaming_tensor_core_kernels_at_tile_edges(B):
     cache = B.Cache(s, [bank], 48, max_tokens=T)
     out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
     assert cache.last_path() == B.PATH_TENSOR_SMALL_N and cache.status() == 0
+    assert cache.last_tensor_kernels() == B.TENSOR_STREAM
     sample = set()
     for e in range(48):
         rows = (ids[:, 0] == e).nonzero()[:, 0].tolist()
@@ -506,6 +567,78 @@ def test_streaming_tensor_core_kernels_at_tile_edges(B):
     again = part.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
     assert torch.equal(out.view(torch.int16), again.view(torch.int16)) and part.status() == 0
     part.close()
+    for miss in (B.MISS_DEVICE_FETCH, B.MISS_HOST_COPIES):         # 18 experts fit 20 slots: several waves need a smaller cap
+        part = B.Cache(s, [bank], 20, max_tokens=T, wave_cap=7)
+        part.set_miss_path(miss)
+        again = part.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+        assert part.last_tensor_kernels() == B.TENSOR_STREAM and part.last_plan(0, T)["n_waves"] == 3
+        assert torch.equal(out.view(torch.int16), again.view(torch.int16)) and part.status() == 0
+        part.close()
+
+
+def test_streaming_tensor_core_kernels_with_more_tiles_than_they_list(B):
+    """A CTA keeps the first 128 entries of the tile list in shared memory and reads the rest past L1: 160 experts with rows."""
+    s = synth.Shape(d_model=2048, d_ff=512, num_experts=160, top_k=1)
+    ora, bank = helpers.make_layer(s, seed=4500)
+    T = 900
+    ids = (torch.arange(T, dtype=torch.int32) * 7 % 160)[torch.randperm(T, generator=torch.Generator().manual_seed(3))].view(T, 1).contiguous()
+    hidden = synth.hidden_states(s, T, seed=4510)
+    p = torch.rand((T, 1), generator=torch.Generator().manual_seed(4)) + 0.5
+    cache = B.Cache(s, [bank], 160, max_tokens=T)
+    out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    assert cache.last_tensor_kernels() == B.TENSOR_STREAM and (cache.last_plan(0, T)["counts"] > 0).sum() == 160
+    sample = [int((ids[:, 0] == e).nonzero()[0]) for e in range(160)]
+    y, ref = ora.forward(hidden[sample], ids[sample], p[sample])
+    helpers.check_output(out[sample], y, ref, "a row of every expert")
+    assert cache.status() == 0
+    cache.close()
+
+
+@pytest.mark.parametrize("slots", [64, 20])
+def test_streaming_tensor_core_kernels_with_invalid_ids(B, olmoe_layer, slots):
+    """Pairs with an id outside the experts add nothing and are reported; a call without any valid id gives zeros, and the next
+    good call is right again."""
+    ora, bank = olmoe_layer
+    s, T = synth.OLMOE, 100
+    hidden, ids, p = helpers.routed_inputs(s, T, seed=4600, alpha=0.5)
+    bad = ids.clone()
+    bad[::3, 2], bad[1::7, 5], bad[50] = -1, 64, 1 << 30
+    cache = B.Cache(s, [bank], slots, max_tokens=T)
+    sample = list(range(0, T, 10)) + [1, 49, 51, 99]
+    for what in (bad, torch.full_like(ids, -7), ids):
+        out = cache.forward(0, hidden.cuda(), what.cuda(), p.cuda())
+        assert cache.last_tensor_kernels() == B.TENSOR_STREAM
+        assert cache.status() == (0 if what is ids else B.EXMOE_ERR_BAD_EXPERT_ID)
+        y, ref = ora.forward(hidden[sample], what[sample], p[sample])
+        if (what == -7).all():
+            assert not out.any()
+        else:
+            helpers.check_output(out[sample], y, ref, "ids")
+            assert not (what is bad and out[50].any())
+    cache.close()
+
+
+@pytest.mark.parametrize("slots", [16, 6])
+def test_chunked_grouping_after_a_call_with_an_invalid_id(B, slots):
+    """More than 8192 pairs: the arrival counter and the bad-id word of the chunked grouping are ready again for the next call, and
+    neither keeps what an earlier call found, with the experts resident or not."""
+    s, T = synth.MID, 2100
+    _, bank = helpers.make_layer(s, seed=5)
+    hidden, ids, p = (x.cuda() for x in helpers.routed_inputs(s, T, seed=4700, alpha=0.5))
+    bad = ids.clone()
+    bad[T - 1, 3] = 16
+    fresh = B.Cache(s, [bank], slots, max_tokens=T)
+    good = fresh.forward(0, hidden, ids, p)
+    cache = B.Cache(s, [bank], slots, max_tokens=T)
+    for what in (bad, ids, bad, bad, ids):
+        out = cache.forward(0, hidden, what, p)
+        assert cache.status() == (0 if what is ids else B.EXMOE_ERR_BAD_EXPERT_ID)
+        plan = cache.last_plan(0, ids.numel())
+        assert plan["counts"].sum() == ids.numel() - (what is bad)
+        assert torch.equal(out[:-1].view(torch.int16), good[:-1].view(torch.int16))
+        assert torch.equal(out[-1].view(torch.int16), good[-1].view(torch.int16)) == (what is ids)
+    fresh.close()
+    cache.close()
 
 
 @pytest.mark.parametrize("T", [96, 140])
