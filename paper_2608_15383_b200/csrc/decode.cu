@@ -1183,10 +1183,9 @@ void launch_decode(const GemmArgs& a, const SmallArgs& sa, const __nv_bfloat16* 
 }
 
 // out[t] = bf16( sum_{j=0..k-1} Y[t*k + j] ), binary32, fixed order; pairs with an invalid id add nothing.
-// A thread requests AHEAD rows before it adds the first.  (With every load behind the id and the addition of the one before it,
-// OLMoE-shaped layers: 5 tokens 27.6 us, now 26.3; 16 tokens 41.7, now 39.6; the kernel alone 2.4 us, now 1.6.)  Eight while the
-// threads are few and the time is latency; four where they fill the chip several times over: the kernel alone at 2048 and
-// 8192 tokens 25.8 and 101.5 us before, 28.6 and 119 with eight, 24.2 and 90.6 (6.3 TB/s) with four.
+// A thread requests AHEAD rows before it adds the first: with every load behind the id and the addition of the one before it, an
+// OLMoE-shaped layer of 16 tokens took 41.7 us and not 39.6.  More rows in flight take registers and with them threads of an SM, so
+// eight only where the threads are few (launch_combine).
 template <int AHEAD>
 __global__ void __launch_bounds__(256)
 combine_kernel(const float* y, const int32_t* __restrict__ ids, int E, int T, int k, int H,
@@ -1215,7 +1214,7 @@ combine_kernel(const float* y, const int32_t* __restrict__ ids, int E, int T, in
         float4 v[AHEAD];
 #pragma unroll
         for (int j = 0; j < AHEAD; ++j)
-            if (valid[j]) v[j] = load_behind_wait(row + (size_t)(j0 + j) * per_row);
+            if (valid[j]) v[j] = row[(size_t)(j0 + j) * per_row];
 #pragma unroll
         for (int j = 0; j < AHEAD; ++j)
             if (valid[j]) {
@@ -1231,8 +1230,16 @@ combine_kernel(const float* y, const int32_t* __restrict__ ids, int E, int T, in
 
 }  // namespace
 
-// about what the chip holds at once: 148 SMs x 2048 threads (592 tokens of d_model 2048)
-constexpr long long kCombineFewThreads = 148 * 2048;
+// Rows requested together, by the rows of a token and by the threads (a quarter of the output's values).  The kernel alone, us, one after
+// the other as at first / two / four / eight:
+//   d_model 2048, top-8:   16 tokens 2.4 / 1.9 / 1.7 / 1.6    200 (102 k threads) 3.6 / 3.2 / 2.6 / 2.4    333 (170 k) 4.3 / 3.9 / 3.0 / 3.5
+//                          592 4.1 / 3.8 / 4.1 / 5.2    2048 25.1 / 23.4 / 22.7 / 25.0    8192 88.9 / 84.2 / 83.1 / 91.5
+//   d_model 2048, top-4:   24 tokens 1.8 / 1.5 / 1.3 / 1.4    400 3.0 / 2.6 / 2.2 / 3.4    2000 8.3 / 7.7 / 7.4 / 13.2
+//   d_model 1024, top-2:   13 tokens 1.4 / 1.2 / 1.2 / 1.4    1000 2.4 / 2.0 / 2.4 / 3.8    d_model 2048, 4000 10.8 / 10.6 / 12.6 / 24.6
+//   d_model 896, top-5:    400 tokens (90 k) 3.2 / 2.9 / 2.6 / 2.1    1000 (224 k) 3.5 / 3.1 / 2.8 / 3.6
+constexpr long long kCombineFewThreads = 1 << 17;
+constexpr int combine_ahead(int k, long long threads) { return k <= 2 ? 2 : k >= 5 && threads <= kCombineFewThreads ? 8 : 4; }
+static_assert(combine_ahead(2, 16) == 2 && combine_ahead(3, 16) == 4 && combine_ahead(8, 128 * 1024) == 8 && combine_ahead(8, 128 * 1024 + 1) == 4);
 void launch_combine(const float* y, const int32_t* ids, int E, int T, int k, int H, __nv_bfloat16* out,
                     cudaStream_t st) {
     const long long n = (long long)T * (H / 4);
@@ -1248,7 +1255,8 @@ void launch_combine(const float* y, const int32_t* ids, int E, int T, int k, int
 #ifdef EXMOE_DISABLE_PDL
     lc.numAttrs = 0;
 #endif
-    cudaLaunchKernelEx(&lc, n <= kCombineFewThreads ? combine_kernel<8> : combine_kernel<4>, y, ids, E, T, k, H, out);
+    const int ahead = combine_ahead(k, n);
+    cudaLaunchKernelEx(&lc, ahead == 2 ? combine_kernel<2> : ahead == 4 ? combine_kernel<4> : combine_kernel<8>, y, ids, E, T, k, H, out);
     count_launch();
 }
 

@@ -94,11 +94,6 @@ __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepco
 // compiler takes for read-only may move in front of the wait), and where many such loads are issued together, these.  It may
 // stand where the data are complete before the kernel starts: weights, a router's matrix and bias, tensor maps; and what the kernels
 // in front of a down or a combine kernel have waited for before they let it start (ids, routing weights).
-__device__ __forceinline__ float4 load_behind_wait(const float4* p) {
-    float4 v;
-    asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
-    return v;
-}
 __device__ __forceinline__ int4 load_behind_wait_cg(const int4* p) {       // past L1
     int4 v;
     asm volatile("ld.global.cg.v4.s32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");

@@ -707,3 +707,21 @@ def test_streaming_tensor_core_kernels_with_large_activations(B):
     helpers.check_output(out[sample], y, ref, "activations of 3e38")
     assert cache.status() == 0
     cache.close()
+
+
+@pytest.mark.parametrize("k, T", [(1, 300), (2, 300), (3, 61), (3, 300), (5, 256), (5, 257), (8, 256), (8, 257), (11, 130), (11, 300)])
+def test_combine_with_its_rows_requested_ahead(B, k, T):
+    """Two, four and eight rows requested together, by top_k and on both sides of 131,072 threads (256 tokens of d_model 2048), where
+    top_k is less than that, equal, and no multiple; some pairs without a valid id."""
+    s = synth.Shape(d_model=2048, d_ff=128, num_experts=16, top_k=k)
+    ora, bank = helpers.make_layer(s, seed=4800 + k)
+    hidden, ids, p = helpers.routed_inputs(s, T, seed=4810 + T)
+    ids[T // 2, k - 1] = -1
+    ids[T - 1, 0] = 16
+    cache = B.Cache(s, [bank], 16, max_tokens=T)
+    out = cache.forward(0, hidden.cuda(), ids.cuda(), p.cuda())
+    sample = sorted({0, 1, T // 2, T // 2 + 1, T - 2, T - 1} | set(range(0, T, 37)))
+    y, ref = ora.forward(hidden[sample], ids[sample], p[sample])
+    helpers.check_output(out[sample], y, ref, f"top-{k}, {T} tokens")
+    assert cache.status() == B.EXMOE_ERR_BAD_EXPERT_ID
+    cache.close()
