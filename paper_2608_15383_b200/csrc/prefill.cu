@@ -599,8 +599,11 @@ __device__ void build_tile_list(const int32_t* counts, const int32_t* offsets, c
             s_weight[warp] = incl_w;
         }
         __syncthreads();
+        // over the warps that have groups only: each step is a read from shared memory that the next one waits for (8 groups, all 32
+        // warps: 1.0 us more of a layer's latency)
+        const int live = min(nwarp, (ng - base + 31) >> 5);
         int wbase = 0, total = 0, wbase_w = 0, total_w = 0;
-        for (int w = 0; w < nwarp; ++w) {
+        for (int w = 0; w < live; ++w) {
             if (w < warp) {
                 wbase += s_warp[w];
                 wbase_w += s_weight[w];
