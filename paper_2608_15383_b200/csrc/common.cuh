@@ -190,7 +190,7 @@ bool tc_stream_runs();
 // 144 tokens (an expert has no more rows than that).  Of the other kernels' time, routing uniform / Zipf 0.5 / 1.0 / 1.25 / 1.5, means
 // of four routings:
 //   64 experts of 2048 x 1024, top-8: 100 tokens 0.82 / 0.81 / 0.87 / 0.89 / 1.02    128: 0.87 / 0.81 / 0.91 / 0.93 / 0.94    144: 0.86 / 0.87 / 0.92 / 0.98 / 1.00
-//                                     160: 0.87 / 0.88 / 0.94 / 0.99 / 1.02 (not taken)   192: 0.86 / 0.88 / 0.91 / 1.02 / 1.03 (not taken)   top-6, 192: Zipf 1.5 1.10 (not taken)
+//                                     160: 0.87 / 0.88 / 0.94 / 0.99 / 1.02 (not taken)   192: 0.86 / 0.88 / 0.91 / 1.02 / 1.03 (not taken)   top-6, 192 tokens: 1.10 at Zipf 1.5 (not taken)
 //   60 of 2048 x 1408, top-4: 170 tokens 0.78 / 0.83 / 0.86 / 0.93 / 0.92    256: 0.83 / 0.82 / 0.88 / 0.91 / 0.98    300: 0.83 / 0.85 / 0.92 / - / 1.17 (not taken)
 //   96 of 4096 x 512, top-2: 400 tokens 0.79 / 0.84 / 0.95 / 0.87 / 1.04    1150: 0.85 / 0.89 / 1.01 / - / 1.19 (not taken)
 //   48 of 2304 x 1536, top-2: 500 tokens 0.84 / 0.82 / 0.89 / 0.94 / 0.93    570: 0.83 / 0.89 / 0.98 / - / 1.27 (not taken)

@@ -687,7 +687,7 @@ gather_rows_kernel(const __nv_bfloat16* hidden, const int32_t* perm,
 }
 
 // Grouping and the grouped copy of the hidden rows in ONE launch, for calls of up to kPlanGatherPairs pairs.  Alone the
-// grouping kernels are latency (one CTA: 11 us at 1024 pairs; count, arrival counter and scatter: 11 us and a memset),
+// grouping kernels are latency (one CTA: 11 us at 1024 pairs; count, arrival counter and scatter: 11 us),
 // so here every CTA counts ALL pairs itself - one shared-memory atomic per pair, in whose low half the key's pairs are
 // counted and in whose high half those in front of the CTA's own segment - and needs no other CTA to place the rows of its
 // segment.  The last CTA takes no segment; it publishes the plan and, for a call of one wave, the tile list.

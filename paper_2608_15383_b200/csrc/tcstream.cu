@@ -9,10 +9,12 @@
 //   - the packed bytes come through a ring of bulk copies, 135 KB deep, in copies of two blocks (eight copies of one block per A
 //     block took the issuing warp 480 cycles, more than HBM needs for the block).
 // With A in shared memory a 128 x 128 block costs 256 cycles of stores and 256 of operand reads of the 128 B per clock that the
-// shared memory moves, next to the tokens' 100 to 200, and an MMA of 16 rows 40 cycles; with A in tensor memory the MMAs take N / 2
-// cycles down to 10 (alone), and a block with 16 rows 450 to 500 here against 1000.  Bound: instruction issue, 0.74 per cycle and
-// scheduler (codes 40 %, waits and polls 25 %); HBM would deliver a block every 377 cycles.  OLMoE-shaped layer, uniform routing /
-// Zipf 0.5: 100 tokens 97 -> 77 / 105 -> 83 us, 150 tokens 100 -> 86 / 102 -> 90.
+// shared memory moves, next to the tokens' 100 to 200; with A in tensor memory the weights touch it once, as packed bytes.  A block
+// takes 617 / 524 cycles (gate/up / down) with 16 rows against 893 / 851 in the other tensor-core kernels, 773 / 989 against
+// 972 / 1003 with 64; HBM would deliver one every 377.  Bound: instructions, 1,700 of a warp per block, 0.62 issued per cycle and
+// scheduler (43 % of them on the ALU pipe, 28 % on the FMA pipe); the split leaves the compiler 72 registers: it spills 12 bytes
+// (gate/up) and 36 (down).  OLMoE-shaped layer, uniform routing / Zipf 0.5: 100 tokens 94 -> 78 /
+// 102 -> 82 us, 128 tokens 95 -> 82 / 103 -> 84.
 // Built and no faster: eight conversion warps of two panels, sixteen of one; a barrier per A block, accumulator and token slot
 // (1,800 cycles per 128 of K); barrier waits with a suspend hint (+3 %) or in tight loops (+4 %); 16x256b stores (+2 %).
 //
@@ -77,8 +79,7 @@ __device__ __forceinline__ void tc_mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// 16 lanes x 32 columns: lane (q, c) gives, for i = 0..7, column 4i + c: r[2i] = row q, r[2i+1] = row q + 8 (124 B per clock and
-// subpartition; 16x256b, 64)
+// 16 lanes x 32 columns: lane (q, c) gives, for i = 0..7, column 4i + c: r[2i] = row q, r[2i+1] = row q + 8
 __device__ __forceinline__ void tc_st_16x128b_x8(uint32_t taddr, const uint32_t (&r)[16]) {
     asm volatile("tcgen05.st.sync.aligned.16x128b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
                  ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
